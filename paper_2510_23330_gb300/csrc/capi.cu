@@ -77,19 +77,17 @@ static void free_particles(gnb_ctx *c)
 
 static void free_gas(gnb_ctx *c)
 {
-    void *all[] = {c->gslot, c->gkey, c->gcx, c->gcy, c->gcz, c->ggrank, c->grx, c->gry, c->grz, c->gx, c->gy,
-                   c->gz, c->gm, c->gvx, c->gvy, c->gvz, c->gu, c->gh2, c->gh, c->g64, c->grho, c->gP, c->gcs,
+    void *all[] = {c->gslot, c->gkey, c->ggrank, c->gx, c->gy, c->gz, c->gvx, c->gvy, c->gvz, c->gu, c->gh2, c->gh, c->g64, c->grho, c->gP, c->gcs,
                    c->gRprev, c->gE, c->nbr, c->nd2, c->mut, c->rcnt, c->roff, c->rfill, c->rlist, c->hax,
-                   c->hay, c->haz, c->hdu, c->kflag, c->kR, c->kRb, c->kitem, c->gvsig, c->kwl[0], c->kwl[1],
+                   c->hay, c->haz, c->hdu, c->kR, c->kitem, c->gvsig,
                    c->gh2lo, c->gh2hi, c->fC, c->fR, c->fV, c->fQ};
     for (void *q : all) dfree(c, q);
-    c->gslot = nullptr; c->gkey = nullptr; c->gcx = c->gcy = c->gcz = c->ggrank = nullptr;
-    c->grx = c->gry = c->grz = nullptr; c->gx = c->gy = c->gz = nullptr;
-    c->gm = c->gvx = c->gvy = c->gvz = c->gu = nullptr; c->gh2 = nullptr; c->gh = nullptr; c->g64 = nullptr;
+    c->gslot = nullptr; c->gkey = nullptr; c->ggrank = nullptr;
+    c->gx = c->gy = c->gz = nullptr;
+    c->gvx = c->gvy = c->gvz = c->gu = nullptr; c->gh2 = nullptr; c->gh = nullptr; c->g64 = nullptr;
     c->grho = c->gP = c->gcs = c->gRprev = c->gE = nullptr; c->nbr = nullptr; c->nd2 = nullptr; c->mut = nullptr;
     c->rcnt = c->roff = c->rfill = c->rlist = nullptr; c->hax = c->hay = c->haz = c->hdu = nullptr;
-    c->kflag = nullptr; c->kR = nullptr; c->kRb = nullptr; c->kitem = nullptr; c->gvsig = nullptr;
-    c->kwl[0] = c->kwl[1] = nullptr;
+    c->kR = nullptr; c->kitem = nullptr; c->gvsig = nullptr;
     c->gh2lo = c->gh2hi = nullptr;
     c->fC = nullptr; c->fR = nullptr; c->fV = nullptr; c->fQ = nullptr;
     tree_free(c, c->gt);
@@ -125,11 +123,9 @@ static int alloc_gas(gnb_ctx *c, int64_t ng)
     free_gas(c);
     size_t G = (size_t)(ng > 0 ? ng : 1);
     GNB_TRY(dalloc(c, &c->gslot, G)); GNB_TRY(dalloc(c, &c->gkey, G));
-    GNB_TRY(dalloc(c, &c->gcx, G)); GNB_TRY(dalloc(c, &c->gcy, G)); GNB_TRY(dalloc(c, &c->gcz, G));
     GNB_TRY(dalloc(c, &c->ggrank, G));
-    GNB_TRY(dalloc(c, &c->grx, G)); GNB_TRY(dalloc(c, &c->gry, G)); GNB_TRY(dalloc(c, &c->grz, G));
     GNB_TRY(dalloc(c, &c->gx, G)); GNB_TRY(dalloc(c, &c->gy, G)); GNB_TRY(dalloc(c, &c->gz, G));
-    GNB_TRY(dalloc(c, &c->gm, G)); GNB_TRY(dalloc(c, &c->gvx, G)); GNB_TRY(dalloc(c, &c->gvy, G));
+    GNB_TRY(dalloc(c, &c->gvx, G)); GNB_TRY(dalloc(c, &c->gvy, G));
     GNB_TRY(dalloc(c, &c->gvz, G)); GNB_TRY(dalloc(c, &c->gu, G));
     GNB_TRY(dalloc(c, &c->gh2, G)); GNB_TRY(dalloc(c, &c->gh, G)); GNB_TRY(dalloc(c, &c->g64, G));
     GNB_TRY(dalloc(c, &c->grho, G)); GNB_TRY(dalloc(c, &c->gP, G)); GNB_TRY(dalloc(c, &c->gcs, G));
@@ -140,9 +136,7 @@ static int alloc_gas(gnb_ctx *c, int64_t ng)
     cudaMemsetAsync(c->nbr, 0, sizeof(int) * G * 64, c->s);  // list entries are always valid indices
     GNB_TRY(dalloc(c, &c->hax, G)); GNB_TRY(dalloc(c, &c->hay, G)); GNB_TRY(dalloc(c, &c->haz, G));
     GNB_TRY(dalloc(c, &c->hdu, G));
-    GNB_TRY(dalloc(c, &c->kflag, 2 * G + 1)); GNB_TRY(dalloc(c, &c->kR, 2 * G + 1));
-    GNB_TRY(dalloc(c, &c->kRb, 2 * G + 1)); GNB_TRY(dalloc(c, &c->kitem, 2 * G + 1));
-    GNB_TRY(dalloc(c, &c->kwl[0], 2 * G + 1)); GNB_TRY(dalloc(c, &c->kwl[1], 2 * G + 1));
+    GNB_TRY(dalloc(c, &c->kR, G)); GNB_TRY(dalloc(c, &c->kitem, G));
     GNB_TRY(dalloc(c, &c->gh2lo, G)); GNB_TRY(dalloc(c, &c->gh2hi, G));
     GNB_TRY(dalloc(c, &c->fC, G)); GNB_TRY(dalloc(c, &c->fR, G)); GNB_TRY(dalloc(c, &c->fV, G));
     GNB_TRY(dalloc(c, &c->fQ, G));

@@ -127,10 +127,9 @@ struct gnb_ctx {
     int *gas_flag = nullptr, *ngas_d = nullptr;
     uint64_t *gkey = nullptr;
     gnb::Tree gt;                 // hydro tree over gas
-    int *gcx = nullptr, *gcy = nullptr, *gcz = nullptr, *ggrank = nullptr;
-    float *grx = nullptr, *gry = nullptr, *grz = nullptr;
+    int *ggrank = nullptr;
     double *gx = nullptr, *gy = nullptr, *gz = nullptr;
-    float *gm = nullptr, *gvx = nullptr, *gvy = nullptr, *gvz = nullptr, *gu = nullptr;
+    float *gvx = nullptr, *gvy = nullptr, *gvz = nullptr, *gu = nullptr;
     double *gh2 = nullptr;        // exact FP64 d^2 of the n_ngb-th neighbour
     float *gh = nullptr;          // h in FP32
     int *g64 = nullptr;           // gas rank of the n_ngb-th neighbour
@@ -145,18 +144,14 @@ struct gnb_ctx {
     int *rtot_d = nullptr;
     int64_t rlist_cap = 0;
     float *hax = nullptr, *hay = nullptr, *haz = nullptr, *hdu = nullptr;
-    int *kflag = nullptr;         // per hydro group: needs another pass
-    float *kR = nullptr;          // per hydro group search radius
-    float2 *kRb = nullptr;        // per hydro group radius bracket (too small, too large)
-    int2 *kitem = nullptr;        // kNN work items (first, count); groups then split particles
-    int *kwl[2] = {nullptr, nullptr};  // kNN worklists: items a pass hands to the next (ping-pong)
+    float *kR = nullptr;          // kNN work items: starting radius without a previous support
+    int2 *kitem = nullptr;        // kNN work items (first, count)
     float *gh2lo = nullptr, *gh2hi = nullptr;  // h^2 rounded down / up to FP32 (per gas)
-    // per-gas records the hydro force gathers for neighbour j (one pass packs them)
+    // per-gas records the kernel-size search and the hydro force gather for particle j
     int4 *fC = nullptr;           // cell x, y, z, mass bits
-    float4 *fR = nullptr;         // residual x, y, z, 1/h
+    float4 *fR = nullptr;         // residual x, y, z, and 1/h once the force pass packs it
     float4 *fV = nullptr;         // v x, y, z, sound speed
     float4 *fQ = nullptr;         // rho, Y, U, - (pair coefficient U_j Y_i of gW(h_i); see sph.cu)
-    int *kcount_d = nullptr;
 
     // supernova surrogate (surrogate.cu)
     int *sreg = nullptr;          // region of each particle slot (-1: none)

@@ -5,26 +5,37 @@
 // Kernel size: the support h_i of gas particle i is the distance to its
 // n_ngb-th nearest gas neighbour (self included), neighbours ordered by
 // (d^2, gas rank) with d^2 = (dx*dx + dy*dy) + dz*dz in FP64.  The paper
-// iterates a search until it converges; here one CTA per hydro-tree group
-// gathers every gas particle within a search radius R of the group into
-// shared memory, and each warp selects the neighbours of one particle:
-//   1. FP32 distances d from FP32 offsets to the group's reference cell,
+// iterates a search until it converges; here one warp takes a run of
+// consecutive gas particles of one hydro-tree group and gathers every gas
+// particle within a search radius R of the run into its shared memory, then
+// selects the neighbours of one member after another:
+//   1. FP32 distances d from FP32 offsets to the run's reference cell,
 //      with |d - D| <= E(D) = 2^-23 (4 sqrt(3) A' sqrt(D) + 5 D), A' = the
-//      largest offset in the group plus two grid units: each offset carries
+//      largest offset in the run plus two grid units: each offset carries
 //      one rounding (<= 2^-24 A') plus the residual's (<= 2^-24 unit), the
 //      difference and the three fused multiply-adds one rounding each, and
 //      the factor 2 over the first-order bound covers the second-order terms,
-//   2. a 64-bin histogram and an in-bucket rank give the exact 64th smallest
-//      FP32 value t,
+//   2. the candidates within the member's own radius (its previous support
+//      times a margin: about 66 of them) are compacted into a list, and the
+//      few largest removed one by one give the exact 64th smallest FP32
+//      value t,
 //   3. entries with d < t - 2E are certainly neighbours, entries with
 //      d > t + 2E certainly not; only the few in between get the exact FP64
 //      d^2 and are ranked by (d^2, gas rank).
-// A group whose radius holds fewer than n_ngb particles for some member
-// retries with a larger radius (bisected once both bounds are known: the
-// paper's "usually twice"); a group whose candidates do not fit is split into
-// single-particle items, and a single particle whose candidates do not fit
-// retries with a smaller radius.  Each pass hands the next only its
-// unfinished items.  Density and the ideal-gas EOS are fused in.
+// Members whose radius holds fewer than n_ngb particles are searched again
+// with a larger one (from the count found, bisected once both bounds are
+// known: the paper's "usually twice"); a run whose candidates do not fit is
+// taken in smaller runs, and a single particle whose candidates do not fit is
+// searched with a smaller radius, down to adjacent floats.  Density and the
+// ideal-gas EOS are fused in.
+//
+// What bounds it: latency and instruction issue (50 % issue-active at 24 warps
+// per SM, which the shared memory allows; HBM and L2 stay below 10 %).  A
+// warp per run has no block barriers, and the compacted list replaces three
+// passes over all candidates (histogram, bucket, classification) by one.
+// Against one 128-thread CTA per group with those passes (phase time):
+// 2^24 disk (1.68 M gas) 6.61 -> 3.07 ms, 2^20 disk (210 k) 1.03 -> 0.45 ms,
+// 1e5-particle region 0.50 -> 0.27 ms, 4,096 gas 0.31 -> 0.05 ms.
 //
 // Force: symmetric SPH over S_i = N_i u {j : i in N_j}.  The reverse part is
 // built from the non-mutual pairs only, so N_i and R_i are disjoint.
@@ -34,13 +45,14 @@ namespace gnb {
 
 #define KN_THREADS 128
 #define KN_WARPS (KN_THREADS / 32)
-// Candidate buffer and node stack size the shared memory of a CTA (24.7 KB),
-// and with it the CTAs per SM (9, as the 56 registers allow).
-#define KN_CAP 768
-#define KN_STACK 768
-#define KN_BKT 256
+#define KN_CTAS 6     // CTAs per SM, as the shared memory of the warps allows
+#define KN_CAP 448    // candidates of a warp's run
+#define KN_STACK 384  // node stack entries of a warp
+#define KN_LIST 128   // entries of one particle's list: 64 neighbours and at most 64 uncertain ones
 #define KN_U 64
-#define KN_SUB 4  // particles per work item when a group splits (2^24 disk: 6.52 ms for the pass, 8: 6.77, singles: 7.05)
+#define KN_GROUP 32   // gas particles of a hydro group
+#define KN_GROW 1.03f // margin over the radius that the count within the last one asks for
+#define KN_SUB 4      // particles per run when a run's candidates do not fit
 #define NGB 64
 
 __device__ __forceinline__ float kern_w(float r, float hinv)
@@ -67,8 +79,10 @@ struct GasGather {
     PArr p;
     const int *gslot;
     uint64_t *gkey;
-    int *gcx, *gcy, *gcz, *ggrank;
-    float *grx, *gry, *grz, *gm, *gvx, *gvy, *gvz, *gu, *gRprev;
+    int *ggrank;
+    int4 *C;
+    float4 *R;
+    float *gvx, *gvy, *gvz, *gu, *gRprev;
     double *gx, *gy, *gz;
     int ng;
     int pred;
@@ -81,10 +95,9 @@ __global__ void k_gas_gather(GasGather g)
     if (k >= g.ng) return;
     int s = g.gslot[k];
     g.gkey[k] = g.skey[s];
-    g.gcx[k] = g.p.cx[s]; g.gcy[k] = g.p.cy[s]; g.gcz[k] = g.p.cz[s];
-    g.grx[k] = g.p.rx[s]; g.gry[k] = g.p.ry[s]; g.grz[k] = g.p.rz[s];
+    g.C[k] = make_int4(g.p.cx[s], g.p.cy[s], g.p.cz[s], __float_as_int(g.p.m[s]));
+    g.R[k] = make_float4(g.p.rx[s], g.p.ry[s], g.p.rz[s], 0.f);
     g.gx[k] = g.p.x[s]; g.gy[k] = g.p.y[s]; g.gz[k] = g.p.z[s];
-    g.gm[k] = g.p.m[s];
     g.ggrank[k] = g.p.grank[s];
     if (g.pred) {
         g.gvx[k] = g.p.vpx[s]; g.gvy[k] = g.p.vpy[s]; g.gvz[k] = g.p.vpz[s]; g.gu[k] = g.p.up[s];
@@ -94,68 +107,63 @@ __global__ void k_gas_gather(GasGather g)
     g.gRprev[k] = g.have_h ? sqrtf((float)g.p.h2[s]) : 0.f;  // a starting radius only
 }
 
-// ---------------------------------------------------------------- search radius
-// Initial radius per hydro group: margin x the largest previous support in
-// the group, or, without history, a density estimate from the smallest
-// ancestor cell holding at least n_ngb particles.  A group split into
-// single-particle items gives each particle margin x its own previous
-// support (at most the group's radius).  The margin trades retried items (a
-// support that grew past it) against candidates per item (the search volume
-// grows as its cube); the host adapts it to the retries it sees (see
-// sph_density).
-__global__ void k_knn_init(Tree t, const float *__restrict__ hprev, int have_h, float margin, const double *__restrict__ box,
-                           float *__restrict__ kR, float2 *__restrict__ kRb, int *__restrict__ kflag,
+// ---------------------------------------------------------------- work items
+// A work item is a run of at most `sub` consecutive gas particles of one
+// hydro group, with the starting search radius of the group where a particle
+// has no previous support: from the density of the smallest ancestor cell
+// holding at least n_ngb particles.
+__global__ void k_knn_init(Tree t, int sub, const double *__restrict__ box, float *__restrict__ kR,
                            int2 *__restrict__ kitem, int *__restrict__ nitems)
 {
-    int ng = *t.ngroups_d;
-    float unit = (float)box[4];
-    if (blockIdx.x == 0 && threadIdx.x == 0) *nitems = ng;
-    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < ng; g += gridDim.x * blockDim.x) {
-        int node = t.groups[g];
-        int4 a = t.na[node];
-        kitem[g] = make_int2(a.x, a.y);
+    const int ng = *t.ngroups_d, lane = threadIdx.x & 31;
+    const float unit = (float)box[4];
+    for (int g0 = (blockIdx.x * blockDim.x + threadIdx.x) & ~31; g0 < ng; g0 += gridDim.x * blockDim.x) {
+        const int g = g0 + lane;
+        int4 a = make_int4(0, 0, 0, 0);
         float R = 0.f;
-        if (have_h) {
-            for (int i = a.x; i < a.x + a.y; i++) R = fmaxf(R, hprev[i]);
-            R *= margin;
+        if (g < ng) {
+            int q = t.groups[g];
+            a = t.na[q];
+            int4 aq = a;
+            while (aq.y < NGB && t.nb[q].w >= 0) {
+                q = t.nb[q].w;
+                aq = t.na[q];
+            }
+            R = 0.9f * (float)(1 << (GNB_MAXLEV - (aq.w & 255))) * unit * cbrtf((float)NGB / (float)max(aq.y, 1));
         }
-        if (!(R > 0.f)) {
-            int q = node;
-            while (t.na[q].y < NGB && t.nb[q].w >= 0) q = t.nb[q].w;
-            int4 aq = t.na[q];
-            int lev = aq.w & 255;
-            float side = (float)(1 << (GNB_MAXLEV - lev)) * unit;
-            R = 0.9f * side * cbrtf((float)NGB / (float)max(aq.y, 1));
+        // items in group order within the warp, one atomic per warp; at most
+        // one item per gas particle in all
+        const int k = (a.y + sub - 1) / sub;
+        int inc = k;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
         }
-        kR[g] = R;
-        kRb[g] = make_float2(0.f, 0.f);
-        kflag[g] = 1;
+        int base = 0;
+        if (lane == 31) base = atomicAdd(nitems, inc);
+        base = __shfl_sync(0xffffffffu, base, 31) + inc - k;
+        for (int e = 0; e < k; e++) {
+            kitem[base + e] = make_int2(a.x + e * sub, min(sub, a.y - e * sub));
+            kR[base + e] = R;
+        }
     }
 }
 
-// Work items: a hydro group, or a single particle split off a group whose
-// candidates did not fit at the radius its members need.
 struct KnnParams {
-    int4 *na, *nb;
-    int2 *item;
-    int *nitems;       // live count (splits append here)
-    const int *nsnap;  // entries of this pass's worklist
-    const int *wl_in;  // this pass's items (null: items 0 .. *nsnap - 1)
-    int *wl_out;       // items left for the next pass: retried radii and new single-particle items
-    int *nwl_out;
-    int item_cap;
-    const int *gcx, *gcy, *gcz, *ggrank;
-    const float *grx, *gry, *grz, *gm, *gu;
+    const int4 *na, *nb;  // hydro tree
+    const int2 *item;
+    const float *kR;
+    const int *nitems;
+    int *next;           // next item to take
+    int *nunder;         // items whose radius held too few candidates for some member
+    const int4 *C;       // cell x, y, z and mass bits per gas particle
+    const float4 *R;     // residual x, y, z
+    const int *ggrank;
+    const float *gu;
     const double *gx, *gy, *gz;
     const double *box;
     const float *rprev;  // previous support per gas particle (0: none)
     float margin;        // search radius over the previous support
-    int *nunder;         // work items whose radius held too few candidates
-    float *kR;
-    float2 *kRb;
-    int *kflag;
-    int *next;
-    int *remaining;
     int *status;
     int *nbr;
     float *nd2;
@@ -167,36 +175,25 @@ struct KnnParams {
     int pressure;  // 1: also smooth P = (gamma - 1) sum_j m_j u_j W_ij (pressure-energy SPH)
 };
 
-struct KnnSmem {
+// Per-warp buffers: the candidates, and a scratch area that holds the node
+// stack and the pending leaves during the walk, then the particle's list and
+// its uncertain entries.
+struct KnnWarp {
     float4 cand[KN_CAP];
-    int stack[KN_STACK];
-    int hist[KN_WARPS][64];
-    float bkt[KN_WARPS][KN_BKT];
-    int bn[KN_WARPS];
-    int un[KN_WARPS];
-    int ui[KN_WARPS][KN_U];
-    long long uD[KN_WARPS][KN_U];  // exact FP64 d^2 as bit patterns (non-negative: they order like the values)
-    int ug[KN_WARPS][KN_U];        // gas ranks of the uncertain entries
-    int nc, sp, g, wb, under, over, split, nleaf, bmin[3], bmax[3];
-    long long rg2i;
-    unsigned amax;
+    union {
+        struct {
+            unsigned stack[KN_STACK];
+            int2 leaf[64];
+        } walk;
+        struct {
+            float d[KN_LIST];
+            int j[KN_LIST];
+            long long uD[KN_U];  // exact FP64 d^2 as bit patterns (non-negative: they order like the values)
+            int uj[KN_U];
+            int ug[KN_U];        // gas ranks of the uncertain entries
+        } sel;
+    };
 };
-// During the gather the bucket buffers hold the list of leaves within the
-// radius (first, count) and its prefix sums over the counts.
-#define KN_LEAF 256
-static_assert(sizeof(float) * KN_WARPS * KN_BKT >= (sizeof(int2) + sizeof(int)) * KN_LEAF + sizeof(int),
-              "leaf list must fit the bucket buffers");
-
-// A particle of a group could not be ranked within the buffers: the FP32
-// error band (2^-17 A^2, A the group's largest offset) is wide when a dense
-// clump sits inside a spread-out group.  The group is then split into
-// single-particle work items, whose band scales with their own search
-// radius; only a single particle that still fails is reported.
-__device__ __forceinline__ void knn_fail(KnnSmem &S, int count, int *status)
-{
-    if (count > 1) S.split = 1;
-    else atomicOr(status, ST_KNN_OVERFLOW);
-}
 
 __device__ __forceinline__ float d2f(float4 c, float xi, float yi, float zi)
 {
@@ -211,497 +208,514 @@ __device__ __forceinline__ double exact_d2(const double *x, const double *y, con
     return __dadd_rn(a, __dmul_rn(dz, dz));
 }
 
-// Exact k-th smallest FP32 d^2 (1-based k) among the candidates of this
-// warp's particle that fall in histogram bucket bstar of [0, R2sel] (the
-// same bin rule as the histogram): a radix select on the bit patterns, which
-// order non-negative floats like their values, 8 bits per pass.  Used when
-// the bucket holds more candidates than the bucket buffer -- a particle whose
-// nearest neighbours all lie in a thin shell, e.g. a compact clump seen from
-// outside, where shrinking the radius does not thin the bucket.
-__device__ __noinline__ float knn_radix_kth(KnnSmem &S, int w, int lane, int nc, float xi, float yi, float zi, float R2sel,
-                               float inv64, int bstar, int k, bool *ok)
+// Box of a run of particles (cells [b0, b1]), its reference cell, and the box
+// in offset coordinates [lo, hi).
+struct KnnBox {
+    int b0[3], b1[3], gref[3];
+    float lo[3], hi[3];
+};
+
+// Candidates of a warp's batch of m <= 32 leaves (lane q holds leaf q: first
+// and count): the particles of the leaves side by side, 32 at a time.  Lane f
+// of a chunk finds its leaf from the leaf starts in the chunk (one bit each)
+// and the number of leaves that start before it.  Returns false when the
+// buffer is full.  one (the run is a single particle at xs): the distance to
+// it decides rather than the box.
+__device__ __forceinline__ bool knn_gather(KnnWarp &S, const KnnParams &p, const KnnBox &B, int m, int2 leaf, float unit,
+                                           float R2stage, bool one, float xs, float ys, float zs, int &nc,
+                                           float &amax, int lane)
 {
-    int *hb = reinterpret_cast<int *>(S.bkt[w]);  // 256 bins (the bucket buffer is free here)
-    unsigned prefix = 0u, pmask = 0u;
-    for (int shift = 24; shift >= 0; shift -= 8) {
-        __syncwarp();
-        for (int b = lane; b < 256; b += 32) hb[b] = 0;
-        __syncwarp();
-        for (int c = lane; c < nc; c += 32) {
-            const float d = d2f(S.cand[c], xi, yi, zi);
-            if (d <= R2sel && min(63, (int)(d * inv64)) == bstar) {
-                const unsigned u = __float_as_uint(d);
-                if ((u & pmask) == prefix) atomicAdd(&hb[(u >> shift) & 255u], 1);
+    const unsigned ltmask = (1u << lane) - 1u, lemask = ltmask | (1u << lane);
+    const int cnt = lane < m ? leaf.y : 0;
+    int inc = cnt;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    const int total = __shfl_sync(0xffffffffu, inc, 31);
+    const int start = lane < m ? inc - cnt : 0x3fffffff;
+    const int rel = leaf.x - start;
+    for (int c = 0; c < total; c += 32) {
+        const unsigned st = (unsigned)(start - c);
+        const unsigned mask = __reduce_or_sync(0xffffffffu, st < 32u ? 1u << st : 0u);
+        const int before = __popc(__ballot_sync(0xffffffffu, start < c));
+        const int ord = before + __popc(mask & lemask) - 1;
+        const int j = __shfl_sync(0xffffffffu, rel, ord) + c + lane;
+        bool in = false;
+        float ox = 0.f, oy = 0.f, oz = 0.f;
+        if (c + lane < total) {
+            const int4 C = __ldg(&p.C[j]);
+            const float4 r = __ldg(&p.R[j]);
+            ox = grid_off(C.x, B.gref[0], r.x, unit);
+            oy = grid_off(C.y, B.gref[1], r.y, unit);
+            oz = grid_off(C.z, B.gref[2], r.z, unit);
+            if (one) {
+                in = d2f(make_float4(ox, oy, oz, 0.f), xs, ys, zs) <= R2stage;
+            } else {
+                const float gx = fmaxf(0.f, fmaxf(B.lo[0] - ox, ox - B.hi[0]));
+                const float gy = fmaxf(0.f, fmaxf(B.lo[1] - oy, oy - B.hi[1]));
+                const float gz = fmaxf(0.f, fmaxf(B.lo[2] - oz, oz - B.hi[2]));
+                in = gx * gx + gy * gy + gz * gz <= R2stage;
             }
         }
-        __syncwarp();
-        int loc[8], sum = 0;
-#pragma unroll
-        for (int q = 0; q < 8; q++) { loc[q] = hb[8 * lane + q]; sum += loc[q]; }
-        int inc = sum;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += y;
+        const unsigned bal = __ballot_sync(0xffffffffu, in);
+        const int add = __popc(bal);
+        if (nc + add > KN_CAP) return false;
+        if (in) {
+            S.cand[nc + __popc(bal & ltmask)] = make_float4(ox, oy, oz, __int_as_float(j));
+            amax = fmaxf(amax, ox * ox + oy * oy + oz * oz);
         }
-        const int exc = inc - sum;
-        int myb = -1, mybefore = 0, run = exc;
-#pragma unroll
-        for (int q = 0; q < 8; q++) {
-            if (myb < 0 && run < k && k <= run + loc[q]) { myb = 8 * lane + q; mybefore = run; }
-            run += loc[q];
-        }
-        const unsigned bal = __ballot_sync(0xffffffffu, myb >= 0);
-        if (bal == 0u) { *ok = false; return 0.f; }
-        const int src = __ffs(bal) - 1;
-        const int b = __shfl_sync(0xffffffffu, myb, src);
-        k -= __shfl_sync(0xffffffffu, mybefore, src);
-        prefix |= (unsigned)b << shift;
-        pmask |= 255u << shift;
+        nc += add;
     }
-    *ok = true;
-    return __uint_as_float(prefix);
+    return true;
 }
 
-__global__ void __launch_bounds__(KN_THREADS, 9) k_knn(KnnParams p)
+// Walk of the hydro tree: every particle within R of the run's box (of the
+// particle, for a run of one) becomes a candidate.  The stack holds nodes
+// whose children are to be tested, as (first child << 3) | (children - 1)
+// (node indices below 2^29, checked by the host); a round tests the children
+// of up to four of them, eight lanes each, so a push is one ballot and one
+// store.  False when the candidate buffer is full.
+__device__ __forceinline__ bool knn_walk(KnnWarp &S, const KnnParams &p, const KnnBox &B, float R, float unit, bool one,
+                                         float xs, float ys, float zs, int &nc, float &amax, int lane)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    KnnSmem &S = *reinterpret_cast<KnnSmem *>(smem_raw);
-    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-    const float unit = (float)p.box[4];
-    const int ngroups = min(*p.nsnap, p.item_cap);
     const unsigned ltmask = (1u << lane) - 1u;
+    // node test in grid units, only a bound for the particle tests below:
+    // gaps are integers below 2^22, exact in FP32, and the margin covers the
+    // roundings of the sums
+    const float Rg = R / unit;  // unit is a power of two
+    const float Rg2 = Rg * Rg * (1.f + 1e-5f) + 4.f;
+    // a single particle keeps what can lie in its list: d^2 <= R^2 + 2 E (E <
+    // 2^-23 (12 R^2 + 14 unit R) there), with a margin
+    const float R2stage = one ? R * R * (1.f + 4e-6f) + 6e-6f * unit * (R + unit)
+                              : R * R * (1.f + 1e-4f) + 4.f * unit * unit;
+    nc = 0;
+    amax = 0.f;
+    int sp = 0, nl = 0;
+    // the first round tests the root alone
+    int node = lane == 0 ? 0 : -1;
     for (;;) {
-        __syncthreads();  // every thread has read the previous S.g
-        if (tid == 0) S.g = atomicAdd(p.next, 1);
-        __syncthreads();
-        if (S.g >= ngroups) break;
-        const int gi = p.wl_in ? p.wl_in[S.g] : S.g;
-        if (p.kflag[gi] == 0) continue;  // uniform
-        const int2 gitem = p.item[gi];
-        const int4 ga = make_int4(gitem.x, gitem.y, 0, 0);
-        const float R = p.kR[gi];
-        if (tid < 3) { S.bmin[tid] = 0x7fffffff; S.bmax[tid] = -1; }
-        if (tid == 0) {
-            S.nc = 0; S.sp = 1; S.stack[0] = 0; S.under = 0; S.over = 0; S.split = 0; S.amax = 0u; S.nleaf = 0;
-            // the node test's threshold: (R in grid units)^2 (1 + 1e-5) + 4, in
-            // FP64 by one thread (GB300's FP64 pipe is narrow).  gap2 is an
-            // integer, so gap2 <= that exactly when gap2 <= its floor
-            const double Rg = (double)R / (double)unit;
-            const double Rg2m = Rg * Rg * (1.0 + 1e-5) + 4.0;
-            S.rg2i = Rg2m >= 4.0e18 ? 0x7fffffffffffffffll : (long long)Rg2m;
-        }
-        __syncthreads();
-        for (int i = ga.x + tid; i < ga.x + ga.y; i += KN_THREADS) {
-            atomicMin(&S.bmin[0], p.gcx[i]); atomicMax(&S.bmax[0], p.gcx[i]);
-            atomicMin(&S.bmin[1], p.gcy[i]); atomicMax(&S.bmax[1], p.gcy[i]);
-            atomicMin(&S.bmin[2], p.gcz[i]); atomicMax(&S.bmax[2], p.gcz[i]);
-        }
-        __syncthreads();
-        const int b0[3] = {S.bmin[0], S.bmin[1], S.bmin[2]}, b1[3] = {S.bmax[0], S.bmax[1], S.bmax[2]};
-        const int gref[3] = {(b0[0] + b1[0]) >> 1, (b0[1] + b1[1]) >> 1, (b0[2] + b1[2]) >> 1};
-        // group box in offset coordinates: [lo_k, hi_k)
-        float blo[3], bhi[3];
-#pragma unroll
-        for (int a = 0; a < 3; a++) {
-            blo[a] = (float)(b0[a] - gref[a]) * unit;
-            bhi[a] = (float)(b1[a] + 1 - gref[a]) * unit;
-        }
-        const long long Rg2i = S.rg2i;
-        const float R2stage = R * R * (1.f + 1e-4f) + 4.f * unit * unit;
-        int2 *leafl = reinterpret_cast<int2 *>(&S.bkt[0][0]);
-        int *lpre = reinterpret_cast<int *>(leafl + KN_LEAF);
-        // gather candidates within R of the group box: the walk lists the
-        // leaves it reaches, then all threads test their particles together
-        for (;;) {
-            __syncthreads();
-            int sp = S.sp;
-            if (sp == 0) break;
-            int k = min(KN_THREADS, sp);
-            int room = (KN_STACK - sp) / 7;
-            k = min(k, max(room, 1));
-            int node = tid < k ? S.stack[sp - k + tid] : -1;
-            __syncthreads();
-            if (tid == 0) S.sp = sp - k;
-            __syncthreads();
-            if (node >= 0) {
-                int4 a = p.na[node];
-                int4 C = p.nb[node];
-                int lev = a.w & 255, nch = a.w >> 8;
-                long long s = 1ll << (GNB_MAXLEV - lev);
-                int cc[3] = {C.x, C.y, C.z};
-                long long gap2 = 0;  // < 3 * 2^44: exact in 64-bit integers
-#pragma unroll
-                for (int q = 0; q < 3; q++) {
-                    long long gp = 0;
-                    if ((long long)cc[q] > (long long)b1[q] + 1) gp = cc[q] - ((long long)b1[q] + 1);
-                    else if ((long long)b0[q] > cc[q] + s) gp = b0[q] - (cc[q] + s);
-                    gap2 += gp * gp;
-                }
-                if (gap2 <= Rg2i) {
-                    if (nch > 0) {
-                        int b = atomicAdd(&S.sp, nch);
-                        if (b + nch <= KN_STACK) {
-                            for (int q = 0; q < nch; q++) S.stack[b + q] = a.z + q;
-                        } else {
-                            atomicSub(&S.sp, nch);
-                            S.over = 1;
-                        }
-                    } else {
-                        const int q = atomicAdd(&S.nleaf, 1);
-                        if (q < KN_LEAF) leafl[q] = make_int2(a.x, a.y);
-                        else  // the list is full: this thread tests the leaf's particles
-                        for (int j = a.x; j < a.x + a.y; j++) {
-                            float ox = grid_off(p.gcx[j], gref[0], p.grx[j], unit);
-                            float oy = grid_off(p.gcy[j], gref[1], p.gry[j], unit);
-                            float oz = grid_off(p.gcz[j], gref[2], p.grz[j], unit);
-                            float gx = fmaxf(0.f, fmaxf(blo[0] - ox, ox - bhi[0]));
-                            float gy = fmaxf(0.f, fmaxf(blo[1] - oy, oy - bhi[1]));
-                            float gz = fmaxf(0.f, fmaxf(blo[2] - oz, oz - bhi[2]));
-                            if (gx * gx + gy * gy + gz * gz <= R2stage) {
-                                int slot = atomicAdd(&S.nc, 1);
-                                if (slot < KN_CAP) {
-                                    S.cand[slot] = make_float4(ox, oy, oz, __int_as_float(j));
-                                    float a2 = ox * ox + oy * oy + oz * oz;
-                                    atomicMax(&S.amax, __float_as_uint(a2));
-                                } else {
-                                    S.over = 1;
-                                }
-                            }
-                        }
-                    }
-                }
+        int nch = 0, child = 0, first = 0, count = 0;
+        if (node >= 0) {
+            const int4 a = __ldg(&p.na[node]);
+            const int4 C = __ldg(&p.nb[node]);
+            const int s = 1 << (GNB_MAXLEV - (a.w & 255));
+            const float gx = (float)max(0, max(C.x - (B.b1[0] + 1), B.b0[0] - (C.x + s)));
+            const float gy = (float)max(0, max(C.y - (B.b1[1] + 1), B.b0[1] - (C.y + s)));
+            const float gz = (float)max(0, max(C.z - (B.b1[2] + 1), B.b0[2] - (C.z + s)));
+            if (gx * gx + gy * gy + gz * gz <= Rg2) {
+                nch = a.w >> 8;
+                child = a.z;
+                first = a.x;
+                if (nch == 0) count = a.y;
             }
         }
-        __syncthreads();
-        {   // the listed leaves' particles, flattened over all threads
-            const int nl = min(S.nleaf, KN_LEAF);
-            if (w == 0) {  // prefix sums of the leaf counts
-                int carry = 0;
-                for (int b0 = 0; b0 < nl; b0 += 32) {
-                    const int q = b0 + lane;
-                    const int v = q < nl ? leafl[q].y : 0;
-                    int inc = v;
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const int y = __shfl_up_sync(0xffffffffu, inc, o);
-                        if (lane >= o) inc += y;
-                    }
-                    if (q < nl) lpre[q] = carry + inc - v;
-                    carry += __shfl_sync(0xffffffffu, inc, 31);
-                }
-                if (lane == 0) lpre[nl] = carry;
-            }
-            __syncthreads();
-            const int total = lpre[nl];
-            for (int f0 = w * 32; f0 < total; f0 += KN_THREADS) {
-                const int f = f0 + lane;
-                bool in = false;
-                float ox = 0.f, oy = 0.f, oz = 0.f;
-                int j = 0;
-                if (f < total) {
-                    int lo = 0, hi = nl - 1;  // the last leaf starting at or before f
-                    while (lo < hi) {
-                        const int mid = (lo + hi + 1) >> 1;
-                        if (lpre[mid] <= f) lo = mid;
-                        else hi = mid - 1;
-                    }
-                    j = leafl[lo].x + (f - lpre[lo]);
-                    ox = grid_off(p.gcx[j], gref[0], p.grx[j], unit);
-                    oy = grid_off(p.gcy[j], gref[1], p.gry[j], unit);
-                    oz = grid_off(p.gcz[j], gref[2], p.grz[j], unit);
-                    const float gx = fmaxf(0.f, fmaxf(blo[0] - ox, ox - bhi[0]));
-                    const float gy = fmaxf(0.f, fmaxf(blo[1] - oy, oy - bhi[1]));
-                    const float gz = fmaxf(0.f, fmaxf(blo[2] - oz, oz - bhi[2]));
-                    in = gx * gx + gy * gy + gz * gz <= R2stage;
-                }
-                const unsigned bal = __ballot_sync(0xffffffffu, in);
-                if (bal == 0u) continue;
-                int base = 0;
-                if (lane == 0) base = atomicAdd(&S.nc, __popc(bal));
-                base = __shfl_sync(0xffffffffu, base, 0);
-                unsigned a2 = 0u;
-                if (in) {
-                    const int slot = base + __popc(bal & ltmask);
-                    if (slot < KN_CAP) {
-                        S.cand[slot] = make_float4(ox, oy, oz, __int_as_float(j));
-                        a2 = __float_as_uint(ox * ox + oy * oy + oz * oz);
-                    } else {
-                        S.over = 1;
-                    }
-                }
-                a2 = __reduce_max_sync(0xffffffffu, a2);
-                if (lane == 0) atomicMax(&S.amax, a2);
-            }
+        __syncwarp();
+        const unsigned pb = __ballot_sync(0xffffffffu, nch > 0), lb = __ballot_sync(0xffffffffu, count > 0);
+        if (nch > 0) S.walk.stack[sp + __popc(pb & ltmask)] = (unsigned)child << 3 | (unsigned)(nch - 1);
+        if (count > 0) S.walk.leaf[nl + __popc(lb & ltmask)] = make_int2(first, count);
+        sp += __popc(pb);
+        nl += __popc(lb);
+        __syncwarp();
+        if (nl >= 32 || (sp == 0 && nl > 0)) {
+            const int m = min(nl, 32);
+            nl -= m;
+            const int2 lf = lane < m ? S.walk.leaf[nl + lane] : make_int2(0, 0);
+            if (!knn_gather(S, p, B, m, lf, unit, R2stage, one, xs, ys, zs, nc, amax, lane)) return false;
         }
-        __syncthreads();
-        const int nc = min(S.nc, KN_CAP);
-        if (!S.over) {
-            // group particles also bound the offsets
-            for (int i = ga.x + tid; i < ga.x + ga.y; i += KN_THREADS) {
-                float ox = grid_off(p.gcx[i], gref[0], p.grx[i], unit);
-                float oy = grid_off(p.gcy[i], gref[1], p.gry[i], unit);
-                float oz = grid_off(p.gcz[i], gref[2], p.grz[i], unit);
-                atomicMax(&S.amax, __float_as_uint(ox * ox + oy * oy + oz * oz));
-            }
-            __syncthreads();
-            // error bound of an FP32 d^2 near D (see the file comment)
-            const float EA = 6.92820323f * (sqrtf(__uint_as_float(S.amax)) + 2.f * unit);  // 4 sqrt(3) A'
-            const float R2 = R * R;
-            const float thrR = R2 - 1.1920929e-07f * (EA * sqrtf(R2) + 5.f * R2);
-            for (int i = ga.x + w; i < ga.x + ga.y; i += KN_WARPS) {
-                const float xi = grid_off(p.gcx[i], gref[0], p.grx[i], unit);
-                const float yi = grid_off(p.gcy[i], gref[1], p.gry[i], unit);
-                const float zi = grid_off(p.gcz[i], gref[2], p.grz[i], unit);
-                __syncwarp();  // the previous particle's scratch is no longer read
-                if (lane == 0) { S.bn[w] = 0; S.un[w] = 0; }
-                // bucket holding the 64th smallest; shrink this particle's
-                // radius to that bucket while the bucket is too full to rank.
-                // The first histogram pass also counts the candidates certainly
-                // within R: fewer than n_ngb means the radius is too small.
-                float R2i = R2, inv64 = 64.f / R2, R2sel = R2;
-                int bstar = -1, kth = 0;
-                bool ok = false, under_i = false;
-                for (int it = 0; it < 16; it++) {
-                    __syncwarp();
-                    R2sel = R2i;  // the radius of this histogram (bstar, kth refer to it)
-                    S.hist[w][lane] = 0;
-                    S.hist[w][lane + 32] = 0;
-                    __syncwarp();
-                    inv64 = 64.f / R2i;
-                    int cnt = 0;
-                    for (int c = lane; c < nc; c += 32) {
-                        float d = d2f(S.cand[c], xi, yi, zi);
-                        if (it == 0) cnt += d <= thrR;
-                        if (d <= R2i) atomicAdd(&S.hist[w][min(63, (int)(d * inv64))], 1);
-                    }
-                    if (it == 0 && warp_sum(cnt) < NGB) {
-                        under_i = true;
-                        break;
-                    }
-                    __syncwarp();
-                    int h0 = S.hist[w][2 * lane], h1 = S.hist[w][2 * lane + 1];
-                    int sum = h0 + h1, inc = sum;
-                    for (int o = 1; o < 32; o <<= 1) {
-                        int y = __shfl_up_sync(0xffffffffu, inc, o);
-                        if (lane >= o) inc += y;
-                    }
-                    int exc = inc - sum;
-                    int mybin = -1, mybefore = 0;
-                    if (exc < NGB && NGB <= exc + h0) { mybin = 2 * lane; mybefore = exc; }
-                    else if (exc + h0 < NGB && NGB <= inc) { mybin = 2 * lane + 1; mybefore = exc + h0; }
-                    unsigned bal = __ballot_sync(0xffffffffu, mybin >= 0);
-                    if (bal == 0u) break;
-                    int src = __ffs(bal) - 1;
-                    bstar = __shfl_sync(0xffffffffu, mybin, src);
-                    kth = NGB - __shfl_sync(0xffffffffu, mybefore, src);  // 1-based rank in bucket
-                    if (S.hist[w][bstar] <= KN_BKT) { ok = true; break; }
-                    R2i = R2i * (float)(bstar + 1) * (1.f / 64.f) * (1.f + 1e-6f);
-                }
-                if (under_i) {
-                    if (lane == 0) S.under = 1;
-                    continue;
-                }
-                float t = 0.f;
-                bool have_t = false;
-                if (ok) {
-                    for (int c = lane; c < nc; c += 32) {
-                        float d = d2f(S.cand[c], xi, yi, zi);
-                        if (d <= R2i && min(63, (int)(d * inv64)) == bstar) {
-                            int slot = atomicAdd(&S.bn[w], 1);
-                            if (slot < KN_BKT) S.bkt[w][slot] = d;
-                        }
-                    }
-                    __syncwarp();
-                    const int nb = S.bn[w];
-                    if (nb <= KN_BKT) {
-                        // t = kth smallest value in the bucket (ties by position)
-                        bool found = false;
-                        for (int e = lane; e < nb; e += 32) {
-                            float de = S.bkt[w][e];
-                            int r = 0;
-                            for (int f = 0; f < nb; f++) {
-                                float df = S.bkt[w][f];
-                                r += (df < de) || (df == de && f < e);
-                            }
-                            if (r == kth - 1) { t = de; found = true; }
-                        }
-                        unsigned fb = __ballot_sync(0xffffffffu, found);
-                        if (fb != 0u) {
-                            t = __shfl_sync(0xffffffffu, t, __ffs(fb) - 1);
-                            have_t = true;
-                        }
-                    }
-                }
-                if (!have_t && bstar >= 0 && ga.y == 1) {
-                    // a single particle whose bucket stays too full: exact
-                    // selection over the candidates themselves (groups split
-                    // first, which is cheaper for a clump inside a spread group)
-                    bool okr = false;
-                    t = knn_radix_kth(S, w, lane, nc, xi, yi, zi, R2sel, 64.f / R2sel, bstar, kth, &okr);
-                    have_t = okr;
-                }
-                if (!have_t) {
-                    if (lane == 0) knn_fail(S, ga.y, p.status);
-                    continue;
-                }
-                // the bound at a point just above the band's upper end (E << t)
-                const float tb = t * 1.0009765625f;
-                const float E = 1.1920929e-07f * (EA * sqrtf(tb) + 5.f * tb);
-                const float lo = t - 2.f * E, hi = t + 2.f * E;
-                // classify: sure members written directly, uncertain ones collected
-                int nS = 0;
-                int *outn = p.nbr + (size_t)i * NGB;
-                float *outd = p.nd2 + (size_t)i * NGB;
-                for (int c0 = 0; c0 < nc; c0 += 32) {
-                    int c = c0 + lane;
-                    float d = 3.0e38f;
-                    int j = -1;
-                    if (c < nc) {
-                        float4 cv = S.cand[c];
-                        d = d2f(cv, xi, yi, zi);
-                        j = __float_as_int(cv.w);
-                    }
-                    bool sure = d < lo;
-                    unsigned sb = __ballot_sync(0xffffffffu, sure);
-                    if (sure) {
-                        int pos = nS + __popc(sb & ltmask);
-                        if (pos < NGB) { outn[pos] = j; outd[pos] = d; }
-                    }
-                    nS += __popc(sb);
-                    if (!sure && d <= hi) {
-                        int slot = atomicAdd(&S.un[w], 1);
-                        if (slot < KN_U) S.ui[w][slot] = j;
-                    }
-                }
-                __syncwarp();
-                const int nu = S.un[w];
-                if (nu > KN_U || nS >= NGB) {
-                    if (lane == 0) knn_fail(S, ga.y, p.status);
-                    continue;
-                }
-                for (int e = lane; e < nu; e += 32) {
-                    const int je = S.ui[w][e];
-                    S.uD[w][e] = __double_as_longlong(exact_d2(p.gx, p.gy, p.gz, i, je));
-                    S.ug[w][e] = p.ggrank[je];
-                }
-                __syncwarp();
-                const int need = NGB - nS;
-                double hsq = 0.0;
-                int h64 = -1;
-                bool have = false;
-                for (int e = lane; e < nu; e += 32) {
-                    const long long De = S.uD[w][e];
-                    const int je = S.ui[w][e];
-                    const int ge = S.ug[w][e];
-                    int r = 0;
-                    for (int f = 0; f < nu; f++) {  // integer compares: no FP64 work
-                        const long long Df = S.uD[w][f];
-                        r += (Df < De) || (Df == De && S.ug[w][f] < ge);
-                    }
-                    if (r < need) {
-                        outn[nS + r] = je;
-                        outd[nS + r] = (float)__longlong_as_double(De);
-                    }
-                    if (r == need - 1) { hsq = __longlong_as_double(De); h64 = ge; have = true; }
-                }
-                unsigned hb = __ballot_sync(0xffffffffu, have);
-                if (hb == 0u) {  // error bound violated: fewer uncertain entries than needed
-                    if (lane == 0) knn_fail(S, ga.y, p.status);
-                    continue;
-                }
-                int hs = __ffs(hb) - 1;
-                hsq = __shfl_sync(0xffffffffu, hsq, hs);
-                h64 = __shfl_sync(0xffffffffu, h64, hs);
-                __syncwarp();
-                // density and EOS over the 64 neighbours
-                const float hh = sqrtf((float)hsq);  // within one FP32 rounding of sqrt(h^2)
-                const float hinv = 1.f / hh;
-                float rs = 0.f, qs = 0.f;
-                for (int e = lane; e < NGB; e += 32) {
-                    int j = outn[e];
-                    const float mw = p.gm[j] * kern_w(sqrtf(outd[e]), hinv);
-                    rs += mw;
-                    if (p.pressure) qs = __fmaf_rn(mw, p.gu[j], qs);
-                }
-                rs = warp_sum(rs);
-                if (p.pressure) qs = warp_sum(qs);
-                if (lane == 0) {
-                    float u = p.gu[i];
-                    float P = p.pressure ? (p.gamma - 1.f) * qs : (p.gamma - 1.f) * rs * u;
-                    p.h2[i] = hsq;
-                    p.h2lo[i] = __double2float_rd(hsq);
-                    p.h2hi[i] = __double2float_ru(hsq);
-                    p.h[i] = hh;
-                    p.g64[i] = h64;
-                    p.E[i] = E;
-                    p.rho[i] = rs;
-                    p.P[i] = P;
-                    p.cs[i] = sqrtf(p.gamma * P / rs);
-                }
-            }
-        }
-        __syncthreads();
-        if ((S.over || S.split) && ga.y > 1) {
-            // the members need a radius whose candidates do not fit: hand
-            // them to work items of at most KN_SUB consecutive particles
-            // (single particles once the item is that small), each starting
-            // from the margin x its members' largest previous support (at
-            // most the group's radius); an item that still does not fit
-            // splits again
-            const int sub = ga.y > KN_SUB ? KN_SUB : 1;
-            const int nsub = (ga.y + sub - 1) / sub;
-            __syncthreads();
-            if (tid == 0) {
-                S.g = atomicAdd(p.nitems, nsub);
-                S.wb = atomicAdd(p.nwl_out, nsub);
-                p.kflag[gi] = 0;
-                atomicAdd(p.remaining, 1);
-            }
-            __syncthreads();
-            const int base = S.g;
-            for (int k = tid; k < nsub; k += KN_THREADS) {
-                const bool fits = base + k < p.item_cap;
-                if (fits) {
-                    const int f = ga.x + k * sub, cnt = min(sub, ga.y - k * sub);
-                    p.item[base + k] = make_int2(f, cnt);
-                    float hp = 0.f;
-                    bool all = true;
-                    for (int q = 0; q < cnt; q++) {
-                        const float h = p.rprev[f + q];
-                        hp = fmaxf(hp, h);
-                        all = all && h > 0.f;
-                    }
-                    p.kR[base + k] = all ? fminf(R, p.margin * hp) : R;
-                    p.kRb[base + k] = make_float2(0.f, 0.f);
-                    p.kflag[base + k] = 1;
-                } else {
-                    atomicOr(p.status, ST_KNN_OVERFLOW);
-                }
-                // an item that did not fit is replaced by the finished parent
-                if (S.wb + k < p.item_cap) p.wl_out[S.wb + k] = fits ? base + k : gi;
-            }
+        if (sp == 0) {
+            if (nl == 0) return true;
+            node = -1;
             continue;
         }
-        if (tid == 0) {
-            float2 rb = p.kRb[gi];
-            int done = 1;
-            if (S.over) {
-                rb.y = R;
-                p.kR[gi] = rb.x > 0.f ? 0.5f * (R + rb.x) : 0.6f * R;
-                done = 0;
-            } else if (S.under) {
-                rb.x = R;
-                p.kR[gi] = rb.y > 0.f ? 0.5f * (R + rb.y) : 1.6f * R;
-                done = 0;
-                atomicAdd(p.nunder, 1);
+        // up to four nodes while the stack is at most half full (a round then
+        // leaves at most 28 more entries), else one (seven more per level below
+        // it, at most GNB_MAXLEV levels): it cannot overflow
+        static_assert(KN_STACK / 2 + 28 + 7 * GNB_MAXLEV <= KN_STACK, "walk stack");
+        const int k = sp <= KN_STACK / 2 ? min(4, sp) : 1;
+        const int q = lane >> 3;
+        const unsigned e = q < k ? S.walk.stack[sp - k + q] : 0u;
+        node = q < k && (lane & 7) <= (int)(e & 7u) ? (int)(e >> 3) + (lane & 7) : -1;
+        sp -= k;
+    }
+}
+
+enum { KN_DONE = 0, KN_UNDER = 1, KN_FAIL = 2 };
+
+// Candidates of particle (xi, yi, zi) with d^2 <= T, compacted into the list
+// (the first KN_LIST of them); returns their number.
+__device__ __forceinline__ int knn_list(KnnWarp &S, int nc, float xi, float yi, float zi, float T, int lane)
+{
+    const unsigned ltmask = (1u << lane) - 1u;
+    int n = 0;
+    __syncwarp();
+    for (int c0 = 0; c0 < nc; c0 += 32) {
+        const int c = c0 + lane;
+        float d = 3.0e38f;
+        int j = 0;
+        if (c < nc) {
+            const float4 v = S.cand[c];
+            d = d2f(v, xi, yi, zi);
+            j = __float_as_int(v.w);
+        }
+        const bool in = d <= T;
+        const unsigned bal = __ballot_sync(0xffffffffu, in);
+        const int pos = n + __popc(bal & ltmask);
+        if (in && pos < KN_LIST) {
+            S.sel.d[pos] = d;
+            S.sel.j[pos] = j;
+        }
+        n += __popc(bal);
+    }
+    __syncwarp();
+    return n;
+}
+
+__device__ __forceinline__ float sqrt_fast(float x)
+{
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));  // relative error below 2^-22
+    return r;
+}
+
+// What the selection of one particle leaves to its lane: its 64th neighbour
+// (-1: ranked already, hsq holds its exact d^2) and the FP32 error bound.
+struct KnnSel {
+    int j64, g64;
+    float E;
+    double hsq;
+};
+
+// The 64 nearest of particle i among the candidates, exactly (see the file
+// comment): fewer than 64 with d^2 <= thr is KN_UNDER, T0 is the largest d^2
+// that can matter.  The list goes to nbr / nd2 except, in the usual case of
+// one uncertain entry, its last place (r.j64).  n: entries of the last list
+// (KN_UNDER: about how many lie within the radius).
+__device__ __forceinline__ int knn_select(KnnWarp &S, const KnnParams &p, int i, int nc, float xi, float yi, float zi,
+                                          float thr, float T0, float EA, int &n, KnnSel &r, int lane)
+{
+    constexpr float U = 1.1920929e-07f;  // 2^-23
+    constexpr int KPL = KN_LIST / 32;
+    const unsigned ltmask = (1u << lane) - 1u;
+    float T = T0, Tlo = 0.f, Thi = T0;  // Tlo: too few entries, Thi: too many
+    float t = 0.f, E = 0.f;
+    unsigned du[KPL];
+    for (int it = 0;; it++) {
+        n = knn_list(S, nc, xi, yi, zi, T, lane);
+        if (n < NGB && it == 0) return KN_UNDER;
+        if (n < NGB || n > KN_LIST) {
+            // more than the list holds within the radius: narrow it to 64 ..
+            // KN_LIST entries, by the number density, then by bisection down
+            // to adjacent floats
+            if (n > KN_LIST) Thi = T;
+            else Tlo = T;
+            float q = T * __powf(88.f / (float)max(n, 1), 0.6666667f);
+            if (it >= 6 || !(q > Tlo && q < Thi)) q = 0.5f * (Tlo + Thi);
+            if (!(q > Tlo && q < Thi) || it >= 64) return KN_FAIL;
+            T = q;
+            continue;
+        }
+        // t = the 64th smallest: the largest after n - 64 removals, or, when
+        // the list holds many more, bit by bit (float bits order like values)
+#pragma unroll
+        for (int k = 0; k < KPL; k++) {
+            const int e = lane + 32 * k;
+            du[k] = e < n ? __float_as_uint(S.sel.d[e]) : 0u;
+        }
+        unsigned tb = 0u;
+        if (n - NGB <= 20) {
+            unsigned w[KPL];
+#pragma unroll
+            for (int k = 0; k < KPL; k++) w[k] = du[k];
+            for (int r = n - NGB;; r--) {
+                unsigned m = w[0];
+#pragma unroll
+                for (int k = 1; k < KPL; k++) m = max(m, w[k]);
+                tb = __reduce_max_sync(0xffffffffu, m);
+                if (r == 0) break;
+                const unsigned who = __ballot_sync(0xffffffffu, m == tb);
+                if (lane == __ffs(who) - 1) {
+                    bool gone = false;
+#pragma unroll
+                    for (int k = 0; k < KPL; k++)
+                        if (!gone && w[k] == tb) { w[k] = 0u; gone = true; }
+                }
             }
-            p.kRb[gi] = rb;
-            p.kflag[gi] = done ? 0 : 1;
-            if (!done) {
-                atomicAdd(p.remaining, 1);
-                const int w = atomicAdd(p.nwl_out, 1);
-                if (w < p.item_cap) p.wl_out[w] = gi;
+        } else {
+            // the largest v with fewer than 64 entries below it
+#pragma unroll 1
+            for (int b = 30; b >= 0; b--) {
+                const unsigned v = tb | (1u << b);
+                int c = 0;
+#pragma unroll
+                for (int k = 0; k < KPL; k++) c += (lane + 32 * k < n && du[k] < v) ? 1 : 0;
+                if (__reduce_add_sync(0xffffffffu, c) < NGB) tb = v;
             }
         }
+        t = __uint_as_float(tb);
+        if (t > thr) return KN_UNDER;  // fewer than 64 certainly within R
+        // the bound at a point just above the band's upper end (E << t)
+        const float te = t * 1.0009765625f;
+        E = U * (EA * sqrt_fast(te) + 5.f * te);
+        if (t + 2.f * E <= T) break;
+        T = t + 2.f * E;  // the band reaches past a narrowed radius
+        Tlo = Thi = 0.f;  // (no further narrowing: more entries than the list holds fail)
+    }
+    const float lo = t - 2.f * E, hi = t + 2.f * E;
+    // sure members (fewer than 64 lie below t) to the list, uncertain ones
+    // collected
+    int *outn = p.nbr + (size_t)i * NGB;
+    float *outd = p.nd2 + (size_t)i * NGB;
+    int nS = 0, nu = 0, ju = 0;
+#pragma unroll
+    for (int k = 0; k < KPL; k++) {
+        if (32 * k < n) {  // (uniform)
+            const bool have = lane + 32 * k < n;
+            const float d = __uint_as_float(du[k]);
+            const int j = have ? S.sel.j[lane + 32 * k] : 0;
+            const bool sure = have && d < lo, unc = have && !sure && d <= hi;
+            const unsigned sb = __ballot_sync(0xffffffffu, sure), ub = __ballot_sync(0xffffffffu, unc);
+            if (sure) {
+                const int pos = nS + __popc(sb & ltmask);
+                outn[pos] = j;
+                outd[pos] = d;
+            }
+            if (unc) {
+                const int pos = nu + __popc(ub & ltmask);
+                if (pos < KN_U) S.sel.uj[pos] = j;
+            }
+            nS += __popc(sb);
+            nu += __popc(ub);
+        }
+    }
+    r.E = E;
+    if (nu > KN_U) return KN_FAIL;
+    __syncwarp();
+    if (nu == 1) {  // t itself: nS is 63
+        r.j64 = S.sel.uj[0];
+        return KN_DONE;
+    }
+    const int need = NGB - nS;
+    double hsq = 0.0;
+    int h64 = -1;
+    bool have = false;
+#pragma unroll 1
+    for (int e = lane; e < nu; e += 32) {
+        const int je = S.sel.uj[e];
+        S.sel.uD[e] = __double_as_longlong(exact_d2(p.gx, p.gy, p.gz, i, je));
+        S.sel.ug[e] = p.ggrank[je];
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int e = lane; e < nu; e += 32) {
+        const long long De = S.sel.uD[e];
+        const int ge = S.sel.ug[e];
+        int rk = 0;
+#pragma unroll 1
+        for (int f = 0; f < nu; f++) {  // integer compares: no FP64 work
+            const long long Df = S.sel.uD[f];
+            rk += (Df < De) || (Df == De && S.sel.ug[f] < ge);
+        }
+        if (rk < need) {
+            outn[nS + rk] = S.sel.uj[e];
+            outd[nS + rk] = (float)__longlong_as_double(De);
+        }
+        if (rk == need - 1) { hsq = __longlong_as_double(De); h64 = ge; have = true; }
+    }
+    const unsigned hb = __ballot_sync(0xffffffffu, have);
+    if (hb == 0u) return KN_FAIL;  // error bound violated: fewer uncertain entries than needed
+    const int hs = __ffs(hb) - 1;
+    r.hsq = __shfl_sync(0xffffffffu, hsq, hs);
+    r.g64 = __shfl_sync(0xffffffffu, h64, hs);
+    r.j64 = -1;
+    return KN_DONE;
+}
+
+// The results of the members `done` of a run whose neighbours are selected
+// (lane k: member k, particle first + k, its selection in r): the exact
+// support, lane by lane, then each member's density and pressure sums over
+// the warp, then the equation of state, again lane by lane.
+__device__ __forceinline__ void knn_finish(const KnnParams &p, int first, unsigned done, const KnnSel &r, int lane)
+{
+    const bool mine = (done >> lane) & 1u;
+    const int i = first + lane;
+    float hinv = 0.f;
+    if (mine) {
+        double hsq = r.hsq;
+        int g64 = r.g64;
+        if (r.j64 >= 0) {
+            hsq = exact_d2(p.gx, p.gy, p.gz, i, r.j64);
+            g64 = p.ggrank[r.j64];
+            p.nbr[(size_t)i * NGB + NGB - 1] = r.j64;
+            p.nd2[(size_t)i * NGB + NGB - 1] = (float)hsq;
+        }
+        const float hh = sqrtf((float)hsq);  // within one FP32 rounding of sqrt(h^2)
+        hinv = 1.f / hh;
+        p.h2[i] = hsq;
+        p.h2lo[i] = __double2float_rd(hsq);
+        p.h2hi[i] = __double2float_ru(hsq);
+        p.h[i] = hh;
+        p.g64[i] = g64;
+        p.E[i] = r.E;
+    }
+    __syncwarp();
+    float rho = 0.f, qsum = 0.f;
+#pragma unroll 1
+    for (unsigned m = done; m; m &= m - 1u) {
+        const int k = __ffs(m) - 1;
+        const float hk = __shfl_sync(0xffffffffu, hinv, k);
+        const int *nb = p.nbr + (size_t)(first + k) * NGB;
+        const float *nd = p.nd2 + (size_t)(first + k) * NGB;
+        float rs = 0.f, qs = 0.f;
+#pragma unroll
+        for (int q = 0; q < NGB / 32; q++) {
+            const int j = nb[lane + 32 * q];
+            const float mw = __int_as_float(p.C[j].w) * kern_w(sqrtf(nd[lane + 32 * q]), hk);
+            rs += mw;
+            if (p.pressure) qs = __fmaf_rn(mw, p.gu[j], qs);
+        }
+        rs = warp_sum(rs);
+        if (p.pressure) qs = warp_sum(qs);
+        if (lane == k) { rho = rs; qsum = qs; }
+    }
+    if (mine) {
+        const float P = p.pressure ? (p.gamma - 1.f) * qsum : (p.gamma - 1.f) * rho * p.gu[i];
+        p.rho[i] = rho;
+        p.P[i] = P;
+        p.cs[i] = sqrtf(p.gamma * P / rho);
+    }
+}
+
+// Kernel-size search of the run [first, first + len), len <= 32, from radius
+// R0 (see the file comment).  KN_FAIL: some member could not be ranked within
+// the buffers.
+__device__ __forceinline__ int knn_run(KnnWarp &S, const KnnParams &p, int first, int len, float R0, float unit,
+                                       bool &widened, int lane)
+{
+    KnnBox B;
+    const bool mine = lane < len;
+    int4 C = make_int4(0, 0, 0, 0);
+    float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
+    float hp = 0.f;
+    if (mine) {
+        C = p.C[first + lane];
+        r = p.R[first + lane];
+        hp = p.rprev[first + lane];
+    }
+    const int cc[3] = {C.x, C.y, C.z};
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        B.b0[a] = __reduce_min_sync(0xffffffffu, mine ? cc[a] : 0x7fffffff);
+        B.b1[a] = __reduce_max_sync(0xffffffffu, mine ? cc[a] : -1);
+        B.gref[a] = (B.b0[a] + B.b1[a]) >> 1;
+        B.lo[a] = (float)(B.b0[a] - B.gref[a]) * unit;
+        B.hi[a] = (float)(B.b1[a] + 1 - B.gref[a]) * unit;
+    }
+    const float xo = grid_off(C.x, B.gref[0], r.x, unit);
+    const float yo = grid_off(C.y, B.gref[1], r.y, unit);
+    const float zo = grid_off(C.z, B.gref[2], r.z, unit);
+    const bool known = __all_sync(0xffffffffu, !mine || hp > 0.f);
+    const unsigned hmax = __reduce_max_sync(0xffffffffu, __float_as_uint(hp));
+    float R = known ? p.margin * __uint_as_float(hmax) : R0;
+    const float xs = __shfl_sync(0xffffffffu, xo, 0), ys = __shfl_sync(0xffffffffu, yo, 0),
+                zs = __shfl_sync(0xffffffffu, zo, 0);
+    unsigned todo = len == 32 ? 0xffffffffu : (1u << len) - 1u;
+    float Rlo = 0.f, Rhi = 0.f;  // radii known to be too small and too large
+    for (int it = 0; it < 96; it++) {
+        int nc;
+        float amax;
+        if (!knn_walk(S, p, B, R, unit, len == 1, xs, ys, zs, nc, amax, lane)) {
+            if (len > 1) return KN_FAIL;
+            Rhi = R;
+            R = Rlo > 0.f ? 0.5f * (R + Rlo) : 0.6f * R;
+            if (!(R > Rlo && R < Rhi)) return KN_FAIL;
+            continue;
+        }
+        // the run's own particles also bound the offsets
+        if (mine) amax = fmaxf(amax, xo * xo + yo * yo + zo * zo);
+        amax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(amax)));
+        // error bound of an FP32 d^2 near D (see the file comment)
+        const float EA = 6.92820323f * (sqrtf(amax) + 2.f * unit);  // 4 sqrt(3) A'
+        // lane k: member k's radius (its own previous support's, or R), thr
+        // and T0: fewer than 64 with d^2 <= thr lie certainly within it, and
+        // t + 2 E(t) <= T0 for every t <= thr
+        unsigned left = 0u, done = 0u;
+        float grow = 1.f;  // the factor by which R falls short, from the counts within it
+        KnnSel sel;
+        sel.j64 = -1; sel.g64 = 0; sel.E = 0.f; sel.hsq = 0.0;
+        const float Rk = hp > 0.f ? fminf(R, p.margin * hp) : R;
+        unsigned m = todo;
+        bool wide = false;  // the member found too few within its own radius: now within R
+#pragma unroll 1
+        while (m) {
+            const int k = __ffs(m) - 1;
+            const float rk = __shfl_sync(0xffffffffu, Rk, k), Ri = wide ? R : rk;
+            const float xi = __shfl_sync(0xffffffffu, xo, k), yi = __shfl_sync(0xffffffffu, yo, k),
+                        zi = __shfl_sync(0xffffffffu, zo, k);
+            constexpr float U = 1.1920929e-07f;  // 2^-23
+            const float R2 = Ri * Ri;
+            const float thr = R2 - U * (EA * Ri + 5.f * R2);
+            const float T0 = R2 + 2.f * U * (EA * (Ri * 1.0005f) + 5.01f * R2);
+            KnnSel one;
+            int n = 0;
+            const int rc = knn_select(S, p, first + k, nc, xi, yi, zi, thr, T0, EA, n, one, lane);
+            if (rc == KN_FAIL) return KN_FAIL;
+            if (rc == KN_UNDER && Ri < R) {
+                wide = true;
+                continue;
+            }
+            if (rc == KN_UNDER) {
+                left |= 1u << k;
+                grow = fmaxf(grow, KN_GROW * cbrtf((float)NGB / (float)max(min(n, NGB), 1)));
+            } else {
+                done |= 1u << k;
+                if (lane == k) sel = one;
+            }
+            wide = false;
+            m &= m - 1u;
+        }
+        knn_finish(p, first, done, sel, lane);
+        if (left == 0u) return KN_DONE;
+        widened = true;
+        todo = left;
+        Rlo = R;
+        R = Rhi > 0.f ? 0.5f * (R + Rhi) : fminf(grow, 1.6f) * R;
+        if (Rhi > 0.f && !(R > Rlo && R < Rhi)) return KN_FAIL;
+    }
+    return KN_FAIL;
+}
+
+__global__ void __launch_bounds__(KN_THREADS, KN_CTAS) k_knn(KnnParams p)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    KnnWarp &S = reinterpret_cast<KnnWarp *>(smem_raw)[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    const float unit = (float)p.box[4];
+    const int nitems = *p.nitems;
+    for (;;) {
+        int it = 0;
+        if (lane == 0) it = atomicAdd(p.next, 1);
+        it = __shfl_sync(0xffffffffu, it, 0);
+        if (it >= nitems) break;
+        const int2 item = p.item[it];
+        const float R0 = p.kR[it];
+        bool widened = false;
+        const int end = item.x + item.y;
+        int step = item.y;
+        for (int pos = item.x; pos < end;) {
+            const int len = min(step, end - pos);
+            if (knn_run(S, p, pos, len, R0, unit, widened, lane) == KN_DONE) {
+                pos += len;
+            } else if (len > 1) {
+                // the members do not fit the buffers together: smaller runs
+                // (each with the radius of its own members), then singles
+                step = len > KN_SUB ? KN_SUB : 1;
+            } else {
+                if (lane == 0) atomicOr(p.status, ST_KNN_OVERFLOW);
+                pos++;
+            }
+        }
+        if (widened && lane == 0) atomicAdd(p.nunder, 1);
     }
 }
 
@@ -782,19 +796,16 @@ struct ForceParams {
 // U = 1 for density-energy SPH; Y = (gamma-1) u / P, U = (gamma-1) u for
 // pressure-energy SPH with the smoothed P, whose pair coefficients are
 // (gamma-1)^2 u_i u_j / P_i and / P_j.
-__global__ void k_force_pack(int ng, const int *__restrict__ gcx, const int *__restrict__ gcy,
-                             const int *__restrict__ gcz, const float *__restrict__ grx, const float *__restrict__ gry,
-                             const float *__restrict__ grz, const float *__restrict__ gm, const float *__restrict__ gvx,
-                             const float *__restrict__ gvy, const float *__restrict__ gvz, const float *__restrict__ h,
+__global__ void k_force_pack(int ng, const float *__restrict__ gvx, const float *__restrict__ gvy,
+                             const float *__restrict__ gvz, const float *__restrict__ h,
                              const float *__restrict__ rho, const float *__restrict__ P, const float *__restrict__ cs,
-                             const float *__restrict__ gu, float gamma, int pressure, int4 *__restrict__ C,
-                             float4 *__restrict__ R, float4 *__restrict__ V, float4 *__restrict__ Q)
+                             const float *__restrict__ gu, float gamma, int pressure, float4 *__restrict__ R,
+                             float4 *__restrict__ V, float4 *__restrict__ Q)
 {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= ng) return;
     const float rj = rho[j];
-    C[j] = make_int4(gcx[j], gcy[j], gcz[j], __float_as_int(gm[j]));
-    R[j] = make_float4(grx[j], gry[j], grz[j], 1.f / h[j]);
+    R[j].w = 1.f / h[j];  // the rest of R, and C, come from the gas gather
     V[j] = make_float4(gvx[j], gvy[j], gvz[j], cs[j]);
     if (pressure) {
         const float U = (gamma - 1.f) * gu[j];
@@ -914,40 +925,18 @@ int sph_density(gnb_ctx *c)
     GNB_TRY(gas_slots(c, a.type, c->n_d, c->gslot));
     GasGather gg;
     gg.skey = c->skey; gg.p = a; gg.gslot = c->gslot; gg.gkey = c->gkey;
-    gg.gcx = c->gcx; gg.gcy = c->gcy; gg.gcz = c->gcz; gg.ggrank = c->ggrank;
-    gg.grx = c->grx; gg.gry = c->gry; gg.grz = c->grz; gg.gm = c->gm;
+    gg.ggrank = c->ggrank; gg.C = c->fC; gg.R = c->fR;
     gg.gvx = c->gvx; gg.gvy = c->gvy; gg.gvz = c->gvz; gg.gu = c->gu; gg.gRprev = c->gRprev;
     gg.gx = c->gx; gg.gy = c->gy; gg.gz = c->gz;
     gg.ng = ng; gg.pred = c->use_pred ? 1 : 0; gg.have_h = c->have_h ? 1 : 0;
     gnb::counted(k_gas_gather)<<<gb, 256, 0, c->s>>>(gg);
     GNB_LAUNCH_CHECK(c, "gas gather");
-    // hydro tree and groups of <= 32 gas particles (measured on the 2^24 disk
-    // with the adaptive search margin: 7.05 ms for the kernel-size pass
-    // against 7.12 with 24, 7.17 with 48 and 7.57 with 16; with the fixed
-    // 1.1 margin 16 was best, since a wider radius makes a larger group's
-    // candidates overflow)
-    GNB_TRY(build_tree(c, c->gt, c->gkey, ng, c->ngas_d, c->cfg.n_leaf, 32, c->gcx, c->gcy, c->gcz, c->grx,
-                       c->gry, c->grz, c->gm, c->gm, false));
+    // hydro tree and groups of at most 32 gas particles (a lane each in the search)
+    GNB_TRY(build_tree(c, c->gt, c->gkey, ng, c->ngas_d, c->cfg.n_leaf, KN_GROUP, nullptr, nullptr, nullptr, nullptr,
+                       nullptr, nullptr, nullptr, nullptr, false));
+    if (c->gt.nnodes >= 1 << 29) return fail(c, GNB_ECAPACITY, "hydro tree nodes");
     phase_begin(c, GNB_T_KNN);
-    // work_d: [0] next item, [1] items left unfinished, [2] live item count, [3] per-pass snapshot
-    gnb::counted(k_knn_init)<<<304, 256, 0, c->s>>>(c->gt, c->gRprev, c->have_h ? 1 : 0, c->knn_margin, c->box_d, c->kR,
-                                      c->kRb, c->kflag, c->kitem, c->work_d + 2);
-    GNB_LAUNCH_CHECK(c, "knn init");
-    KnnParams p;
-    p.na = c->gt.na; p.nb = c->gt.nb; p.item = c->kitem; p.nitems = c->work_d + 2; p.nsnap = c->work_d + 3;
-    p.item_cap = (int)(2 * c->gcap + 1);
-    p.gcx = c->gcx; p.gcy = c->gcy; p.gcz = c->gcz; p.ggrank = c->ggrank;
-    p.grx = c->grx; p.gry = c->gry; p.grz = c->grz; p.gm = c->gm; p.gu = c->gu;
-    p.gx = c->gx; p.gy = c->gy; p.gz = c->gz; p.box = c->box_d;
-    p.kR = c->kR; p.kRb = c->kRb; p.kflag = c->kflag;
-    p.rprev = c->gRprev;
-    p.margin = c->knn_margin;
-    p.nunder = c->work_d + 6;
-    cudaMemsetAsync(c->work_d + 6, 0, sizeof(int), c->s);
-    p.next = c->work_d; p.remaining = c->work_d + 1; p.status = c->status_d;
-    p.nbr = c->nbr; p.nd2 = c->nd2; p.h2 = c->gh2; p.h2lo = c->gh2lo; p.h2hi = c->gh2hi; p.h = c->gh; p.E = c->gE; p.rho = c->grho; p.P = c->gP;
-    p.cs = c->gcs; p.g64 = c->g64; p.gamma = (float)c->cfg.gamma; p.pressure = c->cfg.sph_variant;
-    size_t smem = sizeof(KnnSmem);
+    size_t smem = KN_WARPS * sizeof(KnnWarp);
     cudaError_t e = cudaFuncSetAttribute(k_knn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_check(c, e, "knn smem attribute");
     if (g_knn_blocks == 0) {
@@ -957,47 +946,41 @@ int sph_density(gnb_ctx *c)
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_knn, KN_THREADS, smem);
         g_knn_blocks = sms * (per > 0 ? per : 1);
     }
-    int passes = 0;
-    const int rounds = 12;
-    for (int round = 0; round < rounds; round++) {
-        // four device passes per host check; each pass takes the worklist
-        // the previous one wrote (the first takes every item)
-        for (int q = 0; q < 4; q++) {
-            const int o = passes & 1;
-            cudaMemsetAsync(c->work_d, 0, 2 * sizeof(int), c->s);
-            cudaMemsetAsync(c->work_d + 4 + o, 0, sizeof(int), c->s);
-            if (passes == 0) {
-                cudaMemcpyAsync(c->work_d + 3, c->work_d + 2, sizeof(int), cudaMemcpyDeviceToDevice, c->s);
-                p.nsnap = c->work_d + 3;
-                p.wl_in = nullptr;
-            } else {
-                p.nsnap = c->work_d + 4 + (o ^ 1);
-                p.wl_in = c->kwl[o ^ 1];
-            }
-            p.wl_out = c->kwl[o];
-            p.nwl_out = c->work_d + 4 + o;
-            gnb::counted(k_knn)<<<g_knn_blocks, KN_THREADS, smem, c->s>>>(p);
-            passes++;
-        }
-        GNB_LAUNCH_CHECK(c, "knn");
-        cudaMemcpyAsync(c->pinned_i, c->work_d + 1, sizeof(int), cudaMemcpyDeviceToHost, c->s);
-        cudaMemcpyAsync(c->pinned_i + 20, c->work_d + 3, sizeof(int), cudaMemcpyDeviceToHost, c->s);
-        cudaMemcpyAsync(c->pinned_i + 21, c->work_d + 6, sizeof(int), cudaMemcpyDeviceToHost, c->s);
-        cudaMemcpyAsync(c->pinned_i + 1, c->status_d, sizeof(int), cudaMemcpyDeviceToHost, c->s);
-        GNB_TRY(cuda_check(c, cudaStreamSynchronize(c->s), "knn sync"));
-        if (c->pinned_i[1] & ST_KNN_OVERFLOW) return fail(c, GNB_ECAPACITY, "kNN selection buffer overflow");
-        if (c->pinned_i[0] == 0) break;
-        if (round == rounds - 1) return fail(c, GNB_ECAPACITY, "kNN search radius did not converge");
-    }
-    c->stats[GNB_S_KNN_PASSES] = passes;
-    // the next evaluation's margin: wider when more than 4 % of the work
-    // items needed a larger radius, narrower (to 1.01) below 1 %.  On the
-    // 2^24 disk (dt = 1e-3) a margin of 1.01 retries no item and takes
-    // 7.57 ms for the pass, 1.05 7.83 ms, 1.1 8.21 ms; 1.0 retries 78 % of
-    // the items (a support that did not shrink needs more than itself) and
-    // takes 16.4 ms
+    // particles per work item (a lane each, at most KN_GROUP).  A longer run
+    // shares its walk and its candidates; a shorter one spreads a small set
+    // over more warps and, in three dimensions, gathers fewer candidates per
+    // member.  Measured at 30 k gas particles: 2 per item 111 us, 4 125, 8 159;
+    // 1e5: 4 270, 8 300, 16 361; 210 k: 4 461, 8 453, 16 506; 1.68 M: 4 3.52
+    // ms, 8 3.07, 16 2.97.
+    const int steps[4] = {4, 12, 40, 256};  // gas particles per resident warp
+    int sub = 1;
+    for (int q : steps)
+        if ((long long)ng > (long long)q * g_knn_blocks * KN_WARPS) sub *= 2;
+    // work_d: [0] next item, [1] items whose radius was widened, [2] items
+    cudaMemsetAsync(c->work_d, 0, 3 * sizeof(int), c->s);
+    gnb::counted(k_knn_init)<<<304, 256, 0, c->s>>>(c->gt, sub, c->box_d, c->kR, c->kitem, c->work_d + 2);
+    KnnParams p;
+    p.na = c->gt.na; p.nb = c->gt.nb; p.item = c->kitem; p.kR = c->kR; p.nitems = c->work_d + 2;
+    p.next = c->work_d; p.nunder = c->work_d + 1;
+    p.C = c->fC; p.R = c->fR; p.ggrank = c->ggrank; p.gu = c->gu;
+    p.gx = c->gx; p.gy = c->gy; p.gz = c->gz; p.box = c->box_d;
+    p.rprev = c->gRprev;
+    p.margin = c->knn_margin;
+    p.status = c->status_d;
+    p.nbr = c->nbr; p.nd2 = c->nd2; p.h2 = c->gh2; p.h2lo = c->gh2lo; p.h2hi = c->gh2hi; p.h = c->gh; p.E = c->gE;
+    p.rho = c->grho; p.P = c->gP; p.cs = c->gcs; p.g64 = c->g64;
+    p.gamma = (float)c->cfg.gamma; p.pressure = c->cfg.sph_variant;
+    gnb::counted(k_knn)<<<g_knn_blocks, KN_THREADS, smem, c->s>>>(p);
+    GNB_LAUNCH_CHECK(c, "knn");
+    cudaMemcpyAsync(c->pinned_i, c->work_d, 3 * sizeof(int), cudaMemcpyDeviceToHost, c->s);
+    cudaMemcpyAsync(c->pinned_i + 20, c->status_d, sizeof(int), cudaMemcpyDeviceToHost, c->s);
+    GNB_TRY(cuda_check(c, cudaStreamSynchronize(c->s), "knn sync"));
+    if (c->pinned_i[20] & ST_KNN_OVERFLOW) return fail(c, GNB_ECAPACITY, "kNN selection buffer overflow");
+    c->stats[GNB_S_KNN_PASSES] = 1;
+    // the next evaluation's margin: wider when more than 4 % of the items
+    // needed a larger radius, narrower (to 1.01) below 1 %
     if (c->have_h) {
-        const double under = (double)c->pinned_i[21] / (double)std::max(1, c->pinned_i[20]);
+        const double under = (double)c->pinned_i[1] / (double)std::max(1, c->pinned_i[2]);
         if (under > 0.04) c->knn_margin = std::min(1.5f, c->knn_margin * 1.05f);
         else if (under < 0.01) c->knn_margin = std::max(1.01f, c->knn_margin / 1.02f);
     }
@@ -1024,10 +1007,8 @@ int sph_force(gnb_ctx *c)
     cudaMemsetAsync(c->rfill, 0, sizeof(int) * ng, c->s);
     gnb::counted(k_rev_fill)<<<gb, 256, 0, c->s>>>(ng, c->nbr, c->mut, c->roff, c->rfill, c->rlist);
     GNB_LAUNCH_CHECK(c, "symmetric lists");
-    gnb::counted(k_force_pack)<<<gb, 256, 0, c->s>>>(ng, c->gcx, c->gcy, c->gcz, c->grx, c->gry, c->grz, c->gm, c->gvx,
-                                                     c->gvy, c->gvz, c->gh, c->grho, c->gP, c->gcs, c->gu,
-                                                     (float)c->cfg.gamma, c->cfg.sph_variant, c->fC, c->fR, c->fV,
-                                                     c->fQ);
+    gnb::counted(k_force_pack)<<<gb, 256, 0, c->s>>>(ng, c->gvx, c->gvy, c->gvz, c->gh, c->grho, c->gP, c->gcs, c->gu,
+                                                     (float)c->cfg.gamma, c->cfg.sph_variant, c->fR, c->fV, c->fQ);
     ForceParams p;
     p.ng = ng; p.nbr = c->nbr; p.roff = c->roff; p.rcnt = c->rcnt; p.rlist = c->rlist;
     p.C = c->fC; p.R = c->fR; p.V = c->fV; p.Q = c->fQ;

@@ -30,3 +30,38 @@ def test_tree_topology_at_tile_edges(G, orc, n):
     links = c.get("NODE_LINKS").reshape(-1, 3)
     assert np.array_equal(links[:, 0], tree["child"]) and np.array_equal(links[:, 1], tree["nchild"])
     assert np.array_equal(np.sort(c.get("GROUPS")), np.sort(orc.groups(tree, 64)))
+
+
+def _clump(seed):
+    """A dense ball inside a wide one: runs whose candidates overflow, and outer
+    particles that see the ball as a thin shell."""
+    rng = np.random.default_rng(seed)
+    d = rng.normal(size=(1400, 3))
+    d /= np.linalg.norm(d, axis=1, keepdims=True)
+    r = np.where(np.arange(1400) < 1200, 1e-3, 3.0) * rng.uniform(0.0, 1.0, 1400) ** (1.0 / 3.0)
+    p = ics.uniform_random(1400, seed=seed)
+    x = d * r[:, None] + 0.3
+    return dict(p, x=x[:, 0].copy(), y=x[:, 1].copy(), z=x[:, 2].copy())
+
+
+# kernel-size search: the smallest sets, runs of 1 | 2 and 2 | 4 particles (4
+# and 12 gas particles per resident warp of 152 SMs x 24), and a clump; then
+# the same particles spread out, so that every support outgrows its search
+# radius
+@pytest.mark.parametrize("case", [64, 66, 14592, 14593, 43777, "clump"])
+def test_kernel_sizes_exact_twice(G, orc, case):
+    p = _clump(5) if case == "clump" else ics.uniform_random(case, seed=case)
+    n = p["x"].size
+    rng = np.random.default_rng(1)
+    sample = np.arange(n) if n <= 2000 else np.sort(rng.choice(n, 600, replace=False))
+    c = G.Context()
+    c.set_particles(p)
+    for k in range(2):
+        if k:
+            s = 1.0 + 0.7 * rng.uniform(0.9, 1.1)
+            p = dict(p, x=s * p["x"], y=s * p["y"], z=1.1 * s * p["z"])
+            c.replace_region({q: p[q] for q in ("id", "x", "y", "z", "vx", "vy", "vz", "u")})
+        c.compute_sph_density()
+        nbr, h2 = orc.knn({q: np.asarray(p[q], np.float64) for q in ("x", "y", "z", "m", "u")}, 64, sample=sample)
+        assert np.array_equal(c.get("NBR")[sample], np.sort(nbr, axis=1))
+        assert np.array_equal(c.get("H2")[sample], h2)
