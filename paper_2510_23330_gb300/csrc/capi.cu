@@ -77,18 +77,17 @@ static void free_particles(gnb_ctx *c)
 
 static void free_gas(gnb_ctx *c)
 {
-    void *all[] = {c->gslot, c->gkey, c->ggrank, c->gx, c->gy, c->gz, c->gvx, c->gvy, c->gvz, c->gu, c->gh2, c->gh, c->g64, c->grho, c->gP, c->gcs,
-                   c->gRprev, c->gE, c->nbr, c->nd2, c->mut, c->rcnt, c->roff, c->rfill, c->rlist, c->hax,
-                   c->hay, c->haz, c->hdu, c->kR, c->kitem, c->gvsig,
-                   c->gh2lo, c->gh2hi, c->fC, c->fR, c->fV, c->fQ};
+    void *all[] = {c->gslot, c->gkey, c->ggrank, c->gx, c->gy, c->gz, c->gvx, c->gvy, c->gvz, c->gu, c->gh2, c->gh, c->g64,
+                   c->gRprev, c->gE, c->nbr, c->nd2, c->mut, c->rcnt, c->roff, c->rcur, c->rlist,
+                   c->kR, c->kitem, c->gvsig, c->gh2b, c->fC, c->fR, c->fV, c->fQ};
     for (void *q : all) dfree(c, q);
     c->gslot = nullptr; c->gkey = nullptr; c->ggrank = nullptr;
     c->gx = c->gy = c->gz = nullptr;
     c->gvx = c->gvy = c->gvz = c->gu = nullptr; c->gh2 = nullptr; c->gh = nullptr; c->g64 = nullptr;
-    c->grho = c->gP = c->gcs = c->gRprev = c->gE = nullptr; c->nbr = nullptr; c->nd2 = nullptr; c->mut = nullptr;
-    c->rcnt = c->roff = c->rfill = c->rlist = nullptr; c->hax = c->hay = c->haz = c->hdu = nullptr;
+    c->gRprev = c->gE = nullptr; c->nbr = nullptr; c->nd2 = nullptr; c->mut = nullptr;
+    c->rcnt = c->roff = c->rcur = c->rlist = nullptr;
     c->kR = nullptr; c->kitem = nullptr; c->gvsig = nullptr;
-    c->gh2lo = c->gh2hi = nullptr;
+    c->gh2b = nullptr;
     c->fC = nullptr; c->fR = nullptr; c->fV = nullptr; c->fQ = nullptr;
     tree_free(c, c->gt);
     c->gcap = 0;
@@ -128,16 +127,13 @@ static int alloc_gas(gnb_ctx *c, int64_t ng)
     GNB_TRY(dalloc(c, &c->gvx, G)); GNB_TRY(dalloc(c, &c->gvy, G));
     GNB_TRY(dalloc(c, &c->gvz, G)); GNB_TRY(dalloc(c, &c->gu, G));
     GNB_TRY(dalloc(c, &c->gh2, G)); GNB_TRY(dalloc(c, &c->gh, G)); GNB_TRY(dalloc(c, &c->g64, G));
-    GNB_TRY(dalloc(c, &c->grho, G)); GNB_TRY(dalloc(c, &c->gP, G)); GNB_TRY(dalloc(c, &c->gcs, G));
     GNB_TRY(dalloc(c, &c->gRprev, G)); GNB_TRY(dalloc(c, &c->gE, G)); GNB_TRY(dalloc(c, &c->gvsig, G));
     GNB_TRY(dalloc(c, &c->nbr, G * 64)); GNB_TRY(dalloc(c, &c->nd2, G * 64)); GNB_TRY(dalloc(c, &c->mut, G));
-    GNB_TRY(dalloc(c, &c->rcnt, G + 1)); GNB_TRY(dalloc(c, &c->roff, G + 1)); GNB_TRY(dalloc(c, &c->rfill, G + 1));
+    GNB_TRY(dalloc(c, &c->rcnt, G + 1)); GNB_TRY(dalloc(c, &c->roff, G + 1)); GNB_TRY(dalloc(c, &c->rcur, G + 1));
     GNB_TRY(dalloc(c, &c->rlist, G * 64));
     cudaMemsetAsync(c->nbr, 0, sizeof(int) * G * 64, c->s);  // list entries are always valid indices
-    GNB_TRY(dalloc(c, &c->hax, G)); GNB_TRY(dalloc(c, &c->hay, G)); GNB_TRY(dalloc(c, &c->haz, G));
-    GNB_TRY(dalloc(c, &c->hdu, G));
     GNB_TRY(dalloc(c, &c->kR, G)); GNB_TRY(dalloc(c, &c->kitem, G));
-    GNB_TRY(dalloc(c, &c->gh2lo, G)); GNB_TRY(dalloc(c, &c->gh2hi, G));
+    GNB_TRY(dalloc(c, &c->gh2b, G));
     GNB_TRY(dalloc(c, &c->fC, G)); GNB_TRY(dalloc(c, &c->fR, G)); GNB_TRY(dalloc(c, &c->fV, G));
     GNB_TRY(dalloc(c, &c->fQ, G));
     c->gcap = ng;

@@ -133,25 +133,22 @@ struct gnb_ctx {
     double *gh2 = nullptr;        // exact FP64 d^2 of the n_ngb-th neighbour
     float *gh = nullptr;          // h in FP32
     int *g64 = nullptr;           // gas rank of the n_ngb-th neighbour
-    float *grho = nullptr, *gP = nullptr, *gcs = nullptr;
     float *gRprev = nullptr;      // search radius hint per gas particle
     float *gE = nullptr;          // FP32 distance error bound used for the particle's list
     float *gvsig = nullptr;       // largest pair signal velocity of the last force pass
     unsigned long long *mut = nullptr;  // per gas particle: mutual-neighbour bits
     int *nbr = nullptr;           // n_gas * 64 gas indices
     float *nd2 = nullptr;         // n_gas * 64 FP32 d^2
-    int *rcnt = nullptr, *roff = nullptr, *rfill = nullptr, *rlist = nullptr;
+    int *rcnt = nullptr, *roff = nullptr, *rcur = nullptr, *rlist = nullptr;
     int *rtot_d = nullptr;
-    int64_t rlist_cap = 0;
-    float *hax = nullptr, *hay = nullptr, *haz = nullptr, *hdu = nullptr;
     float *kR = nullptr;          // kNN work items: starting radius without a previous support
     int2 *kitem = nullptr;        // kNN work items (first, count)
-    float *gh2lo = nullptr, *gh2hi = nullptr;  // h^2 rounded down / up to FP32 (per gas)
+    float2 *gh2b = nullptr;       // h^2 rounded down / up to FP32 (per gas)
     // per-gas records the kernel-size search and the hydro force gather for particle j
     int4 *fC = nullptr;           // cell x, y, z, mass bits
-    float4 *fR = nullptr;         // residual x, y, z, and 1/h once the force pass packs it
+    float4 *fR = nullptr;         // residual x, y, z, -
     float4 *fV = nullptr;         // v x, y, z, sound speed
-    float4 *fQ = nullptr;         // rho, Y, U, - (pair coefficient U_j Y_i of gW(h_i); see sph.cu)
+    float4 *fQ = nullptr;         // rho, Y, U, 1/h (pair coefficient U_j Y_i of gW(h_i); see sph.cu)
 
     // supernova surrogate (surrogate.cu)
     int *sreg = nullptr;          // region of each particle slot (-1: none)

@@ -168,9 +168,14 @@ struct KnnParams {
     int *nbr;
     float *nd2;
     double *h2;
-    float *h2lo, *h2hi;
-    float *h, *E, *rho, *P, *cs;
+    float2 *h2b;         // h^2 rounded down and up to FP32
+    float *h, *E;
     int *g64;
+    const float *gvx, *gvy, *gvz;
+    float4 *V, *Q;       // records of the force pass (see pair_force)
+    const int *gslot;    // particle slot of each gas particle, and the fields per slot
+    float *s_rho, *s_pres, *s_cs;
+    double *s_h2;
     float gamma;
     int pressure;  // 1: also smooth P = (gamma - 1) sum_j m_j u_j W_ij (pressure-energy SPH)
 };
@@ -552,11 +557,11 @@ __device__ __forceinline__ void knn_finish(const KnnParams &p, int first, unsign
         const float hh = sqrtf((float)hsq);  // within one FP32 rounding of sqrt(h^2)
         hinv = 1.f / hh;
         p.h2[i] = hsq;
-        p.h2lo[i] = __double2float_rd(hsq);
-        p.h2hi[i] = __double2float_ru(hsq);
+        p.h2b[i] = make_float2(__double2float_rd(hsq), __double2float_ru(hsq));
         p.h[i] = hh;
         p.g64[i] = g64;
         p.E[i] = r.E;
+        p.s_h2[p.gslot[i]] = hsq;
     }
     __syncwarp();
     float rho = 0.f, qsum = 0.f;
@@ -579,10 +584,20 @@ __device__ __forceinline__ void knn_finish(const KnnParams &p, int first, unsign
         if (lane == k) { rho = rs; qsum = qs; }
     }
     if (mine) {
-        const float P = p.pressure ? (p.gamma - 1.f) * qsum : (p.gamma - 1.f) * rho * p.gu[i];
-        p.rho[i] = rho;
-        p.P[i] = P;
-        p.cs[i] = sqrtf(p.gamma * P / rho);
+        const float u = p.gu[i];
+        const float P = p.pressure ? (p.gamma - 1.f) * qsum : (p.gamma - 1.f) * rho * u;
+        const float cs = sqrtf(p.gamma * P / rho);
+        const int s = p.gslot[i];
+        p.s_rho[s] = rho;
+        p.s_pres[s] = P;
+        p.s_cs[s] = cs;
+        p.V[i] = make_float4(p.gvx[i], p.gvy[i], p.gvz[i], cs);
+        if (p.pressure) {
+            const float U = (p.gamma - 1.f) * u;
+            p.Q[i] = make_float4(rho, U / P, U, hinv);
+        } else {
+            p.Q[i] = make_float4(rho, P / (rho * rho), 1.f, hinv);
+        }
     }
 }
 
@@ -728,53 +743,96 @@ __global__ void __launch_bounds__(KN_THREADS, KN_CTAS) k_knn(KnnParams p)
 // rate).  Only a pair that test leaves open takes the FP64 test and, within
 // its band, the exact FP64 d^2.  Every decision the FP32 test takes is the
 // one the FP64 test would take.
-__global__ void k_mutual(int ng, const int *__restrict__ nbr, const float *__restrict__ nd2,
-                         const float *__restrict__ E, const double *__restrict__ h2, const float *__restrict__ h2lo,
-                         const float *__restrict__ h2hi, const int *__restrict__ g64, const int *__restrict__ grank,
-                         const double *__restrict__ x, const double *__restrict__ y, const double *__restrict__ z,
-                         unsigned long long *__restrict__ mut, int *__restrict__ rcnt)
+//
+// SL lanes share a particle here and in the list fill: a lane takes every
+// SL-th entry, so a row of the list is read in whole sectors and the gathers
+// of a particle overlap (one thread per particle: a chain of 64 reads).
+template <int SL>
+__global__ void __launch_bounds__(256) k_mutual(int ng, const int *__restrict__ nbr, const float *__restrict__ nd2,
+                                                const float *__restrict__ E, const double *__restrict__ h2,
+                                                const float2 *__restrict__ h2b, const int *__restrict__ g64,
+                                                const int *__restrict__ grank, const double *__restrict__ x,
+                                                const double *__restrict__ y, const double *__restrict__ z,
+                                                unsigned long long *__restrict__ mut, int *__restrict__ rcnt,
+                                                int *__restrict__ rtot)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= ng) return;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t == 0) *rtot = 0;  // summed by k_rev_off
+    const int i = t / SL, l = threadIdx.x & (SL - 1), half = (threadIdx.x & 31) / SL;
+    const bool valid = i < ng;
     unsigned long long mask = 0ull;
-    const float Ei = E[i];
+    const float Ei = valid ? E[i] : 0.f;
     const float e2 = 2.f * Ei;  // exact
-    int gi = grank[i];
-    for (int k = 0; k < NGB; k++) {
-        int j = nbr[(size_t)i * NGB + k];
-        if (j == i) { mask |= 1ull << k; continue; }
-        const float df = nd2[(size_t)i * NGB + k];
-        bool m;
-        if (__fadd_ru(df, e2) < h2lo[j]) m = true;
-        else if (__fsub_rd(df, e2) > h2hi[j]) m = false;
-        else {
-            double d = (double)df;
-            double hj = h2[j];
-            double e = 2.0 * (double)Ei;
-            if (d + e < hj) m = true;
-            else if (d - e > hj) m = false;
-            else {
-                double D = exact_d2(x, y, z, i, j);
-                m = (D < hj) || (D == hj && gi <= g64[j]);
-            }
-        }
-        if (m) mask |= 1ull << k;
-        else atomicAdd(&rcnt[j], 1);
+    int jk[NGB / SL];
+    float dk[NGB / SL];
+#pragma unroll
+    for (int q = 0; q < NGB / SL; q++) {
+        jk[q] = valid ? nbr[(size_t)i * NGB + q * SL + l] : 0;
+        dk[q] = valid ? nd2[(size_t)i * NGB + q * SL + l] : 0.f;
     }
-    mut[i] = mask;
+#pragma unroll
+    for (int q = 0; q < NGB / SL; q++) {
+        const int j = jk[q];
+        const float df = dk[q];
+        bool m = true;
+        if (valid && j != i) {
+            const float2 hb = h2b[j];
+            if (__fadd_ru(df, e2) < hb.x) m = true;
+            else if (__fsub_rd(df, e2) > hb.y) m = false;
+            else {
+                double d = (double)df;
+                double hj = h2[j];
+                double e = 2.0 * (double)Ei;
+                if (d + e < hj) m = true;
+                else if (d - e > hj) m = false;
+                else {
+                    double D = exact_d2(x, y, z, i, j);
+                    m = (D < hj) || (D == hj && grank[i] <= g64[j]);
+                }
+            }
+            if (!m) atomicAdd(&rcnt[j], 1);
+        }
+        const unsigned bal = __ballot_sync(0xffffffffu, m);
+        mask |= (unsigned long long)((bal >> (SL * half)) & ((1u << SL) - 1u)) << (q * SL);
+    }
+    if (valid && l == 0) mut[i] = mask;
 }
 
-__global__ void k_rev_fill(int ng, const int *__restrict__ nbr, const unsigned long long *__restrict__ mut,
-                           const int *__restrict__ roff, int *__restrict__ rfill, int *__restrict__ rlist)
+// Storage of the reverse lists: each particle's segment of rlist, taken in
+// blocks of a warp's particles from a running total (their order does not
+// matter, so no scan over all particles is needed).
+__global__ void __launch_bounds__(256) k_rev_off(int ng, const int *__restrict__ rcnt, int *__restrict__ roff,
+                                                 int *__restrict__ rcur, int *__restrict__ rtot)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    const int v = i < ng ? rcnt[i] : 0;
+    int inc = v;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    int base = 0;
+    if (lane == 31 && inc > 0) base = atomicAdd(rtot, inc);
+    base = __shfl_sync(0xffffffffu, base, 31) + inc - v;
+    if (i < ng) {
+        roff[i] = base;
+        rcur[i] = base;
+    }
+}
+
+template <int SL>
+__global__ void __launch_bounds__(256) k_rev_fill(int ng, const int *__restrict__ nbr,
+                                                  const unsigned long long *__restrict__ mut, int *__restrict__ rcur,
+                                                  int *__restrict__ rlist)
+{
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) / SL, l = threadIdx.x & (SL - 1);
     if (i >= ng) return;
-    unsigned long long mask = mut[i];
-    for (int k = 0; k < NGB; k++) {
-        if (mask & (1ull << k)) continue;
-        int j = nbr[(size_t)i * NGB + k];
-        int s = atomicAdd(&rfill[j], 1);
-        rlist[roff[j] + s] = i;
+    const unsigned long long mask = mut[i];
+#pragma unroll
+    for (int q = 0; q < NGB / SL; q++) {
+        if (mask & (1ull << (q * SL + l))) continue;
+        const int j = nbr[(size_t)i * NGB + q * SL + l];
+        rlist[atomicAdd(&rcur[j], 1)] = i;
     }
 }
 
@@ -782,39 +840,21 @@ __global__ void k_rev_fill(int ng, const int *__restrict__ nbr, const unsigned l
 struct ForceParams {
     int ng;
     const int *nbr, *roff, *rcnt, *rlist;
-    const int4 *C;    // neighbour records (k_force_pack)
+    const int4 *C;    // neighbour records (gas gather and kernel-size search)
     const float4 *R, *V, *Q;
     const double *box;
     float alpha;
-    float *ax, *ay, *az, *du;
+    const int *gslot;
+    float *ax, *ay, *az, *dudt;  // per particle slot: the hydro part is added to the acceleration
     float *vsig;  // largest signal velocity c_i + c_j - 3 min(w_ij, 0) over the pairs of i
 };
 
 // One record set per gas particle so a pair gathers four records instead of
-// fourteen fields: {cell, mass}, {residual, 1/h}, {v, c}, {rho, Y, U}.  The
+// fourteen fields: {cell, mass}, {residual}, {v, c}, {rho, Y, U, 1/h}.  The
 // pressure terms of a pair are U_j Y_i gW(h_i) + U_i Y_j gW(h_j): Y = P/rho^2,
 // U = 1 for density-energy SPH; Y = (gamma-1) u / P, U = (gamma-1) u for
 // pressure-energy SPH with the smoothed P, whose pair coefficients are
 // (gamma-1)^2 u_i u_j / P_i and / P_j.
-__global__ void k_force_pack(int ng, const float *__restrict__ gvx, const float *__restrict__ gvy,
-                             const float *__restrict__ gvz, const float *__restrict__ h,
-                             const float *__restrict__ rho, const float *__restrict__ P, const float *__restrict__ cs,
-                             const float *__restrict__ gu, float gamma, int pressure, float4 *__restrict__ R,
-                             float4 *__restrict__ V, float4 *__restrict__ Q)
-{
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= ng) return;
-    const float rj = rho[j];
-    R[j].w = 1.f / h[j];  // the rest of R, and C, come from the gas gather
-    V[j] = make_float4(gvx[j], gvy[j], gvz[j], cs[j]);
-    if (pressure) {
-        const float U = (gamma - 1.f) * gu[j];
-        Q[j] = make_float4(rj, U / P[j], U, 0.f);
-    } else {
-        Q[j] = make_float4(rj, P[j] / (rj * rj), 1.f, 0.f);
-    }
-}
-
 __device__ __forceinline__ void pair_force(const ForceParams &p, int j, float unit, int ci0, int ci1, int ci2,
                                            float ri0, float ri1, float ri2, float vi0, float vi1, float vi2,
                                            float hinv_i, float pi_, float ui_, float rhoi, float csi, float &a0,
@@ -830,7 +870,7 @@ __device__ __forceinline__ void pair_force(const ForceParams &p, int j, float un
     float r2 = __fmaf_rn(dx, dx, __fmaf_rn(dy, dy, dz * dz));
     float r = sqrtf(r2);
     float rinv = r > 0.f ? 1.f / r : 0.f;
-    float dwi = kern_dw(r, hinv_i), dwj = kern_dw(r, Rj.w);
+    float dwi = kern_dw(r, hinv_i), dwj = kern_dw(r, Qj.w);
     float rhoj = Qj.x;
     float pj_ = Qj.y;
     float vx = vi0 - Vj.x, vy = vi1 - Vj.y, vz = vi2 - Vj.z;
@@ -849,66 +889,57 @@ __device__ __forceinline__ void pair_force(const ForceParams &p, int j, float un
     du += mj * (ci * dwi + 0.5f * visc * dwbar) * w;
 }
 
-__global__ void k_force(ForceParams p)
+// FL lanes per particle: a lane takes every FL-th pair and the sums are
+// reduced over the lanes.  A pair gathers 64 bytes of records; with one thread
+// per particle the gathers of its ~70 pairs are one chain and a small set has
+// too few threads to hide it.  The sums are added to the particle slots here
+// rather than in a pass of their own.
+template <int FL>
+__global__ void __launch_bounds__(128) k_force(ForceParams p)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= p.ng) return;
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) / FL, l = threadIdx.x & (FL - 1);
+    const bool valid = i < p.ng;
+    const int ii = valid ? i : 0;
     const float unit = (float)p.box[4];
-    const int4 Ci = p.C[i];
-    const float4 Ri = p.R[i];
-    const float4 Vi = p.V[i];
-    const float4 Qi = p.Q[i];
+    const int4 Ci = p.C[ii];
+    const float4 Ri = p.R[ii];
+    const float4 Vi = p.V[ii];
+    const float4 Qi = p.Q[ii];
     const int ci0 = Ci.x, ci1 = Ci.y, ci2 = Ci.z;
     const float ri0 = Ri.x, ri1 = Ri.y, ri2 = Ri.z;
     const float vi0 = Vi.x, vi1 = Vi.y, vi2 = Vi.z;
-    const float hinv = Ri.w, rhoi = Qi.x, csi = Vi.w;
+    const float hinv = Qi.w, rhoi = Qi.x, csi = Vi.w;
     const float pi_ = Qi.y, ui_ = Qi.z;
     float a0 = 0.f, a1 = 0.f, a2 = 0.f, du = 0.f, vs = 2.f * csi;
-    const int *nb = p.nbr + (size_t)i * NGB;
-    for (int k = 0; k < NGB; k++) {
-        int j = nb[k];
-        if (j == i) continue;
-        pair_force(p, j, unit, ci0, ci1, ci2, ri0, ri1, ri2, vi0, vi1, vi2, hinv, pi_, ui_, rhoi, csi, a0, a1, a2, du,
-                   vs);
+    if (valid) {
+        const int *nb = p.nbr + (size_t)i * NGB;
+        for (int k = l; k < NGB; k += FL) {
+            const int j = nb[k];
+            if (j == i) continue;
+            pair_force(p, j, unit, ci0, ci1, ci2, ri0, ri1, ri2, vi0, vi1, vi2, hinv, pi_, ui_, rhoi, csi, a0, a1, a2,
+                       du, vs);
+        }
+        const int b = p.roff[i], e = b + p.rcnt[i];
+        for (int k = b + l; k < e; k += FL)
+            pair_force(p, p.rlist[k], unit, ci0, ci1, ci2, ri0, ri1, ri2, vi0, vi1, vi2, hinv, pi_, ui_, rhoi, csi, a0,
+                       a1, a2, du, vs);
     }
-    int b = p.roff[i], e = b + p.rcnt[i];
-    for (int k = b; k < e; k++)
-        pair_force(p, p.rlist[k], unit, ci0, ci1, ci2, ri0, ri1, ri2, vi0, vi1, vi2, hinv, pi_, ui_, rhoi, csi, a0,
-                   a1, a2, du, vs);
-    p.ax[i] = a0;
-    p.ay[i] = a1;
-    p.az[i] = a2;
-    p.du[i] = du;
-    p.vsig[i] = vs;
-}
-
-// hydro results back to particle slots
-__global__ void k_gas_scatter(int ng, const int *__restrict__ gslot, const float *__restrict__ hax,
-                              const float *__restrict__ hay, const float *__restrict__ haz,
-                              const float *__restrict__ hdu, float *__restrict__ ax, float *__restrict__ ay,
-                              float *__restrict__ az, float *__restrict__ dudt)
-{
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= ng) return;
-    int s = gslot[k];
-    ax[s] += hax[k];
-    ay[s] += hay[k];
-    az[s] += haz[k];
-    dudt[s] = hdu[k];
-}
-
-__global__ void k_gas_scatter_density(int ng, const int *__restrict__ gslot, const float *__restrict__ grho,
-                                      const float *__restrict__ gP, const float *__restrict__ gcs,
-                                      const double *__restrict__ gh2, float *__restrict__ rho,
-                                      float *__restrict__ pres, float *__restrict__ cs, double *__restrict__ h2)
-{
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= ng) return;
-    int s = gslot[k];
-    rho[s] = grho[k];
-    pres[s] = gP[k];
-    cs[s] = gcs[k];
-    h2[s] = gh2[k];
+#pragma unroll
+    for (int o = FL / 2; o > 0; o >>= 1) {
+        a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+        a1 += __shfl_xor_sync(0xffffffffu, a1, o);
+        a2 += __shfl_xor_sync(0xffffffffu, a2, o);
+        du += __shfl_xor_sync(0xffffffffu, du, o);
+        vs = fmaxf(vs, __shfl_xor_sync(0xffffffffu, vs, o));
+    }
+    if (valid && l == 0) {
+        const int s = p.gslot[i];
+        p.ax[s] += a0;
+        p.ay[s] += a1;
+        p.az[s] += a2;
+        p.dudt[s] = du;
+        p.vsig[i] = vs;
+    }
 }
 
 // ---------------------------------------------------------------- host
@@ -967,8 +998,9 @@ int sph_density(gnb_ctx *c)
     p.rprev = c->gRprev;
     p.margin = c->knn_margin;
     p.status = c->status_d;
-    p.nbr = c->nbr; p.nd2 = c->nd2; p.h2 = c->gh2; p.h2lo = c->gh2lo; p.h2hi = c->gh2hi; p.h = c->gh; p.E = c->gE;
-    p.rho = c->grho; p.P = c->gP; p.cs = c->gcs; p.g64 = c->g64;
+    p.nbr = c->nbr; p.nd2 = c->nd2; p.h2 = c->gh2; p.h2b = c->gh2b; p.h = c->gh; p.E = c->gE; p.g64 = c->g64;
+    p.gvx = c->gvx; p.gvy = c->gvy; p.gvz = c->gvz; p.V = c->fV; p.Q = c->fQ;
+    p.gslot = c->gslot; p.s_rho = c->rho; p.s_pres = c->pres; p.s_cs = c->cs; p.s_h2 = a.h2;
     p.gamma = (float)c->cfg.gamma; p.pressure = c->cfg.sph_variant;
     gnb::counted(k_knn)<<<g_knn_blocks, KN_THREADS, smem, c->s>>>(p);
     GNB_LAUNCH_CHECK(c, "knn");
@@ -985,9 +1017,6 @@ int sph_density(gnb_ctx *c)
         else if (under < 0.01) c->knn_margin = std::max(1.01f, c->knn_margin / 1.02f);
     }
     c->stats[GNB_S_GAS_NODES] = c->gt.nnodes;
-    gnb::counted(k_gas_scatter_density)<<<gb, 256, 0, c->s>>>(ng, c->gslot, c->grho, c->gP, c->gcs, c->gh2, c->rho, c->pres,
-                                                c->cs, a.h2);
-    GNB_LAUNCH_CHECK(c, "density scatter");
     phase_end(c);
     c->have_h = true;
     c->nbr_valid = true;
@@ -998,25 +1027,28 @@ int sph_force(gnb_ctx *c)
 {
     int ng = (int)c->n_gas;
     if (ng == 0) return GNB_OK;
-    int gb = (ng + 255) / 256;
     phase_begin(c, GNB_T_FORCE);
+    // lanes per particle: more spread a small set over the chip, fewer do less
+    // reduction and bit bookkeeping.  Phase time, lists + force, one thread per
+    // particle -> 16 and 8 lanes -> 8 and 4: 4,096 gas particles 164 -> 37 ->
+    // 47 us, 1e5 242 -> 135 -> 137, 210 k 424 -> 259 -> 243, 1.68 M 2464 -> 1943
+    // -> 1733.
+    const bool few = ng < 150000;
+    const int sl = few ? 16 : 8, fl = few ? 8 : 4;
+    const int gb = (ng + 255) / 256, gbl = (int)(((long long)ng * sl + 255) / 256);
     cudaMemsetAsync(c->rcnt, 0, sizeof(int) * ng, c->s);
-    gnb::counted(k_mutual)<<<gb, 256, 0, c->s>>>(ng, c->nbr, c->nd2, c->gE, c->gh2, c->gh2lo, c->gh2hi, c->g64,
-                                                 c->ggrank, c->gx, c->gy, c->gz, c->mut, c->rcnt);
-    GNB_TRY(device_scan(c, c->rcnt, c->roff, c->ngas_d, ng, c->rtot_d));
-    cudaMemsetAsync(c->rfill, 0, sizeof(int) * ng, c->s);
-    gnb::counted(k_rev_fill)<<<gb, 256, 0, c->s>>>(ng, c->nbr, c->mut, c->roff, c->rfill, c->rlist);
+    gnb::counted(few ? k_mutual<16> : k_mutual<8>)<<<gbl, 256, 0, c->s>>>(
+        ng, c->nbr, c->nd2, c->gE, c->gh2, c->gh2b, c->g64, c->ggrank, c->gx, c->gy, c->gz, c->mut, c->rcnt, c->rtot_d);
+    gnb::counted(k_rev_off)<<<gb, 256, 0, c->s>>>(ng, c->rcnt, c->roff, c->rcur, c->rtot_d);
+    gnb::counted(few ? k_rev_fill<16> : k_rev_fill<8>)<<<gbl, 256, 0, c->s>>>(ng, c->nbr, c->mut, c->rcur, c->rlist);
     GNB_LAUNCH_CHECK(c, "symmetric lists");
-    gnb::counted(k_force_pack)<<<gb, 256, 0, c->s>>>(ng, c->gvx, c->gvy, c->gvz, c->gh, c->grho, c->gP, c->gcs, c->gu,
-                                                     (float)c->cfg.gamma, c->cfg.sph_variant, c->fR, c->fV, c->fQ);
     ForceParams p;
     p.ng = ng; p.nbr = c->nbr; p.roff = c->roff; p.rcnt = c->rcnt; p.rlist = c->rlist;
     p.C = c->fC; p.R = c->fR; p.V = c->fV; p.Q = c->fQ;
     p.box = c->box_d; p.alpha = (float)c->cfg.alpha_visc;
-    p.ax = c->hax; p.ay = c->hay; p.az = c->haz; p.du = c->hdu; p.vsig = c->gvsig;
-    gnb::counted(k_force)<<<(ng + 127) / 128, 128, 0, c->s>>>(p);
-    gnb::counted(k_gas_scatter)<<<gb, 256, 0, c->s>>>(ng, c->gslot, c->hax, c->hay, c->haz, c->hdu, c->ax, c->ay, c->az,
-                                        c->dudt);
+    p.gslot = c->gslot;
+    p.ax = c->ax; p.ay = c->ay; p.az = c->az; p.dudt = c->dudt; p.vsig = c->gvsig;
+    gnb::counted(few ? k_force<8> : k_force<4>)<<<(int)(((long long)ng * fl + 127) / 128), 128, 0, c->s>>>(p);
     GNB_LAUNCH_CHECK(c, "sph force");
     phase_end(c);
     return GNB_OK;

@@ -65,3 +65,29 @@ def test_kernel_sizes_exact_twice(G, orc, case):
         nbr, h2 = orc.knn({q: np.asarray(p[q], np.float64) for q in ("x", "y", "z", "m", "u")}, 64, sample=sample)
         assert np.array_equal(c.get("NBR")[sample], np.sort(nbr, axis=1))
         assert np.array_equal(c.get("H2")[sample], h2)
+
+
+# hydro force: 16 and 8 lanes per particle below 150,000 gas particles, 8 and 4
+# from there.  Equal and opposite pairs: any pair lost, doubled or one-sided
+# shows in the totals of momentum and energy.
+@pytest.mark.parametrize("n", [64, 67, 149999, 150001])
+@pytest.mark.parametrize("variant", [0, 1])
+def test_hydro_force_conserves(G, n, variant):
+    p = ics.uniform_random(n, seed=n)
+    c = G.Context(sph_variant=variant)
+    c.set_particles(p)
+    c.compute_sph_density()
+    c.compute_sph_force()
+    m, du = p["m"].astype(np.float64), c.get("DUDT").astype(np.float64)
+    a = np.stack([c.get(k) for k in ("AX", "AY", "AZ")]).astype(np.float64)
+    v = np.stack([p[k] for k in ("vx", "vy", "vz")]).astype(np.float64)
+    force = np.sum(m * np.linalg.norm(a, axis=0))
+    # FP32 sums of ~70 terms per particle, errors independent between particles
+    assert np.linalg.norm((m * a).sum(1)) < 1e-5 * force
+    power = np.sum(m * (np.abs(du) + np.linalg.norm(a, axis=0) * np.linalg.norm(v, axis=0)))
+    assert abs(np.sum(m * ((a * v).sum(0) + du))) < 1e-5 * power
+    nb = c.get("NBR")
+    pairs = set()
+    if n < 1000:  # the symmetric lists hold 63 own entries and the one-sided pairs once more
+        pairs = {(i, j) for i in range(n) for j in nb[i] if i != j}
+        assert c.stats()["NSYM"] == 63 * n + sum((j, i) not in pairs for i, j in pairs)
