@@ -62,14 +62,14 @@ static void free_particles(gnb_ctx *c)
     parr_free(c, c->P[0]);
     parr_free(c, c->P[1]);
     void *all[] = {c->ax, c->ay, c->az, c->pot, c->dudt, c->gax, c->gay, c->gaz, c->pext, c->rho, c->pres,
-                   c->cs, c->kres, c->skey, c->skey2, c->sval, c->sval2, c->slot_of_orig, c->src, c->rs_counts,
+                   c->cs, c->kres, c->skey, c->skey2, c->sval, c->sval2, c->slot_of_orig, c->src,
                    c->gas_flag, c->pscan, c->tmp_out};
     for (void *q : all) dfree(c, q);
     c->ax = c->ay = c->az = c->pot = c->dudt = c->gax = c->gay = c->gaz = c->pext = nullptr;
     c->rho = c->pres = c->cs = nullptr;
     c->kres = nullptr;
     c->skey = c->skey2 = nullptr;
-    c->sval = c->sval2 = c->slot_of_orig = c->src = c->rs_counts = c->gas_flag = c->pscan = nullptr;
+    c->sval = c->sval2 = c->slot_of_orig = c->src = c->gas_flag = c->pscan = nullptr;
     c->tmp_out = nullptr;
     tree_free(c, c->t);
     c->cap = 0;
@@ -110,8 +110,6 @@ static int alloc_particles(gnb_ctx *c, int64_t n)
     GNB_TRY(dalloc(c, &c->slot_of_orig, N)); GNB_TRY(dalloc(c, &c->src, N));
     GNB_TRY(dalloc(c, &c->gas_flag, N + 1)); GNB_TRY(dalloc(c, &c->pscan, N + 1));
     GNB_TRY(dalloc(c, &c->tmp_out, 8 * N + 64));
-    int ntiles = (int)((n + 2047) / 2048);
-    GNB_TRY(dalloc(c, &c->rs_counts, (size_t)ntiles * 256));
     c->cap = n;
     return GNB_OK;
 }
@@ -248,7 +246,7 @@ int gnb_create(gnb_ctx **out, const gnb_config *cfg)
     if ((rc = dalloc(c, &c->status_d, 4)) || (rc = dalloc(c, &c->n_d, 4)) || (rc = dalloc(c, &c->ngas_d, 4)) ||
         (rc = dalloc(c, &c->counters_d, 8)) || (rc = dalloc(c, &c->work_d, 8)) || (rc = dalloc(c, &c->box_d, 8)) ||
         (rc = dalloc(c, &c->mm_d, 8)) || (rc = dalloc(c, &c->red_d, 256 * 10 + 16)) ||
-        (rc = dalloc(c, &c->rs_total, 256)) || (rc = dalloc(c, &c->rtot_d, 4)) ||
+        (rc = dalloc(c, &c->rtot_d, 4)) ||
         (rc = dalloc(c, &c->scan_part, 1100)) || (rc = dalloc(c, &c->scan_poff, 1100))) {
         gnb_destroy(c);
         return rc;
@@ -279,7 +277,7 @@ void gnb_destroy(gnb_ctx *c)
     hier_free(c);
     replace_free(c);
     void *all[] = {c->status_d, c->n_d, c->ngas_d, c->counters_d, c->work_d, c->box_d, c->mm_d, c->red_d,
-                   c->rs_total, c->rtot_d, c->scan_part, c->scan_poff, c->gl_pool, c->gl_next, c->gl_cnt,
+                   c->rs_buf, c->rtot_d, c->scan_part, c->scan_poff, c->gl_pool, c->gl_next, c->gl_cnt,
                    c->gl_top, c->gl_head, c->gl_ref, c->gl_lcum};
     for (void *q : all) dfree(c, q);
     if (c->pinned_i) cudaFreeHost(c->pinned_i);

@@ -113,11 +113,12 @@ struct gnb_ctx {
     int *sval = nullptr, *sval2 = nullptr, *slot_of_orig = nullptr, *src = nullptr;
     int *pscan = nullptr;     // per-slot scan scratch
     unsigned char *tmp_out = nullptr;  // export staging (8 bytes per particle)
-    int *rs_counts = nullptr, *rs_total = nullptr;
-    int rs_tiles_cap = 0;
+    int *rs_buf = nullptr;    // radix sort: histograms, tickets, flags, published counts (sort.cu)
+    size_t rs_words = 0;
     // root box: device {lo[3], L, unit} plus min/max scratch
     double *box_d = nullptr;
     unsigned long long *mm_d = nullptr;
+    bool mm_ready = false;    // the words hold their start values (every pass leaves them so)
     double lo[3] = {0, 0, 0}, L = 1, unit = 1;
     // gravity tree
     gnb::Tree t;
@@ -285,7 +286,7 @@ void phase_end(gnb_ctx *c);
 
 // sort.cu
 int morton_and_sort(gnb_ctx *c);
-int radix_sort_pairs(gnb_ctx *c, uint64_t *k0, int *v0, uint64_t *k1, int *v1, int n, int first_digit);
+int radix_sort_pairs(gnb_ctx *c, uint64_t *k0, int *v0, uint64_t *k1, int *v1, int n);
 // replace.cu
 int replace_particles(gnb_ctx *c, int64_t n, const int64_t *id, const double *x, const double *y, const double *z,
                       const float *vx, const float *vy, const float *vz, const float *u, int on_device);

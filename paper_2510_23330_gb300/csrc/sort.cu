@@ -8,6 +8,7 @@
 // index): a stable LSD radix sort of the keys in their current slot order by
 // the top 48 bits, then the short runs that agree there put in (key, caller
 // index) order (see the ties section).
+#include <algorithm>
 #include <utility>
 
 #include "common.cuh"
@@ -16,31 +17,76 @@
 namespace gnb {
 
 // ---------------------------------------------------------------- root box
-__global__ void k_mm_init(unsigned long long *mm) { minmax_init(mm, threadIdx.x); }
-
-__global__ void k_minmax(const double *__restrict__ x, const double *__restrict__ y,
-                         const double *__restrict__ z, int n, unsigned long long *mm)
+// Min/max words accumulated by all blocks; the last block to finish (a ticket
+// counter, no waiting) forms box = {lo_x, lo_y, lo_z, L, unit} and puts the
+// words and the counter back to their start values for the next call.
+__global__ void k_mm_init(unsigned long long *mm)
 {
-    minmax_accumulate(x, y, z, n, mm);
+    minmax_init(mm, threadIdx.x);
+    if (threadIdx.x == 7) mm[7] = 0ull;  // blocks done
 }
 
-// box = {lo_x, lo_y, lo_z, L, unit}
-__global__ void k_box_finalize(const unsigned long long *mm, double *box, int *status)
+__global__ void __launch_bounds__(256) k_root_box(const double *__restrict__ x, const double *__restrict__ y,
+                                                  const double *__restrict__ z, int n, unsigned long long *mm,
+                                                  double *box, int *status)
 {
-    if (threadIdx.x != 0) return;
-    if (box_from_minmax(mm, box)) atomicOr(status, ST_BAD_INPUT);
+    __shared__ bool last;
+    minmax_accumulate(x, y, z, n, mm);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(&mm[7], 1ull) == gridDim.x - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!last) return;
+    if (threadIdx.x == 0) {
+        unsigned long long w[7];
+        for (int k = 0; k < 7; k++) w[k] = *(volatile unsigned long long *)&mm[k];
+        if (box_from_minmax(w, box)) atomicOr(status, ST_BAD_INPUT);
+    }
+    __syncthreads();
+    if (threadIdx.x < 7) minmax_init(mm, threadIdx.x);
+    if (threadIdx.x == 7) mm[7] = 0ull;
 }
 
 int root_box(gnb_ctx *c)
 {
     int n = (int)c->n;
-    gnb::counted(k_mm_init)<<<1, 32, 0, c->s>>>(c->mm_d);
+    if (!c->mm_ready) {
+        gnb::counted(k_mm_init)<<<1, 32, 0, c->s>>>(c->mm_d);
+        c->mm_ready = true;
+    }
     int blocks = (n + 255) / 256;
     if (blocks > 1216) blocks = 1216;
-    gnb::counted(k_minmax)<<<blocks, 256, 0, c->s>>>(c->P[c->cur].x, c->P[c->cur].y, c->P[c->cur].z, n, c->mm_d);
-    gnb::counted(k_box_finalize)<<<1, 32, 0, c->s>>>(c->mm_d, c->box_d, c->status_d);
+    gnb::counted(k_root_box)<<<blocks, 256, 0, c->s>>>(c->P[c->cur].x, c->P[c->cur].y, c->P[c->cur].z, n, c->mm_d,
+                                                      c->box_d, c->status_d);
     GNB_LAUNCH_CHECK(c, "root box");
     return GNB_OK;
+}
+
+#define TIE_SHIFT 16  // key bits below the sorted ones (see the ties section)
+#define TIE_FIRST_DIGIT (TIE_SHIFT / 8)
+
+// A warp's digits F .. 7 of its keys into the block's histograms.  Near-sorted
+// keys share their high digits: one addition where the warp agrees instead
+// of 32 to one word.
+template <int F>
+__device__ __forceinline__ void digit_count(int (*h)[256], uint64_t k, bool valid)
+{
+    const unsigned vb = __ballot_sync(0xffffffffu, valid);
+    if (vb == 0u) return;
+    const int lead = __ffs(vb) - 1;
+#pragma unroll
+    for (int q = F; q < 8; q++) {
+        const int d = (int)(k >> (8 * q)) & 255;
+        const int d0 = __shfl_sync(0xffffffffu, d, lead);
+        if (__all_sync(0xffffffffu, !valid || d == d0)) {
+            if ((threadIdx.x & 31) == lead) atomicAdd(&h[q - F][d], __popc(vb));
+        } else if (valid) {
+            atomicAdd(&h[q - F][d], 1);
+        }
+    }
 }
 
 // ---------------------------------------------------------------- Morton
@@ -60,26 +106,40 @@ __global__ void k_morton(PArr p, int n, const double *__restrict__ box, uint64_t
     slot_of_orig[o] = i;
 }
 
-// Key of every slot, paired with the slot itself for a sort in slot order
-// (ties are put into caller order afterwards, see k_tie_fix), and the FP32
+// Key of every slot (the first sorting pass pairs it with the slot itself;
+// ties are put into caller order afterwards, see k_tie_fix), the FP32
 // remainder of each coordinate within its grid cell (res: three arrays of n,
-// slot order) for the permutation.
-__global__ void k_keys(const double *__restrict__ x, const double *__restrict__ y, const double *__restrict__ z, int n,
-                       const double *__restrict__ box, uint64_t *__restrict__ key, int *__restrict__ val,
-                       float *__restrict__ res)
+// slot order) for the permutation, and the histograms of the digits to be
+// sorted (hist[8][256], see the radix sort).
+__global__ void __launch_bounds__(256) k_keys(const double *__restrict__ x, const double *__restrict__ y,
+                                              const double *__restrict__ z, int n, const double *__restrict__ box,
+                                              uint64_t *__restrict__ key, float *__restrict__ res,
+                                              int *__restrict__ hist)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    __shared__ int h[8 - TIE_FIRST_DIGIT][256];
+    for (int k = threadIdx.x; k < (8 - TIE_FIRST_DIGIT) * 256; k += blockDim.x) (&h[0][0])[k] = 0;
+    __syncthreads();
     const int lexp = box_lexp(box[3]);
-    float r0, r1, r2;
-    const int c0 = grid_cell(x[i], box[0], lexp, &r0);
-    const int c1 = grid_cell(y[i], box[1], lexp, &r1);
-    const int c2 = grid_cell(z[i], box[2], lexp, &r2);
-    key[i] = morton_key(c0, c1, c2);
-    val[i] = i;
-    res[i] = r0;
-    res[(size_t)n + i] = r1;
-    res[2 * (size_t)n + i] = r2;
+    for (int b = blockIdx.x * blockDim.x; b < n; b += gridDim.x * blockDim.x) {
+        const int i = b + threadIdx.x;
+        const bool valid = i < n;
+        uint64_t k = 0;
+        if (valid) {
+            float r0, r1, r2;
+            const int c0 = grid_cell(x[i], box[0], lexp, &r0);
+            const int c1 = grid_cell(y[i], box[1], lexp, &r1);
+            const int c2 = grid_cell(z[i], box[2], lexp, &r2);
+            k = morton_key(c0, c1, c2);
+            key[i] = k;
+            res[i] = r0;
+            res[(size_t)n + i] = r1;
+            res[2 * (size_t)n + i] = r2;
+        }
+        digit_count<TIE_FIRST_DIGIT>(h, k, valid);
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < (8 - TIE_FIRST_DIGIT) * 256; k += blockDim.x)
+        if ((&h[0][0])[k]) atomicAdd(&hist[TIE_FIRST_DIGIT * 256 + k], (&h[0][0])[k]);
 }
 
 // ---------------------------------------------------------------- ties
@@ -91,8 +151,6 @@ __global__ void k_keys(const double *__restrict__ x, const double *__restrict__ 
 // most TIE_MAX entries.  st[0] = 1 when some run exists, st[1] = the longest
 // (capped at TIE_MAX + 1); a longer run is left to the caller-order sort.
 #define TIE_MAX 4096
-#define TIE_SHIFT 16  // key bits below the sorted ones
-#define TIE_FIRST_DIGIT (TIE_SHIFT / 8)
 
 __device__ __forceinline__ bool tie(uint64_t a, uint64_t b) { return (a >> TIE_SHIFT) == (b >> TIE_SHIFT); }
 
@@ -129,116 +187,91 @@ __global__ void k_tie_fix(uint64_t *__restrict__ k, int n, int *__restrict__ val
 }
 
 // ---------------------------------------------------------------- radix sort
-// Stable LSD radix sort of (64-bit key, 32-bit value), 8 bits per pass.
-// Tiles of RS_TILE keys; per pass: digit histogram per tile, per-digit scan
-// over tiles, stable scatter with per-warp match ranks.
+// Stable LSD radix sort of (64-bit key, 32-bit value), 8 bits per pass, one
+// kernel per pass: the digit histograms of all passes are counted once, up
+// front (they do not depend on the order; the Morton keys' with the keys), and a tile finds where its run of
+// each digit starts from the counts that the tiles before it publish
+// (decoupled look-back).  A tile takes its number from a ticket counter, so
+// every tile it waits for is already running.
+//
+// A tile's pairs are first sorted by digit in shared memory, stably, then
+// written out in that order, so consecutive threads write consecutive
+// addresses of each digit's run instead of one scattered store each.  Each
+// warp ranks its own contiguous ITEMS * 32 pairs of the tile (rounds of 32 in
+// order, lanes in order within a round) against per-warp digit counters, with
+// warp synchronisation only; one block-wide step then turns the counters into
+// each warp's offset within the digit's run of the tile.
 #define RS_THREADS 256
-#define RS_ITEMS 16
-#define RS_TILE (RS_THREADS * RS_ITEMS)
+#define RS_BATCH 8            // published counts read at once in the look-back
+#define RS_AGG (1u << 30)     // the tile's own count of the digit
+#define RS_PRE (2u << 30)     // the count of the digit in this tile and all before it
+#define RS_SPINS (1 << 20)    // look-back reads without progress before giving up
 
-__global__ void __launch_bounds__(RS_THREADS) k_rs_hist(const uint64_t *__restrict__ k, int n, int shift,
-                                                       int *__restrict__ counts, int ntiles,
-                                                       int *__restrict__ total)
-{
-    __shared__ int h[256];
-    int t = threadIdx.x, tile = blockIdx.x;
-    h[t] = 0;
-    __syncthreads();
-    int base = tile * RS_TILE;
-#pragma unroll
-    for (int r = 0; r < RS_ITEMS; r++) {
-        int i = base + r * RS_THREADS + t;
-        if (i < n) atomicAdd(&h[(int)((k[i] >> shift) & 255u)], 1);
-    }
-    __syncthreads();
-    int v = h[t];
-    counts[t * ntiles + tile] = v;
-    if (v) atomicAdd(&total[t], v);
-}
+struct RsState {
+    int *hist;        // [8][256] digit histograms
+    int *ticket;      // [8] tiles started per pass
+    unsigned *state;  // [passes][ntiles][256] published counts
+    int *flag;        // set when a look-back gave up
+};
 
-// One block per digit: offs[d][tile] = base(d) + sum_{t' < tile} counts[d][t'].
-__global__ void __launch_bounds__(1024) k_rs_scan(int *__restrict__ counts, int ntiles,
-                                                  const int *__restrict__ total)
-{
-    __shared__ int wsum[32];
-    __shared__ int s_base, s_carry;
-    int d = blockIdx.x, t = threadIdx.x, lane = t & 31, w = t >> 5;
-    if (t < 32) {
-        int acc = 0;
-        for (int e = lane; e < d; e += 32) acc += total[e];
-        acc = warp_sum(acc);
-        if (lane == 0) { s_base = acc; s_carry = 0; }
-    }
-    __syncthreads();
-    int *row = counts + (size_t)d * ntiles;
-    for (int b0 = 0; b0 < ntiles; b0 += 1024) {
-        int i = b0 + t;
-        int v = i < ntiles ? row[i] : 0;
-        int x = v;
-        for (int o = 1; o < 32; o <<= 1) {
-            int y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) wsum[w] = x;
-        __syncthreads();
-        if (w == 0) {
-            int s = wsum[lane];
-            for (int o = 1; o < 32; o <<= 1) {
-                int y = __shfl_up_sync(0xffffffffu, s, o);
-                if (lane >= o) s += y;
-            }
-            wsum[lane] = s;
-        }
-        __syncthreads();
-        int excl = x - v + (w > 0 ? wsum[w - 1] : 0);
-        if (i < ntiles) row[i] = s_base + s_carry + excl;
-        __syncthreads();
-        if (t == 0) s_carry += wsum[31];
-        __syncthreads();
-    }
-}
-
-// Scatter of one tile: the tile's pairs are first sorted by digit in shared
-// memory, stably, then written out in that order, so consecutive threads
-// write consecutive addresses of each digit's run (about RS_TILE / 256 pairs
-// per digit) instead of one scattered 8-byte store each.  Each warp ranks its
-// own contiguous RS_ITEMS * 32 pairs of the tile (rounds of 32 in order,
-// lanes in order within a round) against per-warp digit counters, with warp
-// synchronisation only; one block-wide step then turns the counters into each
-// warp's offset within the digit's run of the tile.
+template <int ITEMS>
 struct RsSmem {
-    uint64_t k[RS_TILE];
-    int v[RS_TILE];
+    uint64_t k[RS_THREADS * ITEMS];
+    int v[RS_THREADS * ITEMS];
     int wc[RS_THREADS / 32][256];  // per-warp digit counts, then each warp's offset in the digit's run
     int lstart[256];               // first local position of each digit
     int goff[256];                 // global position of each digit's first pair of this tile
-    int ws[RS_THREADS / 32];
+    int ws[RS_THREADS / 32], wh[RS_THREADS / 32];
+    int tile, stop;
 };
 
-__global__ void __launch_bounds__(RS_THREADS, 3) k_rs_scatter(const uint64_t *__restrict__ kin,
-                                                          const int *__restrict__ vin,
-                                                          uint64_t *__restrict__ kout,
+__device__ __forceinline__ unsigned ld_relaxed(const unsigned *p)
+{
+    unsigned v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_relaxed(unsigned *p, unsigned v)
+{
+    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+// FIRST: the values are the slots themselves (vin is not read)
+template <int ITEMS, bool FIRST>
+__global__ void __launch_bounds__(RS_THREADS, 3) k_rs_pass(const uint64_t *__restrict__ kin,
+                                                          const int *__restrict__ vin, uint64_t *__restrict__ kout,
                                                           int *__restrict__ vout, int n, int shift,
-                                                          const int *__restrict__ offs, int ntiles)
+                                                          const int *__restrict__ hist, int *ticket, unsigned *state,
+                                                          int *flag)
 {
     extern __shared__ __align__(16) unsigned char rs_raw[];
-    RsSmem &S = *reinterpret_cast<RsSmem *>(rs_raw);
-    const int t = threadIdx.x, tile = blockIdx.x, w = t >> 5, lane = t & 31;
+    RsSmem<ITEMS> &S = *reinterpret_cast<RsSmem<ITEMS> *>(rs_raw);
+    constexpr int TILE = RS_THREADS * ITEMS;
+    const int t = threadIdx.x, w = t >> 5, lane = t & 31;
     const unsigned lt = (1u << lane) - 1u;
-    const int base = tile * RS_TILE;
-    const int cnt = min(RS_TILE, n - base);
+    if (t == 0) {
+        S.tile = atomicAdd(ticket, 1);
+        S.stop = 0;
+    }
 #pragma unroll
     for (int q = 0; q < RS_THREADS / 32; q++) S.wc[q][t] = 0;
-    S.goff[t] = offs[t * ntiles + tile];
+    const int hd = hist[t];
     __syncthreads();
-    uint64_t key[RS_ITEMS];
-    int val[RS_ITEMS], lr[RS_ITEMS];
+    const int tile = S.tile;
+    const int base = tile * TILE;
+    const int cnt = min(TILE, n - base);
+    uint64_t key[ITEMS];
+    int val[ITEMS], lr[ITEMS];
 #pragma unroll
-    for (int r = 0; r < RS_ITEMS; r++) {
-        const int i = w * (RS_ITEMS * 32) + r * 32 + lane;
+    for (int r = 0; r < ITEMS; r++) {
+        const int i = w * (ITEMS * 32) + r * 32 + lane;
+        key[r] = i < cnt ? kin[base + i] : 0ull;
+        val[r] = FIRST ? base + i : (i < cnt ? vin[base + i] : 0);
+    }
+#pragma unroll
+    for (int r = 0; r < ITEMS; r++) {
+        const int i = w * (ITEMS * 32) + r * 32 + lane;
         const bool valid = i < cnt;
-        key[r] = valid ? kin[base + i] : 0ull;
-        val[r] = valid ? vin[base + i] : 0;
         const int d = valid ? (int)((key[r] >> shift) & 255u) : 256;
         const unsigned peers = __match_any_sync(0xffffffffu, d);
         const int leader = __ffs(peers) - 1;
@@ -252,30 +285,35 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_rs_scatter(const uint64_t *__
         __syncwarp();
     }
     __syncthreads();
-    {   // digit t: offsets of the warps within the digit's run, then the
-        // exclusive scan of the tile histogram over the 256 digits
-        int run = 0;
+    // digit t: offsets of the warps within the digit's run; publish the count
+    int run = 0;
 #pragma unroll
-        for (int q = 0; q < RS_THREADS / 32; q++) {
-            const int c = S.wc[q][t];
-            S.wc[q][t] = run;
-            run += c;
-        }
-        int x = run;
+    for (int q = 0; q < RS_THREADS / 32; q++) {
+        const int c = S.wc[q][t];
+        S.wc[q][t] = run;
+        run += c;
+    }
+    unsigned *mine = state + (size_t)tile * 256 + t;
+    st_relaxed(mine, (tile == 0 ? RS_PRE : RS_AGG) | (unsigned)run);
+    // exclusive scans over the 256 digits: of the tile's counts and of all counts
+    int gbase;
+    {
+        int x = run, y = hd;
         for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
+            const int a = __shfl_up_sync(0xffffffffu, x, o), b = __shfl_up_sync(0xffffffffu, y, o);
+            if (lane >= o) { x += a; y += b; }
         }
-        if (lane == 31) S.ws[w] = x;
+        if (lane == 31) { S.ws[w] = x; S.wh[w] = y; }
         __syncthreads();
-        int pre = 0;
-        for (int q = 0; q < w; q++) pre += S.ws[q];
-        S.lstart[t] = pre + x - run;
+        int px = 0, py = 0;
+        for (int q = 0; q < w; q++) { px += S.ws[q]; py += S.wh[q]; }
+        S.lstart[t] = px + x - run;
+        gbase = py + y - hd;
         __syncthreads();
     }
 #pragma unroll
-    for (int r = 0; r < RS_ITEMS; r++) {
-        const int i = w * (RS_ITEMS * 32) + r * 32 + lane;
+    for (int r = 0; r < ITEMS; r++) {
+        const int i = w * (ITEMS * 32) + r * 32 + lane;
         if (i < cnt) {
             const int d = (int)((key[r] >> shift) & 255u);
             const int lp = S.lstart[d] + S.wc[w][d] + lr[r];
@@ -283,7 +321,31 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_rs_scatter(const uint64_t *__
             S.v[lp] = val[r];
         }
     }
+    // look-back: the digit's count in the tiles before this one
+    int before = 0;
+    for (int p = tile - 1, spins = 0; p >= 0;) {
+        unsigned s[RS_BATCH];
+#pragma unroll
+        for (int q = 0; q < RS_BATCH; q++) s[q] = ld_relaxed(state + (size_t)max(p - q, 0) * 256 + t);
+        bool moved = false;
+#pragma unroll
+        for (int q = 0; q < RS_BATCH; q++) {
+            if (p < 0 || s[q] < RS_AGG) break;  // past the first tile, or not published yet
+            before += (int)(s[q] & (RS_AGG - 1u));
+            p = s[q] >= RS_PRE ? -1 : p - 1;
+            moved = true;
+        }
+        if (moved) spins = 0;
+        else if (++spins > RS_SPINS) {  // cannot happen unless a block was lost
+            S.stop = 1;
+            atomicOr(flag, 1);
+            break;
+        }
+    }
+    if (tile > 0) st_relaxed(mine, RS_PRE | (unsigned)(before + run));
+    S.goff[t] = gbase + before;
     __syncthreads();
+    if (S.stop) return;
     for (int pos = t; pos < cnt; pos += RS_THREADS) {
         const uint64_t k = S.k[pos];
         const int d = (int)((k >> shift) & 255u);
@@ -293,37 +355,107 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_rs_scatter(const uint64_t *__
     }
 }
 
-// The scatter's tile (about 59 KB) needs the opt-in to more than 48 KB of
-// dynamic shared memory.
-static int rs_scatter_attr(gnb_ctx *c)
+// Histograms of all digits from digit F up (the Morton keys' come with the keys).
+template <int F>
+__global__ void __launch_bounds__(256) k_rs_hist(const uint64_t *__restrict__ key, int n, int *__restrict__ hist)
 {
-    cudaError_t e = cudaFuncSetAttribute(k_rs_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sizeof(RsSmem));
-    return e == cudaSuccess ? GNB_OK : cuda_check(c, e, "radix sort shared memory attribute");
+    __shared__ int h[8 - F][256];
+    for (int k = threadIdx.x; k < (8 - F) * 256; k += blockDim.x) (&h[0][0])[k] = 0;
+    __syncthreads();
+    for (int b = blockIdx.x * blockDim.x; b < n; b += gridDim.x * blockDim.x) {
+        const int i = b + threadIdx.x;
+        digit_count<F>(h, i < n ? key[i] : 0ull, i < n);
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < (8 - F) * 256; k += blockDim.x)
+        if ((&h[0][0])[k]) atomicAdd(&hist[F * 256 + k], (&h[0][0])[k]);
 }
 
-// Stable sort of n (64-bit key, 32-bit value) pairs held in (k0, v0) by the
-// key bits from 8 first_digit up (first_digit even), with (k1, v1) as the
-// ping-pong buffers; the sorted pairs end in (k0, v0).
-int radix_sort_pairs(gnb_ctx *c, uint64_t *k0, int *v0, uint64_t *k1, int *v1, int n, int first_digit)
+// Pairs per thread of a tile.  Small tiles spread a small set over the chip and
+// shorten the serial ranking rounds; large ones write longer runs and have
+// fewer predecessors to look back to.  Sort phase with 4 / 8 / 16: 8,192
+// particles 75 / 85 / - us, 150,001 118 / 126 / 139, 300,007 177 / 172 / 184,
+// 2^20 - / 276 / 254 (histogram, scan and scatter kernels per pass: 186, 217,
+// 324 and 330).
+static int rs_items(int n) { return n <= 200000 ? 4 : (n <= 500000 ? 8 : 16); }
+
+// Scratch of a sort of n pairs, cleared: histograms, tickets, the give-up
+// flag and the published counts of eight passes.
+static int rs_begin(gnb_ctx *c, int n, RsState *st)
 {
-    int ntiles = (n + RS_TILE - 1) / RS_TILE;
-    GNB_TRY(rs_scatter_attr(c));
-    uint64_t *kin = k0, *kout = k1;
-    int *vin = v0, *vout = v1;
-    for (int pass = first_digit; pass < 8; pass++) {
-        int shift = 8 * pass;
-        cudaMemsetAsync(c->rs_total, 0, 256 * sizeof(int), c->s);
-        gnb::counted(k_rs_hist)<<<ntiles, RS_THREADS, 0, c->s>>>(kin, n, shift, c->rs_counts, ntiles, c->rs_total);
-        gnb::counted(k_rs_scan)<<<256, 1024, 0, c->s>>>(c->rs_counts, ntiles, c->rs_total);
-        gnb::counted(k_rs_scatter)<<<ntiles, RS_THREADS, sizeof(RsSmem), c->s>>>(kin, vin, kout, vout, n, shift,
-                                                                                  c->rs_counts,
-                                                                    ntiles);
-        uint64_t *tk = kin; kin = kout; kout = tk;
-        int *tv = vin; vin = vout; vout = tv;
+    const int tile = RS_THREADS * rs_items(n);
+    const size_t ntiles = (size_t)((n + tile - 1) / tile);
+    const size_t words = 8 * 256 + 16 + 8 * ntiles * 256;
+    if (c->rs_words < words) {
+        dfree(c, c->rs_buf);
+        c->rs_buf = nullptr;
+        c->rs_words = 0;
+        GNB_TRY(dalloc(c, &c->rs_buf, words));
+        c->rs_words = words;
+    }
+    st->hist = c->rs_buf;
+    st->ticket = c->rs_buf + 8 * 256;
+    st->flag = c->rs_buf + 8 * 256 + 8;
+    st->state = (unsigned *)(c->rs_buf + 8 * 256 + 16);
+    return cuda_check(c, cudaMemsetAsync(c->rs_buf, 0, words * sizeof(int), c->s), "radix sort scratch");
+}
+
+template <int ITEMS, bool FIRST>
+static int rs_pass(gnb_ctx *c, const RsState &st, const uint64_t *kin, const int *vin, uint64_t *kout, int *vout, int n,
+                   int pass)
+{
+    // a tile needs more than the default 48 KB of shared memory
+    const cudaError_t e = cudaFuncSetAttribute(k_rs_pass<ITEMS, FIRST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)sizeof(RsSmem<ITEMS>));
+    if (e != cudaSuccess) return cuda_check(c, e, "radix sort shared memory attribute");
+    const int ntiles = (n + RS_THREADS * ITEMS - 1) / (RS_THREADS * ITEMS);
+    gnb::counted(k_rs_pass<ITEMS, FIRST>)<<<ntiles, RS_THREADS, sizeof(RsSmem<ITEMS>), c->s>>>(
+        kin, vin, kout, vout, n, 8 * pass, st.hist + 256 * pass, st.ticket + pass,
+        st.state + (size_t)pass * ntiles * 256, st.flag);
+    return GNB_OK;
+}
+
+// The passes from digit `first` up over (k0, v0) with (k1, v1) as the
+// ping-pong buffers, histograms counted; 8 - first is even, so the sorted
+// pairs end in (k0, v0).  slots: the values are the slots 0 .. n - 1 (v0 is
+// not read).
+static int rs_passes(gnb_ctx *c, const RsState &st, uint64_t *k0, int *v0, uint64_t *k1, int *v1, int n, int first,
+                     bool slots)
+{
+    for (int pass = first; pass < 8; pass++) {
+        const bool odd = (pass - first) & 1, f = slots && pass == first;
+        const uint64_t *ki = odd ? k1 : k0;
+        const int *vi = odd ? v1 : v0;
+        uint64_t *ko = odd ? k0 : k1;
+        int *vo = odd ? v0 : v1;
+        switch (rs_items(n)) {
+        case 4: GNB_TRY(f ? (rs_pass<4, true>(c, st, ki, vi, ko, vo, n, pass))
+                          : (rs_pass<4, false>(c, st, ki, vi, ko, vo, n, pass))); break;
+        case 8: GNB_TRY(f ? (rs_pass<8, true>(c, st, ki, vi, ko, vo, n, pass))
+                          : (rs_pass<8, false>(c, st, ki, vi, ko, vo, n, pass))); break;
+        default: GNB_TRY(f ? (rs_pass<16, true>(c, st, ki, vi, ko, vo, n, pass))
+                           : (rs_pass<16, false>(c, st, ki, vi, ko, vo, n, pass))); break;
+        }
     }
     GNB_LAUNCH_CHECK(c, "radix sort");
     return GNB_OK;
+}
+
+static int rs_gave_up(gnb_ctx *c) { return fail(c, GNB_ETIMEOUT, "a bounded wait in the radix sort ran out"); }
+
+// Stable sort of n (64-bit key, 32-bit value) pairs held in (k0, v0) by the
+// whole key, with (k1, v1) as the ping-pong buffers; the sorted pairs end in
+// (k0, v0).  Waits for the result.
+int radix_sort_pairs(gnb_ctx *c, uint64_t *k0, int *v0, uint64_t *k1, int *v1, int n)
+{
+    RsState st;
+    GNB_TRY(rs_begin(c, n, &st));
+    gnb::counted(k_rs_hist<0>)<<<std::min((n + 1023) / 1024, 1216), 256, 0, c->s>>>(k0, n, st.hist);
+    GNB_TRY(rs_passes(c, st, k0, v0, k1, v1, n, 0, false));
+    GNB_TRY(cuda_check(c, cudaMemcpyAsync(c->pinned_i + 60, st.flag, sizeof(int), cudaMemcpyDeviceToHost, c->s),
+                       "radix sort flag"));
+    GNB_TRY(cuda_check(c, cudaStreamSynchronize(c->s), "radix sort sync"));
+    return c->pinned_i[60] ? rs_gave_up(c) : GNB_OK;
 }
 
 // ---------------------------------------------------------------- permute
@@ -363,7 +495,10 @@ __global__ void k_permute(PArr a, PArr b, const int *__restrict__ src, int n, co
 // array (at most 8 bytes a particle) in L2 while it is gathered, instead of
 // one pass whose 22 sources together are far larger than L2 (on the 2^24
 // disk the single pass took 7.1 ms against 0.73 ms for the near-sorted
-// permutations of later steps).
+// permutations of later steps).  Up to PERM_ONE_PASS particles all sources fit
+// in L2 together (about 150 bytes a particle) and 22 launches cost more than
+// the single pass.
+#define PERM_ONE_PASS 500000
 template <class T>
 __global__ void k_gather1(const T *__restrict__ a, T *__restrict__ b, const int *__restrict__ src, int n)
 {
@@ -420,39 +555,40 @@ int morton_and_sort(gnb_ctx *c)
     // keys in slot order (the particles are near their previous Morton
     // order), stable sort by the top 48 bits, then runs into (key, caller
     // index) order
-    gnb::counted(k_keys)<<<nb, 256, 0, c->s>>>(a.x, a.y, a.z, n, c->box_d, c->skey, c->sval, c->kres);
+    RsState st;
+    GNB_TRY(rs_begin(c, n, &st));
+    gnb::counted(k_keys)<<<std::min(nb, 1216), 256, 0, c->s>>>(a.x, a.y, a.z, n, c->box_d, c->skey, c->kres, st.hist);
     GNB_LAUNCH_CHECK(c, "keys");
-    GNB_TRY(radix_sort_pairs(c, c->skey, c->sval, c->skey2, c->sval2, n, TIE_FIRST_DIGIT));
-    cudaMemsetAsync(c->work_d + 2, 0, 2 * sizeof(int), c->s);
-    gnb::counted(k_tie_detect)<<<nb, 256, 0, c->s>>>(c->skey, n, c->work_d + 2);
+    GNB_TRY(rs_passes(c, st, c->skey, c->sval, c->skey2, c->sval2, n, TIE_FIRST_DIGIT, true));
+    gnb::counted(k_tie_detect)<<<nb, 256, 0, c->s>>>(c->skey, n, st.flag + 1);
     GNB_LAUNCH_CHECK(c, "tie detect");
-    GNB_TRY(cuda_check(c, cudaMemcpyAsync(c->pinned_i + 60, c->work_d + 2, 2 * sizeof(int), cudaMemcpyDeviceToHost,
-                                          c->s), "tie flag"));
+    GNB_TRY(cuda_check(c, cudaMemcpyAsync(c->pinned_i + 60, st.flag, 3 * sizeof(int), cudaMemcpyDeviceToHost, c->s),
+                       "tie flag"));
     GNB_TRY(cuda_check(c, cudaStreamSynchronize(c->s), "tie flag sync"));
-    const int *src = c->sval;  // the old slot of each sorted particle
-    if (c->pinned_i[60] && c->pinned_i[61] <= TIE_MAX) {
+    const int *flags = c->pinned_i + 60;  // {look-back gave up, some run of ties, the longest}
+    if (flags[0]) return rs_gave_up(c);
+    if (flags[1] && flags[2] <= TIE_MAX) {
         gnb::counted(k_tie_fix)<<<nb, 256, 0, c->s>>>(c->skey, n, c->sval, a.orig);
         GNB_LAUNCH_CHECK(c, "tie fix");
-    } else if (c->pinned_i[60]) {
+        std::swap(c->src, c->sval);
+    } else if (flags[1]) {
         // a run of more than TIE_MAX: sort by the whole key in caller order
         // (keys scattered to the caller index, stable sort, slot map)
         gnb::counted(k_morton)<<<nb, 256, 0, c->s>>>(a, n, c->box_d, c->skey, c->sval, c->slot_of_orig);
         GNB_LAUNCH_CHECK(c, "morton");
-        GNB_TRY(radix_sort_pairs(c, c->skey, c->sval, c->skey2, c->sval2, n, 0));
+        GNB_TRY(radix_sort_pairs(c, c->skey, c->sval, c->skey2, c->sval2, n));
         gnb::counted(k_src)<<<nb, 256, 0, c->s>>>(c->sval, c->slot_of_orig, c->src, n);
-        src = c->src;
+    } else {
+        std::swap(c->src, c->sval);  // the old slot of each sorted particle
     }
-    if (src != c->src)
-        GNB_TRY(cuda_check(c, cudaMemcpyAsync(c->src, src, sizeof(int) * (size_t)n, cudaMemcpyDeviceToDevice, c->s),
-                           "slot map copy"));
     PArr &b = c->P[1 - c->cur];
-    if (c->slots_caller) {
+    if (c->slots_caller && n > PERM_ONE_PASS) {
         GNB_TRY(permute_per_array(c, a, b, c->src, n));
-        c->slots_caller = false;
     } else {
         gnb::counted(k_permute)<<<nb, 256, 0, c->s>>>(a, b, c->src, n, c->skey, c->kres);
         GNB_LAUNCH_CHECK(c, "permute");
     }
+    c->slots_caller = false;
     c->cur = 1 - c->cur;
     if (c->hier_on) GNB_TRY(hier_permute(c));  // per-particle step state follows the particles
     return GNB_OK;

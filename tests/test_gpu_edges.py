@@ -91,3 +91,26 @@ def test_hydro_force_conserves(G, n, variant):
     if n < 1000:  # the symmetric lists hold 63 own entries and the one-sided pairs once more
         pairs = {(i, j) for i in range(n) for j in nb[i] if i != j}
         assert c.stats()["NSYM"] == 63 * n + sum((j, i) not in pairs for i, j in pairs)
+
+
+# radix sort: one tile, tile edges, 4 | 8 | 16 pairs per thread of a tile, and
+# a run of equal keys longer than the tie pass takes (whole-key sort)
+@pytest.mark.parametrize("n", [1, 1023, 1024, 1025, 200001, 500001, "ties"])
+def test_sort_order(G, orc, n):
+    p = ics.plummer(9000 if n == "ties" else max(n, 4), seed=3, n_gas=0)
+    if n == "ties":
+        for k in ("x", "y", "z"):
+            p[k][1000:6000] = p[k][1000]
+    elif n < 4:
+        p = ics.subset(p, range(n))
+    c = G.Context()
+    c.set_particles(p)
+    for k in range(2):  # from the caller's order, then from the sorted one
+        c.build_tree()
+        key = orc.morton(p)[0]
+        assert np.array_equal(c.get("KEY"), key)
+        assert np.array_equal(c.get("ORDER"), np.lexsort((np.arange(key.size), key)))
+        assert np.array_equal(c.get("X"), p["x"]) and np.array_equal(c.get("VZ"), p["vz"])
+        rng = np.random.default_rng(k)
+        p = dict(p, x=p["x"] + 1e-3 * rng.normal(size=key.size))
+        c.replace_region({q: p[q] for q in ("id", "x", "y", "z", "vx", "vy", "vz", "u")})
