@@ -506,14 +506,9 @@ static int do_gravity(gnb_ctx *c, int mode)
         GNB_TRY(gravity_tree(c));
     } else if (mode == GNB_GRAV_DIRECT) {
         GNB_TRY(gravity_direct(c));
-    } else {  // GNB_GRAV_NONE: no self-gravity
-        size_t b = sizeof(float) * (size_t)c->n;
-        cudaMemsetAsync(c->gax, 0, b, c->s); cudaMemsetAsync(c->gay, 0, b, c->s);
-        cudaMemsetAsync(c->gaz, 0, b, c->s); cudaMemsetAsync(c->pot, 0, b, c->s);
     }
     phase_begin(c, GNB_T_EXTERNAL);
-    GNB_TRY(gravity_nfw(c));
-    GNB_TRY(zero_forces(c));
+    GNB_TRY(assemble_forces(c, mode != GNB_GRAV_NONE));
     phase_end(c);
     c->gravity_valid = true;
     c->last_grav_mode = mode;

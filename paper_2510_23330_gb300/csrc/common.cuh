@@ -314,7 +314,7 @@ int load_state(gnb_ctx *c, const char *path);
 // gravity.cu
 int gravity_tree(gnb_ctx *c);
 int gravity_direct(gnb_ctx *c);
-int gravity_nfw(gnb_ctx *c);
+int assemble_forces(gnb_ctx *c, bool self);
 // sph.cu
 int sph_density(gnb_ctx *c);
 int sph_force(gnb_ctx *c);
@@ -341,7 +341,6 @@ int predict(gnb_ctx *c, float hdt);
 int kick_drift_predict(gnb_ctx *c, float hdt, double dt);
 int diagnostics(gnb_ctx *c, double out[10]);
 int scatter_out(gnb_ctx *c, int field, void *dst_dev);
-int zero_forces(gnb_ctx *c);
 
 }  // namespace gnb
 

@@ -108,27 +108,6 @@ int predict(gnb_ctx *c, float hdt)
     return GNB_OK;
 }
 
-// total = external (already in a) + self-gravity; du/dt reset
-__global__ void k_combine(int n, const float *__restrict__ gax, const float *__restrict__ gay,
-                          const float *__restrict__ gaz, float *__restrict__ ax, float *__restrict__ ay,
-                          float *__restrict__ az, float *__restrict__ dudt)
-{
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    ax[i] += gax[i];
-    ay[i] += gay[i];
-    az[i] += gaz[i];
-    dudt[i] = 0.f;
-}
-
-int zero_forces(gnb_ctx *c)
-{
-    int n = (int)c->n;
-    gnb::counted(k_combine)<<<(n + 255) / 256, 256, 0, c->s>>>(n, c->gax, c->gay, c->gaz, c->ax, c->ay, c->az, c->dudt);
-    GNB_LAUNCH_CHECK(c, "combine");
-    return GNB_OK;
-}
-
 // ---------------------------------------------------------------- diagnostics
 #define DG_BLOCKS 256
 __global__ void k_diag_partial(PArr p, const float *__restrict__ pot, const float *__restrict__ pext, int n,
