@@ -215,6 +215,8 @@ struct gnb_ctx {
     int *gl_pool = nullptr, *gl_next = nullptr, *gl_cnt = nullptr, *gl_top = nullptr, *gl_lcum = nullptr;
     int4 *gl_head = nullptr, *gl_ref = nullptr;
     int gl_cap = 0, gl_gcap = 0;
+    float4 *gd_part = nullptr;                 // direct gravity: sums of the source parts [parts][n]
+    int64_t gd_cap = 0;
     int *pinned_i = nullptr;                   // pinned host scratch [64]
     // hierarchical timesteps (integrate.cu): per particle slot, permuted with
     // the particles by every sort while hier_on; [2] = current and scratch

@@ -66,7 +66,6 @@ struct GravSmem {
     float je[GW_JP];
     float4 c0[2][GW_JC], c1[2][GW_JC], c2[2][GW_JC];  // two buffers: one evaluated, one filling
     int4 cnb[GW_JC];  // raw cell corners of the buffer being filled (each thread converts its own slots)
-    float4 red[GW_THREADS];
     int ws[32];
     int g;
 };
@@ -129,18 +128,10 @@ __device__ __forceinline__ void pp_one(float4 q, float e, float xi, float yi, fl
     ph += mr;
 }
 
-template <bool MASK>
-__device__ __forceinline__ void pp_loop(const GravSmem &S, int np, int split, int js, float xi, float yi, float zi,
-                                        float e2i, float &ax, float &ay, float &az, float &ph)
-{
-#pragma unroll 4
-    for (int j = split; j < np; j += js) pp_one<MASK>(S.jp[j], S.je[j], xi, yi, zi, e2i, ax, ay, az, ph);
-}
-
 // NI i-particles per thread: each staged j entry is read from shared memory
 // once for all of them.
-template <int NI, bool MASK>
-__device__ __forceinline__ void pp_loopN(const GravSmem &S, int np, int split, int js, const float4 (&pi)[NI],
+template <int NI, bool MASK, class Smem>
+__device__ __forceinline__ void pp_loopN(const Smem &S, int np, int split, int js, const float4 (&pi)[NI],
                                          float4 (&acc)[NI])
 {
     constexpr int UNR = NI >= 4 ? 2 : (NI == 2 ? 2 : 4);
@@ -291,8 +282,8 @@ __device__ __forceinline__ void pc_two(float4 a, float4 b, float4 d, float2 nx, 
     }
 }
 
-template <int NP, bool MASK, bool UNI>
-__device__ __forceinline__ void pp_loopP(const GravSmem &S, int np, int split, int js, const IPair<NP> &I,
+template <int NP, bool MASK, bool UNI, class Smem>
+__device__ __forceinline__ void pp_loopP(const Smem &S, int np, int split, int js, const IPair<NP> &I,
                                          float2 E2, APair<NP> &A)
 {
 #pragma unroll 4
@@ -777,69 +768,168 @@ __global__ void __launch_bounds__(GW_THREADS, 5) k_grav_eval(GravParams p)
     }
 }
 
-// Direct summation: every group streams all n particles through shared memory.
-template <bool MASK>
-__global__ void __launch_bounds__(GW_THREADS, 4) k_gravity_direct(GravParams p)
+// Direct summation.  A work unit is one group (one particle per thread, two
+// above 4, four above 32, packed pairs from two on: 267 us with these limits
+// for 20,011 particles, 281 with the 16 and 64 of the tree evaluation, whose
+// lists are far shorter) against one of `segs` parts of all n particles, staged through
+// shared memory as offsets from the group's reference cell; the parts' sums go
+// to part[segment][particle] and k_direct_sum adds them up in order.  A group
+// against all particles is far too coarse a unit for a small set (20,011
+// particles: 1,121 groups of very different sizes on 608 resident CTAs), and
+// the pairs are bound by the FMA pipe, which the packed instructions fill with
+// half the issue slots.  20,011 particles: 506 -> 258 us (FMA pipe 60 % active;
+// the pairs alone would keep it busy for 137 us).
+struct DirectSmem {
+    float4 jp[GW_JP];
+    float je[GW_JP];
+    int g;
+};
+
+template <int NI, bool MASK, bool UNI>
+__device__ __forceinline__ void direct_chunk(DirectSmem &S, const GravParams &p, int first, int icnt, int j0, int j1,
+                                             const int *gref, float unit, float4 *__restrict__ out)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    GravSmem &S = *reinterpret_cast<GravSmem *>(smem_raw);
+    const int tid = threadIdx.x;
+    const int ilanes = (icnt + NI - 1) / NI;
+    const int js = GW_THREADS / ilanes;
+    const int islot = tid % ilanes, split = tid / ilanes;
+    const bool ivalid = split < js;
+    constexpr bool PK = NI >= 2;
+    constexpr int NP = PK ? NI / 2 : 1;
+    float4 pi[NI], acc[NI];
+    IPair<NP> I;
+    APair<NP> A;
+    const float2 E2 = bc2(p.e2u);
+#pragma unroll
+    for (int k = 0; k < NI; k++) {
+        const int sl = islot + k * ilanes;
+        const int ip = first + (sl < icnt ? sl : islot);  // an empty slot repeats the first particle
+        const float ep = p.eps[ip];
+        pi[k] = make_float4(grid_off(p.cx[ip], gref[0], p.rx[ip], unit), grid_off(p.cy[ip], gref[1], p.ry[ip], unit),
+                            grid_off(p.cz[ip], gref[2], p.rz[ip], unit), ep * ep);
+        acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    if constexpr (PK) {
+#pragma unroll
+        for (int h = 0; h < NP; h++) {
+            I.nx[h] = make_float2(-pi[2 * h].x, -pi[2 * h + 1].x);
+            I.ny[h] = make_float2(-pi[2 * h].y, -pi[2 * h + 1].y);
+            I.nz[h] = make_float2(-pi[2 * h].z, -pi[2 * h + 1].z);
+            I.e2[h] = make_float2(pi[2 * h].w, pi[2 * h + 1].w);
+            A.ax[h] = A.ay[h] = A.az[h] = A.ph[h] = make_float2(0.f, 0.f);
+        }
+    }
+    for (int c0 = j0; c0 < j1; c0 += GW_JP) {
+        const int np = min(GW_JP, j1 - c0);
+        __syncthreads();
+        for (int k = tid; k < np; k += GW_THREADS) {
+            const int j = c0 + k;
+            const float ej = p.eps[j];
+            S.jp[k] = make_float4(grid_off(p.cx[j], gref[0], p.rx[j], unit), grid_off(p.cy[j], gref[1], p.ry[j], unit),
+                                  grid_off(p.cz[j], gref[2], p.rz[j], unit), -p.m[j]);
+            S.je[k] = ej * ej;
+        }
+        __syncthreads();
+        if (ivalid) {
+            if constexpr (PK) pp_loopP<NP, MASK, UNI>(S, np, split, js, I, E2, A);
+            else pp_loopN<NI, MASK>(S, np, split, js, pi, acc);
+        }
+    }
+    if constexpr (PK) {
+#pragma unroll
+        for (int h = 0; h < NP; h++) {
+            acc[2 * h] = make_float4(A.ax[h].x, A.ay[h].x, A.az[h].x, A.ph[h].x);
+            acc[2 * h + 1] = make_float4(A.ax[h].y, A.ay[h].y, A.az[h].y, A.ph[h].y);
+        }
+    }
+    // reduce the j-splits through the staging buffer
+    static_assert(NI * GW_THREADS <= GW_JP, "reduction buffer");
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < NI; k++) S.jp[k * GW_THREADS + tid] = acc[k];
+    __syncthreads();
+    if (split == 0) {
+#pragma unroll
+        for (int k = 0; k < NI; k++) {
+            const int sl = islot + k * ilanes;
+            if (sl >= icnt) continue;
+            float4 a = acc[k];
+            for (int s2 = 1; s2 < js; s2++) {
+                const float4 r = S.jp[k * GW_THREADS + tid + s2 * ilanes];
+                a.x += r.x; a.y += r.y; a.z += r.z; a.w += r.w;
+            }
+            out[first + sl] = a;
+        }
+    }
+}
+
+template <bool MASK, bool UNI>
+__global__ void __launch_bounds__(GW_THREADS, 5) k_gravity_direct(GravParams p, int segs, float4 *__restrict__ part)
+{
+    __shared__ DirectSmem S;
     const int tid = threadIdx.x;
     const float unit = (float)p.box[4];
     const int ngroups = *p.ngroups;
     for (;;) {
+        __syncthreads();  // the previous unit's sums are read and its number is taken
         if (tid == 0) S.g = atomicAdd(p.next, 1);
         __syncthreads();
-        const int gi = S.g;
-        if (gi >= ngroups) break;
-        const int4 ga = p.na[p.groups[gi]];
+        const int unit_no = S.g;
+        if (unit_no >= ngroups * segs) break;
+        const int seg = unit_no / ngroups;
+        const int4 ga = p.na[p.groups[unit_no - seg * ngroups]];
+        const int j0 = (int)((long long)p.n * seg / segs), j1 = (int)((long long)p.n * (seg + 1) / segs);
+        float4 *out = part + (size_t)seg * p.n;
+        // (at most GW_THREADS particles share a reference cell: the offsets of a
+        // wide group's close pairs would lose digits)
         for (int i0 = 0; i0 < ga.y; i0 += GW_THREADS) {
-            const int icnt = min(GW_THREADS, ga.y - i0);
-            const int ilanes = icnt;
-            const int js = GW_THREADS / ilanes;
-            const int islot = tid % ilanes, split = tid / ilanes;
-            const bool ivalid = split < js;
-            const int ip = ga.x + i0 + islot;
-            const int gref[3] = {p.cx[ga.x + i0], p.cy[ga.x + i0], p.cz[ga.x + i0]};
-            const float xi = grid_off(p.cx[ip], gref[0], p.rx[ip], unit);
-            const float yi = grid_off(p.cy[ip], gref[1], p.ry[ip], unit);
-            const float zi = grid_off(p.cz[ip], gref[2], p.rz[ip], unit);
-            const float e2i = p.eps[ip] * p.eps[ip];
-            float ax = 0.f, ay = 0.f, az = 0.f, ph = 0.f;
-            for (int c0 = 0; c0 < p.n; c0 += GW_JP) {
-                int np = min(GW_JP, p.n - c0);
-                __syncthreads();
-                for (int k = tid; k < np; k += GW_THREADS) {
-                    int j = c0 + k;
-                    float ej = p.eps[j];
-                    S.jp[k] = make_float4(grid_off(p.cx[j], gref[0], p.rx[j], unit),
-                                          grid_off(p.cy[j], gref[1], p.ry[j], unit),
-                                          grid_off(p.cz[j], gref[2], p.rz[j], unit), -p.m[j]);
-                    S.je[k] = ej * ej;
-                }
-                __syncthreads();
-                if (ivalid) pp_loop<MASK>(S, np, split, js, xi, yi, zi, e2i, ax, ay, az, ph);
-            }
-            __syncthreads();
-            ax = -ax; ay = -ay; az = -az; ph = -ph;  // the sums were accumulated negated
-            S.red[tid] = make_float4(ax, ay, az, ph);
-            __syncthreads();
-            if (split == 0 && ivalid) {
-                for (int s2 = 1; s2 < js; s2++) {
-                    float4 r = S.red[tid + s2 * ilanes];
-                    ax += r.x; ay += r.y; az += r.z; ph += r.w;
-                }
-                if (!MASK) ph -= p.m[ip] * rsqrtf(2.f * e2i);
-                p.ax[ip] = p.G * ax;
-                p.ay[ip] = p.G * ay;
-                p.az[ip] = p.G * az;
-                p.pot[ip] = -p.G * ph;
-            }
+            const int first = ga.x + i0, icnt = min(GW_THREADS, ga.y - i0);
+            // reference cell: midway between the ends of the Morton run, which
+            // are far apart in a wide one (the first particle's cell doubles
+            // the largest offset and with it the rounding of a pair's distance)
+            const int last = first + icnt - 1;
+            const int gref[3] = {(p.cx[first] + p.cx[last]) >> 1, (p.cy[first] + p.cy[last]) >> 1,
+                                 (p.cz[first] + p.cz[last]) >> 1};
+            if (icnt > 32) direct_chunk<4, MASK, UNI>(S, p, first, icnt, j0, j1, gref, unit, out);
+            else if (icnt > 4) direct_chunk<2, MASK, UNI>(S, p, first, icnt, j0, j1, gref, unit, out);
+            else direct_chunk<1, MASK, UNI>(S, p, first, icnt, j0, j1, gref, unit, out);
         }
-        __syncthreads();
     }
 }
 
+// the parts' sums (accumulated negated) in order, the j == i term removed
+// unless the pairs at R = 0 were masked
+template <bool MASK>
+__global__ void __launch_bounds__(256) k_direct_sum(GravParams p, int segs, const float4 *__restrict__ part)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= p.n) return;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s = 0; s < segs; s++) {
+        const float4 r = part[(size_t)s * p.n + i];
+        a.x -= r.x; a.y -= r.y; a.z -= r.z; a.w -= r.w;
+    }
+    if (!MASK) {
+        const float ep = p.eps[i];
+        a.w -= p.m[i] * rsqrtf(2.f * (ep * ep));
+    }
+    p.ax[i] = p.G * a.x;
+    p.ay[i] = p.G * a.y;
+    p.az[i] = p.G * a.z;
+    p.pot[i] = -p.G * a.w;
+}
+
 static int g_sms = 0;
+
+static int sm_count()
+{
+    if (g_sms == 0) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&g_sms, cudaDevAttrMultiProcessorCount, dev);
+    }
+    return g_sms;
+}
 
 static GravParams make_params(gnb_ctx *c)
 {
@@ -885,17 +975,12 @@ static int launch_persistent(gnb_ctx *c, K kern, GravParams p, int *next_d)
     size_t smem = sizeof(GravSmem);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_check(c, e, "gravity smem attribute");
-    if (g_sms == 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&g_sms, cudaDevAttrMultiProcessorCount, dev);
-    }
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, GW_THREADS, smem);
     if (per_sm < 1) per_sm = 1;
     p.next = next_d;
     cudaMemsetAsync(next_d, 0, sizeof(int), c->s);
-    gnb::counted(kern)<<<g_sms * per_sm, GW_THREADS, smem, c->s>>>(p);
+    gnb::counted(kern)<<<sm_count() * per_sm, GW_THREADS, smem, c->s>>>(p);
     GNB_LAUNCH_CHECK(c, "gravity kernel");
     return GNB_OK;
 }
@@ -946,14 +1031,9 @@ int gravity_tree(gnb_ctx *c)
         cudaMemsetAsync(c->counters_d, 0, 2 * sizeof(unsigned long long), c->s);
         cudaMemsetAsync(c->gl_top, 0, sizeof(int), c->s);
         cudaMemsetAsync(next_d, 0, sizeof(int), c->s);
-        if (g_sms == 0) {
-            int dev = 0;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&g_sms, cudaDevAttrMultiProcessorCount, dev);
-        }
         int per_sm = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_grav_walk, GL_WARPS * 32, 0);
-        gnb::counted(k_grav_walk)<<<g_sms * std::max(per_sm, 1), GL_WARPS * 32, 0, c->s>>>(p);
+        gnb::counted(k_grav_walk)<<<sm_count() * std::max(per_sm, 1), GL_WARPS * 32, 0, c->s>>>(p);
         GNB_LAUNCH_CHECK(c, "tree walk");
         // the pool must have held every list; otherwise grow it and walk again
         GNB_TRY(cuda_check(c, cudaMemcpyAsync(&c->pinned_i[40], c->gl_top, sizeof(int), cudaMemcpyDeviceToHost, c->s),
@@ -995,8 +1075,32 @@ int gravity_direct(gnb_ctx *c)
 {
     GravParams p = make_params(c);
     int *next_d = (int *)(c->counters_d + 6);
-    if (c->min_eps_zero) return launch_persistent(c, k_gravity_direct<true>, p, next_d);
-    return launch_persistent(c, k_gravity_direct<false>, p, next_d);
+    const int n = (int)c->n;
+    // parts of the sources: about eight units per resident CTA, counting three
+    // groups per n_group particles (cells are a third full on average), at
+    // least one staged batch each and at most 16 (the parts' sums are 16 bytes
+    // a particle each)
+    const double groups = std::max(1.0, 3.0 * n / std::max(1, c->cfg.n_group));
+    const int want = (int)std::min(16.0, 8.0 * 5 * sm_count() / groups + 1.0);
+    const int segs = std::max(1, std::min(want, n / GW_JP));
+    if (c->gd_cap < (int64_t)n * segs) {
+        dfree(c, c->gd_part);
+        c->gd_part = nullptr;
+        c->gd_cap = 0;
+        GNB_TRY(dalloc(c, &c->gd_part, (size_t)n * segs));
+        c->gd_cap = (int64_t)n * segs;
+    }
+    p.next = next_d;
+    cudaMemsetAsync(next_d, 0, sizeof(int), c->s);
+    auto k = c->min_eps_zero ? k_gravity_direct<true, false>
+                             : (c->eps_uniform ? k_gravity_direct<false, true> : k_gravity_direct<false, false>);
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, GW_THREADS, 0);
+    gnb::counted(k)<<<sm_count() * std::max(per_sm, 1), GW_THREADS, 0, c->s>>>(p, segs, c->gd_part);
+    gnb::counted(c->min_eps_zero ? k_direct_sum<true> : k_direct_sum<false>)<<<(n + 255) / 256, 256, 0, c->s>>>(
+        p, segs, c->gd_part);
+    GNB_LAUNCH_CHECK(c, "direct gravity");
+    return GNB_OK;
 }
 
 // ---------------------------------------------------------------- NFW halo

@@ -114,3 +114,22 @@ def test_sort_order(G, orc, n):
         rng = np.random.default_rng(k)
         p = dict(p, x=p["x"] + 1e-3 * rng.normal(size=key.size))
         c.replace_region({q: p[q] for q in ("id", "x", "y", "z", "vx", "vy", "vz", "u")})
+
+
+# direct gravity: one and several parts of the sources, one, two and four
+# particles per thread, a group above 512, the three softening forms
+@pytest.mark.parametrize("n,n_group", [(513, 8), (1023, 64), (1025, 600), (2500, 2500)])
+@pytest.mark.parametrize("eps", ["uniform", "mixed", "zero"])
+def test_direct_gravity_forms(G, orc, n, n_group, eps):
+    p = ics.plummer(n, seed=n, n_gas=0)
+    rng = np.random.default_rng(n)
+    if eps != "uniform":
+        p["eps"] = (0.02 * rng.uniform(0.2, 1.0, n)).astype(np.float32)
+    if eps == "zero":
+        p["eps"][::3] = 0.0
+    c = G.Context(n_group=n_group)
+    c.set_particles(p)
+    c.compute_gravity(G.GNB_GRAV_DIRECT)
+    ref = orc.direct_gravity(p)
+    d = np.sqrt(sum((c.get("AGRAV_" + k) - ref["a" + k.lower()]) ** 2 for k in "XYZ"))
+    assert np.max(d / ref["asum"]) < 1e-5
