@@ -63,13 +63,13 @@ static void free_particles(gnb_ctx *c)
     parr_free(c, c->P[1]);
     void *all[] = {c->ax, c->ay, c->az, c->pot, c->dudt, c->gax, c->gay, c->gaz, c->pext, c->rho, c->pres,
                    c->cs, c->kres, c->skey, c->skey2, c->sval, c->sval2, c->slot_of_orig, c->src,
-                   c->gas_flag, c->pscan, c->tmp_out};
+                   c->tmp_out};
     for (void *q : all) dfree(c, q);
     c->ax = c->ay = c->az = c->pot = c->dudt = c->gax = c->gay = c->gaz = c->pext = nullptr;
     c->rho = c->pres = c->cs = nullptr;
     c->kres = nullptr;
     c->skey = c->skey2 = nullptr;
-    c->sval = c->sval2 = c->slot_of_orig = c->src = c->gas_flag = c->pscan = nullptr;
+    c->sval = c->sval2 = c->slot_of_orig = c->src = nullptr;
     c->tmp_out = nullptr;
     tree_free(c, c->t);
     c->cap = 0;
@@ -108,7 +108,6 @@ static int alloc_particles(gnb_ctx *c, int64_t n)
     GNB_TRY(dalloc(c, &c->kres, 3 * N)); GNB_TRY(dalloc(c, &c->skey, N)); GNB_TRY(dalloc(c, &c->skey2, N));
     GNB_TRY(dalloc(c, &c->sval, N)); GNB_TRY(dalloc(c, &c->sval2, N));
     GNB_TRY(dalloc(c, &c->slot_of_orig, N)); GNB_TRY(dalloc(c, &c->src, N));
-    GNB_TRY(dalloc(c, &c->gas_flag, N + 1)); GNB_TRY(dalloc(c, &c->pscan, N + 1));
     GNB_TRY(dalloc(c, &c->tmp_out, 8 * N + 64));
     c->cap = n;
     return GNB_OK;
@@ -155,41 +154,124 @@ static int check_status(gnb_ctx *c)
 }
 
 // ---------------------------------------------------------------- kernels used by set_particles
-__global__ void k_set_init(PArr p, int n)
+// The caller's arrays into the context's (COPY; else they are there already),
+// the fields that start from them, the validity bits, and each block's gas
+// count: block b takes particles [b chunk, (b + 1) chunk).  One pass instead
+// of eleven copies and three kernels: upload, direct gravity and export of
+// 20,011 particles 627 -> 547 us together with the one-launch export.
+#define LD_THREADS 256
+#define LD_BLOCKS 912  // a multiple of 152 SMs, at most the 1,024 partials of a scan
+
+struct LoadArgs {
+    const int64_t *id;
+    const uint8_t *type;
+    const double *x, *y, *z;
+    const float *vx, *vy, *vz, *m, *eps, *u;
+};
+
+__device__ __forceinline__ int load_chunk(int n)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    p.orig[i] = i;
-    p.h2[i] = 0.0;
-    p.vpx[i] = p.vx[i]; p.vpy[i] = p.vy[i]; p.vpz[i] = p.vz[i];
-    if (p.type[i] != GNB_GAS) p.u[i] = 0.f;
-    p.up[i] = p.u[i];
+    const int per = (n + LD_BLOCKS - 1) / LD_BLOCKS;
+    return (per + LD_THREADS - 1) / LD_THREADS * LD_THREADS;
 }
 
-__global__ void k_validate(PArr p, int n, int *bad)
+template <bool COPY>
+__global__ void __launch_bounds__(LD_THREADS) k_load(LoadArgs s, PArr p, int n, int *__restrict__ n_d,
+                                                     int *__restrict__ bad, float *__restrict__ eps0_d,
+                                                     int *__restrict__ partial)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int b = 0;
-    if (!isfinite(p.x[i]) || !isfinite(p.y[i]) || !isfinite(p.z[i])) b |= 1;
-    if (p.type[i] > 1) b |= 2;
-    if (!(p.m[i] > 0.f) || !isfinite(p.m[i])) b |= 4;
-    if (!(p.eps[i] >= 0.f) || !isfinite(p.eps[i])) b |= 8;
-    if (p.eps[i] == 0.f) b |= 16;
-    if (p.eps[i] != p.eps[0]) b |= 32;
-    if (b) atomicOr(bad, b);
+    __shared__ int gas;
+    if (threadIdx.x == 0) gas = 0;
+    __syncthreads();
+    const int chunk = load_chunk(n), beg = min(n, (int)min((long long)n, (long long)blockIdx.x * chunk));
+    const int end = (int)min((long long)n, (long long)beg + chunk);
+    const float eps0 = s.eps[0];
+    int b = 0, ng = 0;
+    for (int i = beg + threadIdx.x; i < end; i += LD_THREADS) {
+        const double x = s.x[i], y = s.y[i], z = s.z[i];
+        const float vx = s.vx[i], vy = s.vy[i], vz = s.vz[i], m = s.m[i], eps = s.eps[i];
+        const uint8_t t = s.type[i];
+        const float u = t == GNB_GAS ? s.u[i] : 0.f;
+        if (COPY) {
+            p.id[i] = s.id[i];
+            p.type[i] = t;
+            p.x[i] = x; p.y[i] = y; p.z[i] = z;
+            p.vx[i] = vx; p.vy[i] = vy; p.vz[i] = vz;
+            p.m[i] = m; p.eps[i] = eps;
+        }
+        p.u[i] = u;
+        p.orig[i] = i;
+        p.h2[i] = 0.0;
+        p.vpx[i] = vx; p.vpy[i] = vy; p.vpz[i] = vz;
+        p.up[i] = u;
+        if (!isfinite(x) || !isfinite(y) || !isfinite(z)) b |= 1;
+        if (t > 1) b |= 2;
+        if (!(m > 0.f) || !isfinite(m)) b |= 4;
+        if (!(eps >= 0.f) || !isfinite(eps)) b |= 8;
+        if (eps == 0.f) b |= 16;
+        if (eps != eps0) b |= 32;
+        ng += t == GNB_GAS;
+    }
+    ng = warp_sum(ng);
+    b = __reduce_or_sync(0xffffffffu, b);
+    if ((threadIdx.x & 31) == 0) {
+        if (ng) atomicAdd(&gas, ng);
+        if (b) atomicOr(bad, b);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        partial[blockIdx.x] = gas;
+        if (blockIdx.x == 0) {
+            *n_d = n;
+            *eps0_d = eps0;
+        }
+    }
 }
 
-__global__ void k_gas_flag_in(const uint8_t *__restrict__ type, int *__restrict__ flag, int n)
+// Exclusive scan of the block counts (one block; total in ngas and *out).
+__global__ void __launch_bounds__(1024) k_load_scan(int *__restrict__ partial, int *__restrict__ ngas,
+                                                    int *__restrict__ out)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) flag[i] = type[i] == GNB_GAS;
+    __shared__ int ws[32];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const int v = t < LD_BLOCKS ? partial[t] : 0;
+    int x = v;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) ws[w] = x;
+    __syncthreads();
+    int pre = 0;
+    for (int q = 0; q < w; q++) pre += ws[q];
+    if (t < LD_BLOCKS) partial[t] = pre + x - v;
+    if (t == 1023) *ngas = *out = pre + x;
 }
 
-__global__ void k_grank(const uint8_t *__restrict__ type, const int *__restrict__ off, int n, int *__restrict__ grank)
+// Rank of every gas particle among the gas, in the caller's order.
+__global__ void __launch_bounds__(LD_THREADS) k_grank(const uint8_t *__restrict__ type, const int *__restrict__ offs,
+                                                      int n, int *__restrict__ grank)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) grank[i] = type[i] == GNB_GAS ? off[i] : -1;
+    __shared__ int ws[2][LD_THREADS / 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int chunk = load_chunk(n), beg = (int)min((long long)n, (long long)blockIdx.x * chunk);
+    const int end = (int)min((long long)n, (long long)beg + chunk);
+    int carry = offs[blockIdx.x], par = 0;
+    for (int i0 = beg; i0 < end; i0 += LD_THREADS, par ^= 1) {
+        const int i = i0 + threadIdx.x;
+        const bool g = i < end && type[i] == GNB_GAS;
+        const unsigned bal = __ballot_sync(0xffffffffu, g);
+        if (lane == 0) ws[par][w] = __popc(bal);
+        __syncthreads();  // (the other half of ws is read before the next round's barrier)
+        int pre = 0, all = 0;
+        for (int q = 0; q < LD_THREADS / 32; q++) {
+            const int c = ws[par][q];
+            if (q < w) pre += c;
+            all += c;
+        }
+        if (i < end) grank[i] = g ? carry + pre + __popc(bal & ((1u << lane) - 1u)) : -1;
+        carry += all;
+    }
 }
 
 }  // namespace gnb
@@ -325,27 +407,28 @@ int gnb_set_particles(gnb_ctx *c, int64_t n, const int64_t *id, const uint8_t *t
     GNB_TRY(alloc_particles(c, n));
     c->cur = 0;
     PArr &p = c->P[0];
-    cudaMemcpyKind k = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     size_t N = (size_t)n;
+    LoadArgs src{id, type, x, y, z, vx, vy, vz, m, eps, u};
     struct { void *d; const void *s; size_t b; } cp[] = {
-        {p.id, id, 8 * N}, {p.type, type, N}, {p.x, x, 8 * N}, {p.y, y, 8 * N}, {p.z, z, 8 * N},
-        {p.vx, vx, 4 * N}, {p.vy, vy, 4 * N}, {p.vz, vz, 4 * N}, {p.m, m, 4 * N}, {p.eps, eps, 4 * N},
-        {p.u, u, 4 * N}};
-    for (auto &q : cp) GNB_TRY(cuda_check(c, cudaMemcpyAsync(q.d, q.s, q.b, k, c->s), "particle copy"));
+        {p.id, id, 8}, {p.type, type, 1}, {p.x, x, 8}, {p.y, y, 8}, {p.z, z, 8}, {p.vx, vx, 4},
+        {p.vy, vy, 4}, {p.vz, vz, 4}, {p.m, m, 4}, {p.eps, eps, 4}, {p.u, u, 4}};
+    // device arrays are read in place (copied first if one is not aligned to its elements)
+    bool copy = !on_device;
+    for (auto &q : cp) copy = copy || (uintptr_t)q.s % q.b != 0;
+    if (copy) {
+        const cudaMemcpyKind k = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+        for (auto &q : cp) GNB_TRY(cuda_check(c, cudaMemcpyAsync(q.d, q.s, q.b * N, k, c->s), "particle copy"));
+        src = LoadArgs{p.id, p.type, p.x, p.y, p.z, p.vx, p.vy, p.vz, p.m, p.eps, p.u};
+    }
     int ni = (int)n;
-    int nb = (ni + 255) / 256;
-    c->pinned_i[0] = ni;
-    cudaMemcpyAsync(c->n_d, c->pinned_i, sizeof(int), cudaMemcpyHostToDevice, c->s);
+    // work_d: [0] validity bits, [1] gas particles, [2] softening of the first
     cudaMemsetAsync(c->work_d, 0, sizeof(int), c->s);
-    gnb::counted(k_validate)<<<nb, 256, 0, c->s>>>(p, ni, c->work_d);
-    gnb::counted(k_set_init)<<<nb, 256, 0, c->s>>>(p, ni);
-    gnb::counted(k_gas_flag_in)<<<nb, 256, 0, c->s>>>(p.type, c->gas_flag, ni);
-    GNB_TRY(device_scan(c, c->gas_flag, c->pscan, c->n_d, ni, c->ngas_d));
-    gnb::counted(k_grank)<<<nb, 256, 0, c->s>>>(p.type, c->pscan, ni, p.grank);
+    gnb::counted(copy ? k_load<false> : k_load<true>)<<<LD_BLOCKS, LD_THREADS, 0, c->s>>>(
+        src, p, ni, c->n_d, c->work_d, (float *)(c->work_d + 2), c->scan_part);
+    gnb::counted(k_load_scan)<<<1, 1024, 0, c->s>>>(c->scan_part, c->ngas_d, c->work_d + 1);
+    gnb::counted(k_grank)<<<LD_BLOCKS, LD_THREADS, 0, c->s>>>(p.type, c->scan_part, ni, p.grank);
     GNB_LAUNCH_CHECK(c, "set particles");
-    cudaMemcpyAsync(c->pinned_i + 1, c->work_d, sizeof(int), cudaMemcpyDeviceToHost, c->s);
-    cudaMemcpyAsync(c->pinned_i + 2, c->ngas_d, sizeof(int), cudaMemcpyDeviceToHost, c->s);
-    cudaMemcpyAsync(c->pinned_i + 3, p.eps, sizeof(float), cudaMemcpyDeviceToHost, c->s);
+    cudaMemcpyAsync(c->pinned_i + 1, c->work_d, 3 * sizeof(int), cudaMemcpyDeviceToHost, c->s);
     GNB_TRY(cuda_check(c, cudaStreamSynchronize(c->s), "set particles sync"));
     int bad = c->pinned_i[1];
     int ng = c->pinned_i[2];
@@ -933,16 +1016,22 @@ int gnb_get_fields(gnb_ctx *c, int nf, const int *fields, void *const *dst, cons
         own = true;
     }
     int rc = GNB_OK;
-    for (int k = 0; k < nf && rc == GNB_OK; k++) {
-        if (cnt[k] == 0) continue;
-        if (on_device) {
-            rc = scatter_out(c, fields[k], dst[k]);
-        } else {
-            rc = scatter_out(c, fields[k], tmp);
-            if (rc == GNB_OK)
-                rc = cuda_check(c, cudaMemcpyAsync(dst[k], tmp, (size_t)cnt[k] * esz[k], cudaMemcpyDeviceToHost, c->s),
-                                "export copy");
+    if (on_device) {
+        std::vector<int> f;
+        std::vector<void *> d;
+        for (int k = 0; k < nf; k++) {
+            if (cnt[k] == 0) continue;
+            f.push_back(fields[k]);
+            d.push_back(dst[k]);
         }
+        rc = export_fields(c, (int)f.size(), f.data(), d.data());
+    }
+    for (int k = 0; k < nf && rc == GNB_OK && !on_device; k++) {
+        if (cnt[k] == 0) continue;
+        rc = scatter_out(c, fields[k], tmp);
+        if (rc == GNB_OK)
+            rc = cuda_check(c, cudaMemcpyAsync(dst[k], tmp, (size_t)cnt[k] * esz[k], cudaMemcpyDeviceToHost, c->s),
+                            "export copy");
     }
     if (rc == GNB_OK && !on_device) rc = cuda_check(c, cudaStreamSynchronize(c->s), "export sync");
     if (own) cudaFree(tmp);

@@ -111,7 +111,6 @@ struct gnb_ctx {
     uint64_t *skey = nullptr, *skey2 = nullptr;
     float *kres = nullptr;    // remainders of the coordinates within their grid cells [3][cap], slot order
     int *sval = nullptr, *sval2 = nullptr, *slot_of_orig = nullptr, *src = nullptr;
-    int *pscan = nullptr;     // per-slot scan scratch
     unsigned char *tmp_out = nullptr;  // export staging (8 bytes per particle)
     int *rs_buf = nullptr;    // radix sort: histograms, tickets, flags, published counts (sort.cu)
     size_t rs_words = 0;
@@ -125,7 +124,7 @@ struct gnb_ctx {
     // hydro (gas) arrays, gas order = Morton order of the gas particles
     int64_t gcap = 0;
     int *gslot = nullptr;         // particle slot of each gas particle
-    int *gas_flag = nullptr, *ngas_d = nullptr;
+    int *ngas_d = nullptr;        // device copy of n_gas
     uint64_t *gkey = nullptr;
     gnb::Tree gt;                 // hydro tree over gas
     int *ggrank = nullptr;
@@ -343,6 +342,7 @@ int predict(gnb_ctx *c, float hdt);
 int kick_drift_predict(gnb_ctx *c, float hdt, double dt);
 int diagnostics(gnb_ctx *c, double out[10]);
 int scatter_out(gnb_ctx *c, int field, void *dst_dev);
+int export_fields(gnb_ctx *c, int nf, const int *fields, void *const *dst_dev);
 
 }  // namespace gnb
 

@@ -133,3 +133,46 @@ def test_direct_gravity_forms(G, orc, n, n_group, eps):
     ref = orc.direct_gravity(p)
     d = np.sqrt(sum((c.get("AGRAV_" + k) - ref["a" + k.lower()]) ** 2 for k in "XYZ"))
     assert np.max(d / ref["asum"]) < 1e-5
+
+
+# upload: the gas ranks and the copy from device arrays around block chunks, a
+# mixed set, and device arrays that start at odd addresses; export of more
+# fields than one launch takes
+@pytest.mark.parametrize("n", [65, 256 * 912 - 1, 256 * 912 + 1])
+def test_upload_and_export(G, n):
+    import torch
+    p = ics.uniform_random(n, seed=n)
+    p["type"] = (np.random.default_rng(n).uniform(size=n) < 0.7).astype(np.uint8) if n > 100 else p["type"]
+    size = {k: v.dtype.itemsize for k, v in p.items()}
+    dev = {k: torch.from_numpy(v).cuda() for k, v in p.items()}
+    raw = {k: torch.empty(n * size[k] + 1, dtype=torch.uint8, device="cuda") for k in p}  # off by one byte
+    for k in p:
+        raw[k][1:] = dev[k].view(torch.uint8).reshape(-1)
+    keys = ("id", "type", "x", "y", "z", "vx", "vy", "vz", "m", "eps", "u")
+    out = []
+    for how in ("host", "device", "odd"):
+        c = G.Context()
+        if how == "odd":
+            torch.cuda.synchronize()
+            assert G.gnb_set_particles(c.h, n, *[raw[k].data_ptr() + 1 for k in keys], 1) == 0
+            c.n, c.n_gas = n, int(p["type"].sum())
+        else:
+            c.set_particles(p if how == "host" else dev)
+        assert c.stats()["NGAS"] == int(p["type"].sum())
+        c.build_tree()
+        f = {k: torch.empty(n, device="cuda", dtype=torch.float64 if k in "XYZ" else torch.int64 if k == "ID" else
+                            torch.float32) for k in ("X", "Y", "Z", "VX", "VY", "VZ", "U", "ID")}
+        c.get_fields(f)
+        fids, reps = [G.F["VX"], G.F["X"]] * 20, [torch.empty(n, device="cuda", dtype=torch.float64) for _ in range(40)]
+        import ctypes as C
+        assert G.gnb_get_fields(c.h, 40, (C.c_int * 40)(*fids), (C.c_void_p * 40)(*[r.data_ptr() for r in reps]),
+                                (C.c_int64 * 40)(*[n] * 40), 1) == 0
+        assert all(torch.equal(r, f["X"]) for r in reps[1::2])
+        assert all(torch.equal(r.view(torch.float32)[:n], f["VX"]) for r in reps[0::2])
+        c.compute_sph_density()
+        out.append({k: v.cpu().numpy() for k, v in f.items()} | {"NBR": c.get("NBR"), "H2": c.get("H2")})
+    for k in ("X", "Y", "Z", "VX", "VY", "VZ", "ID"):
+        assert np.array_equal(out[0][k], p[k.lower()])
+    assert np.array_equal(out[0]["U"], np.where(p["type"] == 1, p["u"], 0).astype(np.float32))
+    for k in out[0]:
+        assert np.array_equal(out[0][k], out[1][k]) and np.array_equal(out[0][k], out[2][k])
