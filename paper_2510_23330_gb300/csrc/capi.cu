@@ -137,19 +137,17 @@ static int alloc_gas(gnb_ctx *c, int64_t ng)
     return GNB_OK;
 }
 
-// After a synchronisation: translate and clear the device status word.
+// Wait for the stream, then translate and clear the device status word.
 static int check_status(gnb_ctx *c)
 {
+    cudaMemcpyAsync(c->pinned_i + 32, c->status_d, sizeof(int), cudaMemcpyDeviceToHost, c->s);
     GNB_TRY(cuda_check(c, cudaStreamSynchronize(c->s), "stream synchronize"));
     GNB_TRY(cuda_check(c, cudaGetLastError(), "kernel"));
-    int st = 0;
-    GNB_TRY(cuda_check(c, cudaMemcpy(&st, c->status_d, sizeof(int), cudaMemcpyDeviceToHost), "status read"));
+    const int st = c->pinned_i[32];
     if (st == 0) return GNB_OK;
     cudaMemsetAsync(c->status_d, 0, sizeof(int), c->s);
     if (st & ST_BAD_INPUT) return fail(c, GNB_EINVAL, "non-finite particle position");
-    if (st & ST_TREE_OVERFLOW) return fail(c, GNB_ECAPACITY, "tree node capacity exceeded");
     if (st & ST_STACK_OVERFLOW) return fail(c, GNB_ECAPACITY, "tree walk stack overflow");
-    if (st & ST_KNN_OVERFLOW) return fail(c, GNB_ECAPACITY, "kNN selection buffer overflow");
     return fail(c, GNB_ECAPACITY, "device status " + std::to_string(st));
 }
 
@@ -360,7 +358,7 @@ void gnb_destroy(gnb_ctx *c)
     replace_free(c);
     void *all[] = {c->status_d, c->n_d, c->ngas_d, c->counters_d, c->work_d, c->box_d, c->mm_d, c->red_d,
                    c->rs_buf, c->rtot_d, c->scan_part, c->scan_poff, c->gl_pool, c->gl_next, c->gl_cnt,
-                   c->gl_top, c->gl_head, c->gl_ref, c->gl_lcum, c->gd_part};
+                   c->gl_head, c->gl_ref, c->gl_lcum, c->gd_part};
     for (void *q : all) dfree(c, q);
     if (c->pinned_i) cudaFreeHost(c->pinned_i);
     {
@@ -564,6 +562,8 @@ static int do_build(gnb_ctx *c)
     return GNB_OK;
 }
 
+// The group count and the level table of the gravity tree: queued here, taken
+// over by finish() after its wait.
 static int read_groups(gnb_ctx *c)
 {
     if (!c->tree_valid) return GNB_OK;  // no gravity tree for the current positions (gravity off)
@@ -571,19 +571,26 @@ static int read_groups(gnb_ctx *c)
                        "groups count"));
     GNB_TRY(cuda_check(c, cudaMemcpyAsync(c->pinned_i + 9, c->t.lvl, sizeof(int) * (GNB_MAXLEV + 2),
                                           cudaMemcpyDeviceToHost, c->s), "levels"));
-    GNB_TRY(cuda_check(c, cudaStreamSynchronize(c->s), "groups sync"));
+    c->groups_queued = true;
+    return GNB_OK;
+}
+
+static void take_groups(gnb_ctx *c)
+{
+    if (!c->groups_queued) return;
+    c->groups_queued = false;
     c->t.ngroups = c->pinned_i[8];
     c->stats[GNB_S_GROUPS] = c->t.ngroups;
     int maxlev = 0;
     for (int l = 0; l <= GNB_MAXLEV; l++)
         if (c->pinned_i[9 + l + 1] > c->pinned_i[9 + l]) maxlev = l;
     c->stats[GNB_S_MAXLEVEL] = maxlev;
-    return GNB_OK;
 }
 
 static int do_gravity(gnb_ctx *c, int mode)
 {
-    cudaMemsetAsync(c->counters_d, 0, 2 * sizeof(unsigned long long), c->s);
+    // interaction counts, list pool top and work counters (see gravity.cu)
+    cudaMemsetAsync(c->counters_d, 0, 8 * sizeof(unsigned long long), c->s);
     phase_begin(c, GNB_T_GRAVITY);
     if (mode == GNB_GRAV_TREE) {
         GNB_TRY(gravity_tree(c));
@@ -605,6 +612,9 @@ static int do_forces(gnb_ctx *c, int mode)
     GNB_TRY(mode == GNB_GRAV_NONE ? do_sort(c) : do_build(c));
     GNB_TRY(do_gravity(c, mode));
     GNB_TRY(sph_density(c));
+    // the walk's lists fitted their pool (sph_density waits for the stream
+    // when there is gas): else gravity again, before anything is added to it
+    GNB_TRY(gravity_settle(c, c->n_gas > 0));
     c->density_valid = true;
     GNB_TRY(sph_force(c));
     c->force_valid = true;
@@ -633,12 +643,14 @@ static int finish(gnb_ctx *c, int rc)
 {
     if (rc != GNB_OK) {
         cudaStreamSynchronize(c->s);
+        c->groups_queued = c->grav_queued = false;
         cudaGetLastError();
         cudaMemsetAsync(c->status_d, 0, sizeof(int), c->s);
         phase_resolve(c);
         return rc;
     }
     rc = check_status(c);
+    take_groups(c);
     phase_resolve(c);
     return rc;
 }
@@ -668,6 +680,7 @@ int gnb_compute_gravity(gnb_ctx *c, int mode)
     if (!c->tree_valid) rc = do_build(c);
     if (rc == GNB_OK) rc = do_gravity(c, mode);
     if (rc == GNB_OK) rc = read_groups(c);
+    if (rc == GNB_OK) rc = gravity_settle(c, false);
     c->force_valid = false;
     return finish(c, rc);
 }
@@ -1066,14 +1079,15 @@ int gnb_stats(gnb_ctx *c, int64_t out[GNB_S_COUNT_])
 {
     if (!c || !out) return GNB_EINVAL;
     unsigned long long h[2] = {0, 0};
-    if (c->counters_d) {
-        cudaStreamSynchronize(c->s);
-        cudaMemcpy(h, c->counters_d, sizeof(h), cudaMemcpyDeviceToHost);
+    int rt = 0;
+    cudaMemcpyAsync(c->pinned_i + 34, c->counters_d, sizeof(h), cudaMemcpyDeviceToHost, c->s);
+    if (c->n_gas > 0) cudaMemcpyAsync(c->pinned_i + 38, c->rtot_d, sizeof(int), cudaMemcpyDeviceToHost, c->s);
+    if (cudaStreamSynchronize(c->s) == cudaSuccess) {
+        memcpy(h, c->pinned_i + 34, sizeof(h));
+        if (c->n_gas > 0) rt = c->pinned_i[38];
     }
     c->stats[GNB_S_NPP] = (int64_t)h[0];
     c->stats[GNB_S_NPC] = (int64_t)h[1];
-    int rt = 0;
-    if (c->rtot_d && c->n_gas > 0) cudaMemcpy(&rt, c->rtot_d, sizeof(int), cudaMemcpyDeviceToHost);
     c->stats[GNB_S_NSYM] = (int64_t)c->n_gas * 63 + rt;
     for (int k = 0; k < GNB_S_COUNT_; k++) out[k] = c->stats[k];
     return GNB_OK;

@@ -39,10 +39,7 @@ inline K counted(K k)
 
 // Device-side status word bits (set by kernels, read by the host).
 enum : int {
-    ST_TREE_OVERFLOW = 1,
     ST_STACK_OVERFLOW = 2,
-    ST_KNN_OVERFLOW = 4,
-    ST_SYM_OVERFLOW = 8,
     ST_BAD_INPUT = 16,
 };
 
@@ -207,13 +204,15 @@ struct gnb_ctx {
     // status / counters
     int *status_d = nullptr;
     int *n_d = nullptr;                        // device copy of n
-    unsigned long long *counters_d = nullptr;  // [8]
+    unsigned long long *counters_d = nullptr;  // [8]: pp, pc, -, -, -, list pool top, walk's next, evaluation's next
     int *work_d = nullptr;                     // work counters of persistent kernels [8]
     int *scan_part = nullptr, *scan_poff = nullptr;  // device_scan scratch [1100]
     // tree-gravity interaction lists (gravity.cu): chunk pool and per-group heads
-    int *gl_pool = nullptr, *gl_next = nullptr, *gl_cnt = nullptr, *gl_top = nullptr, *gl_lcum = nullptr;
+    int *gl_pool = nullptr, *gl_next = nullptr, *gl_cnt = nullptr, *gl_lcum = nullptr;
     int4 *gl_head = nullptr, *gl_ref = nullptr;
     int gl_cap = 0, gl_gcap = 0;
+    bool grav_queued = false;                  // the walk's pool use is on its way to pinned_i[40] (gravity_settle)
+    bool groups_queued = false;                // group count and levels on their way to pinned_i[8..] (finish)
     float4 *gd_part = nullptr;                 // direct gravity: sums of the source parts [parts][n]
     int64_t gd_cap = 0;
     int *pinned_i = nullptr;                   // pinned host scratch [64]
@@ -314,6 +313,7 @@ int save_state(gnb_ctx *c, const char *path);
 int load_state(gnb_ctx *c, const char *path);
 // gravity.cu
 int gravity_tree(gnb_ctx *c);
+int gravity_settle(gnb_ctx *c, bool waited);
 int gravity_direct(gnb_ctx *c);
 int assemble_forces(gnb_ctx *c, bool self);
 // sph.cu

@@ -747,6 +747,7 @@ __global__ void __launch_bounds__(GW_THREADS, 5) k_grav_eval(GravParams p)
     const int tid = threadIdx.x;
     const float unit = (float)p.box[4];
     const int ngroups = *p.ngroups;
+    if (*p.top > p.cap) return;  // the walk ran out of chunks: gravity_settle repeats it
     for (;;) {
         if (tid == 0) S.g = atomicAdd(p.next, 1);
         __syncthreads();
@@ -979,7 +980,6 @@ static int launch_persistent(gnb_ctx *c, K kern, GravParams p, int *next_d)
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, GW_THREADS, smem);
     if (per_sm < 1) per_sm = 1;
     p.next = next_d;
-    cudaMemsetAsync(next_d, 0, sizeof(int), c->s);
     gnb::counted(kern)<<<sm_count() * per_sm, GW_THREADS, smem, c->s>>>(p);
     GNB_LAUNCH_CHECK(c, "gravity kernel");
     return GNB_OK;
@@ -1012,8 +1012,49 @@ static int lists_alloc(gnb_ctx *c, int chunks)
         GNB_TRY(dalloc(c, &c->gl_cnt, (size_t)chunks));
         c->gl_cap = chunks;
     }
-    if (!c->gl_top) GNB_TRY(dalloc(c, &c->gl_top, 1));
     return GNB_OK;
+}
+
+// The walk and the evaluation, one after the other on the stream; the pool's
+// use is copied to pinned_i[40] for gravity_settle.  counters_d is clear.
+static int gravity_lists(gnb_ctx *c)
+{
+    GravParams p = make_params(c);
+    p.pool = c->gl_pool; p.cnext = c->gl_next; p.ccnt = c->gl_cnt; p.top = (int *)(c->counters_d + 5); p.lcum = c->gl_lcum;
+    p.ghead = c->gl_head; p.gref = c->gl_ref; p.cap = c->gl_cap;
+    p.next = (int *)(c->counters_d + 6);
+    int *next_d = (int *)(c->counters_d + 7);
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_grav_walk, GL_WARPS * 32, 0);
+    gnb::counted(k_grav_walk)<<<sm_count() * std::max(per_sm, 1), GL_WARPS * 32, 0, c->s>>>(p);
+    GNB_LAUNCH_CHECK(c, "tree walk");
+    GNB_TRY(cuda_check(c, cudaMemcpyAsync(&c->pinned_i[40], p.top, sizeof(int), cudaMemcpyDeviceToHost, c->s),
+                       "list pool read"));
+    c->grav_queued = true;
+    const bool q = c->cfg.multipole != 0;
+    // groups of more than 128 particles: eight i-particles per thread
+    if (c->cfg.n_group > 128) {
+        if (c->min_eps_zero) {
+            if (q) return launch_persistent(c, k_grav_eval<true, true, 8, false>, p, next_d);
+            return launch_persistent(c, k_grav_eval<true, false, 8, false>, p, next_d);
+        }
+        if (c->eps_uniform) {
+            if (q) return launch_persistent(c, k_grav_eval<false, true, 8, true>, p, next_d);
+            return launch_persistent(c, k_grav_eval<false, false, 8, true>, p, next_d);
+        }
+        if (q) return launch_persistent(c, k_grav_eval<false, true, 8, false>, p, next_d);
+        return launch_persistent(c, k_grav_eval<false, false, 8, false>, p, next_d);
+    }
+    if (c->min_eps_zero) {
+        if (q) return launch_persistent(c, k_grav_eval<true, true, 4, false>, p, next_d);
+        return launch_persistent(c, k_grav_eval<true, false, 4, false>, p, next_d);
+    }
+    if (c->eps_uniform) {
+        if (q) return launch_persistent(c, k_grav_eval<false, true, 4, true>, p, next_d);
+        return launch_persistent(c, k_grav_eval<false, false, 4, true>, p, next_d);
+    }
+    if (q) return launch_persistent(c, k_grav_eval<false, true, 4, false>, p, next_d);
+    return launch_persistent(c, k_grav_eval<false, false, 4, false>, p, next_d);
 }
 
 int gravity_tree(gnb_ctx *c)
@@ -1022,59 +1063,32 @@ int gravity_tree(gnb_ctx *c)
     // entries per particle
     const int want = 2 * c->t.nnodes + (int)((16 * (long long)c->n) / GL_CH) + 1024;
     GNB_TRY(lists_alloc(c, std::max(c->gl_cap, want)));
-    int *next_d = (int *)(c->counters_d + 6);
+    return gravity_lists(c);
+}
+
+// After a wait for the stream (made here unless `waited`): the pool must have
+// held every list; otherwise grow it, walk and evaluate again (an evaluation
+// of incomplete lists does nothing) and repeat the assembly that followed.
+int gravity_settle(gnb_ctx *c, bool waited)
+{
+    if (!c->grav_queued) return GNB_OK;
     for (int attempt = 0;; attempt++) {
-        GravParams p = make_params(c);
-        p.pool = c->gl_pool; p.cnext = c->gl_next; p.ccnt = c->gl_cnt; p.top = c->gl_top; p.lcum = c->gl_lcum;
-        p.ghead = c->gl_head; p.gref = c->gl_ref; p.cap = c->gl_cap;
-        p.next = next_d;
-        cudaMemsetAsync(c->counters_d, 0, 2 * sizeof(unsigned long long), c->s);
-        cudaMemsetAsync(c->gl_top, 0, sizeof(int), c->s);
-        cudaMemsetAsync(next_d, 0, sizeof(int), c->s);
-        int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_grav_walk, GL_WARPS * 32, 0);
-        gnb::counted(k_grav_walk)<<<sm_count() * std::max(per_sm, 1), GL_WARPS * 32, 0, c->s>>>(p);
-        GNB_LAUNCH_CHECK(c, "tree walk");
-        // the pool must have held every list; otherwise grow it and walk again
-        GNB_TRY(cuda_check(c, cudaMemcpyAsync(&c->pinned_i[40], c->gl_top, sizeof(int), cudaMemcpyDeviceToHost, c->s),
-                           "list pool read"));
-        GNB_TRY(cuda_check(c, cudaStreamSynchronize(c->s), "list pool sync"));
+        if (!waited || attempt > 0) GNB_TRY(cuda_check(c, cudaStreamSynchronize(c->s), "list pool sync"));
+        c->grav_queued = false;
         const int used = c->pinned_i[40];
-        if (used <= c->gl_cap) {
-            const bool q = c->cfg.multipole != 0;
-            // groups of more than 128 particles: eight i-particles per thread
-            if (c->cfg.n_group > 128) {
-                if (c->min_eps_zero) {
-                    if (q) return launch_persistent(c, k_grav_eval<true, true, 8, false>, p, next_d);
-                    return launch_persistent(c, k_grav_eval<true, false, 8, false>, p, next_d);
-                }
-                if (c->eps_uniform) {
-                    if (q) return launch_persistent(c, k_grav_eval<false, true, 8, true>, p, next_d);
-                    return launch_persistent(c, k_grav_eval<false, false, 8, true>, p, next_d);
-                }
-                if (q) return launch_persistent(c, k_grav_eval<false, true, 8, false>, p, next_d);
-                return launch_persistent(c, k_grav_eval<false, false, 8, false>, p, next_d);
-            }
-            if (c->min_eps_zero) {
-                if (q) return launch_persistent(c, k_grav_eval<true, true, 4, false>, p, next_d);
-                return launch_persistent(c, k_grav_eval<true, false, 4, false>, p, next_d);
-            }
-            if (c->eps_uniform) {
-                if (q) return launch_persistent(c, k_grav_eval<false, true, 4, true>, p, next_d);
-                return launch_persistent(c, k_grav_eval<false, false, 4, true>, p, next_d);
-            }
-            if (q) return launch_persistent(c, k_grav_eval<false, true, 4, false>, p, next_d);
-            return launch_persistent(c, k_grav_eval<false, false, 4, false>, p, next_d);
-        }
+        if (used <= c->gl_cap) return GNB_OK;
         if (attempt >= 4) return fail(c, GNB_ECAPACITY, "interaction-list pool");
         GNB_TRY(lists_alloc(c, used + used / 2 + 1024));
+        cudaMemsetAsync(c->counters_d, 0, 8 * sizeof(unsigned long long), c->s);
+        GNB_TRY(gravity_lists(c));
+        GNB_TRY(assemble_forces(c, true));
     }
 }
 
 int gravity_direct(gnb_ctx *c)
 {
     GravParams p = make_params(c);
-    int *next_d = (int *)(c->counters_d + 6);
+    int *next_d = (int *)(c->counters_d + 7);  // clear, as gravity_tree's
     const int n = (int)c->n;
     // parts of the sources: about eight units per resident CTA, counting three
     // groups per n_group particles (cells are a third full on average), at
@@ -1091,7 +1105,6 @@ int gravity_direct(gnb_ctx *c)
         c->gd_cap = (int64_t)n * segs;
     }
     p.next = next_d;
-    cudaMemsetAsync(next_d, 0, sizeof(int), c->s);
     auto k = c->min_eps_zero ? k_gravity_direct<true, false>
                              : (c->eps_uniform ? k_gravity_direct<false, true> : k_gravity_direct<false, false>);
     int per_sm = 0;

@@ -164,7 +164,7 @@ struct KnnParams {
     const double *box;
     const float *rprev;  // previous support per gas particle (0: none)
     float margin;        // search radius over the previous support
-    int *status;
+    int *failed;         // set when a particle could not be ranked
     int *nbr;
     float *nd2;
     double *h2;
@@ -726,7 +726,7 @@ __global__ void __launch_bounds__(KN_THREADS, KN_CTAS) k_knn(KnnParams p)
                 // (each with the radius of its own members), then singles
                 step = len > KN_SUB ? KN_SUB : 1;
             } else {
-                if (lane == 0) atomicOr(p.status, ST_KNN_OVERFLOW);
+                if (lane == 0) atomicOr(p.failed, 1);
                 pos++;
             }
         }
@@ -987,8 +987,9 @@ int sph_density(gnb_ctx *c)
     int sub = 1;
     for (int q : steps)
         if ((long long)ng > (long long)q * g_knn_blocks * KN_WARPS) sub *= 2;
-    // work_d: [0] next item, [1] items whose radius was widened, [2] items
-    cudaMemsetAsync(c->work_d, 0, 3 * sizeof(int), c->s);
+    // work_d: [0] next item, [1] items whose radius was widened, [2] items,
+    // [3] set when a particle could not be ranked
+    cudaMemsetAsync(c->work_d, 0, 4 * sizeof(int), c->s);
     gnb::counted(k_knn_init)<<<304, 256, 0, c->s>>>(c->gt, sub, c->box_d, c->kR, c->kitem, c->work_d + 2);
     KnnParams p;
     p.na = c->gt.na; p.nb = c->gt.nb; p.item = c->kitem; p.kR = c->kR; p.nitems = c->work_d + 2;
@@ -997,17 +998,16 @@ int sph_density(gnb_ctx *c)
     p.gx = c->gx; p.gy = c->gy; p.gz = c->gz; p.box = c->box_d;
     p.rprev = c->gRprev;
     p.margin = c->knn_margin;
-    p.status = c->status_d;
+    p.failed = c->work_d + 3;
     p.nbr = c->nbr; p.nd2 = c->nd2; p.h2 = c->gh2; p.h2b = c->gh2b; p.h = c->gh; p.E = c->gE; p.g64 = c->g64;
     p.gvx = c->gvx; p.gvy = c->gvy; p.gvz = c->gvz; p.V = c->fV; p.Q = c->fQ;
     p.gslot = c->gslot; p.s_rho = c->rho; p.s_pres = c->pres; p.s_cs = c->cs; p.s_h2 = a.h2;
     p.gamma = (float)c->cfg.gamma; p.pressure = c->cfg.sph_variant;
     gnb::counted(k_knn)<<<g_knn_blocks, KN_THREADS, smem, c->s>>>(p);
     GNB_LAUNCH_CHECK(c, "knn");
-    cudaMemcpyAsync(c->pinned_i, c->work_d, 3 * sizeof(int), cudaMemcpyDeviceToHost, c->s);
-    cudaMemcpyAsync(c->pinned_i + 20, c->status_d, sizeof(int), cudaMemcpyDeviceToHost, c->s);
+    cudaMemcpyAsync(c->pinned_i, c->work_d, 4 * sizeof(int), cudaMemcpyDeviceToHost, c->s);
     GNB_TRY(cuda_check(c, cudaStreamSynchronize(c->s), "knn sync"));
-    if (c->pinned_i[20] & ST_KNN_OVERFLOW) return fail(c, GNB_ECAPACITY, "kNN selection buffer overflow");
+    if (c->pinned_i[3]) return fail(c, GNB_ECAPACITY, "kNN selection buffer overflow");
     c->stats[GNB_S_KNN_PASSES] = 1;
     // the next evaluation's margin: wider when more than 4 % of the items
     // needed a larger radius, narrower (to 1.01) below 1 %

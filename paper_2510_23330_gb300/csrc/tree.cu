@@ -432,8 +432,7 @@ __device__ void emit_slot(const Tree &t, const uint64_t *__restrict__ k, int i, 
 
 __global__ void __launch_bounds__(TB_THREADS) k_tb_emit(Tree t, const uint64_t *__restrict__ k, int n,
                                                         const int *__restrict__ span, const int *__restrict__ tcnt,
-                                                        const int *__restrict__ tot, int ntiles, int rounds,
-                                                        int *__restrict__ status)
+                                                        const int *__restrict__ tot, int ntiles, int rounds)
 {
     __shared__ EmitShared S;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -451,11 +450,10 @@ __global__ void __launch_bounds__(TB_THREADS) k_tb_emit(Tree t, const uint64_t *
             S.ok = all <= t.cap;
         }
         if (blockIdx.x == 0) {
-            if (all > t.cap) {
-                if (lane == 0) atomicOr(status, ST_TREE_OVERFLOW);
-            } else {
-                if (lane < TB_NCNT) t.lvl[lane] = inc - v;  // entry TB_NCNT - 1: all nodes
-                if (lane == 0) *t.ngroups_d = tot[TB_NCNT - 1];
+            if (lane < TB_NCNT) t.lvl[lane] = inc - v;  // entry TB_NCNT - 1: all nodes
+            if (lane == 0) {
+                t.lvl[TB_NCNT] = all > t.cap ? 1 : 0;  // read back with the table
+                *t.ngroups_d = tot[TB_NCNT - 1];
             }
         }
     }
@@ -778,20 +776,17 @@ int build_tree(gnb_ctx *c, Tree &t, const uint64_t *skey, int n, const int *n_d,
     const int *lv = c->pinned_i + 1;  // level table copy [GNB_MAXLEV + 2]
     for (int attempt = 0;; attempt++) {
         gnb::counted(k_tb_emit)<<<ntiles, TB_THREADS, 0, c->s>>>(t, skey, n, t.span, t.tcnt, t.tot, ntiles,
-                                                                  rounds, c->status_d);
+                                                                  rounds);
         GNB_LAUNCH_CHECK(c, "tree build");
-        cudaMemcpyAsync(c->pinned_i, c->status_d, sizeof(int), cudaMemcpyDeviceToHost, c->s);
-        cudaMemcpyAsync(c->pinned_i + 1, t.lvl, sizeof(int) * (GNB_MAXLEV + 2), cudaMemcpyDeviceToHost, c->s);
+        cudaMemcpyAsync(c->pinned_i + 1, t.lvl, sizeof(int) * (TB_NCNT + 1), cudaMemcpyDeviceToHost, c->s);
         GNB_TRY(cuda_check(c, cudaStreamSynchronize(c->s), "tree build sync"));
-        if (!(c->pinned_i[0] & ST_TREE_OVERFLOW)) break;
+        if (!lv[TB_NCNT]) break;
         if (attempt > 0) return fail(c, GNB_ECAPACITY, "tree node capacity");
         // more nodes than the arrays hold: grow them to the count and emit again
         int tot_h[TB_NCNT];
         GNB_TRY(cuda_check(c, cudaMemcpy(tot_h, t.tot, sizeof(tot_h), cudaMemcpyDeviceToHost), "node count"));
         long long need = 0;
         for (int l = 0; l < TB_NCNT - 1; l++) need += tot_h[l];
-        const int zero = 0;
-        GNB_TRY(cuda_check(c, cudaMemcpy(c->status_d, &zero, sizeof(int), cudaMemcpyHostToDevice), "status reset"));
         if (need + need / 4 + 1024 > INT32_MAX) return fail(c, GNB_ECAPACITY, "tree node capacity");
         GNB_TRY(tree_alloc(c, t, (int)(need + need / 4 + 1024)));
     }

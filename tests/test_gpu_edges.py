@@ -176,3 +176,26 @@ def test_upload_and_export(G, n):
     assert np.array_equal(out[0]["U"], np.where(p["type"] == 1, p["u"], 0).astype(np.float32))
     for k in out[0]:
         assert np.array_equal(out[0][k], out[1][k]) and np.array_equal(out[0][k], out[2][k])
+
+
+# a nearly direct walk fills the interaction-list pool: grown and repeated after
+# the evaluation, before the forces are used
+@pytest.mark.parametrize("n_gas", [0, 500])
+def test_list_pool_grows(G, n_gas):
+    p = ics.plummer(12000, seed=2, n_gas=n_gas)
+    got = {}
+    for theta in (0.03, 0.5):
+        c = G.Context(theta=theta, n_group=64)
+        c.set_particles(p)
+        c.step_kdk(1e-3, 1, G.GNB_GRAV_TREE)
+        got[theta] = [c.get(k).astype(np.float64) for k in ("AGRAV_X", "AGRAV_Y", "AGRAV_Z", "VX", "X")]
+        if theta < 0.1:
+            assert c.stats()["NPP"] + c.stats()["NPC"] > 256 * 64 * (2 * c.stats()["NODES"] + 1774)
+    d = G.Context(n_group=64)
+    d.set_particles(p)
+    d.step_kdk(1e-3, 1, G.GNB_GRAV_DIRECT)
+    ref = [d.get(k).astype(np.float64) for k in ("AGRAV_X", "AGRAV_Y", "AGRAV_Z", "VX", "X")]
+    scale = np.sqrt(sum(r ** 2 for r in ref[:3]))
+    err = {t: np.sqrt(sum((a - r) ** 2 for a, r in zip(g[:3], ref))) / scale for t, g in got.items()}
+    assert np.median(err[0.03]) < 1e-5 < np.median(err[0.5])
+    assert np.max(np.abs(got[0.03][3] - ref[3])) < 1e-6 and np.max(np.abs(got[0.03][4] - ref[4])) < 1e-8
