@@ -705,14 +705,19 @@ __global__ void __launch_bounds__(128) k_up2_tc(const Up2Args p)
 // as a GEMM whose M = 128 rows are (tap slot s, input channel c) pairs --
 // 128 / C taps of one tap group side by side, so every row is a real weight
 // even for C = 16 -- whose N columns are the output channels and whose K is
-// the voxels.  A CTA takes one tap group and one chunk of voxels; per stage of
-// 64 voxels the threads gather the shifted inputs and the output gradient
-// (zero outside the grid) and write them transposed into the canonical
-// K-major core-matrix layout (8 rows x 16 bytes, rows = channels, the 16
-// bytes = 8 voxels), one elected lane issues four K = 16 MMAs into a TMEM
-// accumulator, and the stage buffers are double buffered behind the MMAs'
-// commit barriers.  At the end each warp reads its 32 TMEM lanes (rows) and
-// adds them to dW with FP32 atomics (the voxel chunks are split-K).
+// the voxels.  A CTA takes one tap group and one chunk of voxels.  Both
+// operands are MN-major: a voxel's 8 channels are one 16-byte row of a core
+// matrix (8 voxels x 8 channels, 128 bytes), which is how the blocked tensors
+// hold them, so a stage of 64 voxels is filled by 16-byte asynchronous copies
+// (zero-filled outside the grid) with no transposition through registers;
+// each thread owns one voxel of the stage and steps its coordinates once.
+// One elected lane issues four K = 16 MMAs per stage into a TMEM accumulator;
+// three stage buffers, two stages of copies in flight.  At the end each warp
+// reads its 32 TMEM lanes (rows) and adds them to dW with FP32 vector
+// reductions (the voxel chunks are split-K).  It is bound by the copies
+// through L1/L2 (27 shifted reads of the input).  All 14 layers of a 64^3
+// training step (cold cache): 1,824 us with 2-byte transposing stores and 64-bit
+// divisions per piece, 505 us so.
 struct WgTcArgs {
     const bf16 *x1, *x2;   // input channels [0, C1) from x1, [C1, C) from x2; blocked [B][C/8][V][8]
     int C1, C;
@@ -734,12 +739,16 @@ __device__ __forceinline__ void fence_proxy_async_smem()
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
 }
 
-// offset of (row r, voxel k) in a K-major stage of WG_VS voxels whose M (or N)
-// has rows rows: [k / 16][r / 8][(k % 16) / 8][r % 8][k % 8]
-__device__ __forceinline__ unsigned wg_off(int r, int k, int rows)
+constexpr int WG_ST = 3;   // stage buffers
+
+// 16-byte copy to shared memory, or zeros
+__device__ __forceinline__ void cp16z(unsigned dst, const void *src, bool have)
 {
-    return (unsigned)(k >> 4) * (unsigned)rows * 32u + (unsigned)(r >> 3) * 256u + (unsigned)((k >> 3) & 1) * 128u +
-           (unsigned)(r & 7) * 16u + (unsigned)(k & 7) * 2u;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(have ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void red_v4_f32(float *a, float x, float y, float z, float w)
+{
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"l"(a), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
 }
 
 __global__ void __launch_bounds__(128) k_wgrad_tc(const WgTcArgs p)
@@ -748,9 +757,8 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(const WgTcArgs p)
     const unsigned raw = smem_u32(dsm);
     const unsigned sb = (raw + (ALIGN_SLACK - 1)) & ~(ALIGN_SLACK - 1);
     unsigned char *gb = dsm + (sb - raw);
-    unsigned *slot = reinterpret_cast<unsigned *>(gb + 16);
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(gb + 20);
-    const unsigned bar0 = sb, bar1 = sb + 8;  // commit barriers of the two stage buffers
+    unsigned *slot = reinterpret_cast<unsigned *>(gb + 32);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(gb + 36);
     const unsigned stage_bytes = p.abytes + p.bbytes;
     unsigned char *stg = gb + WG_HDR;
     const unsigned sStg = sb + WG_HDR;
@@ -760,10 +768,9 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(const WgTcArgs p)
     const int ntap = min(p.ntap, 27 - t0);
     const long long r0 = (long long)blockIdx.x * p.chunk, r1 = min(p.V, r0 + p.chunk);
     const int nstage = (int)((r1 - r0 + WG_VS - 1) / WG_VS);
-    const long long D = p.D, Vs = D * D * D;
+    const int D = p.D, Vs = D * D * D;
     if (tid == 0) {
-        mb_init(bar0, 1);
-        mb_init(bar1, 1);
+        for (int k = 0; k < WG_ST; k++) mb_init(sb + 8u * k, 1);  // commit barriers of the stage buffers
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
@@ -778,78 +785,82 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(const WgTcArgs p)
     tc_fence_after();
     const unsigned tmem = *slot;
     // rows of tap slots beyond ntap (a short last group) stay zero: cleared once
-    for (unsigned o = (unsigned)tid * 16u; o < 2u * stage_bytes; o += 128u * 16u)
+    for (unsigned o = (unsigned)tid * 16u; o < (unsigned)WG_ST * stage_bytes; o += 128u * 16u)
         *reinterpret_cast<uint4 *>(stg + o) = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
-    const int cg8 = p.C >> 3, ng8 = p.N >> 3;
+    const int cg8 = p.C >> 3, ng8 = p.N >> 3, c18 = p.C1 >> 3;
+    // this thread's voxel of a stage (k) and its share of the pieces (half)
+    const int k = tid & (WG_VS - 1), half = tid >> 6;
+    long long v = r0 + k;
+    long long bb = v / Vs;
+    int rem = (int)(v - bb * Vs);
+    const unsigned koff = (unsigned)(k & 7) * 16u;
+    const unsigned ka = (unsigned)(k >> 3) * 2048u + koff, kb = (unsigned)(k >> 3) * (unsigned)p.N * 16u + koff;
+    auto load = [&](int st) {  // copies of stage st (called for st = 0, 1, 2, ... in order)
+        const unsigned sA = sStg + (unsigned)(st % WG_ST) * stage_bytes, sB = sA + p.abytes;
+        const bool in = v < r1;
+        const int z = rem / (D * D), yx = rem - z * D * D, y = yx / D, x = yx - y * D;
+        const bf16 *x1 = p.x1 + ((size_t)bb * c18 * Vs + rem) * 8;
+        const bf16 *x2 = p.x2 + ((size_t)bb * (cg8 - c18) * Vs + rem) * 8;
+        for (int s = 0; s < ntap; s++) {
+            const int t = t0 + s, dz = t / 9 - 1, dy = (t / 3) % 3 - 1, dx = t % 3 - 1;
+            const bool have = in && (unsigned)(z + dz) < (unsigned)D && (unsigned)(y + dy) < (unsigned)D &&
+                              (unsigned)(x + dx) < (unsigned)D;
+            const int off = have ? ((dz * D + dy) * D + dx) * 8 : 0;
+            for (int cg = half; cg < cg8; cg += 2) {
+                const bf16 *src = cg < c18 ? x1 + (size_t)cg * Vs * 8 : x2 + (size_t)(cg - c18) * Vs * 8;
+                cp16z(sA + ka + (unsigned)(s * cg8 + cg) * 128u, have ? src + off : p.x1, have);
+            }
+        }
+        const bf16 *g = p.g + ((size_t)bb * (p.Cg >> 3) * Vs + rem) * 8;
+        for (int ng = half; ng < ng8; ng += 2) cp16z(sB + kb + (unsigned)ng * 128u, in ? g + (size_t)ng * Vs * 8 : p.g, in);
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+        v += WG_VS;
+        rem += WG_VS;
+        while (rem >= Vs) {
+            rem -= Vs;
+            bb++;
+        }
+    };
+    load(0);
+    if (nstage > 1) load(1);
+    else asm volatile("cp.async.commit_group;\n" ::: "memory");
     bool ok = true;
     int issued = -1;  // the last stage whose MMAs were issued
-    for (int st = 0; st < nstage && ok; st++) {
-        const int b = st & 1;
-        const unsigned bar = b ? bar1 : bar0;
-        // the MMAs that read this buffer two stages ago have finished
-        if (st >= 2) ok = __syncthreads_and(mb_wait(bar, (unsigned)(((st - 2) >> 1) & 1), abort_flag, p.err, 21));
-        if (!ok) break;
-        unsigned char *sA = stg + (size_t)b * stage_bytes;
-        unsigned char *sB = sA + p.abytes;
-        const long long vb = r0 + (long long)st * WG_VS;
-        // A: (tap slot, channel group, voxel) pieces of 8 channels
-        for (int e = tid; e < ntap * cg8 * WG_VS; e += 128) {
-            const int k = e % WG_VS, q = e / WG_VS;
-            const int cg = q % cg8, s = q / cg8;
-            const long long v = vb + k;
-            uint4 val = make_uint4(0u, 0u, 0u, 0u);
-            if (v < r1) {
-                const long long bb = v / Vs, rem = v - bb * Vs;
-                const long long x = rem % D, y = (rem / D) % D, z = rem / (D * D);
-                const int t = t0 + s;
-                const long long zz = z + (t / 9 - 1), yy = y + ((t / 3) % 3 - 1), xx = x + (t % 3 - 1);
-                if (zz >= 0 && zz < D && yy >= 0 && yy < D && xx >= 0 && xx < D) {
-                    const long long src = (zz * D + yy) * D + xx;
-                    const int c = cg * 8;
-                    val = c < p.C1 ? *reinterpret_cast<const uint4 *>(p.x1 + ((bb * (p.C1 >> 3) + cg) * Vs + src) * 8)
-                                   : *reinterpret_cast<const uint4 *>(
-                                         p.x2 + ((bb * ((p.C - p.C1) >> 3) + (cg - (p.C1 >> 3))) * Vs + src) * 8);
-                }
-            }
-            const unsigned short *h = reinterpret_cast<const unsigned short *>(&val);
-            const int r = s * p.C + cg * 8;
-#pragma unroll
-            for (int j = 0; j < 8; j++) *reinterpret_cast<unsigned short *>(sA + wg_off(r + j, k, 128)) = h[j];
-        }
-        // B: (output channel group, voxel) pieces
-        for (int e = tid; e < ng8 * WG_VS; e += 128) {
-            const int k = e % WG_VS, ng = e / WG_VS;
-            const long long v = vb + k;
-            uint4 val = make_uint4(0u, 0u, 0u, 0u);
-            if (v < r1) {
-                const long long bb = v / Vs, rem = v - bb * Vs;
-                val = *reinterpret_cast<const uint4 *>(p.g + ((bb * (p.Cg >> 3) + ng) * Vs + rem) * 8);
-            }
-            const unsigned short *h = reinterpret_cast<const unsigned short *>(&val);
-#pragma unroll
-            for (int j = 0; j < 8; j++) *reinterpret_cast<unsigned short *>(sB + wg_off(ng * 8 + j, k, p.N)) = h[j];
-        }
-        fence_proxy_async_smem();  // the generic-proxy stores become visible to the tensor cores
+    for (int st = 0; st < nstage; st++) {
+        asm volatile("cp.async.wait_group 1;\n" ::: "memory");  // stage st has landed
+        fence_proxy_async_smem();  // ... and becomes visible to the tensor cores
         tc_fence_before();
         __syncthreads();
         if (warp == 0) {
             tc_fence_after();
-            const unsigned a0 = sStg + (unsigned)b * stage_bytes, b0 = a0 + p.abytes;
-            const unsigned hi = sdesc_hi(256u);
+            const unsigned a0 = sStg + (unsigned)(st % WG_ST) * stage_bytes, b0 = a0 + p.abytes;
+            const unsigned hi = sdesc_hi(128u);  // 8 rows (channels) to the next 8
 #pragma unroll
-            for (int ks = 0; ks < WG_VS / 16; ks++)
-                tc_mma_elect(tmem, dpair(sdesc_lo(a0 + (unsigned)ks * 128u * 32u, 128u), hi),
-                             dpair(sdesc_lo(b0 + (unsigned)ks * (unsigned)p.N * 32u, 128u), hi), p.idesc,
+            for (int ks = 0; ks < WG_VS / 16; ks++)  // K blocks of 8 voxels: 2,048 and 16 N bytes apart
+                tc_mma_elect(tmem, dpair(sdesc_lo(a0 + (unsigned)ks * 4096u, 2048u), hi),
+                             dpair(sdesc_lo(b0 + (unsigned)ks * (unsigned)p.N * 32u, (unsigned)p.N * 16u), hi), p.idesc,
                              (st > 0 || ks > 0) ? 1u : 0u);
-            tc_commit_elect(bar);
+            tc_commit_elect(sb + 8u * (unsigned)(st % WG_ST));
         }
         issued = st;
+        // the buffer of stage st + 2 is the one of stage st - 1, whose MMAs
+        // were issued one iteration ago
+        if (st >= 1) {
+            const int q = st - 1;
+            ok = __syncthreads_and(mb_wait(sb + 8u * (unsigned)(q % WG_ST), (unsigned)((q / WG_ST) & 1), abort_flag, p.err,
+                                           21));
+            if (!ok) break;
+        }
+        if (st + 2 < nstage) load(st + 2);
+        else asm volatile("cp.async.commit_group;\n" ::: "memory");
     }
+    asm volatile("cp.async.wait_all;\n" ::: "memory");  // no copy outlives the CTA
     // the last stage's MMAs (every commit of a barrier before it completed in order)
     if (ok && nstage > 0) {
         const int sl = nstage - 1;
-        ok = __all_sync(0xffffffffu, mb_wait((sl & 1) ? bar1 : bar0, (unsigned)((sl >> 1) & 1), abort_flag, p.err, 22));
+        ok = __all_sync(0xffffffffu, mb_wait(sb + 8u * (unsigned)(sl % WG_ST), (unsigned)((sl / WG_ST) & 1), abort_flag,
+                                             p.err, 22));
         ok = __syncthreads_and(ok);
     }
     if (ok && nstage > 0) {
@@ -858,19 +869,25 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(const WgTcArgs p)
         const int s = r / p.C, c = r - s * p.C;
         const bool live = s < ntap && c < p.Cw;
         const unsigned lane_addr = (unsigned)(32 * warp) << 16;
+        const bool v4 = (reinterpret_cast<uintptr_t>(p.dw) & 15) == 0;
         for (int n0 = 0; n0 < p.N; n0 += 16) {
             float v[16];
             __syncwarp();
             tc_ld16(tmem + lane_addr + (unsigned)n0, v);
             if (live) {
                 float *d = p.dw + ((long long)(t0 + s) * p.Cw + c) * p.N + n0;
+                if (v4) {
 #pragma unroll
-                for (int j = 0; j < 16; j++) atomicAdd(d + j, v[j]);
+                    for (int j = 0; j < 16; j += 4) red_v4_f32(d + j, v[j], v[j + 1], v[j + 2], v[j + 3]);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 16; j++) atomicAdd(d + j, v[j]);
+                }
             }
         }
     }
     if (!ok && issued >= 0 && tid == 0)  // no MMA outlives the CTA: its last commit covers the earlier ones
-        mb_wait((issued & 1) ? bar1 : bar0, (unsigned)((issued >> 1) & 1), abort_flag, p.err, 23, false);
+        mb_wait(sb + 8u * (unsigned)(issued % WG_ST), (unsigned)((issued / WG_ST) & 1), abort_flag, p.err, 23, false);
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {
@@ -1110,58 +1127,12 @@ int up2_tc(const bf16 *in, const bf16 *w, const float *bias, bf16 *out, int B, i
     return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
 
-// [taps][Npad][Kpad] (K innermost) -> [taps][Kpad / 8][Npad][8]
-__global__ void k_pack_w_tc(const bf16 *__restrict__ src, int taps, int Npad, int Kpad, bf16 *__restrict__ dst)
-{
-    long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    long long tot = (long long)taps * Npad * Kpad;
-    if (e >= tot) return;
-    int j = (int)(e & 7);
-    long long q = e >> 3;
-    int n = (int)(q % Npad);
-    q /= Npad;
-    int kc = (int)(q % (Kpad / 8));
-    int t = (int)(q / (Kpad / 8));
-    dst[e] = src[((long long)t * Npad + n) * Kpad + 8 * kc + j];
-}
-
-// [27][Npad][Kpad] -> [9 (ty, tx)][Kpad / 8][3 Npad (z-taps 2, 1, 0)][8]
-__global__ void k_pack_w_tc_dzn(const bf16 *__restrict__ src, int Npad, int Kpad, bf16 *__restrict__ dst)
-{
-    long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int n3n = 3 * Npad;
-    long long tot = 27LL * Npad * Kpad;
-    if (e >= tot) return;
-    int j = (int)(e & 7);
-    long long q = e >> 3;
-    int n3 = (int)(q % n3n);
-    q /= n3n;
-    int kc = (int)(q % (Kpad / 8));
-    int yx = (int)(q / (Kpad / 8));
-    int tz = 2 - n3 / Npad, n = n3 % Npad;
-    int tap = 9 * tz + yx;
-    dst[e] = src[((long long)tap * Npad + n) * Kpad + 8 * kc + j];
-}
-
-int pack_w_tc(const bf16 *src, int taps, int Npad, int Kpad, bf16 *dst, cudaStream_t s)
-{
-    if (taps == 27 && conv3_tc_dzn(Npad, Kpad)) {
-        long long tot = 27LL * Npad * Kpad;
-        counted(k_pack_w_tc_dzn)<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(src, Npad, Kpad, dst);
-        return cudaGetLastError() == cudaSuccess ? 0 : -1;
-    }
-    long long tot = (long long)taps * Npad * Kpad;
-    counted(k_pack_w_tc)<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(src, taps, Npad, Kpad, dst);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
-}
-
-
 int wgrad3_tc(const bf16 *x1, int C1, const bf16 *x2, int C2, const bf16 *g, int Cg, int N, int Cw, float *dw, int B,
               int D, int *err, cudaStream_t s)
 {
     const int C = C1 + C2;
     if (!(C == 16 || C == 32 || C == 64 || C == 128) || (C1 & 7) || N < 16 || N > 128 || (N & 15) || Cg < N ||
-        (Cg & 7) || Cw > C || B < 1 || D < 1)
+        (Cg & 7) || Cw > C || B < 1 || D < 1 || D > 1024)
         return 0;
     if ((reinterpret_cast<uintptr_t>(x1) & 15) || (C2 > 0 && (reinterpret_cast<uintptr_t>(x2) & 15)) ||
         (reinterpret_cast<uintptr_t>(g) & 15))
@@ -1186,10 +1157,12 @@ int wgrad3_tc(const bf16 *x1, int C1, const bf16 *x2, int C2, const bf16 *g, int
     a.abytes = 128u * WG_VS * 2u;
     a.bbytes = (unsigned)N * WG_VS * 2u;
     a.tmem_cols = pow2_at_least((unsigned)N);
-    a.idesc = (1u << 4) | (1u << 7) | (1u << 10) | (((unsigned)N >> 3) << 17) | ((128u >> 4) << 24);
+    // BF16 x BF16 -> FP32, both operands MN-major (bits 15 and 16)
+    a.idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | (((unsigned)N >> 3) << 17) |
+              ((128u >> 4) << 24);
     a.err = err;
     // at most as many CTAs per SM as their TMEM allocations fit
-    const unsigned need = ALIGN_SLACK + WG_HDR + 2u * (a.abytes + a.bbytes);
+    const unsigned need = ALIGN_SLACK + WG_HDR + (unsigned)WG_ST * (a.abytes + a.bbytes);
     const unsigned per_sm = 512u / a.tmem_cols;
     unsigned smem = TC_SMEM_SM / per_sm - 1024u;
     if (smem > TC_SMEM_MAX) smem = TC_SMEM_MAX;

@@ -56,8 +56,8 @@ int conv3_tc(const TcConv &c, int *err, cudaStream_t s);
 // 2x2x2 transposed convolution with stride 2 (the U-Net's up-sampling) on
 // the tensor cores: out(fine voxel 2 v + (dz, dy, dx))[n] = bias[n] +
 // sum_k in(v)[k] w[t][k][n], t = 4 dz + 2 dy + dx, blocked BF16 tensors on a
-// (B, Dc^3) coarse and (B, (2 Dc)^3) fine grid; w in the layout of pack_w_tc
-// with taps = 1 and 8 N rows (row t N + n).  Returns 1 when launched, 0 when
+// (B, Dc^3) coarse and (B, (2 Dc)^3) fine grid; w packed [K / 8][8 N][8] (row
+// t N + n).  Returns 1 when launched, 0 when
 // the shape is not supported (Dc^3 not a multiple of 128, N > 64, ...),
 // -1 on a launch error.
 bool up2_tc_ok(int N, int K, long long Vc);
@@ -77,10 +77,5 @@ int wgrad3_tc(const __nv_bfloat16 *x1, int C1, const __nv_bfloat16 *x2, int C2, 
 // Whether a 3^3 layer with N output and K input channels runs with its
 // three z-taps in one MMA (N <= 32; see conv_tc.cu).
 bool conv3_tc_dzn(int N, int K);
-
-// Re-layout of packed weights [taps][Npad][Kpad] into the tensor-core
-// layout [taps][Kpad / 8][Npad][8], or, for the layers of conv3_tc_dzn,
-// [9 (y, x)-taps][Kpad / 8][3 Npad (z-taps 2, 1, 0)][8].
-int pack_w_tc(const __nv_bfloat16 *src, int taps, int Npad, int Kpad, __nv_bfloat16 *dst, cudaStream_t s);
 
 }  // namespace gnb

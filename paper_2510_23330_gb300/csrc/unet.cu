@@ -21,6 +21,7 @@
 // GEMM (rows = input channels, K = voxels) split over voxel chunks.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -310,15 +311,17 @@ __global__ void __launch_bounds__(128) k_wgrad(WgArgs p)
 // ----------------------------------------------------------------- elementwise
 // FP32 [V][cin] -> blocked BF16 with 16 channels (zeros beyond cin); Vs
 // voxels per batch entry.
-__global__ void k_pack_input(const float *__restrict__ x, int cin, long long V, long long Vs, bf16 *__restrict__ out)
+__global__ void __launch_bounds__(256) k_pack_input(const float *__restrict__ x, int cin, int B, int Vs,
+                                                    bf16 *__restrict__ out)
 {
     // one voxel per thread: its cin values, two 16-byte channel groups out
-    long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= V) return;
+    const long long b = blockIdx.y + 65535LL * blockIdx.z;
+    const int sv = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b >= B || sv >= Vs) return;
+    const float *xv = x + (b * Vs + sv) * cin;
     float f[16];
 #pragma unroll
-    for (int c = 0; c < 16; c++) f[c] = c < cin ? x[v * cin + c] : 0.f;
-    const long long b = v / Vs, sv = v - b * Vs;
+    for (int c = 0; c < 16; c++) f[c] = c < cin ? xv[c] : 0.f;
 #pragma unroll
     for (int g = 0; g < 2; g++) {
         uint4 o;
@@ -337,25 +340,31 @@ __global__ void k_pack_input(const float *__restrict__ x, int cin, long long V, 
 // forward weight.  One voxel per thread; a block's outputs are staged in
 // shared memory and leave as contiguous 16-byte stores.
 constexpr int HEAD_T = 256;
+template <int NO>
 __global__ void __launch_bounds__(HEAD_T) k_head(const bf16 *__restrict__ in, int C, const bf16 *__restrict__ w,
-                                                 int Kpad, const float *__restrict__ bias, int cout, long long V,
-                                                 long long Vs, float *__restrict__ out)
+                                                 int Kpad, const float *__restrict__ bias, int B, int Vs,
+                                                 float *__restrict__ out)
 {
-    __shared__ float sw[8][32], sbias[8];
-    __shared__ __align__(16) float so[HEAD_T * 8];
-    for (int i = threadIdx.x; i < 8 * 32; i += blockDim.x) {
-        const int n = i >> 5, k = i & 31;
-        sw[n][k] = n < cout && k < C ? __bfloat162float(w[n * Kpad + k]) : 0.f;
+    // a block's voxels lie in one batch entry, given by the grid (a 64-bit
+    // division a thread costs more than the products); weights [k][n]: one input channel's are read together (16 bytes at a
+    // time instead of 128 single reads a voxel: 144 -> 122 us for 32 regions
+    // of 64^3, 65 at the copy rate)
+    constexpr int NP = (NO + 3) / 4 * 4;
+    __shared__ __align__(16) float sw[32][NP], sbias[NP];
+    __shared__ __align__(16) float so[HEAD_T * NO];
+    for (int i = threadIdx.x; i < 32 * NP; i += blockDim.x) {
+        const int k = i / NP, n = i % NP;
+        sw[k][n] = n < NO && k < C ? __bfloat162float(w[n * Kpad + k]) : 0.f;
     }
-    if (threadIdx.x < 8) sbias[threadIdx.x] = threadIdx.x < cout && bias ? bias[threadIdx.x] : 0.f;
+    if (threadIdx.x < NP) sbias[threadIdx.x] = threadIdx.x < NO && bias ? bias[threadIdx.x] : 0.f;
     __syncthreads();
-    const long long v0 = (long long)blockIdx.x * HEAD_T;
-    const long long v = v0 + threadIdx.x;
-    if (v < V) {
-        const long long b = v / Vs, sv = v - b * Vs;
-        float acc[8];
+    const long long b = blockIdx.y + 65535LL * blockIdx.z;
+    if (b >= B) return;
+    const int v0 = blockIdx.x * HEAD_T, sv = v0 + threadIdx.x;
+    if (sv < Vs) {
+        float acc[NO];
 #pragma unroll
-        for (int n = 0; n < 8; n++) acc[n] = sbias[n];
+        for (int n = 0; n < NO; n++) acc[n] = sbias[n];
 #pragma unroll
         for (int g = 0; g < 4; g++) {
             if (g >= (C >> 3)) break;
@@ -364,25 +373,35 @@ __global__ void __launch_bounds__(HEAD_T) k_head(const bf16 *__restrict__ in, in
 #pragma unroll
             for (int q = 0; q < 4; q++) {
                 const float2 f = __bfloat1622float2(h[q]);
+                float w0[NP], w1[NP];
 #pragma unroll
-                for (int n = 0; n < 8; n++) acc[n] += f.x * sw[n][8 * g + 2 * q] + f.y * sw[n][8 * g + 2 * q + 1];
+                for (int n = 0; n < NP; n += 4) {
+                    *reinterpret_cast<float4 *>(w0 + n) = *reinterpret_cast<const float4 *>(&sw[8 * g + 2 * q][n]);
+                    *reinterpret_cast<float4 *>(w1 + n) = *reinterpret_cast<const float4 *>(&sw[8 * g + 2 * q + 1][n]);
+                }
+#pragma unroll
+                for (int n = 0; n < NO; n++) acc[n] += f.x * w0[n] + f.y * w1[n];
             }
         }
 #pragma unroll
-        for (int n = 0; n < 8; n++)
-            if (n < cout) so[threadIdx.x * cout + n] = acc[n];
+        for (int n = 0; n < NO; n++) so[threadIdx.x * NO + n] = acc[n];
     }
     __syncthreads();
-    const long long nv = V - v0 < HEAD_T ? V - v0 : HEAD_T;
-    const long long nf = nv * cout;  // floats of this block, contiguous from out + v0 cout
-    float *dst = out + v0 * cout;
+    const int nf = min(HEAD_T, Vs - v0) * NO;  // floats of this block, contiguous
+    float *dst = out + (b * Vs + v0) * NO;
     if ((reinterpret_cast<uintptr_t>(dst) & 15) == 0) {
-        for (long long i = threadIdx.x; i < nf / 4; i += HEAD_T)
+        for (int i = threadIdx.x; i < nf / 4; i += HEAD_T)
             reinterpret_cast<float4 *>(dst)[i] = reinterpret_cast<const float4 *>(so)[i];
-        for (long long i = (nf / 4) * 4 + threadIdx.x; i < nf; i += HEAD_T) dst[i] = so[i];
+        for (int i = (nf / 4) * 4 + threadIdx.x; i < nf; i += HEAD_T) dst[i] = so[i];
     } else {
-        for (long long i = threadIdx.x; i < nf; i += HEAD_T) dst[i] = so[i];
+        for (int i = threadIdx.x; i < nf; i += HEAD_T) dst[i] = so[i];
     }
+}
+
+// Blocks of T threads over Vs voxels of each of B batch entries (y and z).
+static dim3 batch_grid(long long Vs, int T, int B)
+{
+    return dim3((unsigned)((Vs + T - 1) / T), (unsigned)std::min(B, 65535), (unsigned)((B + 65534) / 65535));
 }
 
 __global__ void k_maxpool(const bf16 *__restrict__ in, bf16 *__restrict__ out, unsigned char *__restrict__ idx, int B,
@@ -423,24 +442,34 @@ __global__ void k_maxpool(const bf16 *__restrict__ in, bf16 *__restrict__ out, u
     *reinterpret_cast<uint2 *>(idx + q * 8) = make_uint2(lo, hi);
 }
 
-// dIn (fine grid) = routed pool gradient + skip gradient
+// dIn (fine grid) = routed pool gradient + skip gradient; a thread takes one
+// fine voxel's group of 8 channels (16-byte pieces)
 __global__ void k_maxpool_bwd(const bf16 *__restrict__ dout, const unsigned char *__restrict__ idx,
                               const bf16 *__restrict__ dskip, bf16 *__restrict__ din, int B, int D, int H, int W, int C)
 {
-    // fine grid (B, 2D, 2H, 2W); e runs over the blocked fine tensor
-    long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    long long tot = (long long)B * 8 * D * H * W * C;
-    if (e >= tot) return;
+    // fine grid (B, 2D, 2H, 2W); q runs over the pieces of the blocked fine tensor
+    const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long Vc = (long long)D * H * W, Vf = 8 * Vc;
-    int j = (int)(e & 7);
-    long long q = e >> 3;
-    long long s = q % Vf, bg = q / Vf;
-    long long x = s % (2 * W), r = s / (2 * W), y = r % (2 * H), z = r / (2 * H);
-    int t = (int)(((z & 1) << 2) | ((y & 1) << 1) | (x & 1));
-    long long cv = (bg * Vc + ((z >> 1) * H + (y >> 1)) * W + (x >> 1)) * 8 + j;
-    float g = idx[cv] == t ? __bfloat162float(dout[cv]) : 0.f;
-    if (dskip) g += __bfloat162float(dskip[e]);
-    din[e] = __float2bfloat16_rn(g);
+    if (q >= B * Vf * (C >> 3)) return;
+    const long long bg = q / Vf;
+    const int s = (int)(q - bg * Vf);
+    const int x = s % (2 * W), r = s / (2 * W), y = r % (2 * H), z = r / (2 * H);
+    const unsigned t = ((z & 1) << 2) | ((y & 1) << 1) | (x & 1);
+    const long long cv = bg * Vc + ((long long)(z >> 1) * H + (y >> 1)) * W + (x >> 1);
+    const uint2 iv = reinterpret_cast<const uint2 *>(idx)[cv];
+    const uint4 dv = reinterpret_cast<const uint4 *>(dout)[cv];
+    uint4 sv = make_uint4(0u, 0u, 0u, 0u), ov;
+    if (dskip) sv = reinterpret_cast<const uint4 *>(dskip)[q];
+    const bf16 *dp = reinterpret_cast<const bf16 *>(&dv), *sp = reinterpret_cast<const bf16 *>(&sv);
+    bf16 *op = reinterpret_cast<bf16 *>(&ov);
+#pragma unroll
+    for (int j = 0; j < 8; j++) {
+        const unsigned i = ((j < 4 ? iv.x : iv.y) >> (8 * (j & 3))) & 255u;
+        float g = i == t ? __bfloat162float(dp[j]) : 0.f;
+        if (dskip) g += __bfloat162float(sp[j]);
+        op[j] = __float2bfloat16_rn(g);
+    }
+    reinterpret_cast<uint4 *>(din)[q] = ov;
 }
 
 // Blocked BF16 [B][C/8][V][8] -> FP32 [B][V][keep] (the first `keep` channels).
@@ -453,53 +482,141 @@ __global__ void k_unblock(const bf16 *__restrict__ in, int B, int C, long long V
     out[e] = __bfloat162float(in[((b * (C >> 3) + (c >> 3)) * V + v) * 8 + (c & 7)]);
 }
 
-__global__ void k_relu_mask(const bf16 *__restrict__ dy, const bf16 *__restrict__ y, bf16 *__restrict__ dz, long long n)
+// MSE over (voxels, cout <= 8): loss partial sums in FP64 and dy = 2 (y - t) /
+// count as BF16 with 16 channels (zeros beyond cout); a voxel per thread, one
+// atomic per block (a fixed number of blocks).
+__global__ void __launch_bounds__(256) k_mse(const float *__restrict__ y, const float *__restrict__ tgt, long long V,
+                                             long long Vs, int cout, bf16 *__restrict__ dy, double *__restrict__ loss)
 {
-    long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e < n) dz[e] = __bfloat162float(y[e]) > 0.f ? dy[e] : __float2bfloat16_rn(0.f);
-}
-
-// MSE over (voxels, cout): loss partial sums in FP64 and dy = 2 (y - t) / count
-// as BF16 with 16 channels (zeros beyond cout).
-__global__ void k_mse(const float *__restrict__ y, const float *__restrict__ tgt, long long V, long long Vs, int cout,
-                      bf16 *__restrict__ dy, double *__restrict__ loss)
-{
-    __shared__ double sh[32];
-    long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ double sh[8];
     double l = 0.0;
-    if (e < V * 16) {
-        long long v = e >> 4;
-        int c = (int)(e & 15);
-        float g = 0.f;
-        if (c < cout) {
-            float d = y[v * cout + c] - tgt[v * cout + c];
-            l = (double)d * d;
-            g = 2.f * d / (float)(V * cout);
+    const float cnt = (float)(V * cout);
+    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < V; v += (long long)gridDim.x * blockDim.x) {
+        uint4 o;
+        bf16 *h = reinterpret_cast<bf16 *>(&o);
+#pragma unroll
+        for (int c = 0; c < 8; c++) {
+            float g = 0.f;
+            if (c < cout) {
+                const float d = y[v * cout + c] - tgt[v * cout + c];
+                l += (double)d * d;
+                g = 2.f * d / cnt;
+            }
+            h[c] = __float2bfloat16_rn(g);
         }
-        dy[blk(v, c, 16, Vs)] = __float2bfloat16_rn(g);
+        const long long b = v / Vs, s = v - b * Vs;
+        uint4 *p = reinterpret_cast<uint4 *>(dy) + b * 2 * Vs + s;
+        p[0] = o;
+        p[Vs] = make_uint4(0u, 0u, 0u, 0u);  // channels 8 .. 15
     }
-    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    l = warp_sum(l);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = l;
     __syncthreads();
     if (threadIdx.x == 0) {
-        double s = 0;
-        for (int q = 0; q < (int)(blockDim.x >> 5); q++) s += sh[q];
-        atomicAdd(loss, s);
+        double t = 0;
+        for (int q = 0; q < 8; q++) t += sh[q];
+        atomicAdd(loss, t);
     }
 }
 
-// column sums of a blocked BF16 tensor with Cs channels (V voxels, Vs per
-// batch entry) into db[0..N)
-__global__ void k_colsum(const bf16 *__restrict__ g, long long V, long long Vs, int Cs, int N, float *__restrict__ db)
+// Column sums of a blocked BF16 tensor g (Vs voxels per batch entry, B entries,
+// cg8 groups of 8 channels) into db[0 .. N), the bias gradient: block row y is a
+// channel group, a thread adds up 16-byte pieces.  MASK: g is first set to
+// zero where y <= 0 (the ReLU's backward) and written to dz, so the mask and
+// the sums are one pass.
+template <bool MASK>
+__global__ void __launch_bounds__(256) k_colsum(const uint4 *__restrict__ g, const uint4 *__restrict__ y,
+                                                uint4 *__restrict__ dz, int B, long long Vs, int cg8, int N,
+                                                float *__restrict__ db)
 {
-    int c = threadIdx.x % Cs;
-    int lanes = blockDim.x / Cs;
-    int sub = threadIdx.x / Cs;
-    if (sub >= lanes) return;
-    float s = 0.f;
-    for (long long v = (long long)blockIdx.x * lanes + sub; v < V; v += (long long)gridDim.x * lanes)
-        s += __bfloat162float(g[blk(v, c, Cs, Vs)]);
-    if (c < N) atomicAdd(&db[c], s);
+    __shared__ float sh[8][8];
+    const int cg = blockIdx.y, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (int b = 0; b < B; b++) {
+        const long long p0 = ((long long)b * cg8 + cg) * Vs;
+        for (long long v = p0 + (long long)blockIdx.x * blockDim.x + threadIdx.x; v < p0 + Vs;
+             v += (long long)gridDim.x * blockDim.x) {
+            const uint4 u = g[v];
+            unsigned gi[4] = {u.x, u.y, u.z, u.w};
+            if (MASK) {
+                const uint4 m = y[v];
+                const unsigned mi[4] = {m.x, m.y, m.z, m.w};
+#pragma unroll
+                for (int q = 0; q < 4; q++) {
+                    const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162 *>(&mi[q]);
+                    gi[q] = (__low2float(h) > 0.f ? gi[q] & 0xffffu : 0u) | (__high2float(h) > 0.f ? gi[q] & 0xffff0000u : 0u);
+                }
+                dz[v] = make_uint4(gi[0], gi[1], gi[2], gi[3]);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162 *>(&gi[q]);
+                s[2 * q] += __low2float(h);
+                s[2 * q + 1] += __high2float(h);
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 8; j++) {
+        const float t = warp_sum(s[j]);
+        if (lane == 0) sh[w][j] = t;
+    }
+    __syncthreads();
+    if (threadIdx.x < 8 && cg * 8 + threadIdx.x < N) {
+        float t = 0.f;
+        for (int q = 0; q < 8; q++) t += sh[q][threadIdx.x];
+        atomicAdd(&db[cg * 8 + threadIdx.x], t);
+    }
+}
+
+// Weight gradient of the 1^3 head, dw[c][n] += sum_v x(v)[c] g(v)[n] with n <
+// N <= 8: block row y is a group of 8 input channels, a thread keeps the 64
+// sums of its voxels in registers.  (As a split-K mma.sync GEMM with 5 of 8
+// columns used: 289 us for one 64^3 region, now 10.)
+__global__ void __launch_bounds__(128) k_wgrad_head(const uint4 *__restrict__ x, int B, long long Vs, int cg8,
+                                                    const uint4 *__restrict__ g, int gg8, int N, int Cw,
+                                                    float *__restrict__ dw)
+{
+    __shared__ float sh[4][64];
+    const int cg = blockIdx.y, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    float acc[8][8];
+#pragma unroll
+    for (int c = 0; c < 8; c++)
+#pragma unroll
+        for (int n = 0; n < 8; n++) acc[c][n] = 0.f;
+    for (int b = 0; b < B; b++) {
+        const uint4 *px = x + ((long long)b * cg8 + cg) * Vs, *pg = g + (long long)b * gg8 * Vs;
+        for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < Vs; v += (long long)gridDim.x * blockDim.x) {
+            const uint4 ux = px[v], ug = pg[v];
+            const __nv_bfloat162 *hx = reinterpret_cast<const __nv_bfloat162 *>(&ux);
+            const __nv_bfloat162 *hg = reinterpret_cast<const __nv_bfloat162 *>(&ug);
+            float fx[8], fg[8];
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                fx[2 * q] = __low2float(hx[q]);
+                fx[2 * q + 1] = __high2float(hx[q]);
+                fg[2 * q] = __low2float(hg[q]);
+                fg[2 * q + 1] = __high2float(hg[q]);
+            }
+#pragma unroll
+            for (int c = 0; c < 8; c++)
+#pragma unroll
+                for (int n = 0; n < 8; n++) acc[c][n] = __fmaf_rn(fx[c], fg[n], acc[c][n]);
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 8; c++)
+#pragma unroll
+        for (int n = 0; n < 8; n++) {
+            const float t = warp_sum(acc[c][n]);
+            if (lane == 0) sh[w][c * 8 + n] = t;
+        }
+    __syncthreads();
+    if (threadIdx.x < 64) {
+        const int c = cg * 8 + (threadIdx.x >> 3), n = threadIdx.x & 7;
+        if (c < Cw && n < N)
+            atomicAdd(&dw[c * N + n], sh[0][threadIdx.x] + sh[1][threadIdx.x] + sh[2][threadIdx.x] + sh[3][threadIdx.x]);
+    }
 }
 
 // Adam (Kingma and Ba): m = b1 m + (1 - b1) g, v = b2 v + (1 - b2) g^2,
@@ -521,34 +638,46 @@ __global__ void k_adam(float *__restrict__ p, const float *__restrict__ g, float
     p[i] -= lr * (mi * ic1) / (sqrtf(vi * ic2) + eps);
 }
 
-// master [taps][cin][cout] FP32 -> forward BF16 [taps][Npad][Kpad] (transposed, zero padded)
-__global__ void k_pack_w_fwd(const float *__restrict__ w, int taps, int cin, int cout, int Npad, int Kpad,
-                             bf16 *__restrict__ out)
-{
-    long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    long long tot = (long long)taps * Npad * Kpad;
-    if (e >= tot) return;
-    int k = (int)(e % Kpad);
-    long long q = e / Kpad;
-    int n = (int)(q % Npad);
-    int t = (int)(q / Npad);
-    out[e] = __float2bfloat16_rn(k < cin && n < cout ? w[((long long)t * cin + k) * cout + n] : 0.f);
-}
+// One packed BF16 copy of a layer's FP32 master weights [taps][cin][cout]:
+// rows n and columns k of each tap (forward: n = output, k = input channel;
+// input gradient: the other way round, the taps of a 3^3 convolution mirrored,
+// t -> taps - 1 - t), zero beyond the layer's channels, stored as
+//   PK_PLAIN [taps][N][K];
+//   PK_TC    [taps][K / 8][N][8], the tensor-core layout (up: one matrix of
+//            the 8 taps' rows, [K / 8][8 N][8]);
+//   PK_DZN   [9 (ty, tx)][K / 8][3 N (z-taps 2, 1, 0)][8], see conv3_tc_dzn.
+enum { PK_PLAIN = 0, PK_TC, PK_UP, PK_DZN };
+struct PackDesc {
+    const float *w;
+    bf16 *dst;
+    int taps, cin, cout, N, K, layout, dgrad, mirror;
+    long long total;
+};
 
-// master -> input-gradient BF16 [taps][Npad = cin_pad][Kpad = cout_pad]; taps of a 3^3
-// convolution are mirrored (tap t -> 26 - t)
-__global__ void k_pack_w_dgrad(const float *__restrict__ w, int taps, int mirror, int cin, int cout, int Npad,
-                               int Kpad, bf16 *__restrict__ out)
+// All copies of a network in one launch, a block row per copy (four kernels a
+// layer, 67 launches of 3.3 us each, before).
+__global__ void __launch_bounds__(256) k_pack_weights(const PackDesc *__restrict__ table)
 {
-    long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    long long tot = (long long)taps * Npad * Kpad;
-    if (e >= tot) return;
-    int k = (int)(e % Kpad);
-    long long q = e / Kpad;
-    int n = (int)(q % Npad);
-    int t = (int)(q / Npad);
-    int ts = mirror ? taps - 1 - t : t;
-    out[e] = __float2bfloat16_rn(k < cout && n < cin ? w[((long long)ts * cin + n) * cout + k] : 0.f);
+    const PackDesc d = table[blockIdx.y];
+    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < d.total; e += (long long)gridDim.x * blockDim.x) {
+        int k, n, t;
+        if (d.layout == PK_PLAIN) {
+            k = (int)(e % d.K);
+            const int q = (int)(e / d.K);
+            n = q % d.N;
+            t = q / d.N;
+        } else {
+            const int rows = d.layout == PK_UP ? 8 * d.N : (d.layout == PK_DZN ? 3 * d.N : d.N);
+            const int j = (int)(e & 7), q = (int)(e >> 3), row = q % rows, r = q / rows;
+            k = 8 * (r % (d.K / 8)) + j;
+            const int m = r / (d.K / 8);
+            n = row % d.N;
+            t = d.layout == PK_UP ? row / d.N : (d.layout == PK_DZN ? 9 * (2 - row / d.N) + m : m);
+        }
+        if (d.mirror) t = d.taps - 1 - t;
+        const int ci = d.dgrad ? n : k, co = d.dgrad ? k : n;
+        d.dst[e] = __float2bfloat16_rn(ci < d.cin && co < d.cout ? d.w[((long long)t * d.cin + ci) * d.cout + co] : 0.f);
+    }
 }
 
 }  // namespace gnb
@@ -592,6 +721,8 @@ struct gnb_unet {
     int *err_d = nullptr;        // device error word of the tcgen05 convolutions
     int conv_impl = GNB_CONV_AUTO;
     unsigned tx_extra = 0;       // wait-timeout test only
+    void *pack_d = nullptr;      // PackDesc table of the packed weight copies
+    int npack = 0;
     bool launch_failed = false;
     bool tuning = false;         // forward passes time every tile plan of each 3^3 layer (gnb_unet_autotune)
     int tuned_layers = 0;
@@ -712,20 +843,40 @@ IgArgs ig_base(int mode, int B, int D, int H, int W)
     return a;
 }
 
+// Table of the network's packed copies (made once, with the network).
+int unet_pack_table(gnb_unet *u)
+{
+    std::vector<PackDesc> t;
+    auto add = [&](const ULayer &l, bf16 *dst, bool dgrad, int layout) {
+        if (!dst) return;
+        PackDesc d;
+        d.w = u->p + l.woff;
+        d.dst = dst;
+        d.taps = l.taps; d.cin = l.cin; d.cout = l.cout;
+        d.N = dgrad ? l.Nd : l.Npad;
+        d.K = dgrad ? l.Kd : l.Kpad;
+        d.layout = layout;
+        d.dgrad = dgrad;
+        d.mirror = dgrad && l.kind == L_CONV3;
+        d.total = (long long)l.taps * d.N * d.K;
+        t.push_back(d);
+    };
+    auto tc = [](int N, int K) { return conv3_tc_dzn(N, K) ? PK_DZN : PK_TC; };
+    for (auto &l : u->L) {
+        add(l, l.wf, false, PK_PLAIN);
+        add(l, l.wd, true, PK_PLAIN);
+        add(l, l.wtc, false, l.kind == L_UP2 ? PK_UP : tc(l.Npad, l.Kpad));
+        add(l, l.wdtc, true, tc(l.Nd, l.Kd));
+    }
+    u->npack = (int)t.size();
+    if (cudaMalloc((void **)&u->pack_d, t.size() * sizeof(PackDesc)) != cudaSuccess) return GNB_ENOMEM;
+    return cudaMemcpy(u->pack_d, t.data(), t.size() * sizeof(PackDesc), cudaMemcpyHostToDevice) == cudaSuccess ? GNB_OK
+                                                                                                             : GNB_ECUDA;
+}
+
 int unet_pack(gnb_unet *u)
 {
-    for (auto &l : u->L) {
-        long long nf = (long long)l.taps * l.Npad * l.Kpad;
-        counted(k_pack_w_fwd)<<<(unsigned)((nf + 255) / 256), 256, 0, u->s>>>(u->p + l.woff, l.taps, l.cin, l.cout,
-                                                                            l.Npad, l.Kpad, l.wf);
-        long long nd = (long long)l.taps * l.Nd * l.Kd;
-        counted(k_pack_w_dgrad)<<<(unsigned)((nd + 255) / 256), 256, 0, u->s>>>(
-            u->p + l.woff, l.taps, l.kind == L_CONV3 ? 1 : 0, l.cin, l.cout, l.Nd, l.Kd, l.wd);
-        // up-sampling: the 8 taps' output channels are the rows of one matrix
-        if (l.wtc && l.kind == L_UP2 && pack_w_tc(l.wf, 1, 8 * l.Npad, l.Kpad, l.wtc, u->s) != 0) return GNB_ECUDA;
-        if (l.wtc && l.kind == L_CONV3 && pack_w_tc(l.wf, l.taps, l.Npad, l.Kpad, l.wtc, u->s) != 0) return GNB_ECUDA;
-        if (l.wdtc && pack_w_tc(l.wd, l.taps, l.Nd, l.Kd, l.wdtc, u->s) != 0) return GNB_ECUDA;
-    }
+    counted(k_pack_weights)<<<dim3(64, (unsigned)u->npack), 256, 0, u->s>>>((const PackDesc *)u->pack_d);
     return cudaGetLastError() == cudaSuccess ? GNB_OK : GNB_ECUDA;
 }
 
@@ -805,9 +956,11 @@ void conv_fwd(gnb_unet *u, const ULayer &ly, int mode, int B, int D, const bf16 
         if (rc != 0) { if (rc < 0) u->launch_failed = true; return; }
     }
     if (mode == IG_CONV1 && outf && !in2 && ly.Npad <= 8 && C1 % 8 == 0 && C1 <= 32 && ly.Kpad <= 32) {
-        const long long V = (long long)B * D * D * D;
-        counted(k_head)<<<(unsigned)((V + HEAD_T - 1) / HEAD_T), HEAD_T, 0, u->s>>>(in1, C1, ly.wf, ly.Kpad, u->p + ly.boff, ly.cout,
-                                                                      V, (long long)D * D * D, outf);
+        const int Vs = D * D * D;
+        using Head = void (*)(const bf16 *, int, const bf16 *, int, const float *, int, int, float *);
+        static const Head heads[8] = {k_head<1>, k_head<2>, k_head<3>, k_head<4>, k_head<5>, k_head<6>, k_head<7>, k_head<8>};
+        counted(heads[ly.cout - 1])<<<batch_grid(Vs, HEAD_T, B), HEAD_T, 0, u->s>>>(in1, C1, ly.wf, ly.Kpad, u->p + ly.boff,
+                                                                                   B, Vs, outf);
         return;
     }
     IgArgs a = ig_base(mode, B, D, D, D);
@@ -847,13 +1000,30 @@ void conv_wgrad(gnb_unet *u, const ULayer &ly, int mode, int B, int D, const bf1
         tc = wgrad3_tc(x1, C1, x2, x2 ? C2 : 0, g, Cg, ly.cout, ly.cin, a.dw, B, D, u->err_d, u->s);
         if (tc < 0) u->launch_failed = true;
     }
+    if (mode == IG_CONV1 && !x2 && ly.cout <= 8 && u->conv_impl == GNB_CONV_AUTO) {
+        const long long Vh = (long long)D * D * D;
+        counted(k_wgrad_head)<<<dim3((unsigned)std::max(1LL, std::min((Vh + 511) / 512, 304LL)), (unsigned)(C1 / 8)), 128, 0,
+                               u->s>>>(reinterpret_cast<const uint4 *>(x1), B, Vh, C1 / 8,
+                                       reinterpret_cast<const uint4 *>(g), Cg / 8, ly.cout, ly.cin, a.dw);
+        tc = 1;
+    }
     if (tc == 0) launch_wg(a, ly.taps, u->s);
-    // bias gradient: column sums of the output gradient
-    long long Vs = mode == IG_UP2 ? 8LL * D * D * D : (long long)D * D * D;
-    long long V = (long long)B * Vs;
-    int threads = 256 / Cg * Cg;
-    if (threads < Cg) threads = Cg;
-    counted(k_colsum)<<<120, threads, 0, u->s>>>(g, V, Vs, Cg, ly.cout, u->g + ly.boff);
+}
+
+// Bias gradient of a layer: column sums of its output gradient g; with y (the
+// layer's stored output) g is masked by the ReLU first and written to dz.
+void conv_bgrad(gnb_unet *u, const ULayer &ly, int B, long long Vs, const bf16 *g, int Cg, const bf16 *y = nullptr,
+                bf16 *dz = nullptr)
+{
+    const int cgs = y ? Cg / 8 : (ly.cout + 7) / 8;  // every group is masked; else those with real columns
+    const int nblk = (int)std::max(1LL, std::min((Vs + 1023) / 1024, 608LL / cgs));
+    const dim3 grid((unsigned)nblk, (unsigned)cgs);
+    const uint4 *g4 = reinterpret_cast<const uint4 *>(g);
+    if (y)
+        counted(k_colsum<true>)<<<grid, 256, 0, u->s>>>(g4, reinterpret_cast<const uint4 *>(y), reinterpret_cast<uint4 *>(dz),
+                                                        B, Vs, Cg / 8, ly.cout, u->g + ly.boff);
+    else
+        counted(k_colsum<false>)<<<grid, 256, 0, u->s>>>(g4, nullptr, nullptr, B, Vs, Cg / 8, ly.cout, u->g + ly.boff);
 }
 
 // Forward pass of B regions from the blocked BF16 input xin to the FP32
@@ -898,13 +1068,14 @@ int unet_backward(gnb_unet *u, int B)
     int G = u->grid, b0 = u->base;
     cudaStream_t s = u->s;
     bf16 *T0 = u->tmp[0], *T1 = u->tmp[1], *T2 = u->tmp[2], *T3 = u->tmp[3];
-    auto relu_mask = [&](const bf16 *dy, const bf16 *y, bf16 *dz, long long n) {
-        counted(k_relu_mask)<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(dy, y, dz, n);
+    auto relu_mask = [&](const ULayer &ly, int D, const bf16 *dy, const bf16 *y, bf16 *dz) {
+        conv_bgrad(u, ly, B, (long long)D * D * D, dy, ly.cout, y, dz);
     };
     // head
     const ULayer &hd = u->L[LI_HEAD(u)];
     const bf16 *top = u->act[S_DECB(u, 0)];
     conv_wgrad(u, hd, IG_CONV1, B, G, top, b0, nullptr, 0, u->dyb, 16);
+    conv_bgrad(u, hd, B, (long long)G * G * G, u->dyb, 16);
     conv_dgrad(u, hd, IG_CONV1, B, G, u->dyb, 16, T0, b0, nullptr);  // T0: d(dec0b.out)
     // decoder levels 0 .. levels-2; skip gradients stay in the ENC slots' spare: use T-buffers per level
     // dskip[l] is stored in place of the decoder's "up" activation gradient area: allocate per level below
@@ -912,12 +1083,11 @@ int unet_backward(gnb_unet *u, int B)
     bf16 *dcur = T0;  // gradient of the current decoder output
     for (int l = 0; l + 1 < u->levels; l++) {
         int D = G >> l, w = width(u, l);
-        long long n = vox(u, l, B) * w;
         // the level-l tensors are at most as large as level 0 with 2 * base channels
-        relu_mask(dcur, u->act[S_DECB(u, l)], T1, n);
+        relu_mask(u->L[LI_DECB(u, l)], D, dcur, u->act[S_DECB(u, l)], T1);
         conv_wgrad(u, u->L[LI_DECB(u, l)], IG_CONV3, B, D, u->act[S_DECA(u, l)], w, nullptr, 0, T1, w);
         conv_dgrad(u, u->L[LI_DECB(u, l)], IG_CONV3, B, D, T1, w, T2, w, nullptr);
-        relu_mask(T2, u->act[S_DECA(u, l)], T1, n);
+        relu_mask(u->L[LI_DECA(u, l)], D, T2, u->act[S_DECA(u, l)], T1);
         conv_wgrad(u, u->L[LI_DECA(u, l)], IG_CONV3, B, D, u->act[S_ENCB(l)], w, u->act[S_UP(u, l)], w, T1, w);
         // dskip -> the level's dec-a slot (its forward value is no longer needed), dup -> T2
         dskip[l] = u->act[S_DECA(u, l)];
@@ -927,6 +1097,7 @@ int unet_backward(gnb_unet *u, int B)
         conv_wgrad(u, u->L[LI_UP(u, l)], IG_UP2, B, Dc, l + 2 < u->levels ? u->act[S_DECB(u, l + 1)]
                                                                           : u->act[S_ENCB(u->levels - 1)],
                    wc, nullptr, 0, T2, w);
+        conv_bgrad(u, u->L[LI_UP(u, l)], B, (long long)D * D * D, T2, w);
         conv_dgrad(u, u->L[LI_UP(u, l)], IG_DOWN2, B, Dc, T2, w, T3, wc, nullptr);
         std::swap(T0, T3);
         dcur = T0;  // gradient of the level-(l+1) decoder output (or the bottleneck)
@@ -937,15 +1108,15 @@ int unet_backward(gnb_unet *u, int B)
         long long n = vox(u, l, B) * w;
         if (l + 1 < u->levels) {
             // dcur is the gradient of pool(l) output; route it and add the skip gradient
-            counted(k_maxpool_bwd)<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(dcur, u->pidx[l], dskip[l], T3, B,
+            counted(k_maxpool_bwd)<<<(unsigned)((n / 8 + 255) / 256), 256, 0, s>>>(dcur, u->pidx[l], dskip[l], T3, B,
                                                                              D / 2, D / 2, D / 2, w);
             std::swap(T0, T3);
             dcur = T0;
         }
-        relu_mask(dcur, u->act[S_ENCB(l)], T1, n);
+        relu_mask(u->L[LI_ENCB(l)], D, dcur, u->act[S_ENCB(l)], T1);
         conv_wgrad(u, u->L[LI_ENCB(l)], IG_CONV3, B, D, u->act[S_ENCA(l)], w, nullptr, 0, T1, w);
         conv_dgrad(u, u->L[LI_ENCB(l)], IG_CONV3, B, D, T1, w, T2, w, nullptr);
-        relu_mask(T2, u->act[S_ENCA(l)], T1, n);
+        relu_mask(u->L[LI_ENCA(l)], D, T2, u->act[S_ENCA(l)], T1);
         const bf16 *xin = l == 0 ? u->xin : u->act[S_POOL(l - 1)];
         int cin = l == 0 ? 16 : width(u, l - 1);
         conv_wgrad(u, u->L[LI_ENCA(l)], IG_CONV3, B, D, xin, cin, nullptr, 0, T1, w);
@@ -1074,7 +1245,7 @@ int gnb_unet_create(gnb_unet **out, int cin, int cout, int base, int levels, int
         if (ok && l.kind == L_CONV3 && conv3_tc_plan(l.Nd, l.Kd, grid, &pl))
             ok = cudaMalloc((void **)&l.wdtc, (size_t)l.taps * l.Nd * l.Kd * 2) == cudaSuccess;
     }
-    if (!ok) {
+    if (!ok || unet_pack_table(u) != GNB_OK) {
         cudaGetLastError();
         gnb_unet_destroy(u);
         return GNB_ENOMEM;
@@ -1103,6 +1274,7 @@ void gnb_unet_destroy(gnb_unet *u)
     for (float *q : a) if (q) cudaFree(q);
     if (u->loss_d) cudaFree(u->loss_d);
     if (u->err_d) cudaFree(u->err_d);
+    if (u->pack_d) cudaFree(u->pack_d);
     delete u;
 }
 
@@ -1338,7 +1510,8 @@ int gnb_unet_forward(gnb_unet *u, int batch, const float *x, float *y, int on_de
         cudaMemcpyAsync(tmpx, x, V * u->cin * 4, cudaMemcpyHostToDevice, u->s);
         xd = tmpx;
     }
-    counted(k_pack_input)<<<(unsigned)((V + 255) / 256), 256, 0, u->s>>>(xd, u->cin, V, vox(u, 0, 1), u->xin);
+    counted(k_pack_input)<<<batch_grid(vox(u, 0, 1), 256, batch), 256, 0, u->s>>>(xd, u->cin, batch, (int)vox(u, 0, 1),
+                                                                                u->xin);
     rc = unet_forward(u, batch);
     if (rc == GNB_OK)
         cudaMemcpyAsync(y, u->yout, V * u->cout * 4, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
@@ -1364,10 +1537,11 @@ int gnb_unet_train_step(gnb_unet *u, int batch, const float *x, const float *tar
     }
     cudaMemcpyAsync(u->tgt, target, V * u->cout * 4, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
                     u->s);
-    counted(k_pack_input)<<<(unsigned)((V + 255) / 256), 256, 0, u->s>>>(xd, u->cin, V, vox(u, 0, 1), u->xin);
+    counted(k_pack_input)<<<batch_grid(vox(u, 0, 1), 256, batch), 256, 0, u->s>>>(xd, u->cin, batch, (int)vox(u, 0, 1),
+                                                                                u->xin);
     rc = unet_forward(u, batch);
     cudaMemsetAsync(u->loss_d, 0, 8, u->s);
-    counted(k_mse)<<<(unsigned)((V * 16 + 255) / 256), 256, 0, u->s>>>(u->yout, u->tgt, V, vox(u, 0, 1), u->cout,
+    counted(k_mse)<<<(unsigned)std::min((V + 255) / 256, 608LL), 256, 0, u->s>>>(u->yout, u->tgt, V, vox(u, 0, 1), u->cout,
                                                                      u->dyb, u->loss_d);
     cudaMemsetAsync(u->g, 0, u->nparam * 4, u->s);
     if (rc == GNB_OK) rc = unet_backward(u, batch);

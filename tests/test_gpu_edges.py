@@ -199,3 +199,53 @@ def test_list_pool_grows(G, n_gas):
     err = {t: np.sqrt(sum((a - r) ** 2 for a, r in zip(g[:3], ref))) / scale for t, g in got.items()}
     assert np.median(err[0.03]) < 1e-5 < np.median(err[0.5])
     assert np.max(np.abs(got[0.03][3] - ref[3])) < 1e-6 and np.max(np.abs(got[0.03][4] - ref[4])) < 1e-8
+
+
+def _bf16(a):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(a, np.float32)).bfloat16().float().numpy()
+
+
+# the head for every output count and width, ragged blocks and several batch
+# entries: forward from the stored last activation, weight and bias gradient
+# from the output gradient (BF16 operands, FP32 sums of G^3 B terms)
+@pytest.mark.parametrize("base,cout", [(16, 1), (32, 2), (16, 3), (32, 4), (16, 5), (32, 6), (16, 7), (32, 8)])
+def test_unet_head_forward_and_gradient(G, base, cout):
+    from paper_2510_23330_gb300 import surrogate
+    grid, B, rng = 20, 3, np.random.default_rng(base + cout)
+    net = G.UNet(3, cout, base, 2, grid)
+    w = surrogate.he_init(3, cout, base, 2, seed=cout)
+    nh = base * cout + cout
+    w[-cout:] = rng.normal(size=cout)
+    net.set_params(w)
+    x = rng.normal(size=(B, grid, grid, grid, 3)).astype(np.float32)
+    t = rng.normal(size=(B, grid, grid, grid, cout)).astype(np.float32)
+    y = net.forward(x)
+    act = net.get_activation(8, B, grid, base).astype(np.float64)  # dec 0 b
+    ref = act @ _bf16(w[-nh:-cout]).astype(np.float64).reshape(base, cout) + w[-cout:]
+    assert np.max(np.abs(y - ref)) < 1e-5 * np.max(np.abs(ref))
+    net.train_step(x, t, 0.0)
+    g = net.get_grads()[-nh:].astype(np.float64)
+    dy = _bf16(2.0 * (y - t) / y.size).astype(np.float64)
+    dw = np.einsum("bzyxc,bzyxn->cn", act, dy)
+    assert np.linalg.norm(g[:-cout].reshape(base, cout) - dw) < 1e-5 * np.linalg.norm(dw)
+    assert np.max(np.abs(g[-cout:] - dy.sum((0, 1, 2, 3)))) < 1e-5 * np.abs(dy).sum((0, 1, 2, 3)).max()
+
+
+# weight gradients of the 3^3 layers: a last voxel chunk of fewer than 64, one
+# stage only, two inputs, against the mma.sync kernel on the same forward state
+@pytest.mark.parametrize("grid,B", [(8, 1), (12, 3)])
+def test_unet_weight_gradients_two_kernels(G, grid, B):
+    from paper_2510_23330_gb300 import surrogate
+    rng = np.random.default_rng(grid)
+    x = rng.normal(size=(B, grid, grid, grid, 5)).astype(np.float32)
+    t = rng.normal(size=x.shape).astype(np.float32)
+    out = []
+    for impl in (G.GNB_CONV_AUTO, G.GNB_CONV_MMA_SYNC):
+        net = G.UNet(5, 5, 16, 3, grid)
+        net.set_params(surrogate.he_init(5, 5, 16, 3, seed=1))
+        net.set_conv_impl(impl)
+        net.train_step(x, t, 0.0)
+        out.append(net.get_grads().astype(np.float64))
+    # both round activations to BF16; a different order of FP32 sums flips some
+    assert np.linalg.norm(out[0] - out[1]) < 5e-2 * np.linalg.norm(out[1])
