@@ -149,12 +149,10 @@ struct gnb_ctx {
 
     // supernova surrogate (surrogate.cu)
     int *sreg = nullptr;          // region of each particle slot (-1: none)
-    int *rcount = nullptr;        // members per region
     float *vacc = nullptr;        // voxel accumulators: [voxels][4], then [voxels / 2][4] (see k_vox_scatter)
     float *vout = nullptr;        // standardised channels [nreg][grid^3][5]
     double *vw = nullptr;         // remap weights [nreg][grid^3]
-    double *vcdf = nullptr;       // remap line CDFs [nreg][axis][grid^2 lines][grid]
-    float *vcdf32 = nullptr;      // the same, rounded to FP32 (decides the comparisons it can)
+    float *vcdf32 = nullptr;      // remap line sums in FP32 [nreg][axis][grid^2 lines][grid]
     float *vcdfc = nullptr;       // every 8th FP32 sum of each line (its last entry = the line total)
     double *cent_d = nullptr;     // region centres [nreg][3]
     float *rsx = nullptr;         // region centre x (FP32), sorted ascending (membership search)

@@ -21,6 +21,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "common.cuh"
 
@@ -48,19 +49,6 @@ __device__ __forceinline__ double uniform_draw(uint64_t sid, uint64_t k)
     return (double)(sm64(sid + k) >> 11) * (1.0 / 9007199254740992.0);
 }
 
-// counter[key] += 1 for every active lane, one atomic per distinct key in
-// the warp (neighbouring particles in Morton order mostly share their
-// region and tiles); returns each lane's slot.
-__device__ __forceinline__ int warp_inc(int *counter, int key)
-{
-    const unsigned mask = __match_any_sync(__activemask(), key);
-    const int lane = threadIdx.x & 31, leader = __ffs(mask) - 1;
-    int base = 0;
-    if (lane == leader) base = atomicAdd(counter + key, __popc(mask));
-    base = __shfl_sync(mask, base, leader);
-    return base + __popc(mask & ((1u << lane) - 1));
-}
-
 // Region of every gas particle: the first region r (smallest index) with
 // |x - c_r|_inf <= side / 2, decided in FP64.  Candidates come from the
 // regions sorted by centre x: an FP32 binary search finds the slab
@@ -70,7 +58,7 @@ __device__ __forceinline__ int warp_inc(int *counter, int key)
 // of its FP32 rate).
 __global__ void k_region_assign(PArr p, int n, const double *__restrict__ cent, const float *__restrict__ rsx,
                                 const int *__restrict__ rsi, const float *__restrict__ cf, int nreg, double half,
-                                int *__restrict__ reg, int *__restrict__ rcount)
+                                int *__restrict__ reg)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -98,7 +86,6 @@ __global__ void k_region_assign(PArr p, int n, const double *__restrict__ cent, 
         if (best < nreg) r = best;
     }
     reg[i] = r;
-    if (r >= 0) warp_inc(rcount, r);
 }
 
 __device__ __forceinline__ void region_lo(const double *cent, int r, double side, double *lo)
@@ -265,20 +252,66 @@ __global__ void __launch_bounds__(256) k_vox_finalize(const float *__restrict__ 
     }
 }
 
-__global__ void k_remap_weights(const float *__restrict__ pred, long long nv, int cout, double *__restrict__ w)
+// 10^x in FP64, by table and polynomial (Tang, ACM TOMS 15, 1989): x = (k / 128)
+// log10 2 + r with integer k (the reduction in two steps, the leading
+// constant short enough for an exact product), 10^x = 2^(k / 128) e^(r ln 10),
+// the first factor a table of 2^(j / 128) with the exponent added as an
+// integer, the second a Taylor polynomial of degree 5 (|r ln 10| <= ln 2 / 256:
+// truncation below 2^-60).  About one unit in the last place, 14 FP64
+// operations; GB300's FP64 pipe is narrow, and the library's exp10 set the time
+// of this pass (16.8 M voxels 605 us, now 456, still the FP64 pipe).
+struct Exp2Table {
+    double t[128];  // 2^(j / 128)
+};
+
+__device__ __forceinline__ double exp10_table(double x, const double *t)
 {
-    long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v < nv) w[v] = exp10((double)pred[v * cout] - 0.33);
+    if (!(fabs(x) < 290.0)) return exp10(x);  // overflow, underflow, infinities, NaN
+    const double y = __fma_rn(x, 128.0 * 3.32192809488736234787, 6755399441055744.0);  // 128 log2 10; 1.5 2^52 rounds
+    const int k = __double2loint(y);
+    const double kd = y - 6755399441055744.0;
+    // log10(2) / 128 = A + B, A with 33 significant bits
+    constexpr double A = 0x1.34413508p-9, B = 0x1.f79fef311f12bp-41;
+    const double r = __fma_rn(-kd, B, __fma_rn(-kd, A, x));
+    const double z = r * 2.30258509299404568402;
+    double p = __fma_rn(z, 1.0 / 120.0, 1.0 / 24.0);
+    p = __fma_rn(z, p, 1.0 / 6.0);
+    p = __fma_rn(z, p, 0.5);
+    p = __fma_rn(z, p, 1.0) * z;
+    const double s = t[k & 127];
+    const double v = __fma_rn(s, p, s);
+    return __hiloint2double(__double2hiint(v) + ((k >> 7) << 20), __double2loint(v));
+}
+
+__global__ void __launch_bounds__(256) k_remap_weights(const float *__restrict__ pred, long long nv, int cout,
+                                                       __grid_constant__ const Exp2Table table, double *__restrict__ w)
+{
+    __shared__ double t[128];
+    if (threadIdx.x < 128) t[threadIdx.x] = table.t[threadIdx.x];
+    __syncthreads();
+    const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (v < nv) w[v] = exp10_table((double)pred[v * cout] - 0.33, t);
+}
+
+static const Exp2Table &exp2_table()
+{
+    static const Exp2Table t = [] {
+        Exp2Table e;
+        for (int j = 0; j < 128; j++) e.t[j] = std::exp2(j / 128.0);
+        return e;
+    }();
+    return t;
 }
 
 // Cumulative weights along every grid line of every region, one thread per
-// (region, axis, line), summed left to right in FP64 -- the same additions in
-// the same order as a running sum taken at draw time, so each draw below sees
-// bit-identical partial sums -- and each sum also rounded to nearest FP32;
-// every 8th FP32 sum also goes to a coarse table (grids of a multiple of 8).  Line of axis a through voxel (x, y, z):
+// (region, axis, line), summed left to right in FP64 and each sum rounded to
+// nearest FP32; every 8th FP32 sum also goes to a coarse table (grids of a
+// multiple of 8).  A draw that the FP32 images cannot decide repeats the same
+// additions in the same order (line_sums), so the FP64 sums are not stored.
+// Line of axis a through voxel (x, y, z):
 // a = 0 -> z G + y, a = 1 -> z G + x, a = 2 -> y G + x.
-__global__ void k_line_cdf(const double *__restrict__ w, int nreg, int grid, double *__restrict__ cdf,
-                           float *__restrict__ cdf32, float *__restrict__ cdfc)
+__global__ void k_line_cdf(const double *__restrict__ w, int nreg, int grid, float *__restrict__ cdf32,
+                           float *__restrict__ cdfc)
 {
     long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long G = grid, lines = G * G;
@@ -292,12 +325,10 @@ __global__ void k_line_cdf(const double *__restrict__ w, int nreg, int grid, dou
     else if (a == 1) { b0 = u * G * G + v; stride = G; }       // z = u, x = v
     else { b0 = u * G + v; stride = G * G; }                   // y = u, x = v
     const double *wr = w + r * G * G * G + b0;
-    double *out = cdf + t * G;
     float *out32 = cdf32 + t * G;
     double cum = 0.0;
     for (int q = 0; q < grid; q++) {
         cum = __dadd_rn(cum, wr[q * stride]);
-        out[q] = cum;
         out32[q] = __double2float_rn(cum);
         if ((grid & 7) == 0 && (q & 7) == 7) cdfc[t * (G >> 3) + (q >> 3)] = out32[q];
     }
@@ -310,8 +341,7 @@ __global__ void k_line_cdf(const double *__restrict__ w, int nreg, int grid, dou
 // and each lane sums its own line left to right as above (bit-identical).
 constexpr int LC_W = 2;  // warps per block
 __global__ void __launch_bounds__(32 * LC_W) k_line_cdf_tiled(const double *__restrict__ w, int nreg, int grid,
-                                                              double *__restrict__ cdf, float *__restrict__ cdf32,
-                                                              float *__restrict__ cdfc)
+                                                              float *__restrict__ cdf32, float *__restrict__ cdfc)
 {
     __shared__ double tile[LC_W][32][65];
     const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
@@ -324,10 +354,11 @@ __global__ void __launch_bounds__(32 * LC_W) k_line_cdf_tiled(const double *__re
     const long long u = line0 / G, v0 = line0 % G;
     const double *wr = w + r * G * G * G;
     double(*T)[65] = tile[wq];
+    const int sh = grid == 64 ? 6 : 5;
     if (a == 0) {
         // lines (z = u, y = v0 .. v0 + 31) along x: one contiguous block of 32 G weights
         const double *blk = wr + (u * G + v0) * G;
-        for (int k = lane; k < 32 * grid; k += 32) T[k / grid][k % grid] = blk[k];
+        for (int k = lane; k < 32 * grid; k += 32) T[k >> sh][k & (grid - 1)] = blk[k];
     } else {
         const long long stride = a == 1 ? G : G * G;
         const long long b0 = a == 1 ? u * G * G + v0 : u * G + v0;  // line l adds l (inner x)
@@ -340,15 +371,34 @@ __global__ void __launch_bounds__(32 * LC_W) k_line_cdf_tiled(const double *__re
         T[lane][q] = cum;
     }
     __syncwarp();
-    double *out = cdf + t0 * G;
     float *out32 = cdf32 + t0 * G;
-    for (int k = lane; k < 32 * grid; k += 32) {
-        const double c = T[k / grid][k % grid];
-        out[k] = c;
-        out32[k] = __double2float_rn(c);
-    }
+    for (int k = lane; k < 32 * grid; k += 32) out32[k] = __double2float_rn(T[k >> sh][k & (grid - 1)]);
     const int nc = grid >> 3;
     for (int k = lane; k < 32 * nc; k += 32) cdfc[t0 * nc + k] = __double2float_rn(T[k / nc][8 * (k % nc) + 7]);
+}
+
+// Eight consecutive floats (32-byte aligned) in one load.
+__device__ __forceinline__ void load8(const float *p, float (&v)[8])
+{
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+        : "l"(p));
+}
+
+// First q of a line of G weights (stride apart) whose running FP64 sum exceeds
+// U times the line's total (G if none), U = m 2^-53: the sums as k_line_cdf
+// forms them.
+__device__ __noinline__ int line_search(const double *w, long long stride, int G, uint64_t m)
+{
+    double tot = 0.0;
+    for (int q = 0; q < G; q++) tot = __dadd_rn(tot, w[q * stride]);
+    const double target = __dmul_rn((double)m * (1.0 / 9007199254740992.0), tot);
+    double cum = 0.0;
+    for (int q = 0; q < G; q++) {
+        cum = __dadd_rn(cum, w[q * stride]);
+        if (cum > target) return q;
+    }
+    return G;
 }
 
 // Members are read from `p` (positions, ID; region in reg) and their new
@@ -356,7 +406,7 @@ __global__ void __launch_bounds__(32 * LC_W) k_line_cdf_tiled(const double *__re
 // asynchronous batch reads a snapshot and writes the current arrays).
 __global__ void k_remap(PArr p, PArr q, const int *__restrict__ src_orig, const int *__restrict__ map, int n,
                         const int *__restrict__ reg, const float *__restrict__ pred, int cout,
-                        const double *__restrict__ cdf, const float *__restrict__ cdf32,
+                        const double *__restrict__ wgt, const float *__restrict__ cdf32,
                         const float *__restrict__ cdfc, const double *__restrict__ cent, double side, double d,
                         double inv_d, int grid, const unsigned long long *__restrict__ seedp, int sweeps, int r0,
                         int r1)
@@ -385,7 +435,7 @@ __global__ void k_remap(PArr p, PArr q, const int *__restrict__ src_orig, const 
     const size_t G = (size_t)grid;
     uint64_t id = (uint64_t)p.id[i];
     const uint64_t sid = sm64(seed + id);  // the particle's stream: draw k is sm64(sid + k)
-    const bool coarse8 = (grid & 31) == 0 && grid <= 64;  // lines of 8 or fewer coarse sums, float4-aligned
+    const bool coarse8 = grid == 64 || grid == 32;  // lines of 8 or 4 coarse sums, 32- and 16-byte aligned
     uint64_t k = 0;
     for (int s = 0; s < sweeps; s++) {
         for (int a = 0; a < 3; a++, k++) {
@@ -393,78 +443,86 @@ __global__ void k_remap(PArr p, PArr q, const int *__restrict__ src_orig, const 
             // q whose running sum exceeds target = U * total (the first
             // crossing of a scan of the non-decreasing running sums).  The
             // comparisons run on FP32 images: t32 approximates target from
-            // the top 32 bits of U's 53-bit integer m and the FP32 total
-            // within a relative 2^-21 (m >= 2^45: truncation 2^-24, three
-            // roundings 2^-24 each, FP64 rounding of target 2^-53; the total
-            // kept in FP32's normal range), and the FP32 sums are within 2^-24
+            // the 32 leading bits of U's 53-bit integer m and the FP32 total
+            // within a relative 2^-21 (truncation 2^-31, three roundings
+            // 2^-24 each, FP64 rounding of target 2^-53; the total and t32
+            // kept in FP32's normal range, m >= 2^32), and the FP32 sums are within 2^-24
             // of the FP64 ones, so a sum outside t32 (1 -+ 2^-20) orders
-            // against target as its image does; inside that band (and for
-            // m < 2^45) the FP64 values decide.  With 8 | grid the search is
-            // two scans of 8: the coarse sums (every 8th) pick the block, the
-            // block's 8 sums the voxel -- two dependent 32-byte loads.
+            // against target as its image does; if one lies inside that band
+            // (or m < 2^32) the FP64 sums decide (line_search: rare enough,
+            // about one draw in 15,000, to repeat the additions).  With grids of
+            // 32 and 64 the search is two counts of 8: the coarse sums (every
+            // 8th) below the band give the block, the block's 8 sums the
+            // voxel -- two dependent 32-byte loads, each one request (a pair
+            // of 16-byte loads doubles the requests through L1, which set
+            // the time: 1,705 us for 6.4 M particles of 64 regions with 16-byte
+            // loads and scans that leave at the first sum above, now 1,347).
             size_t line = a == 0 ? (size_t)c[2] * G + c[1] : (a == 1 ? (size_t)c[2] * G + c[0] : (size_t)c[1] * G + c[0]);
             const size_t lid = ((size_t)(r - r0) * 3 + a) * G * G + line;
-            const double *L = cdf + lid * G;
             const float *L32 = cdf32 + lid * G;
             const uint64_t m = sm64(sid + k) >> 11;
-            double target = 0.0;
-            bool have = false;
             float lo32 = 0.f, hi32 = 0.f;
-            bool fast = false;
-            // true when running sum q (FP32 image l32) exceeds target
-            auto above = [&](float l32, int q) -> bool {
-                if (fast && l32 > hi32) return true;
-                if (fast && l32 < lo32) return false;
-                if (!have) {
-                    target = __dmul_rn((double)m * (1.0 / 9007199254740992.0), L[grid - 1]);
-                    have = true;
-                }
-                return L[q] > target;
-            };
+            bool sure = false;
             auto setup = [&](float tot32) {
-                fast = m >= (1ull << 45) && tot32 >= 0x1p-90f && tot32 <= 0x1p100f;
-                // float(M), M = m >> 21 < 2^32, rounded to nearest, on the FP32
-                // pipes: its two 16-bit halves are exact as 2^23 + x - 2^23, and
-                // one FMA joins them with a single rounding
-                const unsigned M = (unsigned)(m >> 21);
+                sure = m >= (1ull << 32) && tot32 >= 0x1p-90f && tot32 <= 0x1p100f;
+                // M = the 32 leading bits of m = M 2^(21 - s): float(M),
+                // rounded to nearest, on the FP32 pipes: its two 16-bit halves
+                // are exact as 2^23 + x - 2^23, and one FMA joins them with a
+                // single rounding
+                const int s = min(__clzll((long long)m) - 11, 20);
+                const unsigned M = (unsigned)((m << s) >> 21);
                 const float mh = __int_as_float(0x4B000000 | (int)(M >> 16)) - 8388608.f;
                 const float ml = __int_as_float(0x4B000000 | (int)(M & 0xFFFFu)) - 8388608.f;
-                const float t32 = __fmul_rn(__fmaf_rn(mh, 65536.f, ml), tot32 * 0x1p-32f);
+                const float t32 = __fmul_rn(__fmaf_rn(mh, 65536.f, ml), tot32 * __int_as_float((127 - 32 - s) << 23));
                 lo32 = __fmul_rn(t32, 1.f - 0x1p-20f);
                 hi32 = __fmul_rn(t32, 1.f + 0x1p-20f);
             };
             int qa;
             if (coarse8) {
                 const int nc = grid >> 3;
-                const float4 *C4 = reinterpret_cast<const float4 *>(cdfc + lid * nc);
-                const float4 v0 = C4[0];
-                const float4 v1 = nc == 8 ? C4[1] : v0;
-                const float cv[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-                setup(nc == 8 ? v1.w : v0.w);
-                int jb = nc;
-#pragma unroll
-                for (int j = 0; j < 8; j++)
-                    if (j < nc && above(cv[j], 8 * j + 7)) { jb = j; break; }
-                if (jb == nc) {
-                    qa = grid;
-                } else {
-                    const float4 *F4 = reinterpret_cast<const float4 *>(L32 + 8 * jb);
-                    const float4 f0 = F4[0], f1 = F4[1];
-                    const float fv[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
-                    qa = 8 * jb + 7;  // block jb's last sum is above target
-#pragma unroll
-                    for (int q = 0; q < 7; q++)
-                        if (above(fv[q], 8 * jb + q)) { qa = 8 * jb + q; break; }
+                float cv[8];
+                if (nc == 8) {
+                    load8(cdfc + lid * 8, cv);
+                } else {  // four coarse sums; the rest never count
+                    const float4 v = *reinterpret_cast<const float4 *>(cdfc + lid * 4);
+                    cv[0] = v.x; cv[1] = v.y; cv[2] = v.z; cv[3] = v.w;
+                    cv[4] = cv[5] = cv[6] = cv[7] = __int_as_float(0x7f800000);
                 }
+                setup(nc == 8 ? cv[7] : cv[3]);
+                int below = 0, upto = 0;  // coarse sums below the band, and below or inside it
+#pragma unroll
+                for (int j = 0; j < 8; j++) {
+                    below += cv[j] < lo32;
+                    upto += cv[j] <= hi32;
+                }
+                sure = sure && below == upto && below < nc;  // (total above the band: block `below` holds the crossing)
+                float fv[8];
+                load8(L32 + 8 * min(below, nc - 1), fv);
+                int in = 0, into = 0;
+#pragma unroll
+                for (int q = 0; q < 7; q++) {  // the block's last sum is above the band
+                    in += fv[q] < lo32;
+                    into += fv[q] <= hi32;
+                }
+                sure = sure && in == into;
+                qa = 8 * below + in;
             } else {
                 setup(L32[grid - 1]);
                 int qb = grid;
                 qa = 0;
                 while (qa < qb) {
                     int mid = (qa + qb) >> 1;
-                    if (above(L32[mid], mid)) qb = mid;
+                    const float l = L32[mid];
+                    sure = sure && (l < lo32 || l > hi32);
+                    if (l > hi32) qb = mid;
                     else qa = mid + 1;
                 }
+            }
+            if (!sure) {
+                const long long b0 = a == 0 ? ((long long)c[2] * grid + c[1]) * grid
+                                            : (a == 1 ? (long long)c[2] * grid * grid + c[0] : (long long)c[1] * grid + c[0]);
+                const long long stride = a == 0 ? 1 : (a == 1 ? grid : (long long)grid * grid);
+                qa = line_search(wgt + (size_t)(r - r0) * G * G * G + b0, stride, grid, m);
             }
             c[a] = qa < grid ? qa : grid - 1;
         }
@@ -503,17 +561,14 @@ int voxelise_buffers_for(gnb_ctx *c, int nreg, int grid)
     }
     if (c->sur_nv < nv || c->sur_nreg < nreg) {
         c->sur_gen++;
-        dfree(c, c->vacc); dfree(c, c->vw); dfree(c, c->vcdf); dfree(c, c->vcdf32); dfree(c, c->vcdfc);
+        dfree(c, c->vacc); dfree(c, c->vw); dfree(c, c->vcdf32); dfree(c, c->vcdfc);
         dfree(c, c->cent_d);
-        dfree(c, c->rcount);
         dfree(c, c->vout); dfree(c, c->rsx); dfree(c, c->rsi); dfree(c, c->centf);
-        c->vacc = nullptr; c->vw = nullptr; c->vcdf = nullptr; c->vcdf32 = nullptr; c->vcdfc = nullptr;
+        c->vacc = nullptr; c->vw = nullptr; c->vcdf32 = nullptr; c->vcdfc = nullptr;
         c->cent_d = nullptr;
-        c->rcount = nullptr;
         c->vout = nullptr; c->rsx = nullptr; c->rsi = nullptr; c->centf = nullptr;
         GNB_TRY(dalloc(c, &c->vacc, nv * 8));
         GNB_TRY(dalloc(c, &c->vw, nv));
-        GNB_TRY(dalloc(c, &c->vcdf, nv * 3));
         GNB_TRY(dalloc(c, &c->vcdf32, nv * 3));
         GNB_TRY(dalloc(c, &c->vcdfc, nv * 3 / 8 + 1));
         GNB_TRY(dalloc(c, &c->vout, nv * 5));
@@ -521,7 +576,6 @@ int voxelise_buffers_for(gnb_ctx *c, int nreg, int grid)
         GNB_TRY(dalloc(c, &c->rsx, (size_t)nreg));
         GNB_TRY(dalloc(c, &c->rsi, (size_t)nreg));
         GNB_TRY(dalloc(c, &c->centf, (size_t)nreg * 3));
-        GNB_TRY(dalloc(c, &c->rcount, (size_t)nreg));
         c->sur_nv = nv;
         c->sur_nreg = nreg;
     }
@@ -557,9 +611,8 @@ static int upload_centres(gnb_ctx *c, int nreg, const double *centers)
 static void assign_launch(gnb_ctx *c, int nreg, double side, cudaStream_t st)
 {
     int n = (int)c->n;
-    cudaMemsetAsync(c->rcount, 0, sizeof(int) * nreg, st);
     counted(k_region_assign)<<<(n + 255) / 256, 256, 0, st>>>(c->P[c->cur], n, c->cent_d, c->rsx, c->rsi, c->centf,
-                                                              nreg, 0.5 * side, c->sreg, c->rcount);
+                                                              nreg, 0.5 * side, c->sreg);
 }
 
 // Accumulators of regions [r0, r1) (membership already assigned); their
@@ -609,16 +662,15 @@ static int remap_regions_launch(gnb_ctx *c, int r0, int r1, double side, int gri
     const long long V = (long long)grid * grid * grid;
     size_t nv = (size_t)(r1 - r0) * V;
     counted(k_remap_weights)<<<(unsigned)((nv + 255) / 256), 256, 0, st>>>(pred + (size_t)r0 * V * cout,
-                                                                           (long long)nv, cout, c->vw);
+                                                                           (long long)nv, cout, exp2_table(), c->vw);
     long long nl = (long long)(r1 - r0) * 3 * grid * grid;
     if (grid == 32 || grid == 64)
         counted(k_line_cdf_tiled)<<<(unsigned)((nl / 32 + LC_W - 1) / LC_W), 32 * LC_W, 0, st>>>(
-            c->vw, r1 - r0, grid, c->vcdf, c->vcdf32, c->vcdfc);
+            c->vw, r1 - r0, grid, c->vcdf32, c->vcdfc);
     else
-        counted(k_line_cdf)<<<(unsigned)((nl + 127) / 128), 128, 0, st>>>(c->vw, r1 - r0, grid, c->vcdf, c->vcdf32,
-                                                                          c->vcdfc);
+        counted(k_line_cdf)<<<(unsigned)((nl + 127) / 128), 128, 0, st>>>(c->vw, r1 - r0, grid, c->vcdf32, c->vcdfc);
     counted(k_remap)<<<(n + 127) / 128, 128, 0, st>>>(c->P[c->cur], c->P[c->cur], nullptr, nullptr, n, c->sreg, pred,
-                                                      cout, c->vcdf, c->vcdf32,
+                                                      cout, c->vw, c->vcdf32,
                                                       c->vcdfc, c->cent_d, side, side / grid, 1.0 / (side / grid), grid,
                                                       c->seed_d, sweeps, r0, r1);
     GNB_LAUNCH_CHECK(c, "remap");
@@ -648,9 +700,8 @@ int remap_regions(gnb_ctx *c, int nreg, const double *centers, double side, int 
     unsigned long long sd = seed;
     GNB_TRY(cuda_check(c, cudaMemcpyAsync(c->seed_d, &sd, sizeof(sd), cudaMemcpyHostToDevice, c->s), "seed"));
     int n = (int)c->n;
-    cudaMemsetAsync(c->rcount, 0, sizeof(int) * nreg, c->s);
     counted(k_region_assign)<<<(n + 255) / 256, 256, 0, c->s>>>(c->P[c->cur], n, c->cent_d, c->rsx, c->rsi, c->centf,
-                                                                nreg, 0.5 * side, c->sreg, c->rcount);
+                                                                nreg, 0.5 * side, c->sreg);
     phase_begin(c, GNB_T_REMAP);
     GNB_TRY(remap_launch(c, nreg, side, grid, pred_dev, 5, sweeps));
     phase_end(c);
@@ -759,14 +810,13 @@ int sn_async_submit(gnb_ctx *c, gnb_unet *net, int nreg, const double *centers, 
     GNB_TRY(vox_regions_view(c, sna_view(c), n, c->sna_reg, c->sna_rho, 0, nreg, side, grid, nullptr, xin, st));
     GNB_TRY(unet_run(net, nreg, st, nullptr, nullptr));
     const size_t nv = (size_t)nreg * grid * grid * grid;
-    counted(k_remap_weights)<<<(unsigned)((nv + 255) / 256), 256, 0, st>>>(yout, (long long)nv, cout, c->vw);
+    counted(k_remap_weights)<<<(unsigned)((nv + 255) / 256), 256, 0, st>>>(yout, (long long)nv, cout, exp2_table(), c->vw);
     const long long nl = (long long)nreg * 3 * grid * grid;
     if (grid == 32 || grid == 64)
         counted(k_line_cdf_tiled)<<<(unsigned)((nl / 32 + LC_W - 1) / LC_W), 32 * LC_W, 0, st>>>(
-            c->vw, nreg, grid, c->vcdf, c->vcdf32, c->vcdfc);
+            c->vw, nreg, grid, c->vcdf32, c->vcdfc);
     else
-        counted(k_line_cdf)<<<(unsigned)((nl + 127) / 128), 128, 0, st>>>(c->vw, nreg, grid, c->vcdf, c->vcdf32,
-                                                                          c->vcdfc);
+        counted(k_line_cdf)<<<(unsigned)((nl + 127) / 128), 128, 0, st>>>(c->vw, nreg, grid, c->vcdf32, c->vcdfc);
     GNB_LAUNCH_CHECK(c, "surrogate side stream");
     GNB_TRY(cuda_check(c, cudaEventRecord(c->sna_ev_done, st), "event"));
     c->sna_pending = true;
@@ -785,7 +835,7 @@ int sn_async_apply(gnb_ctx *c)
     const int grid = c->sna_grid;
     counted(k_inverse)<<<(n + 255) / 256, 256, 0, c->s>>>(c->P[c->cur].orig, n, c->sna_inv);
     counted(k_remap)<<<(n + 127) / 128, 128, 0, c->s>>>(sna_view(c), c->P[c->cur], c->sna_orig, c->sna_inv, n,
-                                                        c->sna_reg, c->sna_yout, 5, c->vcdf, c->vcdf32, c->vcdfc,
+                                                        c->sna_reg, c->sna_yout, 5, c->vw, c->vcdf32, c->vcdfc,
                                                         c->cent_d, side, side / grid, 1.0 / (side / grid), grid,
                                                         c->sna_seed, c->sna_sweeps, 0, c->sna_nreg);
     GNB_LAUNCH_CHECK(c, "surrogate apply");

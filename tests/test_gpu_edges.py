@@ -249,3 +249,26 @@ def test_unet_weight_gradients_two_kernels(G, grid, B):
         out.append(net.get_grads().astype(np.float64))
     # both round activations to BF16; a different order of FP32 sums flips some
     assert np.linalg.norm(out[0] - out[1]) < 5e-2 * np.linalg.norm(out[1])
+
+
+# remap: lines with empty voxels (weight 0), weights over many decades and grids
+# of each search form, against the oracle's voxel choices
+@pytest.mark.parametrize("grid", [32, 64, 24])
+def test_remap_extreme_weights(G, orc, grid):
+    from oracle import surrogate as S
+    n, side, cen, sweeps = 4000, 60.0, (3.0, 1.0, -2.0), 6
+    rng = np.random.default_rng(grid)
+    p = ics.sn_region(n, seed=grid, grid=16)
+    for k, v in zip("xyz", cen):
+        p[k] = p[k] + v
+    pred = rng.normal(size=(1, grid, grid, grid, 5)).astype(np.float32)
+    pred[..., 0] = rng.uniform(-25.0, 20.0, pred.shape[:-1])
+    pred[..., 0][rng.uniform(size=pred.shape[:-1]) < 0.3] = -400.0
+    pred[..., 0][:, : grid // 4] = 0.0
+    c = G.Context()
+    c.set_particles(p)
+    c.remap_regions([cen], pred, side=side, seed=77, sweeps=sweeps)
+    pos = np.stack([p[k] for k in "xyz"], axis=1)
+    _, rp, _, _ = S.remap(pred[0].reshape(-1, 5).astype(np.float64), p["id"], pos, cen, side, grid, seed=77, sweeps=sweeps)
+    got = np.stack([c.get(k) for k in "XYZ"], axis=1)
+    assert np.max(np.abs(got - rp)) < 1e-12 * side
