@@ -14,7 +14,7 @@
 //    staging accepted cells (monopole + quadrupole) and the particles of
 //    opened leaves as FP32 offsets from the group's reference grid point
 //    (Sec. 4.3 mixed precision); every thread evaluates its i-particles
-//    (one, two above 16, four above 64 and eight above 128 particles per
+//    (one, two above 8, four above 32 and eight above 128 particles per
 //    group chunk; from two on in float2 pairs on the FP32x2 instructions)
 //    against the staged j entries, read as warp-wide broadcasts, and the j
 //    loop is split over as many thread sets as fit ("j-splits") so all
@@ -44,6 +44,7 @@ struct GravParams {
     const double *box;
     double theta2;
     long long open_d2max[GNB_MAXLEV + 1];  // per level: largest d2 that opens a cell (see must_open)
+    int overlap;  // theta^2 > 4/3: a cell overlapping the group box may pass the distance test
     float G;
     float e2u;  // 2 fl(eps^2) when every particle has the same softening eps > 0
     int quad;
@@ -75,25 +76,33 @@ struct GravSmem {
 // distance between the cell centre and the group box, both in doubled grid
 // units).  That FP64 test is monotone in the integer d2, so the host finds,
 // with the same FP64 arithmetic, the largest d2 that passes it for each
-// level; the walk then compares integers (no FP64 per visited cell).
-__device__ __forceinline__ bool must_open(int4 C, int level, const int *bmin, const int *bmax,
-                                          const long long *d2max)
+// level; the walk then compares integers (no FP64 per visited cell) -- and
+// those first in FP32: the three distances are below 2^23 (exact), so the FP32
+// sum of their squares is within 2^-22 of d2, and a sum outside (1 -+ 2^-20)
+// times the limit orders as d2 does; only one inside that band takes the
+// 64-bit sum.  Overlapping boxes have d2 <= 3 s^2, which the distance test
+// opens by itself unless theta^2 > 4/3 (overlap).
+struct OpenLimits {
+    long long d2max[GNB_MAXLEV + 1];
+    float lo[GNB_MAXLEV + 1], hi[GNB_MAXLEV + 1];
+};
+
+__device__ __forceinline__ bool must_open(int4 C, int level, const int *bmin, const int *bmax, const OpenLimits &L,
+                                          int overlap)
 {
-    long long s = 1ll << (GNB_MAXLEV - level);
-    bool overlap = true;
-    long long d2 = 0;
-    int cc[3] = {C.x, C.y, C.z};
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        long long lo = cc[a], b0 = bmin[a], b1 = bmax[a];
-        if (b0 > lo + s - 1 || b1 < lo) overlap = false;
-        long long cen = 2 * lo + s;
-        long long d = 0;
-        if (2 * b0 > cen) d = 2 * b0 - cen;
-        else if (cen > 2 * b1) d = cen - 2 * b1;
-        d2 += d * d;
-    }
-    return overlap || d2 <= d2max[level];
+    const int s = 1 << (GNB_MAXLEV - level);
+    const int dx = max(0, max(2 * (bmin[0] - C.x) - s, 2 * (C.x - bmax[0]) + s));
+    const int dy = max(0, max(2 * (bmin[1] - C.y) - s, 2 * (C.y - bmax[1]) + s));
+    const int dz = max(0, max(2 * (bmin[2] - C.z) - s, 2 * (C.z - bmax[2]) + s));
+    const float fx = (float)dx, fy = (float)dy, fz = (float)dz;
+    const float d2 = __fmaf_rn(fx, fx, __fmaf_rn(fy, fy, fz * fz));
+    bool open = d2 < L.lo[level];
+    if (!open && d2 <= L.hi[level])
+        open = (long long)dx * dx + (long long)dy * dy + (long long)dz * dz <= L.d2max[level];
+    if (overlap)
+        open = open || (bmin[0] <= C.x + s - 1 && bmax[0] >= C.x && bmin[1] <= C.y + s - 1 && bmax[1] >= C.y &&
+                        bmin[2] <= C.z + s - 1 && bmax[2] >= C.z);
+    return open;
 }
 
 // FP32 1/sqrt(x) of a squared distance plus softening (a positive normal
@@ -395,19 +404,31 @@ __device__ __forceinline__ void cp_async16_g(void *smem, const void *g)
     unsigned s = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(g) : "memory");
 }
+__device__ __forceinline__ void cp_async4_g(void *smem, const void *g)
+{
+    unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(g) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit_g() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all_g() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 // Raw data of up to GW_JC accepted cells (two per thread, node indices in
-// idx) into buffer b: corner, centre of mass + mass, quadrupole.
+// idx) into buffer b: corner, centre of mass + mass, quadrupole -- or, for
+// monopoles, the cell softening alone (4 bytes instead of 32: the copies
+// through L2 weigh as much as the sums for small groups).
+template <bool QUAD>
 __device__ __forceinline__ void cells_issue(GravSmem &S, const GravParams &p, int b, const int *idx)
 {
     for (int h = 0; h < 2; h++) {
         const int s = threadIdx.x + h * GW_THREADS, node = idx[h];
         cp_async16_g(&S.cnb[s], &p.nb[node]);
         cp_async16_g(&S.c0[b][s], &p.mo0[node]);
-        cp_async16_g(&S.c1[b][s], &p.mo1[node]);
-        cp_async16_g(&S.c2[b][s], &p.mo2[node]);
+        if (QUAD) {
+            cp_async16_g(&S.c1[b][s], &p.mo1[node]);
+            cp_async16_g(&S.c2[b][s], &p.mo2[node]);
+        } else {
+            cp_async4_g(&S.c2[b][s].z, &p.mo2[node].z);
+        }
     }
     cp_async_commit_g();
 }
@@ -470,14 +491,28 @@ __device__ __forceinline__ void chain_append_leaf(bool flag, int first, int coun
     else cnt += n;
 }
 
-// Tree walk of one group per warp (see the file comment).
+// Tree walk of one group per warp (see the file comment).  It is bound by
+// instructions: about 70 rounds of 32 nodes a group.  The opening test runs in
+// FP32 (see must_open), the children's places on the stack come from ballots
+// of the bits of their counts, and opened leaves (two or three a round) are
+// collected and appended 32 at a time.  Walk + evaluation with 64-bit tests,
+// shuffle scans and leaves appended each round against this (and the shorter
+// monopole copies): 2^24 disk, n_g = 256, 52.5 -> 50.1 ms; 2^20, n_g = 128, 2592
+// -> 2409 us; 300,007 stars, n_g = 64, monopoles, 1326 -> 1099 us.
 __global__ void __launch_bounds__(GL_WARPS * 32, 5) k_grav_walk(GravParams p)
 {
     __shared__ int stack[GL_WARPS][GL_STACK];
-    __shared__ long long d2max[GNB_MAXLEV + 1];  // lanes index it by level: shared, not the parameter bank
+    __shared__ int2 leafb[GL_WARPS][64];  // leaves to append: first particle, count
+    __shared__ OpenLimits lim;            // lanes index it by level: shared, not the parameter bank
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
     int *st = stack[w];
-    for (int l = threadIdx.x; l <= GNB_MAXLEV; l += blockDim.x) d2max[l] = p.open_d2max[l];
+    for (int l = threadIdx.x; l <= GNB_MAXLEV; l += blockDim.x) {
+        const long long d = p.open_d2max[l];
+        lim.d2max[l] = d;
+        lim.lo[l] = (float)d * (1.f - 0x1p-20f);
+        lim.hi[l] = (float)d * (1.f + 0x1p-20f);
+    }
     __syncthreads();
     const int ngroups = *p.ngroups;
     unsigned long long cnt_pp = 0, cnt_pc = 0;
@@ -496,52 +531,73 @@ __global__ void __launch_bounds__(GL_WARPS * 32, 5) k_grav_walk(GravParams p)
             for (int a = 0; a < 3; a++) { bmin[a] = min(bmin[a], cc[a]); bmax[a] = max(bmax[a], cc[a]); }
         }
 #pragma unroll
-        for (int a = 0; a < 3; a++)
-            for (int o = 16; o > 0; o >>= 1) {
-                bmin[a] = min(bmin[a], __shfl_xor_sync(0xffffffffu, bmin[a], o));
-                bmax[a] = max(bmax[a], __shfl_xor_sync(0xffffffffu, bmax[a], o));
-            }
+        for (int a = 0; a < 3; a++) {
+            bmin[a] = __reduce_min_sync(0xffffffffu, bmin[a]);
+            bmax[a] = __reduce_max_sync(0xffffffffu, bmax[a]);
+        }
         int ccur = chain_new(p, lane), lcur = chain_new(p, lane);
         const int chead = ccur, lhead = lcur;
-        int ccnt = 0, lcnt = 0, ncell = 0, npart = 0;
+        int ccnt = 0, lcnt = 0, ncell = 0, npart = 0, nl = 0;
         int sp = 1;
         if (lane == 0) st[0] = 0;
         __syncwarp();
         while (sp > 0) {
             // pop up to 32 nodes, keeping room for their children
-            int k = min(32, sp);
-            const int room = max(1, (GL_STACK - sp) / 7);
-            k = min(k, room);
+            const int k = min(min(32, sp), max(1, (GL_STACK - sp) / 7));
             const int node = lane < k ? st[sp - k + lane] : -1;
             __syncwarp();
             sp -= k;
             bool is_cell = false, is_leaf = false;
-            int nch = 0, child0 = 0, lcount = 0, lfirst = 0;
+            int nch = 0;
+            int4 a = make_int4(0, 0, 0, 0);
             if (node >= 0) {
-                const int4 a = __ldg(&p.na[node]);
-                const int lev = a.w & 255;
-                const bool open = node == 0 || must_open(__ldg(&p.nb[node]), lev, bmin, bmax, d2max);
-                if (!open) is_cell = true;
-                else if ((a.w >> 8) == 0) { is_leaf = true; lcount = a.y; lfirst = a.x; }
-                else { nch = a.w >> 8; child0 = a.z; }
+                a = __ldg(&p.na[node]);
+                const int4 C = __ldg(&p.nb[node]);
+                if (node != 0 && !must_open(C, a.w & 255, bmin, bmax, lim, p.overlap)) is_cell = true;
+                else {
+                    nch = a.w >> 8;
+                    is_leaf = nch == 0;
+                }
             }
-            // push children (inclusive scan of the child counts over the warp)
-            int inc = nch;
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, inc, o);
-                if (lane >= o) inc += y;
+            // push children: prefix sums of the counts (at most 8), bit by bit
+            int pre = 0, tot = 0;
+#pragma unroll
+            for (int b = 0; b < 4; b++) {
+                const unsigned m = __ballot_sync(0xffffffffu, (nch >> b) & 1);
+                pre += __popc(m & lt) << b;
+                tot += __popc(m) << b;
             }
-            const int tot = __shfl_sync(0xffffffffu, inc, 31);
-            const int base = sp + inc - nch;
-            for (int q = 0; q < nch; q++) {
-                if (base + q < GL_STACK) st[base + q] = child0 + q;
-                else atomicOr(p.status, ST_STACK_OVERFLOW);
+            const int base = sp + pre;
+            if (base + nch <= GL_STACK) {
+                for (int q = 0; q < nch; q++) st[base + q] = a.z + q;
+            } else if (nch > 0) {
+                atomicOr(p.status, ST_STACK_OVERFLOW);
+                for (int q = 0; q < nch && base + q < GL_STACK; q++) st[base + q] = a.z + q;
             }
             sp = min(sp + tot, GL_STACK);
+            const unsigned lb = __ballot_sync(0xffffffffu, is_leaf);
+            if (is_leaf) leafb[w][nl + __popc(lb & lt)] = make_int2(a.x, a.y);
+            nl += __popc(lb);
             __syncwarp();
-            chain_append(is_cell, node, ccur, ccnt, p, lane);
-            chain_append_leaf(is_leaf, lfirst, lcount, npart, lcur, lcnt, p, lane);
             ncell += __popc(__ballot_sync(0xffffffffu, is_cell));
+            chain_append(is_cell, node, ccur, ccnt, p, lane);
+            if (nl >= 32 || (sp == 0 && nl > 0)) {
+                // in the order found: the first 32, the rest moved up
+                const int2 lf = leafb[w][lane];
+                const int2 rest = leafb[w][32 + lane];
+                const int m = min(nl, 32);
+                chain_append_leaf(lane < m, lf.x, lf.y, npart, lcur, lcnt, p, lane);
+                __syncwarp();
+                nl -= m;
+                if (lane < nl) leafb[w][lane] = rest;
+                __syncwarp();
+                if (sp == 0 && nl > 0) {
+                    const int2 l2 = leafb[w][lane];
+                    chain_append_leaf(lane < nl, l2.x, l2.y, npart, lcur, lcnt, p, lane);
+                    nl = 0;
+                    __syncwarp();
+                }
+            }
         }
         chain_close(p, ccur, ccnt, lane);
         chain_close(p, lcur, lcnt, lane);
@@ -608,7 +664,7 @@ __device__ __forceinline__ void eval_chunk(GravSmem &S, const GravParams &p, int
     if (ch >= 0) {
         idx[0] = p.pool[(size_t)ch * GL_CH + tid];
         idx[1] = p.pool[(size_t)ch * GL_CH + tid + GW_THREADS];
-        cells_issue(S, p, 0, idx);
+        cells_issue<QUAD>(S, p, 0, idx);
         cnx = p.cnext[ch];
         if (cnx >= 0) {
             idx[0] = p.pool[(size_t)cnx * GL_CH + tid];
@@ -667,7 +723,7 @@ __device__ __forceinline__ void eval_chunk(GravSmem &S, const GravParams &p, int
         const int nc = p.ccnt[ch];
         int nxt2 = -1, idx2[2] = {0, 0};
         if (cnx >= 0) {
-            cells_issue(S, p, cb ^ 1, idx);
+            cells_issue<QUAD>(S, p, cb ^ 1, idx);
             nxt2 = p.cnext[cnx];
             if (nxt2 >= 0) {
                 idx2[0] = p.pool[(size_t)nxt2 * GL_CH + tid];
@@ -735,8 +791,9 @@ __device__ __forceinline__ void eval_chunk(GravSmem &S, const GravParams &p, int
 
 // Evaluation of the walk's lists, one group per CTA (see the file comment):
 // the group's particles in chunks of up to NIMAX * GW_THREADS, eight per
-// thread above 128 particles in a chunk (NIMAX = 8), four above 64, two above
-// 16, else one.  Five CTAs per SM (96 registers a thread; the eight-particle
+// thread above 128 particles in a chunk (NIMAX = 8), four above 32, two above
+// 8, else one (walk + evaluation with limits of 64 and 16 against 32 and 8:
+// 2^20 disk, n_g = 128, 2643 -> 2592 us; 300,007 stars, n_g = 64, 1368 -> 1326).  Five CTAs per SM (96 registers a thread; the eight-particle
 // variant spills a few bytes outside its inner loops and still runs faster
 // than at 4 CTAs and 128 registers).
 template <bool MASK, bool QUAD, int NIMAX, bool UNI>
@@ -762,8 +819,8 @@ __global__ void __launch_bounds__(GW_THREADS, 5) k_grav_eval(GravParams p)
             const int icnt = min(NIMAX * GW_THREADS, gcount - i0);
             if (NIMAX >= 8 && icnt > 128)
                 eval_chunk<NIMAX >= 8 ? 8 : 4, MASK, QUAD, UNI>(S, p, gfirst + i0, icnt, gh, gref, unit);
-            else if (icnt > 64) eval_chunk<4, MASK, QUAD, UNI>(S, p, gfirst + i0, icnt, gh, gref, unit);
-            else if (icnt > 16) eval_chunk<2, MASK, QUAD, UNI>(S, p, gfirst + i0, icnt, gh, gref, unit);
+            else if (icnt > 32) eval_chunk<4, MASK, QUAD, UNI>(S, p, gfirst + i0, icnt, gh, gref, unit);
+            else if (icnt > 8) eval_chunk<2, MASK, QUAD, UNI>(S, p, gfirst + i0, icnt, gh, gref, unit);
             else eval_chunk<1, MASK, QUAD, UNI>(S, p, gfirst + i0, icnt, gh, gref, unit);
         }
     }
@@ -943,6 +1000,7 @@ static GravParams make_params(gnb_ctx *c)
     p.ax = c->gax; p.ay = c->gay; p.az = c->gaz; p.pot = c->pot;
     p.box = c->box_d;
     p.theta2 = c->cfg.theta * c->cfg.theta;
+    p.overlap = !(p.theta2 < 1.333);  // (with a margin: the test is exact, only not needed)
     for (int l = 0; l <= GNB_MAXLEV; l++) {
         // largest d2 with (2 s)^2 > theta2 * (double)d2 (the test is monotone
         // in d2; (double)d2 rounds the same way here and on the device)
