@@ -77,7 +77,8 @@ __device__ __forceinline__ float kern_dw(float r, float hinv)
 struct GasGather {
     const uint64_t *skey;
     PArr p;
-    const int *gslot;
+    int *gslot;
+    int all;  // every particle is gas: slot k itself
     uint64_t *gkey;
     int *ggrank;
     int4 *C;
@@ -93,7 +94,9 @@ __global__ void k_gas_gather(GasGather g)
 {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= g.ng) return;
-    int s = g.gslot[k];
+    int s = k;
+    if (g.all) g.gslot[k] = k;
+    else s = g.gslot[k];
     g.gkey[k] = g.skey[s];
     g.C[k] = make_int4(g.p.cx[s], g.p.cy[s], g.p.cz[s], __float_as_int(g.p.m[s]));
     g.R[k] = make_float4(g.p.rx[s], g.p.ry[s], g.p.rz[s], 0.f);
@@ -952,9 +955,10 @@ int sph_density(gnb_ctx *c)
     phase_begin(c, GNB_T_HYDRO_TREE);
     PArr &a = c->P[c->cur];
     int gb = (ng + 255) / 256;
-    // gas slots in Morton order
-    GNB_TRY(gas_slots(c, a.type, c->n_d, c->gslot));
+    // gas slots in Morton order (a supernova region is all gas: nothing to select)
     GasGather gg;
+    gg.all = c->n_gas == c->n ? 1 : 0;
+    if (!gg.all) GNB_TRY(gas_slots(c, a.type, c->n_d, c->gslot));
     gg.skey = c->skey; gg.p = a; gg.gslot = c->gslot; gg.gkey = c->gkey;
     gg.ggrank = c->ggrank; gg.C = c->fC; gg.R = c->fR;
     gg.gvx = c->gvx; gg.gvy = c->gvy; gg.gvz = c->gvz; gg.gu = c->gu; gg.gRprev = c->gRprev;
