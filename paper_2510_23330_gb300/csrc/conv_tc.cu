@@ -19,15 +19,16 @@
 // The weights of all taps stay resident in shared memory for the whole
 // persistent CTA, packed [tap][channel group][N][8].
 //
-// Roles (192 threads): warp 4 lane 0 issues the TMA loads, warp 5 runs the
-// MMA loop warp-uniformly and one elected lane issues tcgen05.mma (FP32
-// accumulators in TMEM), warps 0..3 read TMEM with
-// tcgen05.ld and apply bias, ReLU and the BF16 store.  Halo buffers and TMEM
-// accumulators are double buffered so the loads of tile i + 1, the MMAs of
-// tile i and the epilogue of tile i - 1 overlap.  Every mbarrier wait is
-// bounded (1 s of %globaltimer); a wait that runs out sets the error word,
-// all roles leave their loops, in-flight copies and MMAs are drained (again
-// bounded) and TMEM is freed before the CTA exits.
+// Roles (352 threads): warp 8 lane 0 issues the TMA loads, warps 9 and 10 run
+// the MMA loop warp-uniformly and one elected lane of each issues tcgen05.mma
+// (FP32 accumulators in TMEM; one warp when the z-taps share an MMA or the tile
+// has one plane), warps 0..7 read TMEM with tcgen05.ld and apply bias, ReLU and
+// the BF16 store.  Halo buffers and TMEM accumulators are double buffered where
+// they fit so the loads of tile i + 1, the MMAs of tile i and the epilogue of
+// tile i - 1 overlap.  Every mbarrier wait is bounded (1 s of %globaltimer); a
+// wait that runs out sets the error word, all roles leave their loops, in-flight
+// copies and MMAs are drained (again bounded) and TMEM is freed before the CTA
+// exits.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -43,12 +44,14 @@ namespace gnb {
 
 namespace {
 
-constexpr int TC_THREADS = 192;
+constexpr int EPI_WARPS = 8, TMA_WARP = 8, MMA_WARP = 9;  // then two MMA warps
+constexpr int TC_THREADS = 32 * (MMA_WARP + 2);
 constexpr int HX = 10, HY = 18;          // halo extent in x and y
 constexpr unsigned ROW_BYTES = 16;       // one voxel of one 8-channel group
 constexpr unsigned YSTRIDE = HX * ROW_BYTES;
 constexpr unsigned ZSTRIDE = HY * YSTRIDE;
-constexpr unsigned HDR = 256;            // barriers, TMEM slot, abort word
+constexpr unsigned BIAS_AT = 256;        // after the barriers, TMEM slot and abort word
+constexpr unsigned HDR = BIAS_AT + 1024; // with the bias of up to 256 output channels
 constexpr int MAX_WSTAGE = 4;            // weight ring stages when the weights are streamed
 constexpr unsigned ALIGN_SLACK = 1024;
 constexpr unsigned long long WAIT_NS = 1000000000ull;
@@ -61,12 +64,12 @@ struct TcArgs {
     bf16 *out1, *out2;
     int N, K, C1, O1, relu;
     int B, D, H, W;
-    int Zt, nbuf, tx, ty, tz;
+    int Zt, nbuf, nacc, tx, ty, tz;  // nbuf halo buffers, nacc accumulator buffers
     int wstages;  // 0: all 27 taps resident; else a ring of this many one-tap stages
     int dzn;      // 1: the three z-taps share one MMA (N = 3 N_out, sliding TMEM windows)
     unsigned acc_cols;  // TMEM columns of one accumulator buffer
     long long ntiles;
-    unsigned wbytes, plane, halo, off_w, off_h, tx_bytes, tmem_cols, idesc;
+    unsigned wbytes, plane, halo, off_w, off_h, tx_bytes, tmem_cols;
     int *err;
 };
 
@@ -104,7 +107,7 @@ __device__ __forceinline__ unsigned long long gtimer()
 // Bounded wait for the phase of `parity`.  Returns false when another role
 // has aborted (honour_abort) or after WAIT_NS, in which case it aborts the
 // CTA and records `code` in the error word.
-__device__ bool mb_wait(unsigned bar, unsigned parity, volatile int *abort_flag, int *err, int code,
+__device__ __noinline__ bool mb_wait(unsigned bar, unsigned parity, volatile int *abort_flag, int *err, int code,
                         bool honour_abort = true)
 {
     unsigned long long t0 = 0;
@@ -121,6 +124,13 @@ __device__ bool mb_wait(unsigned bar, unsigned parity, volatile int *abort_flag,
             }
         }
     }
+}
+
+// The same with the first test inline: between the MMAs of two taps or tiles a
+// call and its return cost more than the tensor core's queue covers.
+__device__ __forceinline__ bool mb_wait_ready(unsigned bar, unsigned parity, volatile int *abort_flag, int *err, int code)
+{
+    return mb_try(bar, parity) || mb_wait(bar, parity, abort_flag, err, code);
 }
 
 __device__ __forceinline__ void tma_load_4d(unsigned dst, const CUtensorMap *m, int c0, int c1, int c2, int c3,
@@ -178,19 +188,42 @@ __device__ __forceinline__ void tc_commit_elect(unsigned bar)
         : "memory");
 }
 
-// 16 consecutive FP32 columns of this thread's TMEM lane; the wait is in the
+// NC consecutive FP32 columns of this thread's TMEM lane; the wait is in the
 // same statement so no use of the registers can be scheduled before it.
+template <int NC>
+__device__ void tc_ld(unsigned taddr, unsigned *r);
+template <>
+__device__ __forceinline__ void tc_ld<16>(unsigned taddr, unsigned *r)
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
+                 "%13, %14, %15}, [%16];\n"
+                 "tcgen05.wait::ld.sync.aligned;\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+                   "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]),
+                   "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                 : "r"(taddr)
+                 : "memory");
+}
+template <>
+__device__ __forceinline__ void tc_ld<32>(unsigned taddr, unsigned *r)
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
+                 "%13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31},"
+                 " [%32];\n"
+                 "tcgen05.wait::ld.sync.aligned;\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+                   "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]),
+                   "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]),
+                   "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+                   "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]),
+                   "=r"(r[30]), "=r"(r[31])
+                 : "r"(taddr)
+                 : "memory");
+}
 __device__ __forceinline__ void tc_ld16(unsigned taddr, float *v)
 {
     unsigned r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-        "%15}, [%16];\n"
-        "tcgen05.wait::ld.sync.aligned;\n"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
+    tc_ld<16>(taddr, r);
 #pragma unroll
     for (int i = 0; i < 16; i++) v[i] = __uint_as_float(r[i]);
 }
@@ -209,18 +242,6 @@ __device__ __forceinline__ void tc_ld8(unsigned taddr, float *v)
     for (int i = 0; i < 8; i++) v[i] = __uint_as_float(r[i]);
 }
 
-// Zeros 16 consecutive FP32 columns of this warp's 32 TMEM lanes.
-__device__ __forceinline__ void tc_st16_zero(unsigned taddr)
-{
-    const unsigned z = 0u;
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, "
-        "%1};\n" ::"r"(taddr),
-        "r"(z)
-        : "memory");
-}
-__device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
-
 __device__ __forceinline__ void decode_tile(const TcArgs &p, int Zt, long long t, int &bb, int &z0, int &y0, int &x0)
 {
     int xt = (int)(t % p.tx);
@@ -234,21 +255,37 @@ __device__ __forceinline__ void decode_tile(const TcArgs &p, int Zt, long long t
     z0 = Zt * zt;
 }
 
+// kind::f16 instruction descriptor without N: FP32 accumulator (bit 4), BF16 A
+// (bits 7-9 = 1) and B (bits 10-12 = 1), both K-major, M >> 4 at bit 24
+// (M = 128); N >> 3 goes to bit 17.
+constexpr unsigned IDESC0 = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 4) << 24);
+
+// Bytes of one channel group of a tile's halo.
+__host__ __device__ constexpr unsigned plane_bytes(int zt) { return ((unsigned)(zt + 2) * ZSTRIDE + 127u) & ~127u; }
+
+// The tensor core needs max(N / 2, 32 + N / 4) cycles for one 128 x N x 16 MMA
+// (measured; the 4 KB of A and the 32 N bytes of B come from shared memory at
+// 128 bytes a cycle), whatever the accumulator, the start address or the
+// stride: 44 at N = 48, 48 at N = 64, 56 at N = 96.  One warp issues that fast
+// only when every operand is a loop-carried base plus a compile-time constant;
+// with N, the plane size or K read from the arguments, and 64-bit divisions by
+// the ring size between the taps, an MMA took 71 (resident weights) to 98
+// (streamed) cycles at N = 64.  So the tile depth, N and the K steps of a block are
+// template parameters; 0 stands for a run-time value.
+
 // The MMAs of one dz-in-N tile.  Input plane j, in-plane tap (ty, tx): one
-// MMA of N = 3 N_out whose column window [j N, (j + 3) N) holds output planes
-// j - 2, j - 1, j (z-taps 2, 1, 0); every MMA accumulates.  Windows of planes
-// j = r, r + 3, ... are disjoint, so issuing them back to back keeps several
-// accumulations in flight instead of a chain of dependent MMAs.  With the
-// tile depth and K / 16 known at compile time the loop nest is straight-line
-// code: a small-N MMA takes only ~40 cycles of the tensor core, and a loop
-// with run-time bounds spends about twice that per MMA on issue.
-template <int ZT, int NKS>
+// MMA whose columns are output planes j - 2, j - 1, j (z-taps 2, 1, 0), less
+// those outside the tile.  Windows of planes j = r, r + 3, ... are disjoint, so
+// every output sums its z-taps in the order of r and, within one, (ty, tx) and
+// the channels in order; those of r = 0 cover every output plane, so its first
+// MMAs start the sums.
+template <int ZT, int NKS, int NN>
 __device__ __forceinline__ void issue_dzn(const TcArgs &p, unsigned alo0, unsigned sW, unsigned d0)
 {
-    const int Zt = ZT ? ZT : p.Zt, nks = NKS ? NKS : (p.K >> 4);
+    const int Zt = ZT ? ZT : p.Zt, nks = NKS ? NKS : (p.K >> 4), N = NN ? NN : p.N;
     const unsigned ahi = sdesc_hi(YSTRIDE), bhi = sdesc_hi(128u);
-    const unsigned zs4 = ZSTRIDE >> 4, pl4 = (2u * p.plane) >> 4;
-    const unsigned n3 = 3u * (unsigned)p.N;
+    const unsigned zs4 = ZSTRIDE >> 4, pl4 = (2u * plane_bytes(Zt)) >> 4;
+    const unsigned n3 = 3u * (unsigned)N;
     const unsigned wyx4 = ((unsigned)nks * 2u * n3 * 16u) >> 4;  // one (ty, tx) slice of weights
     const unsigned bk4 = (2u * n3 * 16u) >> 4;
     const unsigned blo0 = sdesc_lo(sW, n3 * 16u);
@@ -258,20 +295,62 @@ __device__ __forceinline__ void issue_dzn(const TcArgs &p, unsigned alo0, unsign
         for (int yx = 0; yx < 9; yx++) {
             const unsigned aoff = ((unsigned)(yx / 3) * YSTRIDE + (unsigned)(yx % 3) * ROW_BYTES) >> 4;
 #pragma unroll
-            for (int ks = 0; ks < nks; ks++) {
-                const unsigned long long bd = dpair(blo0 + (unsigned)yx * wyx4 + (unsigned)ks * bk4, bhi);
+            for (int ks = 0; ks < nks; ks++)
 #pragma unroll
-                for (int j = r; j < Zt + 2; j += 3)
-                    tc_mma_elect(d0 + (unsigned)(j * p.N), dpair(alo0 + aoff + (unsigned)ks * pl4 + (unsigned)j * zs4, ahi),
-                                 bd, p.idesc, 1u);
-            }
+                for (int j = r; j < Zt + 2; j += 3) {
+                    const int q0 = j < 2 ? 2 - j : 0, q1 = j < Zt ? 3 : Zt + 2 - j;  // z-tap blocks inside the tile
+                    tc_mma_elect(d0 + (unsigned)((j - 2 + q0) * N),
+                                 dpair(alo0 + aoff + (unsigned)ks * pl4 + (unsigned)j * zs4, ahi),
+                                 dpair(blo0 + (unsigned)yx * wyx4 + (unsigned)ks * bk4 + (unsigned)(q0 * N), bhi),
+                                 IDESC0 | ((unsigned)((q1 - q0) * N >> 3) << 17), (unsigned)(r + yx + ks != 0));
+                }
         }
 }
 
+// The MMAs of TAPS consecutive x-taps of one plain tile: per K step (innermost,
+// so every accumulator sums its taps and channels in one fixed order) one MMA
+// for each of this warp's z-planes, in blocks of NKS K steps.  FIRST: the first MMA
+// of each plane starts its sum.
+template <int ZT, int NKS, int NN, int TAPS, bool FIRST>
+__device__ __forceinline__ void issue_taps(const TcArgs &p, unsigned alo, unsigned blo, unsigned d0, int mw)
+{
+    constexpr int U = NKS ? NKS : 1;
+    const int Zt = ZT ? ZT : p.Zt, blocks = (p.K >> 4) / U, N = NN ? NN : p.N, nmma = Zt > 1 ? 2 : 1;
+    alo += (unsigned)mw * (ZSTRIDE >> 4);  // planes mw, mw + 2, ...
+    d0 += (unsigned)(mw * N);
+    const unsigned ahi = sdesc_hi(YSTRIDE), bhi = sdesc_hi(128u);
+    const unsigned zs4 = ZSTRIDE >> 4, pl4 = (2u * plane_bytes(Zt)) >> 4, nb4 = (2u * (unsigned)N * 16u) >> 4;
+    const unsigned idesc = IDESC0 | ((unsigned)(N >> 3) << 17);
+#pragma unroll
+    for (int t = 0; t < TAPS; t++) {
+        unsigned at = alo + (unsigned)t * (ROW_BYTES >> 4);
+#pragma unroll 1
+        for (int kb = 0; kb < blocks; kb++, at += U * pl4, blo += U * nb4) {
+#pragma unroll
+            for (int u = 0; u < U; u++)
+#pragma unroll
+                for (int zz = 0; zz < Zt - (ZT ? 0 : mw); zz += nmma)
+                    tc_mma_elect(d0 + (unsigned)(zz * N), dpair(at + (unsigned)u * pl4 + (unsigned)zz * zs4, ahi),
+                                 dpair(blo + (unsigned)u * nb4, bhi), idesc,
+                                 FIRST && t == 0 && u == 0 ? (unsigned)(kb != 0) : 1u);
+        }
+    }
+}
+
 // DZ: 1 dz-in-N, 0 plain, -1 read from p; ZT: tile depth (0: read from p);
-// NKS: K / 16 (0: read from p).
-template <int DZ, int ZT, int NKS>
-__global__ void __launch_bounds__(TC_THREADS, 1)
+// NKS: K / 16 (plain tiles: the K steps of one straight-line block; 0: read from p);
+// NN: the output channels (0: read from p).
+// CTAs that can share an SM: the registers are limited for two where the shared
+// memory of a dz-in-N tile admits two (32 -> 16 channels, one CTA: 285 us
+// without the limit on 32 x 64^3 voxels, 355 with it; 16 -> 32 channels on
+// 32 x 32^3, two CTAs: 38 us with one, 29 with two).
+__host__ __device__ constexpr int tc_min_ctas(int dz, int zt, int nks, int nn)
+{
+    return dz == 1 && zt && 27u * (unsigned)(nn * nks) * 32u + 4u * (unsigned)nks * plane_bytes(zt) > TC_SMEM_SM / 2u ? 1 : 2;
+}
+
+template <int DZ, int ZT, int NKS, int NN>
+__global__ void __launch_bounds__(TC_THREADS, tc_min_ctas(DZ, ZT, NKS, NN))
     k_conv3_tc(const __grid_constant__ CUtensorMap m1, const __grid_constant__ CUtensorMap m2, const TcArgs p)
 {
     const int Zt = ZT ? ZT : p.Zt;
@@ -286,23 +365,30 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     auto bar = [&](int i) { return sb + 8u * (unsigned)i; };
 
+    // plain tiles of two and more planes are issued by two warps, each with its
+    // share of the planes (the accumulators are independent): one warp spent
+    // 60 to 90 cycles per 48-cycle MMA (N = 64) on the waits and commits of a tap
+    const int nmma = !dzn && Zt > 1 ? 2 : 1;
     if (threadIdx.x == 0) {
         mb_init(bar(B_W), 1);
         for (int b = 0; b < 2; b++) {
             mb_init(bar(B_HF + b), 1);
-            mb_init(bar(B_HE + b), 1);
-            mb_init(bar(B_AF + b), 1);
-            mb_init(bar(B_AE + b), 128);
+            mb_init(bar(B_HE + b), (unsigned)nmma);
+            mb_init(bar(B_AF + b), (unsigned)nmma);
+            mb_init(bar(B_AE + b), 32 * EPI_WARPS);
         }
-        mb_init(bar(B_DR), 1);
+        mb_init(bar(B_DR), (unsigned)nmma);
         for (int q = 0; q < MAX_WSTAGE; q++) {
             mb_init(bar(B_WF + q), 1);
-            mb_init(bar(B_WE + q), 1);
+            mb_init(bar(B_WE + q), (unsigned)nmma);
         }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
-    if (warp == 4) {
+    float *sbias = reinterpret_cast<float *>(gb + BIAS_AT);
+    if (p.bias)
+        for (int n = threadIdx.x; n < p.N; n += TC_THREADS) sbias[n] = p.bias[n];
+    if (warp == TMA_WARP) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(slot)),
                      "r"(p.tmem_cols)
                      : "memory");
@@ -313,20 +399,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     tc_fence_after();
     const unsigned tmem = *slot;
     const int kc8 = p.K >> 3;
-    if (dzn) {
-        // the sliding accumulator windows start from zero: the epilogue warps
-        // clear both buffers here and each buffer again after reading it
-        if (warp < 4) {
-            for (unsigned c = 0; c < (unsigned)p.nbuf * p.acc_cols; c += 16)
-                tc_st16_zero(tmem + ((unsigned)(32 * warp) << 16) + c);
-            tc_wait_st();
-        }
-        tc_fence_before();
-        __syncthreads();
-        tc_fence_after();
-    }
-
-    if (warp == 4) {
+    if (warp == TMA_WARP) {
         if (lane == 0) {
             // ---------------------------------------------------------- producer
             const unsigned wtap = (unsigned)kc8 * (unsigned)p.N * 16u;  // bytes of one tap's weights
@@ -338,7 +411,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 }
             }
             int uses[2] = {0, 0};
-            long long wg = 0;  // weight-tap loads issued (streamed mode)
+            // the weight ring: the next stage and how often it was filled (counted,
+            // as 64-bit divisions by the ring size took as long as a tap's MMAs)
+            int st = 0;
+            unsigned round = 0;
             bool stop = false;
             int i = 0;
             for (long long t = blockIdx.x; t < p.ntiles; t += gridDim.x, i++) {
@@ -361,16 +437,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 }
                 uses[b]++;
                 // streamed weights: the 27 taps of this tile through the ring
-                for (int tap = 0; p.wstages && tap < 27; tap++, wg++) {
-                    const int st = (int)(wg % p.wstages);
-                    const unsigned kk = (unsigned)(wg / p.wstages);
-                    if (kk > 0 && !mb_wait(bar(B_WE + st), (kk - 1) & 1u, abort_flag, p.err, 8)) {
+                for (int tap = 0; p.wstages && tap < 27; tap++) {
+                    if (round > 0 && !mb_wait(bar(B_WE + st), (round - 1) & 1u, abort_flag, p.err, 8)) {
                         stop = true;
                         break;
                     }
                     mb_expect_tx(bar(B_WF + st), wtap);
                     bulk_load(sW + (unsigned)st * wtap, reinterpret_cast<const unsigned char *>(p.w) + (size_t)tap * wtap,
                               wtap, bar(B_WF + st));
+                    if (++st == p.wstages) { st = 0; round++; }
                 }
                 if (stop) break;
             }
@@ -378,88 +453,90 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             if (!p.wstages) mb_wait(bar(B_W), 0, abort_flag, p.err, 2, false);
             for (int b = 0; b < 2; b++)
                 if (uses[b] > 0) mb_wait(bar(B_HF + b), (unsigned)(uses[b] - 1) & 1u, abort_flag, p.err, 2, false);
-            for (int st = 0; p.wstages && st < p.wstages; st++) {
-                // the last load issued into stage st is number (wg - 1 - ((wg - 1 - st) mod S))
-                if (wg > st) {
-                    const long long last = st + ((wg - 1 - st) / p.wstages) * p.wstages;
-                    mb_wait(bar(B_WF + st), (unsigned)(last / p.wstages) & 1u, abort_flag, p.err, 2, false);
-                }
+            for (int q = 0; q < p.wstages; q++) {
+                const unsigned fills = round + (q < st ? 1u : 0u);
+                if (fills > 0) mb_wait(bar(B_WF + q), (fills - 1) & 1u, abort_flag, p.err, 2, false);
             }
         }
-    } else if (warp == 5) {
+    } else if (warp >= MMA_WARP) {
+        const int mw = warp - MMA_WARP;
         // ------------------------------------------------------------------ MMA
         // The Zt z-planes of a tile accumulate into Zt independent TMEM
         // blocks; their MMAs are interleaved so consecutive MMAs never feed
         // the same accumulator.
-        int ok = p.wstages ? 1 : mb_wait(bar(B_W), 0, abort_flag, p.err, 3);
+        int ok = mw >= nmma ? 0 : (p.wstages ? 1 : mb_wait(bar(B_W), 0, abort_flag, p.err, 3));
         if (__all_sync(0xffffffffu, ok)) {
-            long long wg = 0;  // weight taps consumed (streamed mode)
+            const long long first_reuse = blockIdx.x + (long long)p.nacc * gridDim.x;
+            int st = 0;  // the weight ring's next stage and the parity of its fill
+            unsigned wpar = 0;
             const unsigned wtap = (unsigned)kc8 * (unsigned)p.N * 16u;  // bytes of one tap's weights
             const unsigned nbytes16 = (unsigned)p.N * 16u;              // one channel group of weights
-            int i = 0;
-            for (long long t = blockIdx.x; t < p.ntiles; t += gridDim.x, i++) {
-                const int b = i % p.nbuf;
-                const unsigned k = (unsigned)(i / p.nbuf);
-                ok = mb_wait(bar(B_HF + b), k & 1u, abort_flag, p.err, 4);
+            int b = 0, ab = 0;  // halo and accumulator buffer, and the parities of their barriers' phases
+            unsigned hpar = 0, apar = 1;
+            for (long long t = blockIdx.x; t < p.ntiles; t += gridDim.x) {
+                ok = mb_wait_ready(bar(B_HF + b), hpar, abort_flag, p.err, 4);
+                if (t >= first_reuse) ok = ok && mb_wait_ready(bar(B_AE + ab), apar, abort_flag, p.err, 5);
                 if (!__all_sync(0xffffffffu, ok)) break;
-                if (k > 0) {
-                    ok = mb_wait(bar(B_AE + b), (k - 1) & 1u, abort_flag, p.err, 5);
-                    if (!__all_sync(0xffffffffu, ok)) break;
-                }
                 tc_fence_after();
                 const unsigned hb = sH + (unsigned)b * p.halo;
-                const unsigned d0 = tmem + (unsigned)b * p.acc_cols;
+                const unsigned d0 = tmem + (unsigned)ab * p.acc_cols;
                 bool stop = false;
                 // descriptors are stepped as 32-bit low words (start address in
                 // 16-byte units): a few adds per MMA
-                const unsigned ahi = sdesc_hi(YSTRIDE), bhi = sdesc_hi(128u);
                 const unsigned alo0 = sdesc_lo(hb, p.plane);
-                const unsigned zs4 = ZSTRIDE >> 4, pl4 = (2u * p.plane) >> 4;
-                if (dzn) issue_dzn<ZT, NKS>(p, alo0, sW, d0);
-                const unsigned nb4 = (2u * (unsigned)p.N * 16u) >> 4;  // two channel groups of weights
-                for (int tap = 0; !dzn && tap < 27; tap++) {
-                    const int tz = tap / 9, ty = (tap / 3) % 3, tx = tap % 3;
-                    unsigned alo = alo0 + (((unsigned)tz * ZSTRIDE + (unsigned)ty * YSTRIDE + (unsigned)tx * ROW_BYTES) >> 4);
-                    unsigned w0 = sW + (unsigned)tap * wtap;
-                    int st = 0;
-                    if (p.wstages) {
-                        st = (int)(wg % p.wstages);
-                        ok = mb_wait(bar(B_WF + st), (unsigned)(wg / p.wstages) & 1u, abort_flag, p.err, 9);
+                if (dzn) issue_dzn<ZT, NKS, NN>(p, alo0, sW, d0);
+                for (int row = 0; !dzn && row < 9; row++) {  // (tz, ty); the three tx inside
+                    const unsigned alo = alo0 + (((unsigned)(row / 3) * ZSTRIDE + (unsigned)(row % 3) * YSTRIDE) >> 4);
+                    if (!p.wstages) {
+                        const unsigned blo = sdesc_lo(sW + 3u * (unsigned)row * wtap, nbytes16);
+                        if (row) issue_taps<ZT, NKS, NN, 3, false>(p, alo, blo, d0, mw);
+                        else issue_taps<ZT, NKS, NN, 3, true>(p, alo, blo, d0, mw);
+                        continue;
+                    }
+                    for (int tx = 0; tx < 3; tx++) {
+                        ok = mb_wait_ready(bar(B_WF + st), wpar, abort_flag, p.err, 9);
                         if (!__all_sync(0xffffffffu, ok)) { stop = true; break; }
                         tc_fence_after();
-                        w0 = sW + (unsigned)st * wtap;
-                    }
-                    unsigned blo = sdesc_lo(w0, nbytes16);
-                    for (int ks = 0; ks < (p.K >> 4); ks++, alo += pl4, blo += nb4) {
-                        const unsigned long long bd = dpair(blo, bhi);
-                        const unsigned acc = (tap | ks) != 0;
-#pragma unroll
-                        for (int zz = 0; zz < Zt; zz++)
-                            tc_mma_elect(d0 + (unsigned)(zz * p.N), dpair(alo + (unsigned)zz * zs4, ahi), bd, p.idesc, acc);
-                    }
-                    if (p.wstages) {
+                        const unsigned at = alo + (unsigned)tx * (ROW_BYTES >> 4);
+                        const unsigned blo = sdesc_lo(sW + (unsigned)st * wtap, nbytes16);
+                        if (row + tx) issue_taps<ZT, NKS, NN, 1, false>(p, at, blo, d0, mw);
+                        else issue_taps<ZT, NKS, NN, 1, true>(p, at, blo, d0, mw);
                         tc_commit_elect(bar(B_WE + st));  // the stage is free once these MMAs complete
-                        wg++;
+                        if (++st == p.wstages) { st = 0; wpar ^= 1u; }
                     }
+                    if (stop) break;
                 }
                 if (stop) break;
                 tc_commit_elect(bar(B_HE + b));
-                tc_commit_elect(bar(B_AF + b));
+                tc_commit_elect(bar(B_AF + ab));
+                if (++b == p.nbuf) { b = 0; hpar ^= 1u; }
+                if (++ab == p.nacc) { ab = 0; apar ^= 1u; }
             }
         }
-        // drain: all MMAs issued by this warp's elected lane are complete
-        tc_commit_elect(bar(B_DR));
-        mb_wait(bar(B_DR), 0, abort_flag, p.err, 6, false);
+        // drain: all MMAs issued by the MMA warps' elected lanes are complete
+        if (mw < nmma) {
+            tc_commit_elect(bar(B_DR));
+            mb_wait(bar(B_DR), 0, abort_flag, p.err, 6, false);
+        }
         __syncwarp();
     } else {
         // ------------------------------------------------------------ epilogue
-        const int r = 32 * warp + lane;  // TMEM lane = row of the M = 128 block
-        const unsigned lane_addr = (unsigned)(32 * warp) << 16;
+        // The accumulators' columns are plane-major; each of the two warps of a
+        // lane quarter reads every other CH of them.  Bias, ReLU, conversion
+        // and stores are one warp's serial instructions: with one warp per
+        // quarter the 16-channel layers waited for them (4500 of a tile's 5500
+        // cycles).  A buffer is handed back before its last columns are stored.
+        constexpr int COLS = ZT * NN, CH = COLS >= 64 ? 32 : 16;
+        static_assert(COLS % CH == 0, "columns are read in whole chunks");
+        const int N = NN ? NN : p.N;
+        const int r = 32 * (warp & 3) + lane;  // TMEM lane = row of the M = 128 block
+        const unsigned lane_addr = (unsigned)(32 * (warp & 3)) << 16;
         const long long Vs = (long long)p.D * p.H * p.W;
+        const int HW = p.H * p.W;
         int i = 0;
         for (long long t = blockIdx.x; t < p.ntiles; t += gridDim.x, i++) {
-            const int b = i % p.nbuf;
-            const unsigned k = (unsigned)(i / p.nbuf);
+            const int b = i % p.nacc;
+            const unsigned k = (unsigned)(i / p.nacc);
             int ok = mb_wait(bar(B_AF + b), k & 1u, abort_flag, p.err, 7);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
@@ -467,19 +544,35 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             int bb, z0, y0, x0;
             decode_tile(p, Zt, t, bb, z0, y0, x0);
             const int x = x0 + (r & 7), y = y0 + (r >> 3);
-            for (int zz = 0; zz < Zt; zz++) {
-                const int z = z0 + zz;
-                const bool valid = x < p.W && y < p.H && z < p.D;
-                const long long sv = ((long long)z * p.H + y) * p.W + x;
-                for (int c0 = 0; c0 < p.N; c0 += 16) {
+            const bool inxy = x < p.W && y < p.H;
+            const long long sv0 = ((long long)z0 * p.H + y) * p.W + x;
+            const int cols = Zt * N;
+            if ((warp >> 2) * CH >= cols) {
+                tc_fence_before();
+                mb_arrive(bar(B_AE + b));
+            }
+#pragma unroll 1
+            for (int c = (warp >> 2) * CH; c < cols; c += 2 * CH) {
+                unsigned u[CH];
+                __syncwarp();
+                tc_ld<CH>(tmem + lane_addr + (unsigned)b * p.acc_cols + (unsigned)c, u);
+                if (c + 2 * CH >= cols) {
+                    tc_fence_before();
+                    mb_arrive(bar(B_AE + b));
+                }
+#pragma unroll
+                for (int g = 0; g < CH; g += 16) {
+                    const int zz = (c + g) / N, c0 = (c + g) % N;
+                    if (!inxy || z0 + zz >= p.D) continue;
                     float f[16];
-                    __syncwarp();
-                    tc_ld16(tmem + lane_addr + (unsigned)b * p.acc_cols + (unsigned)((zz + (dzn ? 2 : 0)) * p.N + c0),
-                            f);
-                    if (!valid) continue;
+#pragma unroll
+                    for (int q = 0; q < 16; q++) f[q] = __uint_as_float(u[g + q]);
                     if (p.bias) {
 #pragma unroll
-                        for (int q = 0; q < 16; q++) f[q] += __ldg(p.bias + c0 + q);
+                        for (int q = 0; q < 16; q += 4) {
+                            const float4 bq = *reinterpret_cast<const float4 *>(sbias + c0 + q);
+                            f[q] += bq.x; f[q + 1] += bq.y; f[q + 2] += bq.z; f[q + 3] += bq.w;
+                        }
                     }
                     if (p.relu) {
 #pragma unroll
@@ -494,24 +587,18 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     }
                     // two channel groups: two 16-byte pieces, Vs * 8 elements apart
                     const bool lo = c0 < p.O1;
-                    const int Cx = lo ? p.O1 : p.N - p.O1, cc = lo ? c0 : c0 - p.O1;
-                    bf16 *dst = (lo ? p.out1 : p.out2) + (((long long)bb * (Cx >> 3) + (cc >> 3)) * Vs + sv) * 8;
+                    const int Cx = lo ? p.O1 : N - p.O1, cc = lo ? c0 : c0 - p.O1;
+                    bf16 *dst = (lo ? p.out1 : p.out2) +
+                                (((long long)bb * (Cx >> 3) + (cc >> 3)) * Vs + sv0 + (long long)zz * HW) * 8;
                     *reinterpret_cast<uint4 *>(dst) = o[0];
                     *reinterpret_cast<uint4 *>(dst + Vs * 8) = o[1];
                 }
             }
-            if (dzn) {
-                __syncwarp();
-                for (unsigned c = 0; c < p.acc_cols; c += 16) tc_st16_zero(tmem + lane_addr + (unsigned)b * p.acc_cols + c);
-                tc_wait_st();
-            }
-            tc_fence_before();
-            mb_arrive(bar(B_AE + b));
         }
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 4) {
+    if (warp == TMA_WARP) {
         __syncwarp();
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(p.tmem_cols)
@@ -906,13 +993,13 @@ static bool dzn_fits(int N, int K, int zt, int nbuf, unsigned *smem, unsigned *c
                      unsigned *halo, unsigned *off_h)
 {
     const unsigned wbytes = 27u * (unsigned)N * (unsigned)K * 2u;
-    *plane = ((unsigned)(zt + 2) * ZSTRIDE + 127u) & ~127u;
+    *plane = plane_bytes(zt);
     *halo = (unsigned)(K / 8) * *plane;
     *off_h = (HDR + wbytes + 127u) & ~127u;
     *smem = ALIGN_SLACK + *off_h + (unsigned)nbuf * *halo;
-    const unsigned acc = (unsigned)((zt + 4) * N);
+    const unsigned acc = (unsigned)(zt * N);
     *cols = pow2_at_least((unsigned)nbuf * acc);
-    return *smem <= TC_SMEM_MAX && *cols <= 512;
+    return *smem <= TC_SMEM_MAX && zt * N <= 128;
 }
 
 bool conv3_tc_dzn(int N, int K)
@@ -936,6 +1023,7 @@ int conv3_tc_plans(int N, int K, int D, TcPlan *out, int cap)
             TcPlan &pl = out[np];
             pl.Zt = zt;
             pl.nbuf = nbuf;
+            pl.nacc = nbuf;
             pl.wstages = 0;
             pl.dzn = 1;
             pl.plane = plane;
@@ -959,16 +1047,18 @@ int conv3_tc_plans(int N, int K, int D, TcPlan *out, int cap)
         for (int nbuf = 2; nbuf >= 1; nbuf--) {
             for (int zt : zts) {
                 if (zt > 1 && zt > D) continue;
-                const unsigned plane = ((unsigned)(zt + 2) * ZSTRIDE + 127u) & ~127u;
+                const unsigned plane = plane_bytes(zt);
                 const unsigned halo = (unsigned)(K / 8) * plane;
                 const unsigned off_w = HDR;
                 const unsigned off_h = (off_w + wbytes + 127u) & ~127u;
                 const unsigned smem = ALIGN_SLACK + off_h + (unsigned)nbuf * halo;
-                const unsigned cols = pow2_at_least((unsigned)(nbuf * zt * N));
+                const int nacc = 2 * zt * N <= 512 ? 2 : 1;
+                const unsigned cols = pow2_at_least((unsigned)(nacc * zt * N));
                 if (smem > TC_SMEM_MAX || cols > 512) continue;
                 TcPlan &pl = out[np];
                 pl.Zt = zt;
                 pl.nbuf = nbuf;
+                pl.nacc = nacc;
                 pl.wstages = stages;
                 pl.dzn = 0;
                 pl.plane = plane;
@@ -992,24 +1082,60 @@ bool conv3_tc_plan(int N, int K, int D, TcPlan *pl)
 
 using TcKernel = void (*)(const CUtensorMap, const CUtensorMap, const TcArgs);
 
-// The instantiations: the hot tile shapes with compile-time loop bounds, and
+// The instantiations: the usual tile shapes with compile-time operands, and
 // one run-time variant per mode for the rest.
-const TcKernel TC_KERNELS[] = {k_conv3_tc<1, 8, 1>, k_conv3_tc<1, 4, 1>, k_conv3_tc<1, 4, 2>, k_conv3_tc<1, 0, 0>,
-                               k_conv3_tc<0, 4, 0>, k_conv3_tc<0, 2, 0>, k_conv3_tc<0, 1, 0>, k_conv3_tc<0, 0, 0>};
+struct TcVariant {
+    int dzn, zt, nks, n;
+    TcKernel k;
+};
+#define TC_V(dz, zt, nks, n) {dz, zt, nks, n, k_conv3_tc<dz, zt, nks, n>}
+#define TC_PLAIN(n) \
+    TC_V(0, 4, 2, n), TC_V(0, 2, 2, n), TC_V(0, 1, 2, n), TC_V(0, 4, 4, n), TC_V(0, 2, 4, n), TC_V(0, 1, 4, n)
+const TcVariant TC_VARIANTS[] = {TC_V(1, 8, 1, 16), TC_V(1, 4, 1, 16), TC_V(1, 4, 2, 16), TC_V(1, 4, 1, 32),
+                                 TC_V(1, 4, 2, 32), TC_PLAIN(32),      TC_PLAIN(64),      TC_PLAIN(128),
+                                 TC_V(1, 0, 0, 0),  TC_V(0, 0, 0, 0)};
+#undef TC_PLAIN
+#undef TC_V
 
-TcKernel pick_kernel(const TcPlan &pl, int K)
+TcKernel pick_kernel(const TcPlan &pl, int N, int K)
 {
-    const int nks = K >> 4;
-    if (pl.dzn) {
-        if (pl.Zt == 8 && nks == 1) return TC_KERNELS[0];
-        if (pl.Zt == 4 && nks == 1) return TC_KERNELS[1];
-        if (pl.Zt == 4 && nks == 2) return TC_KERNELS[2];
-        return TC_KERNELS[3];
+    const int nks = K >> 4, block = pl.dzn ? nks : (nks % 4 == 0 ? 4 : (nks % 2 == 0 ? 2 : 1));
+    for (const TcVariant &v : TC_VARIANTS)
+        if (v.dzn == pl.dzn && (!v.n || (v.zt == pl.Zt && v.nks == block && v.n == N))) return v.k;
+    return nullptr;
+}
+
+// CTAs of a plan that fit on an SM, by shared memory and by TMEM.
+static int ctas_by_smem(const TcPlan &pl) { return (int)(TC_SMEM_SM / (pl.smem + 1024u)); }
+static int ctas_by_tmem(const TcPlan &pl) { return (int)(512u / pl.tmem_cols); }
+
+// The rule's choice among the plain plans, by an estimate of the time of the SM
+// with the most tiles in units of one z-plane's MMAs: every tile costs its
+// planes plus what its start and end leave the tensor core idle, least with two
+// CTAs on the SM (0.45), more with one and two halo buffers (0.6), most with one
+// halo buffer (1.1), and 0.15 for streamed weights.  Measured (tile depth,
+// buffers, weights): 64 -> 32 channels on 32 x 32^3 voxels 212 us with 2, 1,
+// resident, 180 with 2, 1, streamed (two CTAs on an SM); 128 -> 64 on 32 x 16^3
+// 85 with 1, 1, streamed, 71 with 2, 1, streamed, but on one 16^3 region 16
+// against 22.  The dz-in-N plans keep their order: their depth decides the order
+// of the sums.
+static int choose_plan(const TcPlan *pl, int np, const TcConv &c)
+{
+    int best = 0;
+    double least = 1e300;
+    for (int k = 0; k < np; k++) {
+        if (pl[k].dzn) return 0;
+        const long long t = (long long)((c.W + 7) / 8) * ((c.H + 15) / 16) * ((c.D + pl[k].Zt - 1) / pl[k].Zt) * c.B;
+        const int per_sm = std::max(1, std::min(2, std::min(ctas_by_smem(pl[k]), ctas_by_tmem(pl[k]))));
+        const long long slots = (long long)device_sms() * per_sm;
+        const double idle = per_sm > 1 ? 0.45 : (pl[k].nbuf > 1 ? 0.6 : 1.1);
+        const double est = (double)(per_sm * ((t + slots - 1) / slots)) * (pl[k].Zt + idle + (pl[k].wstages ? 0.15 : 0.0));
+        if (est < least * 0.999) {
+            least = est;
+            best = k;
+        }
     }
-    if (pl.Zt == 4) return TC_KERNELS[4];
-    if (pl.Zt == 2) return TC_KERNELS[5];
-    if (pl.Zt == 1) return TC_KERNELS[6];
-    return TC_KERNELS[7];
+    return best;
 }
 
 int conv3_tc(const TcConv &c, int *err, cudaStream_t s)
@@ -1018,7 +1144,7 @@ int conv3_tc(const TcConv &c, int *err, cudaStream_t s)
     TcPlan plans[TC_MAX_PLANS];
     const int np = conv3_tc_plans(N, K, c.D, plans, TC_MAX_PLANS);
     if ((c.C1 % 8) || (c.C2 % 8) || (c.O1 % 16) || c.O1 > N || np < 1) return 0;
-    const TcPlan pl = plans[c.plan >= 0 && c.plan < np ? c.plan : 0];
+    const TcPlan pl = plans[c.plan >= 0 && c.plan < np ? c.plan : choose_plan(plans, np, c)];
     if ((reinterpret_cast<uintptr_t>(c.w) & 15) || (reinterpret_cast<uintptr_t>(c.in1) & 15) ||
         (c.C2 && (reinterpret_cast<uintptr_t>(c.in2) & 15)))
         return 0;
@@ -1034,8 +1160,8 @@ int conv3_tc(const TcConv &c, int *err, cudaStream_t s)
     static std::once_flag once;
     static cudaError_t attr_err = cudaSuccess;
     std::call_once(once, []() {
-        for (TcKernel k : TC_KERNELS) {
-            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM_MAX);
+        for (const TcVariant &v : TC_VARIANTS) {
+            cudaError_t e = cudaFuncSetAttribute(v.k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM_MAX);
             if (e != cudaSuccess) attr_err = e;
         }
     });
@@ -1053,9 +1179,10 @@ int conv3_tc(const TcConv &c, int *err, cudaStream_t s)
     a.B = c.B; a.D = c.D; a.H = c.H; a.W = c.W;
     a.Zt = pl.Zt;
     a.nbuf = pl.nbuf;
+    a.nacc = pl.nacc;
     a.wstages = pl.wstages;
     a.dzn = pl.dzn;
-    a.acc_cols = (unsigned)((pl.dzn ? pl.Zt + 4 : pl.Zt) * N);
+    a.acc_cols = (unsigned)(pl.Zt * N);
     a.tx = (c.W + 7) / 8;
     a.ty = (c.H + 15) / 16;
     a.tz = (c.D + pl.Zt - 1) / pl.Zt;
@@ -1067,20 +1194,19 @@ int conv3_tc(const TcConv &c, int *err, cudaStream_t s)
     a.off_h = pl.off_h;
     a.tx_bytes = (unsigned)(K / 8) * (unsigned)zh * ZSTRIDE + c.tx_extra;
     a.tmem_cols = pl.tmem_cols;
-    // kind::f16 instruction descriptor: FP32 accumulator (bit 4), BF16 A
-    // (bits 7-9 = 1) and B (bits 10-12 = 1), both K-major, N >> 3 at bit 17,
-    // M >> 4 at bit 24 (M = 128).
-    const int nmma = pl.dzn ? 3 * N : N;
-    a.idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((unsigned)(nmma >> 3) << 17) | ((128u >> 4) << 24);
     a.err = err;
-    const int per_sm_smem = (int)(TC_SMEM_SM / (pl.smem + 1024u));
-    const int per_sm_tmem = (int)(512u / pl.tmem_cols);
+    const int per_sm_smem = ctas_by_smem(pl), per_sm_tmem = ctas_by_tmem(pl);
     int per_sm = per_sm_smem < per_sm_tmem ? per_sm_smem : per_sm_tmem;
     if (per_sm < 1) per_sm = 1;
+    // never more CTAs on an SM than their TMEM allocations fit
+    unsigned smem = pl.smem;
+    if (per_sm_smem > per_sm_tmem && smem < TC_SMEM_SM / (unsigned)per_sm_tmem - 1024u)
+        smem = TC_SMEM_SM / (unsigned)per_sm_tmem - 1024u;
+    if (smem > TC_SMEM_MAX) smem = TC_SMEM_MAX;
     long long grid = (long long)device_sms() * per_sm;
     if (grid > a.ntiles) grid = a.ntiles;
     if (grid < 1) return 1;
-    counted(pick_kernel(pl, K))<<<(unsigned)grid, TC_THREADS, pl.smem, s>>>(m1, m2, a);
+    counted(pick_kernel(pl, N, K))<<<(unsigned)grid, TC_THREADS, smem, s>>>(m1, m2, a);
     return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
 

@@ -251,6 +251,27 @@ def test_unet_weight_gradients_two_kernels(G, grid, B):
     assert np.linalg.norm(out[0] - out[1]) < 5e-2 * np.linalg.norm(out[1])
 
 
+# the tensor-core forward with partial tiles in x, y and z, one to three levels of
+# each width, and batches on both sides of the plan rule's and of the head's
+# lines: every plan sums in one order, so a region's output has the same bits
+# alone and in a batch; against the mma.sync kernel a sum in another order moves
+# a BF16 activation by at most one place (2^-8 of it), so a tenth of the rms is
+# far above what a few layers make of it and far below a wrong tap or plane
+@pytest.mark.parametrize("grid,base,levels,B", [(64, 16, 4, 4), (40, 32, 3, 5), (24, 32, 4, 3), (20, 16, 3, 2)])
+def test_unet_forward_plans(G, grid, base, levels, B):
+    from paper_2510_23330_gb300 import surrogate
+    rng = np.random.default_rng(grid + base)
+    net = G.UNet(5, 5, base, levels, grid)
+    net.set_params(surrogate.he_init(5, 5, base, levels, seed=2))
+    x = rng.normal(size=(B, grid, grid, grid, 5)).astype(np.float32)
+    y = net.forward(x)
+    for b in range(B):
+        assert np.array_equal(net.forward(x[b : b + 1])[0], y[b])
+    net.set_conv_impl(G.GNB_CONV_MMA_SYNC)
+    ref = net.forward(x[:1])[0].astype(np.float64)
+    assert np.max(np.abs(y[0] - ref)) < 0.1 * np.sqrt(np.mean(ref**2))
+
+
 # remap: lines with empty voxels (weight 0), weights over many decades and grids
 # of each search form, against the oracle's voxel choices
 @pytest.mark.parametrize("grid", [32, 64, 24])
