@@ -114,13 +114,20 @@ __device__ __forceinline__ long long ig_dst(const IgArgs &p, long long r, int t)
 }
 
 #define IG_M 64
-// NB = number of 8-column blocks per CTA (N tile = 8 NB)
+#define IG_ST 4  // staged K steps
+#define IG_CTAS 152  // CTAs below which a launch takes fewer output channels per CTA
+// NB = number of 8-column blocks per CTA (N tile = 8 NB).  What bounds it is the
+// latency of a K step (few CTAs at the coarse levels, 8 at 8^3): four steps are
+// in flight, and a thread decodes its row once and steps tap and channel by
+// counters (with 64-bit divisions in every step and two steps in flight the
+// input gradient of the 128 -> 64 channel up-sampling of one 8^3 grid took 52 us,
+// now 13).
 template <int NB>
 __global__ void __launch_bounds__(128) k_igemm(IgArgs p)
 {
     constexpr int NT = 8 * NB;
-    __shared__ __align__(16) bf16 sA[2][IG_M][16];
-    __shared__ __align__(16) bf16 sB[2][NT][16];
+    __shared__ __align__(16) bf16 sA[IG_ST][IG_M][16];
+    __shared__ __align__(16) bf16 sB[IG_ST][NT][16];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gid = lane >> 2, tig = lane & 3;
     const long long M = (long long)p.B * p.D * p.H * p.W;
     const long long row0 = (long long)blockIdx.x * IG_M;
@@ -137,41 +144,56 @@ __global__ void __launch_bounds__(128) k_igemm(IgArgs p)
 #pragma unroll
     for (int j = 0; j < NB; j++) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
 
-    auto stage = [&](int s, int buf) {
-        int t = s / kch, c0 = (s % kch) * 16;
-        int wt = p.mode == IG_UP2 ? tapz : t;
+    // the row this thread stages, and the next step to stage
+    const int sr = tid >> 1, half = tid & 1;
+    const bool row_in = row0 + sr < M;
+    const long long gr0 = row_in ? row0 + sr : 0, b0 = gr0 / Vrow;
+    const int sv0 = (int)(gr0 - b0 * Vrow);
+    const int x = sv0 % p.W, y = sv0 / p.W % p.H, z = sv0 / p.W / p.H;
+    int st_t = 0, st_c = 0, slot = 0;
+    long long src_v = -1;  // source voxel within the batch entry (-1: zero padding)
+    auto tap_voxel = [&](int t) -> long long {
+        if (!row_in) return -1;
+        if (p.mode == IG_CONV3) {
+            const int zz = z + c_taps[t][0], yy = y + c_taps[t][1], xx = x + c_taps[t][2];
+            if (zz < 0 || zz >= p.D || yy < 0 || yy >= p.H || xx < 0 || xx >= p.W) return -1;
+            return ((long long)zz * p.H + yy) * p.W + xx;
+        }
+        if (p.mode == IG_DOWN2)  // gather from the grid twice as fine
+            return ((long long)(2 * z + ((t >> 2) & 1)) * 2 * p.H + (2 * y + ((t >> 1) & 1))) * 2 * p.W + (2 * x + (t & 1));
+        return sv0;  // IG_CONV1, IG_UP2: the row's own voxel
+    };
+    auto stage = [&]() {
+        if (st_c == 0) src_v = tap_voxel(st_t);
         {   // A: 64 rows x 16 channels, one 16-byte piece per thread
-            int r = tid >> 1, half = tid & 1;
-            long long gr = row0 + r;
-            long long v = gr < M ? ig_src(p, gr, t) : -1;
-            int c = c0 + 8 * half;
+            const int c = st_c + 8 * half;
             const bf16 *src = p.in1;
-            int bytes = 0;
-            if (v >= 0) {
-                src = c < p.C1 ? p.in1 + blk(v, c, p.C1, VsA) : p.in2 + blk(v, c - p.C1, p.C2, VsA);
-                bytes = 16;
-            }
-            cp_async16(&sA[buf][r][8 * half], src, bytes);
+            if (src_v >= 0)
+                src = c < p.C1 ? p.in1 + ((b0 * (p.C1 >> 3) + (c >> 3)) * VsA + src_v) * 8
+                               : p.in2 + ((b0 * (p.C2 >> 3) + ((c - p.C1) >> 3)) * VsA + src_v) * 8;
+            cp_async16(&sA[slot][sr][8 * half], src, src_v >= 0 ? 16 : 0);
         }
+        const int wt = p.mode == IG_UP2 ? tapz : st_t;
         for (int q = tid; q < NT * 2; q += 128) {  // B: NT rows x 16 k
-            int n = q >> 1, half = q & 1;
-            bool in = (n0 + n) < p.Npad;
-            const bf16 *src = in ? p.w + ((long long)wt * p.Npad + n0 + n) * K + c0 + 8 * half : p.w;
-            cp_async16(&sB[buf][n][8 * half], src, in ? 16 : 0);
+            const int n = q >> 1;
+            const bool in = (n0 + n) < p.Npad;
+            const bf16 *src = in ? p.w + ((long long)wt * p.Npad + n0 + n) * K + st_c + 8 * half : p.w;
+            cp_async16(&sB[slot][n][8 * half], src, in ? 16 : 0);
         }
-        cp_async_commit();
+        if ((st_c += 16) >= 16 * kch) { st_c = 0; st_t++; }
+        slot = slot + 1 == IG_ST ? 0 : slot + 1;
     };
 
-    stage(0, 0);
+    for (int s = 0; s < IG_ST - 1; s++) {
+        if (s < nsteps) stage();
+        cp_async_commit();
+    }
     for (int s = 0; s < nsteps; s++) {
-        const int buf = s & 1;
-        if (s + 1 < nsteps) {
-            stage(s + 1, buf ^ 1);
-            cp_async_wait<1>();
-        } else {
-            cp_async_wait<0>();
-        }
-        __syncthreads();
+        const int buf = s % IG_ST;
+        cp_async_wait<IG_ST - 2>();
+        __syncthreads();  // step s has landed, and every warp is done with the slot staged next
+        if (s + IG_ST - 1 < nsteps) stage();
+        cp_async_commit();
         unsigned a[4];
         const int ra = 16 * warp + gid;
         a[0] = *reinterpret_cast<const unsigned *>(&sA[buf][ra][2 * tig]);
@@ -185,7 +207,6 @@ __global__ void __launch_bounds__(128) k_igemm(IgArgs p)
             b[1] = *reinterpret_cast<const unsigned *>(&sB[buf][8 * j + gid][2 * tig + 8]);
             mma_bf16(acc[j], a, b);
         }
-        __syncthreads();
     }
     // epilogue: bias, ReLU, BF16 (or FP32) store
 #pragma unroll
@@ -821,13 +842,20 @@ void launch_ig_nb(const IgArgs &a, int ntiles_n, int gz, cudaStream_t s)
 
 void launch_ig(const IgArgs &a, cudaStream_t s)
 {
-    int gz = a.mode == IG_UP2 ? 8 : 1;
-    int Np = a.Npad;
-    if (Np <= 8) launch_ig_nb<1>(a, 1, gz, s);
-    else if (Np <= 16) launch_ig_nb<2>(a, 1, gz, s);
-    else if (Np <= 32) launch_ig_nb<4>(a, 1, gz, s);
-    else if (Np <= 64) launch_ig_nb<8>(a, 1, gz, s);
-    else launch_ig_nb<16>(a, (Np + 127) / 128, gz, s);
+    // 8 NB output channels a CTA: all of them (at most 128), but while that
+    // leaves most of the chip idle narrower ones, down to 16 (a training step of
+    // one 64^3 region 1386 -> 1350 us, of two 32^3 regions 959 -> 924).
+    const int gz = a.mode == IG_UP2 ? 8 : 1;
+    const long long mt = ((long long)a.B * a.D * a.H * a.W + IG_M - 1) / IG_M * gz;
+    int nb = 1;
+    while (nb < 16 && 8 * nb < a.Npad) nb *= 2;
+    while (nb > 2 && mt * ((a.Npad + 8 * nb - 1) / (8 * nb)) < IG_CTAS) nb /= 2;
+    const int nt = (a.Npad + 8 * nb - 1) / (8 * nb);
+    if (nb == 1) launch_ig_nb<1>(a, nt, gz, s);
+    else if (nb == 2) launch_ig_nb<2>(a, nt, gz, s);
+    else if (nb == 4) launch_ig_nb<4>(a, nt, gz, s);
+    else if (nb == 8) launch_ig_nb<8>(a, nt, gz, s);
+    else launch_ig_nb<16>(a, nt, gz, s);
 }
 
 template <int NB>
