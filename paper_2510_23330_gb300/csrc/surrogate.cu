@@ -445,8 +445,10 @@ __global__ void k_remap(PArr p, PArr q, const int *__restrict__ src_orig, const 
             // comparisons run on FP32 images: t32 approximates target from
             // the 32 leading bits of U's 53-bit integer m and the FP32 total
             // within a relative 2^-21 (truncation 2^-31, three roundings
-            // 2^-24 each, FP64 rounding of target 2^-53; the total and t32
-            // kept in FP32's normal range, m >= 2^32), and the FP32 sums are within 2^-24
+            // 2^-24 each, FP64 rounding of target 2^-53; every factor and
+            // product in FP32's normal range: U's image is scaled to
+            // [2^-21, 1) by itself, exactly, and the total, from 2^-90 on,
+            // multiplies it last), and the FP32 sums are within 2^-24
             // of the FP64 ones, so a sum outside t32 (1 -+ 2^-20) orders
             // against target as its image does; if one lies inside that band
             // (or m < 2^32) the FP64 sums decide (line_search: rare enough,
@@ -473,7 +475,8 @@ __global__ void k_remap(PArr p, PArr q, const int *__restrict__ src_orig, const 
                 const unsigned M = (unsigned)((m << s) >> 21);
                 const float mh = __int_as_float(0x4B000000 | (int)(M >> 16)) - 8388608.f;
                 const float ml = __int_as_float(0x4B000000 | (int)(M & 0xFFFFu)) - 8388608.f;
-                const float t32 = __fmul_rn(__fmaf_rn(mh, 65536.f, ml), tot32 * __int_as_float((127 - 32 - s) << 23));
+                const float u32 = __fmul_rn(__fmaf_rn(mh, 65536.f, ml), __int_as_float((127 - 32 - s) << 23));
+                const float t32 = __fmul_rn(u32, tot32);
                 lo32 = __fmul_rn(t32, 1.f - 0x1p-20f);
                 hi32 = __fmul_rn(t32, 1.f + 0x1p-20f);
             };

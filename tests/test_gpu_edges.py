@@ -293,3 +293,46 @@ def test_remap_extreme_weights(G, orc, grid):
     _, rp, _, _ = S.remap(pred[0].reshape(-1, 5).astype(np.float64), p["id"], pos, cen, side, grid, seed=77, sweeps=sweeps)
     got = np.stack([c.get(k) for k in "XYZ"], axis=1)
     assert np.max(np.abs(got - rp)) < 1e-12 * side
+
+
+def _splitmix64(x):
+    x = x + np.uint64(0x9E3779B97F4A7C15)
+    x = (x ^ (x >> np.uint64(30))) * np.uint64(0xBF58476D1CE4E5B9)
+    x = (x ^ (x >> np.uint64(27))) * np.uint64(0x94D049BB133111EB)
+    return x ^ (x >> np.uint64(31))
+
+
+# remap: draws below 2^-16 on lines whose weights add up to about 2^-89.5, just
+# inside the range decided in FP32, and whose first weight is the draw's share of
+# the total but for 1e-4: U times the total is a normal FP32 number only if no
+# factor on the way is smaller than either
+@pytest.mark.parametrize("grid", [64, 24])
+def test_remap_small_draws_on_small_totals(G, orc, grid):
+    from oracle import surrogate as S
+    seed, n, side = 5, 200, 60.0
+    rng = np.random.default_rng(grid)
+    ids = np.arange(1 << 24, dtype=np.uint64)
+    m = _splitmix64(_splitmix64(ids + np.uint64(seed))) >> np.uint64(11)  # 53-bit draw 0 of each ID
+    ids = ids[m < (1 << 37)][:n].astype(np.int64)
+    U = np.array([S.uniform(seed, int(i), 0) for i in ids])
+    assert ids.size == n and np.all(U < 2.0**-16)
+    line = rng.permutation(grid * grid)[:n]  # (z, y) of the particle's x line
+    T = 2.0**-90 * rng.uniform(1.05, 2.0, n)
+    w = np.full((grid * grid, grid), 2.0**-89.5 / (grid - 1))
+    w[line, 1:] = (T / (grid - 1))[:, None]
+    w[line, 0] = U * T * (1.0 + rng.choice([-1e-4, 1e-4], n))
+    pred = np.zeros((1, grid, grid, grid, 5), np.float32)
+    pred[..., 0] = np.log10(w).reshape(1, grid, grid, grid) + 0.33
+    p = ics.sn_region(n, seed=1, grid=16)
+    p["id"] = ids
+    d = side / grid
+    pos = np.stack([np.full(n, 5), line % grid, line // grid], axis=1) * d + 0.5 * d - 0.5 * side
+    for a, k in enumerate("xyz"):
+        p[k] = np.ascontiguousarray(pos[:, a])
+    c = G.Context()
+    c.set_particles(p)
+    c.remap_regions([(0.0, 0.0, 0.0)], pred, side=side, seed=seed, sweeps=1)
+    _, rp, _, _ = S.remap(pred[0].reshape(-1, 5).astype(np.float64), ids, pos, (0.0, 0.0, 0.0), side, grid, seed=seed,
+                          sweeps=1)
+    got = np.stack([c.get(k) for k in "XYZ"], axis=1)
+    assert np.max(np.abs(got - rp)) < 1e-12 * side
