@@ -21,6 +21,13 @@ extern "C" {
  * seconds.  Errors: GNB_EINVAL (NULL, or the mma.sync path selected). */
 int gnb_unet_test_wait_timeout(gnb_unet *net);
 
+/* Out of device memory: after `after` further device allocations of the
+ * context the next one fails, once, as cudaMalloc does without memory left
+ * (the call that made it returns GNB_ENOMEM); -1 puts this off.  Returns what
+ * was left of the former count (-1: no failure was due, or it has happened;
+ * -2: NULL context). */
+int64_t gnb_test_fail_alloc(gnb_ctx *ctx, int64_t after);
+
 #ifdef __cplusplus
 }
 #endif

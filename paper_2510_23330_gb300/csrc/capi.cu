@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "../../include/galnb_testing.h"
 
 namespace gnb {
 
@@ -1073,6 +1074,14 @@ int gnb_diagnostics(gnb_ctx *c, double out[10])
     c->err.clear();
     if (!c->gravity_valid) return fail(c, GNB_ESTATE, "forces not computed");
     return finish(c, diagnostics(c, out));
+}
+
+int64_t gnb_test_fail_alloc(gnb_ctx *c, int64_t after)
+{
+    if (!c) return -2;
+    const int64_t left = c->alloc_left;
+    c->alloc_left = after < 0 ? -1 : after;
+    return left;
 }
 
 int gnb_stats(gnb_ctx *c, int64_t out[GNB_S_COUNT_])

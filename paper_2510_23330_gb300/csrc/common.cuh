@@ -214,6 +214,7 @@ struct gnb_ctx {
     float4 *gd_part = nullptr;                 // direct gravity: sums of the source parts [parts][n]
     int64_t gd_cap = 0;
     int *pinned_i = nullptr;                   // pinned host scratch [64]
+    int64_t alloc_left = -1;                   // device allocations before one fails (tests; -1: none does)
     // hierarchical timesteps (integrate.cu): per particle slot, permuted with
     // the particles by every sort while hier_on; [2] = current and scratch
     bool hier_on = false, hier_valid = false;
@@ -262,13 +263,24 @@ int fail(gnb_ctx *c, int code, const std::string &msg);
 int cuda_check(gnb_ctx *c, cudaError_t e, const char *what);
 void dfree(gnb_ctx *c, void *p);
 
+// Frees arrays that are about to be replaced.  Their pointers become null and
+// the caller sets their capacity to 0, so that a failed allocation leaves
+// neither a dangling pointer nor a capacity that nothing stands behind.
+template <class... T>
+inline void drop(gnb_ctx *c, T *&...p)
+{
+    ((dfree(c, p), p = nullptr), ...);
+}
+
 // Device allocation of count elements; GNB_ENOMEM on failure.
 template <class T>
 inline int dalloc(gnb_ctx *c, T **p, size_t count)
 {
     *p = nullptr;
     if (count == 0) count = 1;
-    cudaError_t e = cudaMalloc((void **)p, count * sizeof(T));
+    const bool refuse = c->alloc_left == 0;  // (set by tests)
+    if (c->alloc_left >= 0) c->alloc_left--;
+    cudaError_t e = refuse ? cudaErrorMemoryAllocation : cudaMalloc((void **)p, count * sizeof(T));
     if (e != cudaSuccess) {
         cudaGetLastError();
         *p = nullptr;

@@ -1050,8 +1050,8 @@ static int lists_alloc(gnb_ctx *c, int chunks)
 {
     const int ng = std::max(c->t.nnodes, 1);
     if (c->gl_gcap < ng) {
-        dfree(c, c->gl_head); dfree(c, c->gl_ref);
-        c->gl_head = nullptr; c->gl_ref = nullptr;
+        drop(c, c->gl_head, c->gl_ref);
+        c->gl_gcap = 0;
         const int cap = ng + ng / 4 + 64;
         GNB_TRY(dalloc(c, &c->gl_head, (size_t)cap));
         GNB_TRY(dalloc(c, &c->gl_ref, (size_t)cap));
@@ -1062,8 +1062,8 @@ static int lists_alloc(gnb_ctx *c, int chunks)
         // count, which drifts from step to step, and a reallocation (cudaFree
         // synchronises the device) must not recur every step
         chunks = std::max(chunks + chunks / 4, c->gl_cap + c->gl_cap / 2);
-        dfree(c, c->gl_pool); dfree(c, c->gl_next); dfree(c, c->gl_cnt); dfree(c, c->gl_lcum);
-        c->gl_pool = nullptr; c->gl_next = nullptr; c->gl_cnt = nullptr; c->gl_lcum = nullptr;
+        drop(c, c->gl_pool, c->gl_next, c->gl_cnt, c->gl_lcum);
+        c->gl_cap = 0;
         GNB_TRY(dalloc(c, &c->gl_pool, (size_t)chunks * GL_CH));
         GNB_TRY(dalloc(c, &c->gl_lcum, (size_t)chunks * GL_CH));
         GNB_TRY(dalloc(c, &c->gl_next, (size_t)chunks));

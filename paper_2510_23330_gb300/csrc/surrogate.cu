@@ -553,8 +553,8 @@ int voxelise_buffers_for(gnb_ctx *c, int nreg, int grid)
     size_t nv = (size_t)nreg * grid * grid * grid;
     if (c->sur_pcap < c->cap) {
         c->sur_gen++;
-        dfree(c, c->sreg); dfree(c, c->vpa); dfree(c, c->vpb); dfree(c, c->vpc); dfree(c, c->vbox);
-        c->sreg = nullptr; c->vpa = nullptr; c->vpb = nullptr; c->vpc = nullptr; c->vbox = nullptr;
+        drop(c, c->sreg, c->vpa, c->vpb, c->vpc, c->vbox);
+        c->sur_pcap = 0;
         GNB_TRY(dalloc(c, &c->sreg, (size_t)c->cap + 1));
         GNB_TRY(dalloc(c, &c->vpa, (size_t)c->cap + 1));
         GNB_TRY(dalloc(c, &c->vpb, (size_t)c->cap + 1));
@@ -564,12 +564,9 @@ int voxelise_buffers_for(gnb_ctx *c, int nreg, int grid)
     }
     if (c->sur_nv < nv || c->sur_nreg < nreg) {
         c->sur_gen++;
-        dfree(c, c->vacc); dfree(c, c->vw); dfree(c, c->vcdf32); dfree(c, c->vcdfc);
-        dfree(c, c->cent_d);
-        dfree(c, c->vout); dfree(c, c->rsx); dfree(c, c->rsi); dfree(c, c->centf);
-        c->vacc = nullptr; c->vw = nullptr; c->vcdf32 = nullptr; c->vcdfc = nullptr;
-        c->cent_d = nullptr;
-        c->vout = nullptr; c->rsx = nullptr; c->rsi = nullptr; c->centf = nullptr;
+        drop(c, c->vacc, c->vw, c->vcdf32, c->vcdfc, c->cent_d, c->vout, c->rsx, c->rsi, c->centf);
+        c->sur_nv = 0;
+        c->sur_nreg = 0;
         GNB_TRY(dalloc(c, &c->vacc, nv * 8));
         GNB_TRY(dalloc(c, &c->vw, nv));
         GNB_TRY(dalloc(c, &c->vcdf32, nv * 3));
@@ -768,9 +765,9 @@ static int sna_buffers(gnb_ctx *c)
         GNB_TRY(cuda_check(c, cudaEventCreateWithFlags(&c->sna_ev_done, cudaEventDisableTiming), "event"));
     if (!c->sna_seed) GNB_TRY(dalloc(c, &c->sna_seed, 1));
     if (c->sna_cap >= c->cap) return GNB_OK;
-    void *old[] = {c->sna_x, c->sna_y, c->sna_z, c->sna_h2, c->sna_m, c->sna_u, c->sna_vx, c->sna_vy, c->sna_vz,
-                   c->sna_rho, c->sna_reg, c->sna_orig, c->sna_pos, c->sna_inv, c->sna_id};
-    for (void *q : old) dfree(c, q);
+    drop(c, c->sna_x, c->sna_y, c->sna_z, c->sna_h2, c->sna_m, c->sna_u, c->sna_vx, c->sna_vy, c->sna_vz, c->sna_rho,
+         c->sna_reg, c->sna_orig, c->sna_pos, c->sna_inv, c->sna_id);
+    c->sna_cap = 0;
     const size_t m = (size_t)c->cap + 1;
     GNB_TRY(dalloc(c, &c->sna_x, m)); GNB_TRY(dalloc(c, &c->sna_y, m)); GNB_TRY(dalloc(c, &c->sna_z, m));
     GNB_TRY(dalloc(c, &c->sna_h2, m)); GNB_TRY(dalloc(c, &c->sna_m, m)); GNB_TRY(dalloc(c, &c->sna_u, m));

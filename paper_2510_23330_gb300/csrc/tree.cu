@@ -716,32 +716,33 @@ __global__ void __cluster_dims__(MC_CTAS, 1, 1) __launch_bounds__(MC_THREADS)
 int tree_alloc(gnb_ctx *c, Tree &t, int cap)
 {
     // node arrays only; the per-slot scratch survives a regrow
-    dfree(c, t.na); dfree(c, t.nb); dfree(c, t.mo0); dfree(c, t.mo1); dfree(c, t.mo2); dfree(c, t.head);
-    t.cap = cap;
+    drop(c, t.na, t.nb, t.mo0, t.mo1, t.mo2, t.head);
+    t.cap = 0;
     GNB_TRY(dalloc(c, &t.na, cap));
     GNB_TRY(dalloc(c, &t.nb, cap));
     GNB_TRY(dalloc(c, &t.mo0, cap));
     GNB_TRY(dalloc(c, &t.mo1, cap));
     GNB_TRY(dalloc(c, &t.mo2, cap));
     GNB_TRY(dalloc(c, &t.head, cap));
+    t.cap = cap;
     return GNB_OK;
 }
 
 static int tree_scratch(gnb_ctx *c, Tree &t, int n, int ntiles)
 {
-    if (!t.lvl) {
-        GNB_TRY(dalloc(c, &t.lvl, GNB_MAXLEV + 4));
-        GNB_TRY(dalloc(c, &t.tot, TB_NCNT));
-        GNB_TRY(dalloc(c, &t.ngroups_d, 4));
-    }
+    if (!t.lvl) GNB_TRY(dalloc(c, &t.lvl, GNB_MAXLEV + 4));
+    if (!t.tot) GNB_TRY(dalloc(c, &t.tot, TB_NCNT));
+    if (!t.ngroups_d) GNB_TRY(dalloc(c, &t.ngroups_d, 4));
     if (n + 1 > t.scap) {
-        dfree(c, t.span); dfree(c, t.groups);
+        drop(c, t.span, t.groups);
+        t.scap = 0;
         GNB_TRY(dalloc(c, &t.span, (size_t)n + 1));
         GNB_TRY(dalloc(c, &t.groups, (size_t)n + 1));
         t.scap = n + 1;
     }
     if (ntiles * TB_NCNT > t.tcap) {
-        dfree(c, t.tcnt);
+        drop(c, t.tcnt);
+        t.tcap = 0;
         GNB_TRY(dalloc(c, &t.tcnt, (size_t)ntiles * TB_NCNT));
         t.tcap = ntiles * TB_NCNT;
     }

@@ -147,6 +147,8 @@ def _declare(L):
     L.gnb_unet_set_conv_impl.restype = C.c_int
     L.gnb_unet_test_wait_timeout.argtypes = [_vp]
     L.gnb_unet_test_wait_timeout.restype = C.c_int
+    L.gnb_test_fail_alloc.argtypes = [_vp, C.c_int64]
+    L.gnb_test_fail_alloc.restype = C.c_int64
     for name in ("gnb_save", "gnb_load", "gnb_unet_save", "gnb_unet_load"):
         getattr(L, name).argtypes = [_vp, C.c_char_p]
         getattr(L, name).restype = C.c_int
@@ -287,6 +289,10 @@ def gnb_unet_set_conv_impl(net, impl):
 
 def gnb_unet_test_wait_timeout(net):
     return lib().gnb_unet_test_wait_timeout(net)
+
+
+def gnb_test_fail_alloc(h, after):
+    return lib().gnb_test_fail_alloc(h, after)
 
 
 def gnb_unet_get_params(net, dst, on_device):

@@ -1,0 +1,80 @@
+"""Calls that fail part-way: what they leave behind.
+
+Device allocations are made to fail on the host (gnb_test_fail_alloc), one
+after the other; nothing here makes a kernel fail."""
+import numpy as np
+import pytest
+
+from paper_2510_23330_gb300 import ics
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def G():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2510_23330_gb300 import galnb
+    return galnb
+
+
+FIELDS = ("X", "Y", "Z", "AX", "AY", "AZ", "POT", "DUDT", "RHO", "H2")
+
+
+def _calls(G, c, net, p, cen, rep):
+    return [
+        lambda: c.set_particles(p),
+        lambda: c.compute_forces(G.GNB_GRAV_DIRECT),
+        lambda: c.compute_forces(G.GNB_GRAV_TREE),
+        lambda: c.voxelise([cen], grid=12),
+        lambda: c.sn_async_submit(net, [cen], seed=3, sweeps=1),
+        lambda: c.sn_async_apply(),
+        lambda: c.replace_region(rep),
+        lambda: c.compute_forces(G.GNB_GRAV_TREE),
+    ]
+
+
+def test_calls_after_a_failed_allocation(G):
+    """Whichever allocation of a context fails, the call that made it returns
+    GNB_ENOMEM and the same call works when it is repeated: no array is used
+    whose replacement was not allocated, and the results are those of a
+    context without a failure."""
+    from paper_2510_23330_gb300 import surrogate
+    n, cen, big = 2000, (0.0, 0.0, 0.0), 1 << 40
+    p = ics.sn_region(n, seed=2, grid=16)
+    rng = np.random.default_rng(0)
+    pick = rng.permutation(n)[:50]
+    rep = {k: p[k][pick].copy() for k in ("id", "x", "y", "z", "vx", "vy", "vz", "u")}
+    for k in "xyz":
+        rep[k] += rng.uniform(-1.0, 1.0, 50)
+    net = G.UNet(5, 5, 16, 2, 8)
+    net.set_params(surrogate.he_init(5, 5, 16, 2, seed=1))
+
+    def run(after):
+        c = G.Context()
+        G.gnb_test_fail_alloc(c.h, after)
+        failed = 0
+        for call in _calls(G, c, net, p, cen, rep):
+            try:
+                call()
+            except G.GalnbError as e:
+                assert e.code == G.GNB_ENOMEM and failed == 0
+                failed += 1
+                call()
+        out = {k: c.get(k).astype(np.float64) for k in FIELDS}
+        if after < big:
+            # from arrays of this size to larger ones: everything is replaced once more
+            assert failed == 1
+            c.set_particles({k: np.concatenate([v, v]) for k, v in p.items()})
+            c.compute_forces(G.GNB_GRAV_TREE)
+        left = G.gnb_test_fail_alloc(c.h, -1)
+        c.close()
+        return out, left
+
+    ref, left = run(big)
+    for after in range(big - left):
+        got, _ = run(after)
+        for k in FIELDS:
+            # (the symmetric SPH sums have no fixed order)
+            assert np.max(np.abs(got[k] - ref[k])) <= 1e-4 * np.max(np.abs(ref[k])), (after, k)
