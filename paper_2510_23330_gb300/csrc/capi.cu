@@ -593,6 +593,8 @@ static int do_gravity(gnb_ctx *c, int mode)
     // interaction counts, list pool top and work counters (see gravity.cu)
     cudaMemsetAsync(c->counters_d, 0, 8 * sizeof(unsigned long long), c->s);
     phase_begin(c, GNB_T_GRAVITY);
+    // tree gravity is valid once its lists are known to be complete (gravity_settle)
+    c->gravity_valid = false;
     if (mode == GNB_GRAV_TREE) {
         GNB_TRY(gravity_tree(c));
     } else if (mode == GNB_GRAV_DIRECT) {
@@ -601,7 +603,7 @@ static int do_gravity(gnb_ctx *c, int mode)
     phase_begin(c, GNB_T_EXTERNAL);
     GNB_TRY(assemble_forces(c, mode != GNB_GRAV_NONE));
     phase_end(c);
-    c->gravity_valid = true;
+    c->gravity_valid = !c->grav_queued;
     c->last_grav_mode = mode;
     return GNB_OK;
 }
@@ -611,11 +613,16 @@ static int do_forces(gnb_ctx *c, int mode)
     // without self-gravity only the hydro tree is needed, which the sorted
     // gas particles give
     GNB_TRY(mode == GNB_GRAV_NONE ? do_sort(c) : do_build(c));
+    // the accelerations and du/dt are overwritten from here on
+    c->force_valid = c->sphf_valid = false;
     GNB_TRY(do_gravity(c, mode));
-    GNB_TRY(sph_density(c));
+    const int rc = sph_density(c);
     // the walk's lists fitted their pool (sph_density waits for the stream
-    // when there is gas): else gravity again, before anything is added to it
-    GNB_TRY(gravity_settle(c, c->n_gas > 0));
+    // when there is gas): else gravity again, before anything is added to it;
+    // gravity is complete by itself, also when the density is not
+    const int settled = gravity_settle(c, rc == GNB_OK && c->n_gas > 0);
+    if (rc != GNB_OK) return rc;
+    GNB_TRY(settled);
     c->density_valid = true;
     GNB_TRY(sph_force(c));
     c->force_valid = true;
@@ -683,6 +690,7 @@ int gnb_compute_gravity(gnb_ctx *c, int mode)
     if (rc == GNB_OK) rc = read_groups(c);
     if (rc == GNB_OK) rc = gravity_settle(c, false);
     c->force_valid = false;
+    if (rc != GNB_OK) c->sphf_valid = false;  // its sums may have been overwritten
     return finish(c, rc);
 }
 

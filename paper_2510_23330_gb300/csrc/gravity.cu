@@ -1127,6 +1127,8 @@ int gravity_tree(gnb_ctx *c)
 // After a wait for the stream (made here unless `waited`): the pool must have
 // held every list; otherwise grow it, walk and evaluate again (an evaluation
 // of incomplete lists does nothing) and repeat the assembly that followed.
+// Only then are the accelerations marked valid: if the pool cannot grow they
+// are sums of the fields' former contents.
 int gravity_settle(gnb_ctx *c, bool waited)
 {
     if (!c->grav_queued) return GNB_OK;
@@ -1134,7 +1136,10 @@ int gravity_settle(gnb_ctx *c, bool waited)
         if (!waited || attempt > 0) GNB_TRY(cuda_check(c, cudaStreamSynchronize(c->s), "list pool sync"));
         c->grav_queued = false;
         const int used = c->pinned_i[40];
-        if (used <= c->gl_cap) return GNB_OK;
+        if (used <= c->gl_cap) {
+            c->gravity_valid = true;
+            return GNB_OK;
+        }
         if (attempt >= 4) return fail(c, GNB_ECAPACITY, "interaction-list pool");
         GNB_TRY(lists_alloc(c, used + used / 2 + 1024));
         cudaMemsetAsync(c->counters_d, 0, 8 * sizeof(unsigned long long), c->s);

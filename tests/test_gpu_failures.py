@@ -78,3 +78,38 @@ def test_calls_after_a_failed_allocation(G):
         for k in FIELDS:
             # (the symmetric SPH sums have no fixed order)
             assert np.max(np.abs(got[k] - ref[k])) <= 1e-4 * np.max(np.abs(ref[k])), (after, k)
+
+
+@pytest.mark.parametrize("n_gas", [0, 500])
+def test_list_pool_that_cannot_grow(G, n_gas):
+    """A nearly direct walk of small groups over single-particle leaves outgrows
+    the first interaction-list pool; when the larger one cannot be allocated
+    the accelerations were never evaluated and are not handed out, and the next
+    call finds memory again."""
+    p = ics.plummer(6000, seed=2, n_gas=n_gas)
+    names = ("AGRAV_X", "AGRAV_Y", "AGRAV_Z", "POT", "AX")
+    c, d = G.Context(theta=0.03, n_leaf=1, n_group=8), G.Context(theta=0.03, n_leaf=1, n_group=8)
+    for q in (c, d):
+        q.set_particles(p)
+        q.compute_sph_density()  # every other array of the calls below
+    call = {0: "compute_gravity", 500: "compute_forces"}[n_gas]
+    G.gnb_test_fail_alloc(c.h, 6)  # the pool's six arrays, not the larger pool
+    with pytest.raises(G.GalnbError) as e:
+        getattr(c, call)(G.GNB_GRAV_TREE)
+    assert e.value.code == G.GNB_ENOMEM and G.gnb_test_fail_alloc(c.h, -1) == -1
+    for k in names:
+        with pytest.raises(G.GalnbError) as e:
+            c.get(k)
+        assert e.value.code == G.GNB_ESTATE
+    with pytest.raises(G.GalnbError):
+        c.diagnostics()
+    if n_gas:
+        c.compute_sph_force()  # of the density that was there; not a force to step with
+        with pytest.raises(G.GalnbError):
+            c.get("POT")
+    for q in (c, d):
+        getattr(q, call)(G.GNB_GRAV_TREE)
+    for k in names:
+        assert np.allclose(c.get(k), d.get(k), rtol=1e-5, atol=1e-6)
+    d.compute_gravity(G.GNB_GRAV_DIRECT)
+    assert np.median(np.abs(c.get("AGRAV_X") / d.get("AGRAV_X") - 1.0)) < 1e-4
