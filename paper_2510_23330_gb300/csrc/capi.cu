@@ -619,11 +619,14 @@ static int do_forces(gnb_ctx *c, int mode)
     const int rc = sph_density(c);
     // the walk's lists fitted their pool (sph_density waits for the stream
     // when there is gas): else gravity again, before anything is added to it;
-    // gravity is complete by itself, also when the density is not
+    // either is complete by itself, also when the other is not
     const int settled = gravity_settle(c, rc == GNB_OK && c->n_gas > 0);
     if (rc != GNB_OK) return rc;
-    GNB_TRY(settled);
     c->density_valid = true;
+    if (settled != GNB_OK) {
+        sph_keep_support(c);
+        return settled;
+    }
     GNB_TRY(sph_force(c));
     c->force_valid = true;
     c->sphf_valid = true;
@@ -702,6 +705,7 @@ int gnb_compute_sph_density(gnb_ctx *c)
     int rc = GNB_OK;
     if (!c->tree_valid) rc = do_build(c);
     if (rc == GNB_OK) rc = sph_density(c);
+    if (rc == GNB_OK) rc = sph_keep_support(c);
     if (rc == GNB_OK) c->density_valid = true;
     c->force_valid = false;
     return finish(c, rc);

@@ -328,6 +328,7 @@ int gravity_direct(gnb_ctx *c);
 int assemble_forces(gnb_ctx *c, bool self);
 // sph.cu
 int sph_density(gnb_ctx *c);
+int sph_keep_support(gnb_ctx *c);
 int sph_force(gnb_ctx *c);
 // surrogate.cu
 int voxelise_buffers_for(gnb_ctx *c, int nreg, int grid);

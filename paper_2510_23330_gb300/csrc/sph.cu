@@ -178,7 +178,6 @@ struct KnnParams {
     float4 *V, *Q;       // records of the force pass (see pair_force)
     const int *gslot;    // particle slot of each gas particle, and the fields per slot
     float *s_rho, *s_pres, *s_cs;
-    double *s_h2;
     float gamma;
     int pressure;  // 1: also smooth P = (gamma - 1) sum_j m_j u_j W_ij (pressure-energy SPH)
 };
@@ -564,7 +563,6 @@ __device__ __forceinline__ void knn_finish(const KnnParams &p, int first, unsign
         p.h[i] = hh;
         p.g64[i] = g64;
         p.E[i] = r.E;
-        p.s_h2[p.gslot[i]] = hsq;
     }
     __syncwarp();
     float rho = 0.f, qsum = 0.f;
@@ -747,6 +745,8 @@ __global__ void __launch_bounds__(KN_THREADS, KN_CTAS) k_knn(KnnParams p)
 // its band, the exact FP64 d^2.  Every decision the FP32 test takes is the
 // one the FP64 test would take.
 //
+// The particles' supports are stored here too.
+//
 // SL lanes share a particle here and in the list fill: a lane takes every
 // SL-th entry, so a row of the list is read in whole sectors and the gathers
 // of a particle overlap (one thread per particle: a chain of 64 reads).
@@ -757,7 +757,8 @@ __global__ void __launch_bounds__(256) k_mutual(int ng, const int *__restrict__ 
                                                 const int *__restrict__ grank, const double *__restrict__ x,
                                                 const double *__restrict__ y, const double *__restrict__ z,
                                                 unsigned long long *__restrict__ mut, int *__restrict__ rcnt,
-                                                int *__restrict__ rtot)
+                                                int *__restrict__ rtot, const int *__restrict__ gslot,
+                                                double *__restrict__ s_h2)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t == 0) *rtot = 0;  // summed by k_rev_off
@@ -798,7 +799,10 @@ __global__ void __launch_bounds__(256) k_mutual(int ng, const int *__restrict__ 
         const unsigned bal = __ballot_sync(0xffffffffu, m);
         mask |= (unsigned long long)((bal >> (SL * half)) & ((1u << SL) - 1u)) << (q * SL);
     }
-    if (valid && l == 0) mut[i] = mask;
+    if (valid && l == 0) {
+        mut[i] = mask;
+        s_h2[gslot[i]] = h2[i];  // see sph_keep_support
+    }
 }
 
 // Storage of the reverse lists: each particle's segment of rlist, taken in
@@ -948,6 +952,28 @@ __global__ void __launch_bounds__(128) k_force(ForceParams p)
 // ---------------------------------------------------------------- host
 static int g_knn_blocks = 0;
 
+__global__ void __launch_bounds__(256) k_keep_support(int ng, const int *__restrict__ gslot,
+                                                      const double *__restrict__ h2, double *__restrict__ s_h2)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < ng) s_h2[gslot[i]] = h2[i];
+}
+
+// The supports of a search that succeeded become the particles': they are the
+// next search's starting radii and part of the saved state, so one that fails
+// must not touch them (density, pressure and sound speed, which it may have
+// overwritten in part, are marked invalid instead).  sph_force does the same
+// on its way (k_mutual).
+int sph_keep_support(gnb_ctx *c)
+{
+    const int ng = (int)c->n_gas;
+    if (ng == 0) return GNB_OK;
+    gnb::counted(k_keep_support)<<<(ng + 255) / 256, 256, 0, c->s>>>(ng, c->gslot, c->gh2, c->P[c->cur].h2);
+    GNB_LAUNCH_CHECK(c, "supports");
+    c->have_h = true;
+    return GNB_OK;
+}
+
 int sph_density(gnb_ctx *c)
 {
     int ng = (int)c->n_gas;
@@ -1005,8 +1031,9 @@ int sph_density(gnb_ctx *c)
     p.failed = c->work_d + 3;
     p.nbr = c->nbr; p.nd2 = c->nd2; p.h2 = c->gh2; p.h2b = c->gh2b; p.h = c->gh; p.E = c->gE; p.g64 = c->g64;
     p.gvx = c->gvx; p.gvy = c->gvy; p.gvz = c->gvz; p.V = c->fV; p.Q = c->fQ;
-    p.gslot = c->gslot; p.s_rho = c->rho; p.s_pres = c->pres; p.s_cs = c->cs; p.s_h2 = a.h2;
+    p.gslot = c->gslot; p.s_rho = c->rho; p.s_pres = c->pres; p.s_cs = c->cs;
     p.gamma = (float)c->cfg.gamma; p.pressure = c->cfg.sph_variant;
+    c->density_valid = c->nbr_valid = false;  // overwritten from here on
     gnb::counted(k_knn)<<<g_knn_blocks, KN_THREADS, smem, c->s>>>(p);
     GNB_LAUNCH_CHECK(c, "knn");
     cudaMemcpyAsync(c->pinned_i, c->work_d, 4 * sizeof(int), cudaMemcpyDeviceToHost, c->s);
@@ -1022,7 +1049,6 @@ int sph_density(gnb_ctx *c)
     }
     c->stats[GNB_S_GAS_NODES] = c->gt.nnodes;
     phase_end(c);
-    c->have_h = true;
     c->nbr_valid = true;
     return GNB_OK;
 }
@@ -1042,7 +1068,9 @@ int sph_force(gnb_ctx *c)
     const int gb = (ng + 255) / 256, gbl = (int)(((long long)ng * sl + 255) / 256);
     cudaMemsetAsync(c->rcnt, 0, sizeof(int) * ng, c->s);
     gnb::counted(few ? k_mutual<16> : k_mutual<8>)<<<gbl, 256, 0, c->s>>>(
-        ng, c->nbr, c->nd2, c->gE, c->gh2, c->gh2b, c->g64, c->ggrank, c->gx, c->gy, c->gz, c->mut, c->rcnt, c->rtot_d);
+        ng, c->nbr, c->nd2, c->gE, c->gh2, c->gh2b, c->g64, c->ggrank, c->gx, c->gy, c->gz, c->mut, c->rcnt, c->rtot_d,
+        c->gslot, c->P[c->cur].h2);
+    c->have_h = true;
     gnb::counted(k_rev_off)<<<gb, 256, 0, c->s>>>(ng, c->rcnt, c->roff, c->rcur, c->rtot_d);
     gnb::counted(few ? k_rev_fill<16> : k_rev_fill<8>)<<<gbl, 256, 0, c->s>>>(ng, c->nbr, c->mut, c->rcur, c->rlist);
     GNB_LAUNCH_CHECK(c, "symmetric lists");

@@ -113,3 +113,33 @@ def test_list_pool_that_cannot_grow(G, n_gas):
         assert np.allclose(c.get(k), d.get(k), rtol=1e-5, atol=1e-6)
     d.compute_gravity(G.GNB_GRAV_DIRECT)
     assert np.median(np.abs(c.get("AGRAV_X") / d.get("AGRAV_X") - 1.0)) < 1e-4
+
+
+def test_search_that_fails_leaves_the_supports(G, tmp_path):
+    """Three hundred gas particles at one point cannot be ranked: the
+    kernel-size search fails for them, after it has found the supports of the
+    others.  The supports of the state stay those it came with, and the density
+    of the failed call is not handed out."""
+    p = ics.sn_region(3000, seed=4, grid=16)
+    for k in "xyz":
+        p[k][:300] = p[k][0]
+    n = p["x"].size
+    rng = np.random.default_rng(1)
+    p["h2"] = rng.uniform(1.0, 2.0, n)
+    for k in ("ax", "ay", "az", "dudt"):
+        p[k] = np.zeros(n, np.float32)
+    c = G.Context()
+    c.set_state(p, G.GNB_GRAV_NONE)
+    for call in (c.compute_sph_density, lambda: c.compute_forces(G.GNB_GRAV_NONE)):
+        with pytest.raises(G.GalnbError) as e:
+            call()
+        assert e.value.code == G.GNB_ECAPACITY
+        for k in ("RHO", "H2", "NBR"):
+            with pytest.raises(G.GalnbError):
+                c.get(k)
+        path = str(tmp_path / "state")
+        c.save(path)
+        # after the header: id, type, 3 positions, 6 floats, then h2 and 12 floats
+        raw = open(path, "rb").read()
+        at = len(raw) - n * (8 + 12 * 4)
+        assert np.array_equal(np.frombuffer(raw, np.float64, n, at), p["h2"])
