@@ -399,7 +399,7 @@ int gnb_set_particles(gnb_ctx *c, int64_t n, const int64_t *id, const uint8_t *t
     if (!id || !type || !x || !y || !z || !vx || !vy || !vz || !m || !eps || !u)
         return fail(c, GNB_EINVAL, "null array");
     c->have_particles = c->sorted_valid = c->tree_valid = c->gravity_valid = c->density_valid = c->force_valid = false;
-    c->sphf_valid = false;
+    c->sphf_valid = c->nbr_valid = false;
     c->have_h = false;
     c->hier_on = c->hier_valid = false;
     c->rid_valid = false;
@@ -543,6 +543,10 @@ static void phase_resolve(gnb_ctx *c)
 static int do_sort(gnb_ctx *c)
 {
     phase_begin(c, GNB_T_SORT);
+    // results are held by slot: those that came with a state in the caller's
+    // order do not follow its particles to their new slots
+    if (!c->sorted_valid)
+        c->gravity_valid = c->density_valid = c->force_valid = c->sphf_valid = c->nbr_valid = false;
     GNB_TRY(morton_and_sort(c));
     phase_end(c);
     c->sorted_valid = true;
@@ -633,6 +637,28 @@ static int do_forces(gnb_ctx *c, int mode)
     return GNB_OK;
 }
 
+// A state from a file or from gnb_set_state has no neighbour lists and no signal
+// velocities: the forces it came with are evaluated here (those of gravity
+// only if it had them).
+static int forces_with_lists(gnb_ctx *c)
+{
+    if (c->gravity_valid) return do_forces(c, c->last_grav_mode);
+    GNB_TRY(do_build(c));
+    GNB_TRY(sph_density(c));
+    const size_t b = sizeof(float) * (size_t)c->n;
+    for (float *a : {c->ax, c->ay, c->az, c->dudt}) cudaMemsetAsync(a, 0, b, c->s);
+    GNB_TRY(sph_force(c));
+    c->density_valid = c->sphf_valid = true;
+    return GNB_OK;
+}
+
+static int ensure_lists(gnb_ctx *c)
+{
+    if (c->n_gas == 0 || c->nbr_valid) return GNB_OK;
+    GNB_TRY(forces_with_lists(c));
+    return read_groups(c);
+}
+
 // One kick-drift-kick step; forces at the start of the step must be current.
 static int kdk_one(gnb_ctx *c, double dt, int mode)
 {
@@ -716,6 +742,7 @@ int gnb_compute_sph_force(gnb_ctx *c)
     if (!c) return GNB_EINVAL;
     c->err.clear();
     if (!c->density_valid) return fail(c, GNB_ESTATE, "SPH density not computed for the current positions");
+    if (c->n_gas > 0 && !c->nbr_valid) return finish(c, ensure_lists(c));
     int rc = GNB_OK;
     if (!c->gravity_valid) {
         size_t b = sizeof(float) * (size_t)c->n;
@@ -779,7 +806,8 @@ int gnb_cfl_timestep(gnb_ctx *c, double courant, double *dt)
     if (!(courant > 0.0)) return fail(c, GNB_EINVAL, "courant factor");
     if (!c->sphf_valid) return fail(c, GNB_ESTATE, "SPH force not computed");
     double m = 0.0;
-    int rc = cfl_min_h_over_vsig(c, &m);
+    int rc = ensure_lists(c);
+    if (rc == GNB_OK) rc = cfl_min_h_over_vsig(c, &m);
     *dt = courant * m;
     return finish(c, rc);
 }
@@ -795,7 +823,7 @@ int gnb_integrate_cfl(gnb_ctx *c, double t_span, double courant, int max_steps, 
     if (!c->have_particles) return fail(c, GNB_ESTATE, "no particles");
     if (c->n_gas == 0) return fail(c, GNB_ESTATE, "no gas: the CFL timestep is undefined");
     int rc = GNB_OK;
-    if (!c->force_valid || c->last_grav_mode != mode) rc = do_forces(c, mode);
+    if (!c->force_valid || c->last_grav_mode != mode || !c->nbr_valid) rc = do_forces(c, mode);
     double t = 0.0;
     int64_t steps = 0;
     while (rc == GNB_OK && t < t_span && steps < max_steps) {
@@ -832,7 +860,7 @@ int gnb_integrate_hier(gnb_ctx *c, double t_span, double courant, int max_level,
     if (c->sna_pending) return fail(c, GNB_ESTATE, "an asynchronous surrogate batch is pending");
     c->hier_on = c->hier_valid = false;
     int rc = hier_buffers(c);
-    if (rc == GNB_OK && (!c->force_valid || c->last_grav_mode != mode)) rc = do_forces(c, mode);
+    if (rc == GNB_OK && (!c->force_valid || c->last_grav_mode != mode || !c->nbr_valid)) rc = do_forces(c, mode);
     const int K = max_level;
     const long long NT = 1ll << (K + 1);
     const double tick = std::ldexp(t_span, -(K + 1));
