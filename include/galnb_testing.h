@@ -28,6 +28,12 @@ int gnb_unet_test_wait_timeout(gnb_unet *net);
  * -2: NULL context). */
 int64_t gnb_test_fail_alloc(gnb_ctx *ctx, int64_t after);
 
+/* A bounded wait of the radix sort that runs out: the context's next sort
+ * starts with its pass `pass` (the key's byte, 0 .. 7; the particles' sort
+ * takes 2 .. 7) marked as given up.  The later passes do nothing and the call
+ * returns GNB_ETIMEOUT.  -1 puts this off.  Errors: GNB_EINVAL. */
+int gnb_test_sort_give_up(gnb_ctx *ctx, int pass);
+
 #ifdef __cplusplus
 }
 #endif

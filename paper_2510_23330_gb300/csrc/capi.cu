@@ -1124,6 +1124,13 @@ int64_t gnb_test_fail_alloc(gnb_ctx *c, int64_t after)
     return left;
 }
 
+int gnb_test_sort_give_up(gnb_ctx *c, int pass)
+{
+    if (!c || pass < -1 || pass > 7) return GNB_EINVAL;
+    c->sort_gives_up = pass;
+    return GNB_OK;
+}
+
 int gnb_stats(gnb_ctx *c, int64_t out[GNB_S_COUNT_])
 {
     if (!c || !out) return GNB_EINVAL;

@@ -214,6 +214,7 @@ struct gnb_ctx {
     float4 *gd_part = nullptr;                 // direct gravity: sums of the source parts [parts][n]
     int64_t gd_cap = 0;
     int *pinned_i = nullptr;                   // pinned host scratch [64]
+    int sort_gives_up = -1;                    // pass of the next radix sort that counts as given up (tests)
     int64_t alloc_left = -1;                   // device allocations before one fails (tests; -1: none does)
     // hierarchical timesteps (integrate.cu): per particle slot, permuted with
     // the particles by every sort while hier_on; [2] = current and scratch

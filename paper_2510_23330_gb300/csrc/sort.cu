@@ -211,7 +211,7 @@ struct RsState {
     int *hist;        // [8][256] digit histograms
     int *ticket;      // [8] tiles started per pass
     unsigned *state;  // [passes][ntiles][256] published counts
-    int *flag;        // set when a look-back gave up
+    int *flag;        // bit p set when a look-back of pass p gave up
 };
 
 template <int ITEMS>
@@ -269,7 +269,12 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_rs_pass(const uint64_t *__res
 #pragma unroll
     for (int q = 0; q < RS_THREADS / 32; q++) S.wc[q][t] = 0;
     const int hd = hist[t];
+    // an earlier pass that gave up left places unwritten: its output no longer
+    // has the digits that were counted, and their positions could lie beyond
+    // the arrays (the earlier passes' bits are final: every thread sees the same)
+    const unsigned gave_up = *(volatile int *)flag & ((1u << (shift >> 3)) - 1u);
     __syncthreads();
+    if (gave_up) return;
     const int tile = S.tile;
     const int base = tile * TILE;
     const int cnt = min(TILE, n - base);
@@ -368,7 +373,7 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_rs_pass(const uint64_t *__res
         if (moved) spins = 0;
         else if (++spins > RS_SPINS) {  // cannot happen unless a block was lost
             S.stop = 1;
-            atomicOr(flag, 1);
+            atomicOr(flag, 1 << (shift >> 3));
             break;
         }
     }
@@ -427,7 +432,13 @@ static int rs_begin(gnb_ctx *c, int n, RsState *st)
     st->ticket = c->rs_buf + 8 * 256;
     st->flag = c->rs_buf + 8 * 256 + 8;
     st->state = (unsigned *)(c->rs_buf + 8 * 256 + 16);
-    return cuda_check(c, cudaMemsetAsync(c->rs_buf, 0, words * sizeof(int), c->s), "radix sort scratch");
+    GNB_TRY(cuda_check(c, cudaMemsetAsync(c->rs_buf, 0, words * sizeof(int), c->s), "radix sort scratch"));
+    if (c->sort_gives_up >= 0) {  // (set by tests)
+        const int bit = 1 << c->sort_gives_up;
+        c->sort_gives_up = -1;
+        return cuda_check(c, cudaMemsetAsync(st->flag, bit, 1, c->s), "radix sort flag");
+    }
+    return GNB_OK;
 }
 
 template <int ITEMS, bool FIRST>

@@ -149,6 +149,8 @@ def _declare(L):
     L.gnb_unet_test_wait_timeout.restype = C.c_int
     L.gnb_test_fail_alloc.argtypes = [_vp, C.c_int64]
     L.gnb_test_fail_alloc.restype = C.c_int64
+    L.gnb_test_sort_give_up.argtypes = [_vp, C.c_int]
+    L.gnb_test_sort_give_up.restype = C.c_int
     for name in ("gnb_save", "gnb_load", "gnb_unet_save", "gnb_unet_load"):
         getattr(L, name).argtypes = [_vp, C.c_char_p]
         getattr(L, name).restype = C.c_int
@@ -293,6 +295,10 @@ def gnb_unet_test_wait_timeout(net):
 
 def gnb_test_fail_alloc(h, after):
     return lib().gnb_test_fail_alloc(h, after)
+
+
+def gnb_test_sort_give_up(h, pass_):
+    return lib().gnb_test_sort_give_up(h, pass_)
 
 
 def gnb_unet_get_params(net, dst, on_device):

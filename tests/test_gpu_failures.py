@@ -1,7 +1,8 @@
 """Calls that fail part-way: what they leave behind.
 
 Device allocations are made to fail on the host (gnb_test_fail_alloc), one
-after the other; nothing here makes a kernel fail."""
+after the other, and a sort is told that a wait ran out
+(gnb_test_sort_give_up); nothing here makes a kernel fault or hang."""
 import numpy as np
 import pytest
 
@@ -185,3 +186,24 @@ def test_hydro_calls_on_a_loaded_state(G, tmp_path):
     b.compute_sph_density()
     with pytest.raises(G.GalnbError):
         b.get("AX")
+
+
+@pytest.mark.parametrize("last", [2, 4, 7])
+def test_sort_that_gave_up(G, orc, last):
+    """After a pass whose wait ran out the later passes leave their arrays
+    alone (places that were never written have other digits than were
+    counted); the call reports it and the next one sorts."""
+    p = ics.plummer(5000, seed=last, n_gas=0)
+    c = G.Context()
+    c.set_particles(p)
+    assert G.gnb_test_sort_give_up(c.h, last) == G.GNB_OK
+    with pytest.raises(G.GalnbError) as e:
+        c.build_tree()
+    assert e.value.code == G.GNB_ETIMEOUT
+    for k in ("KEY", "NODES"):
+        with pytest.raises(G.GalnbError):
+            c.get(k)
+    c.build_tree()
+    key, _, _, _ = orc.morton(p)
+    assert np.array_equal(c.get("KEY"), key.astype(np.int64))
+    assert np.array_equal(c.get("ORDER"), orc.sort_order(key))
