@@ -6,6 +6,8 @@
 // SPH density and force (Table 3); shared-timestep leapfrog (Sec. 3.2).
 // All device work runs on cfg.cuda_stream; each call ends with one stream
 // synchronisation and a check of the device status word.
+#include <cuda.h>
+
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -25,6 +27,7 @@ int fail(gnb_ctx *c, int code, const std::string &msg)
 int cuda_check(gnb_ctx *c, cudaError_t e, const char *what)
 {
     if (e == cudaSuccess) return GNB_OK;
+    cudaGetLastError();  // reported here: a later call's launch check does not find it again
     std::string m = std::string(what) + ": " + cudaGetErrorString(e);
     if (e == cudaErrorMemoryAllocation) return fail(c, GNB_ENOMEM, m);
     return fail(c, GNB_ECUDA, m);
@@ -247,6 +250,35 @@ __global__ void __launch_bounds__(1024) k_load_scan(int *__restrict__ partial, i
     if (t == 1023) *ngas = *out = pre + x;
 }
 
+// Whether [p, p + bytes) lies in one allocation of this device, so that a kernel
+// can read it.  What does not (host or managed memory, another device's, an
+// array shorter than the count asks for) goes through a copy, which reaches
+// what the device cannot read in place and refuses what is not there.
+static bool readable_in_place(const void *p, size_t bytes)
+{
+    typedef CUresult (*range_fn)(CUdeviceptr *, size_t *, CUdeviceptr);
+    static const range_fn range = []() -> range_fn {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        return reinterpret_cast<range_fn>(f);
+    }();
+    cudaPointerAttributes a;
+    int dev = -1;
+    if (!range || cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    return a.type == cudaMemoryTypeDevice && a.device == dev &&
+           range(&base, &size, (CUdeviceptr)(uintptr_t)p) == CUDA_SUCCESS && (uintptr_t)p + bytes <= base + size;
+}
+
 // Rank of every gas particle among the gas, in the caller's order.
 __global__ void __launch_bounds__(LD_THREADS) k_grank(const uint8_t *__restrict__ type, const int *__restrict__ offs,
                                                       int n, int *__restrict__ grank)
@@ -411,9 +443,10 @@ int gnb_set_particles(gnb_ctx *c, int64_t n, const int64_t *id, const uint8_t *t
     struct { void *d; const void *s; size_t b; } cp[] = {
         {p.id, id, 8}, {p.type, type, 1}, {p.x, x, 8}, {p.y, y, 8}, {p.z, z, 8}, {p.vx, vx, 4},
         {p.vy, vy, 4}, {p.vz, vz, 4}, {p.m, m, 4}, {p.eps, eps, 4}, {p.u, u, 4}};
-    // device arrays are read in place (copied first if one is not aligned to its elements)
+    // device arrays are read in place (copied first if one is not aligned to its elements
+    // or not all there)
     bool copy = !on_device;
-    for (auto &q : cp) copy = copy || (uintptr_t)q.s % q.b != 0;
+    for (auto &q : cp) copy = copy || (uintptr_t)q.s % q.b != 0 || !readable_in_place(q.s, q.b * N);
     if (copy) {
         const cudaMemcpyKind k = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
         for (auto &q : cp) GNB_TRY(cuda_check(c, cudaMemcpyAsync(q.d, q.s, q.b * N, k, c->s), "particle copy"));

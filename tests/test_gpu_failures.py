@@ -207,3 +207,31 @@ def test_sort_that_gave_up(G, orc, last):
     key, _, _, _ = orc.morton(p)
     assert np.array_equal(c.get("KEY"), key.astype(np.int64))
     assert np.array_equal(c.get("ORDER"), orc.sort_order(key))
+
+
+def test_upload_of_arrays_that_are_not_all_there(G):
+    """Device arrays are read in place only where the whole of each lies in one
+    allocation: pinned and managed memory is taken as before, an array of half
+    the length is refused by the copy it then goes through."""
+    import ctypes as C
+    import torch
+    p = ics.plummer(1 << 15, seed=1, n_gas=0)
+    n = p["x"].size
+    dev = {k: torch.from_numpy(np.ascontiguousarray(p[k], dtype=t)).cuda() for k, t in G.Context._DT.items()}
+    managed, half = C.c_void_p(), C.c_void_p()
+    L = G.lib()
+    assert L.cudaMallocManaged(C.byref(managed), C.c_size_t(8 * n), 1) == 0
+    assert L.cudaMalloc(C.byref(half), C.c_size_t(4 * n)) == 0
+    C.memmove(managed, p["x"].ctypes.data, 8 * n)
+    pinned = torch.from_numpy(p["x"].copy()).pin_memory()
+    torch.cuda.synchronize()
+    for x, ok in ((dev["x"].data_ptr(), True), (pinned.data_ptr(), True), (managed.value, True), (half.value, False)):
+        c = G.Context()
+        c.n = n
+        rc = G.gnb_set_particles(c.h, n, *[x if k == "x" else dev[k].data_ptr() for k in dev], 1)
+        assert rc == (G.GNB_OK if ok else G.GNB_ECUDA)
+        if not ok:  # and the refused call leaves nothing for the next
+            c.set_particles(p)
+        assert np.array_equal(c.get("X"), p["x"])
+        c.close()
+    assert L.cudaFree(managed) == 0 and L.cudaFree(half) == 0
