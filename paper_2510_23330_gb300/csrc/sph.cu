@@ -292,8 +292,10 @@ __device__ __forceinline__ bool knn_walk(KnnWarp &S, const KnnParams &p, const K
     // roundings of the sums
     const float Rg = R / unit;  // unit is a power of two
     const float Rg2 = Rg * Rg * (1.f + 1e-5f) + 4.f;
-    // a single particle keeps what can lie in its list: d^2 <= R^2 + 2 E (E <
-    // 2^-23 (12 R^2 + 14 unit R) there), with a margin
+    // a single particle keeps what can lie in its list: d^2 <= R^2 + 2 E, with a
+    // margin (E < 2^-23 (12 R^2 + 26 unit R) there: A' is at most R, sqrt(3)
+    // units to the particle and two more; 2 E < 2.9e-6 R^2 + 6.2e-6 unit R,
+    // below the margin by (1.1 R^2 - 0.2 unit R + 6 unit^2) 1e-6 > 0)
     const float R2stage = one ? R * R * (1.f + 4e-6f) + 6e-6f * unit * (R + unit)
                               : R * R * (1.f + 1e-4f) + 4.f * unit * unit;
     nc = 0;
@@ -406,10 +408,14 @@ __device__ __forceinline__ int knn_select(KnnWarp &S, const KnnParams &p, int i,
     const unsigned ltmask = (1u << lane) - 1u;
     float T = T0, Tlo = 0.f, Thi = T0;  // Tlo: too few entries, Thi: too many
     float t = 0.f, E = 0.f;
+    bool band = false;  // T is the upper end of the uncertain band
     unsigned du[KPL];
     for (int it = 0;; it++) {
         n = knn_list(S, nc, xi, yi, zi, T, lane);
         if (n < NGB && it == 0) return KN_UNDER;
+        // fewer than 64 lie below the band, so more than KN_U of the list's
+        // entries are in it: narrowing would find the same t and band again
+        if (n > KN_LIST && band) return KN_FAIL;
         if (n < NGB || n > KN_LIST) {
             // more than the list holds within the radius: narrow it to 64 ..
             // KN_LIST entries, by the number density, then by bisection down
@@ -466,7 +472,7 @@ __device__ __forceinline__ int knn_select(KnnWarp &S, const KnnParams &p, int i,
         E = U * (EA * sqrt_fast(te) + 5.f * te);
         if (t + 2.f * E <= T) break;
         T = t + 2.f * E;  // the band reaches past a narrowed radius
-        Tlo = Thi = 0.f;  // (no further narrowing: more entries than the list holds fail)
+        band = true;
     }
     const float lo = t - 2.f * E, hi = t + 2.f * E;
     // sure members (fewer than 64 lie below t) to the list, uncertain ones

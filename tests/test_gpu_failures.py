@@ -235,3 +235,34 @@ def test_upload_of_arrays_that_are_not_all_there(G):
         assert np.array_equal(c.get("X"), p["x"])
         c.close()
     assert L.cudaFree(managed) == 0 and L.cudaFree(half) == 0
+
+
+def test_particle_inside_a_thin_shell(G, orc):
+    """A particle that sees its 64th neighbour among equal distances: 60 in a
+    shell a millionth thick are ranked, 200 are more than the uncertain entries
+    that can be (they fail at once: the band of the 64th reaches past the list)."""
+    rng = np.random.default_rng(3)
+    for m, ok in ((60, True), (200, False)):
+        p = ics.uniform_random(4000, seed=9)
+        x = np.stack([p[k] for k in "xyz"], axis=1)
+        at = x.mean(0)
+        far = np.argsort(((x - at) ** 2).sum(1))[::-1]
+        hole = 0.5 * np.sqrt(((x - at) ** 2).sum(1)).max()
+        d = x - at
+        r = np.sqrt((d**2).sum(1))
+        x = at + d * np.maximum(1.0, hole / np.maximum(r, 1e-12))[:, None] * rng.uniform(1.0, 1.2, (x.shape[0], 1))
+        x[far[0]] = at
+        v = rng.normal(size=(m, 3))
+        x[far[1 : m + 1]] = at + 0.4 * hole * (1.0 + 5e-7 * rng.uniform(-1.0, 1.0, (m, 1))) * v / np.sqrt((v**2).sum(1))[:, None]
+        for k, a in zip("xyz", range(3)):
+            p[k] = np.ascontiguousarray(x[:, a])
+        c = G.Context()
+        c.set_particles(p)
+        if ok:
+            c.compute_sph_density()
+            d2 = np.sort(((x - at) ** 2).sum(1))
+            assert abs(c.get("H2")[far[0]] - d2[63]) < 1e-12 * d2[63]
+        else:
+            with pytest.raises(G.GalnbError) as e:
+                c.compute_sph_density()
+            assert e.value.code == G.GNB_ECAPACITY
