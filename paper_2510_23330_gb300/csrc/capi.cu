@@ -113,6 +113,7 @@ static int alloc_particles(gnb_ctx *c, int64_t n)
     GNB_TRY(dalloc(c, &c->sval, N)); GNB_TRY(dalloc(c, &c->sval2, N));
     GNB_TRY(dalloc(c, &c->slot_of_orig, N)); GNB_TRY(dalloc(c, &c->src, N));
     GNB_TRY(dalloc(c, &c->tmp_out, 8 * N + 64));
+    GNB_TRY(sort_reserve(c, (int)n));
     c->cap = n;
     return GNB_OK;
 }

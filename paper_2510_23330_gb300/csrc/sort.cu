@@ -414,20 +414,32 @@ __global__ void __launch_bounds__(256) k_rs_hist(const uint64_t *__restrict__ ke
 // 324 and 330).
 static int rs_items(int n) { return n <= 200000 ? 4 : (n <= 500000 ? 8 : 16); }
 
-// Scratch of a sort of n pairs, cleared: histograms, tickets, the give-up
-// flag and the published counts of eight passes.
-static int rs_begin(gnb_ctx *c, int n, RsState *st)
+// Words of a sort of n pairs: histograms, tickets, the give-up flag and the
+// published counts of eight passes.
+static size_t rs_words(int n)
 {
     const int tile = RS_THREADS * rs_items(n);
-    const size_t ntiles = (size_t)((n + tile - 1) / tile);
-    const size_t words = 8 * 256 + 16 + 8 * ntiles * 256;
-    if (c->rs_words < words) {
-        dfree(c, c->rs_buf);
-        c->rs_buf = nullptr;
-        c->rs_words = 0;
-        GNB_TRY(dalloc(c, &c->rs_buf, words));
-        c->rs_words = words;
-    }
+    return 8 * 256 + 16 + 8 * (size_t)((n + tile - 1) / tile) * 256;
+}
+
+// Scratch for sorts of up to n pairs (smaller tiles below the lines of
+// rs_items): allocated with the particles, about 8 bytes each.
+int sort_reserve(gnb_ctx *c, int n)
+{
+    const size_t words = std::max({rs_words(n), rs_words(std::min(n, 200000)), rs_words(std::min(n, 500000))});
+    if (c->rs_words >= words) return GNB_OK;
+    drop(c, c->rs_buf);
+    c->rs_words = 0;
+    GNB_TRY(dalloc(c, &c->rs_buf, words));
+    c->rs_words = words;
+    return GNB_OK;
+}
+
+// The scratch of a sort of n pairs, cleared.
+static int rs_begin(gnb_ctx *c, int n, RsState *st)
+{
+    const size_t words = rs_words(n);
+    GNB_TRY(sort_reserve(c, n));
     st->hist = c->rs_buf;
     st->ticket = c->rs_buf + 8 * 256;
     st->flag = c->rs_buf + 8 * 256 + 8;

@@ -266,3 +266,20 @@ def test_particle_inside_a_thin_shell(G, orc):
             with pytest.raises(G.GalnbError) as e:
                 c.compute_sph_density()
             assert e.value.code == G.GNB_ECAPACITY
+
+
+@pytest.mark.parametrize("n", [100, 250000])
+def test_scratch_of_the_sort_comes_with_the_particles(G, n):
+    """The first tree of a context allocates the tree's twelve arrays and
+    nothing else, also for fewer particles than the context has held, and the
+    sort still orders them."""
+    big = 1 << 40
+    p = ics.uniform_random(n, seed=n, gas_frac=0.0)
+    c = G.Context()
+    c.set_particles(ics.uniform_random(n + 1, seed=1, gas_frac=0.0))
+    c.set_particles(p)
+    G.gnb_test_fail_alloc(c.h, big)
+    c.build_tree()
+    assert big - G.gnb_test_fail_alloc(c.h, -1) == 12
+    key = c.get("KEY")
+    assert np.array_equal(c.get("ORDER"), np.lexsort((np.arange(n), key)))
