@@ -46,7 +46,7 @@ struct IgArgs {
     int mode;
     const bf16 *in1, *in2;  // input channels [0, C1) from in1, [C1, C1 + C2) from in2
     int C1, C2;
-    const bf16 *w;          // [taps][Npad][K], K = C1 + C2
+    const bf16 *w;          // [taps][Npad][Kp], Kp = C1 + C2 rounded up to 16 (zeros beyond)
     const float *bias;      // [N] or null
     int N, Npad;
     bf16 *out1, *out2;      // channels [0, O1) -> out1, [O1, N) -> out2
@@ -135,7 +135,8 @@ __global__ void __launch_bounds__(128) k_igemm(IgArgs p)
     const int K = p.C1 + p.C2;
     const int ntap = p.mode == IG_CONV3 ? 27 : (p.mode == IG_DOWN2 ? 8 : 1);
     const int tapz = p.mode == IG_UP2 ? (int)blockIdx.z : 0;
-    const int kch = K / 16;
+    const int kch = (K + 15) / 16;  // (a width of an odd multiple of 8 leaves the last step half empty)
+    const int Kp = 16 * kch;
     const int nsteps = ntap * kch;
     const long long Vrow = (long long)p.D * p.H * p.W;
     const long long VsA = p.mode == IG_DOWN2 ? 8 * Vrow : Vrow;  // voxels per batch entry of the source grid
@@ -168,19 +169,20 @@ __global__ void __launch_bounds__(128) k_igemm(IgArgs p)
         {   // A: 64 rows x 16 channels, one 16-byte piece per thread
             const int c = st_c + 8 * half;
             const bf16 *src = p.in1;
-            if (src_v >= 0)
+            const bool in = src_v >= 0 && c < K;
+            if (in)
                 src = c < p.C1 ? p.in1 + ((b0 * (p.C1 >> 3) + (c >> 3)) * VsA + src_v) * 8
                                : p.in2 + ((b0 * (p.C2 >> 3) + ((c - p.C1) >> 3)) * VsA + src_v) * 8;
-            cp_async16(&sA[slot][sr][8 * half], src, src_v >= 0 ? 16 : 0);
+            cp_async16(&sA[slot][sr][8 * half], src, in ? 16 : 0);
         }
         const int wt = p.mode == IG_UP2 ? tapz : st_t;
         for (int q = tid; q < NT * 2; q += 128) {  // B: NT rows x 16 k
             const int n = q >> 1;
             const bool in = (n0 + n) < p.Npad;
-            const bf16 *src = in ? p.w + ((long long)wt * p.Npad + n0 + n) * K + st_c + 8 * half : p.w;
+            const bf16 *src = in ? p.w + ((long long)wt * p.Npad + n0 + n) * Kp + st_c + 8 * half : p.w;
             cp_async16(&sB[slot][n][8 * half], src, in ? 16 : 0);
         }
-        if ((st_c += 16) >= 16 * kch) { st_c = 0; st_t++; }
+        if ((st_c += 16) >= Kp) { st_c = 0; st_t++; }
         slot = slot + 1 == IG_ST ? 0 : slot + 1;
     };
 
