@@ -34,6 +34,16 @@ int64_t gnb_test_fail_alloc(gnb_ctx *ctx, int64_t after);
  * returns GNB_ETIMEOUT.  -1 puts this off.  Errors: GNB_EINVAL. */
 int gnb_test_sort_give_up(gnb_ctx *ctx, int pass);
 
+/* The tile plan of the network's tensor-core 3^3 forward convolutions: number
+ * `plan` of each layer's list of supported plans instead of the rule's (or the
+ * autotuner's) choice, where the list is that long; -1 gives the choice back
+ * to the rule.  Returns the longest list's length, or GNB_EINVAL. */
+int gnb_unet_test_set_plan(gnb_unet *net, int plan);
+
+/* y[i] = 10^x[i] as the remap forms its voxel weights (host arrays of n
+ * doubles).  Errors: GNB_EINVAL, GNB_ENOMEM, GNB_ECUDA. */
+int gnb_test_exp10(int64_t n, const double *x, double *y);
+
 #ifdef __cplusplus
 }
 #endif

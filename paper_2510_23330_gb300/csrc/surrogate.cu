@@ -24,6 +24,7 @@
 #include <cmath>
 
 #include "common.cuh"
+#include "../../include/galnb_testing.h"
 
 typedef __nv_bfloat16 bf16;
 
@@ -291,6 +292,16 @@ __global__ void __launch_bounds__(256) k_remap_weights(const float *__restrict__
     __syncthreads();
     const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (v < nv) w[v] = exp10_table((double)pred[v * cout] - 0.33, t);
+}
+
+__global__ void __launch_bounds__(256) k_exp10(const double *__restrict__ x, long long n,
+                                               __grid_constant__ const Exp2Table table, double *__restrict__ y)
+{
+    __shared__ double t[128];
+    if (threadIdx.x < 128) t[threadIdx.x] = table.t[threadIdx.x];
+    __syncthreads();
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) y[i] = exp10_table(x[i], t);
 }
 
 static const Exp2Table &exp2_table()
@@ -944,3 +955,20 @@ int sn_surrogate_batch(gnb_ctx *c, gnb_unet *net, int nreg, const double *center
 }
 
 }  // namespace gnb
+
+// (the remap's voxel weights by themselves, for the tests of their 10^x)
+extern "C" int gnb_test_exp10(int64_t n, const double *x, double *y)
+{
+    if (n < 1 || n > (1 << 28) || !x || !y) return GNB_EINVAL;
+    double *d = nullptr;
+    if (cudaMalloc((void **)&d, 16 * (size_t)n) != cudaSuccess) {
+        cudaGetLastError();
+        return GNB_ENOMEM;
+    }
+    cudaMemcpy(d, x, 8 * (size_t)n, cudaMemcpyHostToDevice);
+    gnb::counted(gnb::k_exp10)<<<(unsigned)((n + 255) / 256), 256>>>(d, (long long)n, gnb::exp2_table(), d + n);
+    const bool ok = cudaMemcpy(y, d + n, 8 * (size_t)n, cudaMemcpyDeviceToHost) == cudaSuccess &&
+                    cudaGetLastError() == cudaSuccess;
+    cudaFree(d);
+    return ok ? GNB_OK : GNB_ECUDA;
+}

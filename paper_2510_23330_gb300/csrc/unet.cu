@@ -1343,6 +1343,20 @@ int gnb_unet_test_wait_timeout(gnb_unet *u)
     return unet_check(u, rc);
 }
 
+int gnb_unet_test_set_plan(gnb_unet *u, int plan)
+{
+    if (!u || plan < -1) return GNB_EINVAL;
+    int most = 0;
+    for (auto &l : u->L) {
+        if (l.kind != L_CONV3) continue;
+        TcPlan plans[TC_MAX_PLANS];
+        // (the coarsest grid's list is the shortest, the finest's the longest)
+        most = std::max(most, conv3_tc_plans(l.Npad, l.Kpad, u->grid, plans, TC_MAX_PLANS));
+        l.plan_f = plan;
+    }
+    return most;
+}
+
 int gnb_unet_set_conv_impl(gnb_unet *u, int impl)
 {
     if (!u || (impl != GNB_CONV_AUTO && impl != GNB_CONV_MMA_SYNC)) return GNB_EINVAL;

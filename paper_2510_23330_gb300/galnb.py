@@ -151,6 +151,10 @@ def _declare(L):
     L.gnb_test_fail_alloc.restype = C.c_int64
     L.gnb_test_sort_give_up.argtypes = [_vp, C.c_int]
     L.gnb_test_sort_give_up.restype = C.c_int
+    L.gnb_unet_test_set_plan.argtypes = [_vp, C.c_int]
+    L.gnb_unet_test_set_plan.restype = C.c_int
+    L.gnb_test_exp10.argtypes = [C.c_int64, C.POINTER(C.c_double), C.POINTER(C.c_double)]
+    L.gnb_test_exp10.restype = C.c_int
     for name in ("gnb_save", "gnb_load", "gnb_unet_save", "gnb_unet_load"):
         getattr(L, name).argtypes = [_vp, C.c_char_p]
         getattr(L, name).restype = C.c_int
@@ -299,6 +303,14 @@ def gnb_test_fail_alloc(h, after):
 
 def gnb_test_sort_give_up(h, pass_):
     return lib().gnb_test_sort_give_up(h, pass_)
+
+
+def gnb_unet_test_set_plan(net, plan):
+    return lib().gnb_unet_test_set_plan(net, plan)
+
+
+def gnb_test_exp10(n, x, y):
+    return lib().gnb_test_exp10(n, x, y)
 
 
 def gnb_unet_get_params(net, dst, on_device):

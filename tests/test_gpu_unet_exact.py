@@ -81,3 +81,38 @@ def test_training_step_is_exact(G, grid, B, base, levels):
             got = g[at : at + ref[k].size].reshape(ref[k].shape)
             at += ref[k].size
             assert np.array_equal(got, ref[k]), (k, np.argwhere(got != ref[k])[:4], np.max(np.abs(got - ref[k])))
+
+
+# every tile plan of every layer's list, forced, with ragged tiles in x, y and z
+@pytest.mark.parametrize("grid,B,base,levels", [(40, 2, 16, 4), (20, 3, 32, 3), (24, 1, 24, 3)])
+def test_forward_is_exact_under_every_plan(G, grid, B, base, levels):
+    p, x = _params(base + grid, base, levels), _input(grid, B, grid)
+    y, _ = U.forward(p, x, levels=levels, bf=True)
+    net = _net(G, p, base, levels, grid)
+    most = G.gnb_unet_test_set_plan(net.h, -1)
+    assert 3 <= most <= 24
+    for plan in range(-1, most):
+        assert G.gnb_unet_test_set_plan(net.h, plan) == most
+        assert np.array_equal(net.forward(x.astype(np.float32)), y), plan
+
+
+# 10^x of the remap's weights against 113-bit arithmetic: the table's entry and
+# the last multiply-add round once each (2^-53 of the result), the reduction and
+# the polynomial add less than a twentieth of that; outside +-290 the library's
+def test_remap_exp10(G):
+    import ctypes as C
+    if np.finfo(np.longdouble).nmant < 100:
+        pytest.skip("long double is not quadruple precision here")
+    rng = np.random.default_rng(0)
+    x = np.concatenate([rng.uniform(-40.0, 40.0, 60000), rng.uniform(-289.9, 289.9, 30000), np.arange(-280.0, 281.0),
+                        rng.normal(size=5000) * 1e-6, np.log10(2.0) / 256.0 * np.arange(-3001.0, 3002.0, 2.0)])
+    sp = np.array([0.0, 400.0, -400.0, np.inf, -np.inf, np.nan, 308.0, -320.0])
+    v = np.ascontiguousarray(np.concatenate([x, sp]))
+    y = np.empty_like(v)
+    ptr = C.POINTER(C.c_double)
+    assert G.gnb_test_exp10(v.size, v.ctypes.data_as(ptr), y.ctypes.data_as(ptr)) == G.GNB_OK
+    ref = np.power(np.longdouble(10.0), x.astype(np.longdouble))
+    assert np.max(np.abs(y[: x.size].astype(np.longdouble) / ref - 1)) < 2.1 * 2.0**-53
+    s = y[x.size :]
+    assert s[0] == 1.0 and s[1] == np.inf and s[2] == 0.0 and s[3] == np.inf and s[4] == 0.0 and np.isnan(s[5])
+    assert abs(s[6] / 1e308 - 1.0) < 1e-15 and 0.0 < s[7] < 1.1e-320
