@@ -197,6 +197,7 @@ struct gnb_ctx {
     int64_t sn_n = 0;
     int sn_cur = -1;
     uint64_t sn_gen = 0;          // sur_gen when the graph was captured
+    uint64_t sn_net_gen = 0;      // and the network's generation (its buffers are in the graph too)
     int64_t sn_graph_replays = 0;
 
     // status / counters

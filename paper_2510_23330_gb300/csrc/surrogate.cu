@@ -31,6 +31,7 @@ typedef __nv_bfloat16 bf16;
 namespace gnb {
 
 int unet_prepare(gnb_unet *u, int batch, bf16 **xin, float **yout, int *grid, int *cout);
+uint64_t unet_generation(const gnb_unet *u);
 int unet_run(gnb_unet *u, int batch, cudaStream_t stream, const bf16 *xin, float *yout);
 
 #define SUR_T_PER_U 48.45894937815476  // (gamma - 1) mu m_H / k_B, K per (km/s)^2, mu = 0.6
@@ -889,7 +890,7 @@ int sn_surrogate_batch(gnb_ctx *c, gnb_unet *net, int nreg, const double *center
     bool same = c->sn_graph && c->sn_key[0] == nreg && c->sn_key[1] == grid && c->sn_key[2] == sweeps &&
                 c->sn_key[3] == nch &&
                 c->sn_net == (void *)net && c->sn_side == side && c->sn_n == c->n && c->sn_cur == c->cur &&
-                c->sn_gen == c->sur_gen;
+                c->sn_gen == c->sur_gen && c->sn_net_gen == unet_generation(net);
     if (use_graph && same) {
         c->sn_graph_replays++;
         return cuda_check(c, cudaGraphLaunch(c->sn_graph, c->s), "surrogate graph launch");
@@ -951,6 +952,7 @@ int sn_surrogate_batch(gnb_ctx *c, gnb_unet *net, int nreg, const double *center
     GNB_TRY(cuda_check(c, e, "graph instantiate"));
     c->sn_key[0] = nreg; c->sn_key[1] = grid; c->sn_key[2] = sweeps; c->sn_key[3] = nch;
     c->sn_net = net; c->sn_side = side; c->sn_n = c->n; c->sn_cur = c->cur; c->sn_gen = c->sur_gen;
+    c->sn_net_gen = unet_generation(net);
     return cuda_check(c, cudaGraphLaunch(c->sn_graph, c->s), "surrogate graph launch");
 }
 

@@ -22,6 +22,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -767,13 +768,23 @@ struct gnb_unet {
     bool launch_failed = false;
     bool tuning = false;         // forward passes time every tile plan of each 3^3 layer (gnb_unet_autotune)
     int tuned_layers = 0;
+    uint64_t gen = 0;            // of the buffers and kernels a captured forward pass has in it (unet_generation)
     std::string err;
 };
 
 namespace {
 
+// A number that no network has had before: of a new network, of new activation
+// buffers or of another choice of kernels.
+void new_generation(gnb_unet *u)
+{
+    static std::atomic<uint64_t> last{0};
+    u->gen = ++last;
+}
+
 void unet_free_acts(gnb_unet *u)
 {
+    new_generation(u);
     for (auto *a : u->act) if (a) cudaFree(a);
     for (auto *a : u->pidx) if (a) cudaFree(a);
     for (auto *a : u->tmp) if (a) cudaFree(a);
@@ -1217,6 +1228,8 @@ int unet_prepare(gnb_unet *u, int batch, bf16 **xin, float **yout, int *grid, in
     return GNB_OK;
 }
 
+uint64_t unet_generation(const gnb_unet *u) { return u->gen; }
+
 int unet_poll_error(gnb_unet *u)
 {
     int e = 0;
@@ -1249,6 +1262,7 @@ int gnb_unet_create(gnb_unet **out, int cin, int cout, int base, int levels, int
     if (!u) return GNB_ENOMEM;
     u->cin = cin; u->cout = cout; u->base = base; u->levels = levels; u->grid = grid;
     u->s = (cudaStream_t)stream;
+    new_generation(u);
     // layers in the order of the flat parameter array
     auto add = [&](int kind, int ci, int co) {
         ULayer l;
@@ -1354,6 +1368,7 @@ int gnb_unet_test_set_plan(gnb_unet *u, int plan)
         most = std::max(most, conv3_tc_plans(l.Npad, l.Kpad, u->grid, plans, TC_MAX_PLANS));
         l.plan_f = plan;
     }
+    new_generation(u);
     return most;
 }
 
@@ -1361,6 +1376,7 @@ int gnb_unet_set_conv_impl(gnb_unet *u, int impl)
 {
     if (!u || (impl != GNB_CONV_AUTO && impl != GNB_CONV_MMA_SYNC)) return GNB_EINVAL;
     u->conv_impl = impl;
+    new_generation(u);
     return GNB_OK;
 }
 
@@ -1467,6 +1483,7 @@ int gnb_unet_autotune(gnb_unet *u, int batch, double out_ms[2])
     if (rc == GNB_OK) rc = timed(&after);
     if (rc == GNB_OK && after > before)  // the timings of single layers did not add up: keep the rule
         for (auto &ly : u->L) ly.plan_f = -1;
+    new_generation(u);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (out_ms) {

@@ -283,3 +283,35 @@ def test_scratch_of_the_sort_comes_with_the_particles(G, n):
     assert big - G.gnb_test_fail_alloc(c.h, -1) == 12
     key = c.get("KEY")
     assert np.array_equal(c.get("ORDER"), np.lexsort((np.arange(n), key)))
+
+
+@pytest.mark.parametrize("change", ["kernels", "buffers"])
+def test_captured_batch_follows_the_network(G, change):
+    """The graph of a surrogate batch holds the network's buffers and kernels:
+    after another choice of kernels, or a larger batch that moved the buffers,
+    the next call captures again instead of replaying what is no longer there."""
+    import torch
+    from paper_2510_23330_gb300 import surrogate
+    stream = torch.cuda.Stream()
+    p, cen = ics.sn_region(3000, seed=5, grid=16), [(0.0, 0.0, 0.0)]
+    with torch.cuda.stream(stream):
+        net = G.UNet(5, 5, 16, 2, 8, stream=stream.cuda_stream)
+        net.set_params(surrogate.he_init(5, 5, 16, 2, seed=1))
+        c = G.Context(stream=stream.cuda_stream)
+        out, launches = [], []
+        for step in range(3):
+            if step == 2 and change == "kernels":
+                net.set_conv_impl(G.GNB_CONV_MMA_SYNC)
+            elif step == 2:
+                net.forward(np.zeros((40, 8, 8, 8, 5), np.float32))
+            c.set_particles(p)
+            c.compute_sph_density()
+            before = c.phase_times()[2]
+            c.sn_surrogate_batch(net, cen, seed=3, sweeps=0, use_graph=True)
+            launches.append(c.phase_times()[2] - before)
+            out.append({k: c.get(k).astype(np.float64) for k in ("X", "U")})
+        stream.synchronize()
+    assert launches[0] > 10 and launches[1] == 0 and launches[2] > 10
+    for o in out[1:]:
+        assert np.array_equal(o["X"], out[0]["X"])  # no sweeps: positions do not depend on the prediction
+        assert np.all(np.abs(np.log10(o["U"] / out[0]["U"])) < 0.3)
