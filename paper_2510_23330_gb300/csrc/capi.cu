@@ -255,8 +255,16 @@ __global__ void __launch_bounds__(1024) k_load_scan(int *__restrict__ partial, i
 // can read it.  What does not (host or managed memory, another device's, an
 // array shorter than the count asks for) goes through a copy, which reaches
 // what the device cannot read in place and refuses what is not there.
-static bool readable_in_place(const void *p, size_t bytes)
+// [lo, hi): the allocation found last, which several arrays may share (a
+// pointer's attributes and range take about half a microsecond).
+struct DeviceRange {
+    uintptr_t lo = 0, hi = 0;
+};
+
+static bool readable_in_place(DeviceRange &r, const void *p, size_t bytes)
 {
+    const uintptr_t at = (uintptr_t)p;
+    if (at >= r.lo && at < r.hi) return bytes <= r.hi - at;
     typedef CUresult (*range_fn)(CUdeviceptr *, size_t *, CUdeviceptr);
     static const range_fn range = []() -> range_fn {
         void *f = nullptr;
@@ -276,8 +284,11 @@ static bool readable_in_place(const void *p, size_t bytes)
     }
     CUdeviceptr base = 0;
     size_t size = 0;
-    return a.type == cudaMemoryTypeDevice && a.device == dev &&
-           range(&base, &size, (CUdeviceptr)(uintptr_t)p) == CUDA_SUCCESS && (uintptr_t)p + bytes <= base + size;
+    if (a.type != cudaMemoryTypeDevice || a.device != dev || range(&base, &size, (CUdeviceptr)at) != CUDA_SUCCESS)
+        return false;
+    r.lo = (uintptr_t)base;
+    r.hi = r.lo + size;
+    return bytes <= r.hi - at;
 }
 
 // Rank of every gas particle among the gas, in the caller's order.
@@ -447,7 +458,8 @@ int gnb_set_particles(gnb_ctx *c, int64_t n, const int64_t *id, const uint8_t *t
     // device arrays are read in place (copied first if one is not aligned to its elements
     // or not all there)
     bool copy = !on_device;
-    for (auto &q : cp) copy = copy || (uintptr_t)q.s % q.b != 0 || !readable_in_place(q.s, q.b * N);
+    DeviceRange range;
+    for (auto &q : cp) copy = copy || (uintptr_t)q.s % q.b != 0 || !readable_in_place(range, q.s, q.b * N);
     if (copy) {
         const cudaMemcpyKind k = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
         for (auto &q : cp) GNB_TRY(cuda_check(c, cudaMemcpyAsync(q.d, q.s, q.b * N, k, c->s), "particle copy"));
