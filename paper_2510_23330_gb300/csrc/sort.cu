@@ -206,12 +206,13 @@ __global__ void k_tie_fix(uint64_t *__restrict__ k, int n, int *__restrict__ val
 #define RS_AGG (1u << 30)     // the tile's own count of the digit
 #define RS_PRE (2u << 30)     // the count of the digit in this tile and all before it
 #define RS_SPINS (1 << 20)    // look-back reads without progress before giving up
+#define RS_DEAD (1 << 30)     // in a pass's ticket counter: an earlier pass gave up
 
 struct RsState {
     int *hist;        // [8][256] digit histograms
     int *ticket;      // [8] tiles started per pass
     unsigned *state;  // [passes][ntiles][256] published counts
-    int *flag;        // bit p set when a look-back of pass p gave up
+    int *flag;        // set when a look-back gave up
 };
 
 template <int ITEMS>
@@ -269,13 +270,12 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_rs_pass(const uint64_t *__res
 #pragma unroll
     for (int q = 0; q < RS_THREADS / 32; q++) S.wc[q][t] = 0;
     const int hd = hist[t];
+    __syncthreads();
+    const int tile = S.tile;
     // an earlier pass that gave up left places unwritten: its output no longer
     // has the digits that were counted, and their positions could lie beyond
-    // the arrays (the earlier passes' bits are final: every thread sees the same)
-    const unsigned gave_up = *(volatile int *)flag & ((1u << (shift >> 3)) - 1u);
-    __syncthreads();
-    if (gave_up) return;
-    const int tile = S.tile;
+    // the arrays
+    if (tile >= RS_DEAD) return;
     const int base = tile * TILE;
     const int cnt = min(TILE, n - base);
     uint64_t key[ITEMS];
@@ -373,7 +373,8 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_rs_pass(const uint64_t *__res
         if (moved) spins = 0;
         else if (++spins > RS_SPINS) {  // cannot happen unless a block was lost
             S.stop = 1;
-            atomicOr(flag, 1 << (shift >> 3));
+            atomicOr(flag, 1);
+            for (int q = (shift >> 3) + 1; q < 8; q++) atomicOr(ticket + q - (shift >> 3), RS_DEAD);
             break;
         }
     }
@@ -446,9 +447,11 @@ static int rs_begin(gnb_ctx *c, int n, RsState *st)
     st->state = (unsigned *)(c->rs_buf + 8 * 256 + 16);
     GNB_TRY(cuda_check(c, cudaMemsetAsync(c->rs_buf, 0, words * sizeof(int), c->s), "radix sort scratch"));
     if (c->sort_gives_up >= 0) {  // (set by tests)
-        const int bit = 1 << c->sort_gives_up;
+        const int later = c->sort_gives_up + 1;
         c->sort_gives_up = -1;
-        return cuda_check(c, cudaMemsetAsync(st->flag, bit, 1, c->s), "radix sort flag");
+        GNB_TRY(cuda_check(c, cudaMemsetAsync(st->flag, 1, 1, c->s), "radix sort flag"));
+        GNB_TRY(cuda_check(c, cudaMemsetAsync(st->ticket + later, RS_DEAD >> 24, (8 - later) * sizeof(int), c->s),
+                           "radix sort flag"));
     }
     return GNB_OK;
 }
