@@ -793,9 +793,10 @@ __device__ __forceinline__ void eval_chunk(GravSmem &S, const GravParams &p, int
 // the group's particles in chunks of up to NIMAX * GW_THREADS, eight per
 // thread above 128 particles in a chunk (NIMAX = 8), four above 32, two above
 // 8, else one (walk + evaluation with limits of 64 and 16 against 32 and 8:
-// 2^20 disk, n_g = 128, 2643 -> 2592 us; 300,007 stars, n_g = 64, 1368 -> 1326).  Five CTAs per SM (96 registers a thread; the eight-particle
-// variant spills a few bytes outside its inner loops and still runs faster
-// than at 4 CTAs and 128 registers).
+// 2^20 disk, n_g = 128, 2643 -> 2592 us; 300,007 stars, n_g = 64, 1368 -> 1326).
+// Five CTAs per SM (96 registers a thread; the eight-particle variant spills a
+// few bytes outside its inner loops and still runs faster than at 4 CTAs and
+// 128 registers).
 template <bool MASK, bool QUAD, int NIMAX, bool UNI>
 __global__ void __launch_bounds__(GW_THREADS, 5) k_grav_eval(GravParams p)
 {
@@ -1022,7 +1023,7 @@ static GravParams make_params(gnb_ctx *c)
     p.e2u = c->eps_uniform ? 2.f * (c->eps0 * c->eps0) : 0.f;
     p.quad = c->cfg.multipole;
     p.n = (int)c->n;
-    p.next = c->pinned_i ? nullptr : nullptr;
+    p.next = nullptr;  // set by each launch
     p.status = c->status_d;
     p.counters = c->counters_d;
     return p;

@@ -189,10 +189,13 @@ __global__ void k_tie_fix(uint64_t *__restrict__ k, int n, int *__restrict__ val
 // ---------------------------------------------------------------- radix sort
 // Stable LSD radix sort of (64-bit key, 32-bit value), 8 bits per pass, one
 // kernel per pass: the digit histograms of all passes are counted once, up
-// front (they do not depend on the order; the Morton keys' with the keys), and a tile finds where its run of
-// each digit starts from the counts that the tiles before it publish
-// (decoupled look-back).  A tile takes its number from a ticket counter, so
-// every tile it waits for is already running.
+// front (they do not depend on the order; those of the Morton keys come with
+// the keys), and a tile finds where its run of each digit starts from the
+// counts that the tiles before it publish.  The scheme is the single-pass scan
+// with decoupled look-back of Merrill and Garland (NVIDIA technical report
+// NVR-2016-002), applied to every digit as in the one-sweep radix sort of
+// Adinets and Merrill (arXiv 2206.01784).  A tile takes its number from a
+// ticket counter, so every tile it waits for is already running.
 //
 // A tile's pairs are first sorted by digit in shared memory, stably, then
 // written out in that order, so consecutive threads write consecutive

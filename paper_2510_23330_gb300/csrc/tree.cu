@@ -686,8 +686,9 @@ __global__ void __launch_bounds__(TB_THREADS) k_moments_inner(Tree t, int b, int
 // to every block of the cluster) between them.  A level of at most MC_NODES
 // nodes costs a few dependent reads either way; in a launch of its own it
 // costs a launch on top: inner nodes 45 -> 28 us (cold cache) for 8,192
-// particles (10 levels), 60 -> 49 us for the 2^20 disk (12 levels).  Above MC_NODES the cluster's 1,024 four-lane groups need several
-// rounds and a level is better off with the whole chip.
+// particles (10 levels), 60 -> 49 us for the 2^20 disk (12 levels).  Above
+// MC_NODES the cluster's 1,024 four-lane groups need several rounds and a level
+// is better off with the whole chip.
 #define MC_CTAS 8
 #define MC_THREADS 512
 #define MC_NODES 2048

@@ -370,11 +370,11 @@ __global__ void __launch_bounds__(HEAD_T) k_head(const bf16 *__restrict__ in, in
                                                  float *__restrict__ out)
 {
     // a block's voxels lie in one batch entry, given by the grid (a 64-bit
-    // division a thread costs more than the products); weights [k][n]: one input channel's are read together (16 bytes at a
-    // time instead of 128 single reads a voxel: 144 -> 122 us for 32 regions
-    // of 64^3, 65 at the copy rate).  Eight voxels per thread pay once for
-    // staging the weights, and the next voxel's loads are under way while one is
-    // summed (124 -> 93 us).
+    // division a thread costs more than the products); weights [k][n]: one
+    // input channel's are read together (16 bytes at a time instead of 128
+    // single reads a voxel: 144 -> 122 us for 32 regions of 64^3, 65 at the copy
+    // rate).  Eight voxels per thread pay once for staging the weights, and the
+    // next voxel's loads are under way while one is summed (124 -> 93 us).
     constexpr int NP = (NO + 3) / 4 * 4;
     __shared__ __align__(16) float sw[32][NP], sbias[NP];
     __shared__ __align__(16) float so[2][HEAD_T * NO];
