@@ -801,10 +801,12 @@ __global__ void __launch_bounds__(128) k_up2_tc(const Up2Args p)
 // One elected lane issues four K = 16 MMAs per stage into a TMEM accumulator;
 // three stage buffers, two stages of copies in flight.  At the end each warp
 // reads its 32 TMEM lanes (rows) and adds them to dW with FP32 vector
-// reductions (the voxel chunks are split-K).  It is bound by the copies
-// through L1/L2 (27 shifted reads of the input).  All 14 layers of a 64^3
-// training step (cold cache): 1,824 us with 2-byte transposing stores and 64-bit
-// divisions per piece, 505 us so.
+// reductions (the voxel chunks are split-K).  It is bound by the instructions
+// that address the copies (27 shifted 16-byte pieces per voxel and channel
+// group, each with its bounds test: 56 % issue-active on a 16-channel 64^3
+// layer, where L1 is at 15 %, L2 at 22 and the tensor pipe at 2.5).  All 14
+// layers of a 64^3 training step (cold cache): 1,824 us with 2-byte transposing
+// stores and 64-bit divisions per piece, 505 us so.
 struct WgTcArgs {
     const bf16 *x1, *x2;   // input channels [0, C1) from x1, [C1, C) from x2; blocked [B][C/8][V][8]
     int C1, C;
