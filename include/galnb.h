@@ -213,7 +213,10 @@ int gnb_compute_sph_density(gnb_ctx *ctx);
 /* SPH pressure force, artificial viscosity and du/dt over the symmetric
  * neighbour sets (Table 3 "hydro force").  Adds the hydro acceleration to
  * the total acceleration.  Requires gnb_compute_sph_density since the last
- * change of positions.  Errors: GNB_ESTATE, GNB_ECUDA. */
+ * change of positions.  A state from gnb_load holds no neighbour lists: this
+ * call, gnb_cfl_timestep and the first step of gnb_integrate_cfl and
+ * gnb_integrate_hier (also after gnb_set_state) evaluate its forces first.
+ * Errors: GNB_ESTATE, GNB_ECUDA. */
 int gnb_compute_sph_force(gnb_ctx *ctx);
 
 /* Total force evaluation: sort and tree build, gravity (mode), NFW, SPH
